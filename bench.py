@@ -102,6 +102,8 @@ def solve_layout(r):
     if r["shape"] in (2, 3, 4):
         return {"fused": {2: "register", 3: "lean", 4: "lean, two-warp CTAs"}[r["shape"]],
                 "tile": r["slots"] % 256, "pole_groups": r["slots"] // 256, "layout_shape": r["shape"]}
+    if r["shape"] == 5:
+        return {"digits": "contractions on the tensor cores", "pole_slots": r["slots"], "layout_shape": 5}
     return {"pole_slots": r["slots"], "layout_shape": r["shape"]}
 
 

@@ -124,8 +124,10 @@ typedef struct {
   int32_t pole_slots;   /* 0: the default solve -- for batches of up to four states with
                            binary64 solves of the delta solver on the rotating sphere, the
                            fused solve that keeps the pole sum on chip (one kernel, every
-                           output written once), else the pole-slot solve (rexi_tune picks
-                           per batch); > 0: the pole-slot solve with this many pole groups
+                           output written once), for larger ones the digit solve (the
+                           contractions exactly on the tensor cores; needs device memory
+                           for 292 B per row and pole and poles of like scale), else the
+                           pole-slot solve (rexi_tune picks per batch); > 0: the pole-slot solve with this many pole groups
                            summed separately, then reduced in slot order (a deterministic
                            tuning knob, any >= 1) */
   const double *alpha;  /* optional: P complex poles (re, im interleaved); NULL -> computed */
@@ -265,7 +267,8 @@ rexi_status rexi_get_coefficients(const rexi_plan *plan, double *alpha, double *
  * 1 for batches of 1 and 2) and, for batches up to 8, with each tile's poles split over
  * 1, 2, 3, 4, 6 or 8 CTAs, and shapes 3 and 4: its lean forms (see rexi_set_pole_slots).
  * Keeps the fastest for later steps with this batch (the fused solve unless a slot layout
- * is more than 0.5 % faster: it needs no reduction) and writes its slot count (for shapes
+ * is more than 0.5 % faster: it needs no reduction) or, if faster still and available, the
+ * digit solve (shape 5), and writes its slot count (for shapes
  * 2 to 4: tile + 256 x pole groups, as rexi_set_pole_slots takes it) to *slots and its
  * shape to *shape (either may be NULL).  Synchronous; uses the plan's workspaces, so no
  * step of this plan may be in flight. */
@@ -280,7 +283,10 @@ rexi_status rexi_tune(rexi_plan *plan, int32_t batch, int32_t *slots, int32_t *s
  * split over `groups` CTAs in whole passes of the CTA's pole lanes (0: the default, more
  * than one only when a batch is too small to fill the GPU; a request is capped at the
  * passes), the last CTA of a tile to finish adding the groups' partial sums in group
- * order, or shape 3 for its lean form (three or four CTAs of four warps per SM, fewer
+ * order, or shape 5 for the digit solve (binary64 delta solver on the rotating sphere, plans
+ * with max_batch >= 5: the right-hand sides and the pole sums as exact fixed-point products
+ * on the tensor cores; slots: the items each system's poles are split over, 0: the default;
+ * the default solve above four states), or shape 3 for its lean form (three or four CTAs of four warps per SM, fewer
  * registers, the next rows prefetched into the caches; tiles of up to 8 states), or shape
  * 4 for the lean form on CTAs of two warps (seven or eight per SM; tiles of up to 4
  * states; a tile of 2 states puts each state on a warp of its own, so no CTA splits its

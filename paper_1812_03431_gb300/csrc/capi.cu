@@ -24,6 +24,7 @@ rexi_status step_static(Plan &pl, const void *in, void *out, int B, cudaStream_t
 rexi_status tune_layout(Plan &pl, int B, int *slots_out, int *shape_out);
 rexi_status set_layout(Plan &pl, int B, int slots, int shape, int *used);
 const FusedLayout *fused_layout(Plan &pl, int B);
+const DigitLayout *digit_layout(Plan &pl, int B, bool adjoint);
 
 namespace {
 
@@ -102,7 +103,15 @@ rexi_status check_io2(const Plan &pl, const void *in, const void *out, int B, bo
 }
 
 rexi_status ensure_adjoint_factors(Plan &pl) {
-  if (pl.fac_adj || pl.prm.fsphere) return REXI_OK;
+  if (pl.fac_adj || pl.prm.fsphere) {
+    if (pl.fac_adj && pl.dig_fwd.fwd && !pl.dig_adj_tried) {
+      pl.dig_adj_tried = true;
+      cudaError_t e = build_digit_factors(pl, pl.fac_adj, pl.dig_adj);
+      if (e != cudaSuccess) return cuda_fail("adjoint digit factors", e);
+      if (pl.dig_adj.fwd) pl.bytes += digit_factor_bytes(pl);
+    }
+    return REXI_OK;
+  }
   const size_t n = (size_t)fac_ncomp(pl) * pl.nrows * pl.P;
   cudaError_t e = cudaMalloc(&pl.fac_adj, n * sizeof(double2));
   if (e != cudaSuccess) {
@@ -123,7 +132,7 @@ rexi_status ensure_adjoint_factors(Plan &pl) {
       return r;
     }
   }
-  return REXI_OK;
+  return ensure_adjoint_factors(pl);  // then the same factors as digits
 }
 
 // Spectral REXI core on the plan's internal layout: s_in -> s_out.
@@ -132,6 +141,14 @@ rexi_status core(Plan &pl, int B, bool adjoint, cudaStream_t st, Marks &mk) {
     mk.mark(ST_SOLVE);
     cudaError_t e = launch_fsphere(pl, adjoint, pl.s_in, pl.s_out, B, false, 0, st);
     return e == cudaSuccess ? REXI_OK : cuda_fail("f-sphere solve", e);
+  }
+  if (const DigitLayout *dl = digit_layout(pl, B, adjoint)) {  // both contractions on the tensor cores
+    mk.mark(ST_SOLVE);
+    cudaError_t e = launch_solve_digits(pl, *dl, adjoint, pl.s_in, B, st);
+    if (e != cudaSuccess) return cuda_fail("digit solve", e);
+    mk.mark(ST_REDUCE);
+    e = launch_finish_digits(pl, *dl, adjoint, pl.s_in, pl.s_out, B, st);
+    return e == cudaSuccess ? REXI_OK : cuda_fail("digit sums", e);
   }
   SolveLayout *lay = nullptr;
   rexi_status r = get_layout(pl, B, false, &lay);
@@ -477,14 +494,14 @@ rexi_status rexi_tune(rexi_plan *plan, int32_t batch, int32_t *slots, int32_t *s
 rexi_status rexi_set_pole_slots(rexi_plan *plan, int32_t batch, int32_t slots, int32_t shape, int32_t *used) {
   if (!plan || !plan->pl) { set_error("null plan"); return REXI_EINVAL; }
   Plan &pl = *plan->pl;
-  if (batch < 1 || batch > pl.prm.max_batch || (shape < 2 && slots < 1) || slots < 0 || shape < 0 || shape > 4) {
-    set_error("rexi_set_pole_slots: batch must be in [1, max_batch], shape 0 to 4, slots >= 1 for "
-              "shapes 0 and 1 and >= 0 for shapes 2 to 4");
+  if (batch < 1 || batch > pl.prm.max_batch || (shape < 2 && slots < 1) || slots < 0 || shape < 0 || shape > 5) {
+    set_error("rexi_set_pole_slots: batch must be in [1, max_batch], shape 0 to 5, slots >= 1 for "
+              "shapes 0 and 1 and >= 0 for shapes 2 to 5");
     return REXI_EINVAL;
   }
   if (pl.prm.fsphere) {  // no banded solves, no layout
     if (shape >= 2) {
-      set_error("rexi_set_pole_slots: the fused solve (shapes 2 to 4) does not apply to f-sphere plans");
+      set_error("rexi_set_pole_slots: the fused solve (shapes 2 to 5) does not apply to f-sphere plans");
       return REXI_EINVAL;
     }
     if (used) *used = 0;

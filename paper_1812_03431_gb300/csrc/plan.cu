@@ -101,6 +101,13 @@ __global__ void alp_tables_kernel(const double *mu_all, int N, int J, double *ta
 
 void free_plan(Plan *pl);
 
+// The smallest batch the digit solve takes by default: its warps carry tiles of eight states;
+// five of them still take a third of the pole-slot solve's time (T85: 0.20 / 0.62 ms); up to
+// four the fused solve is the default.  Then the most device memory its factors may take: 2336 B per
+// row and eight poles, twice the binary64 factors.
+constexpr int kDigitMinBatch = 5;
+constexpr size_t kDigitMostBytes = (size_t)32 << 30;
+
 rexi_status build_plan(const rexi_params &prm, Plan *pl) {
   pl->prm = prm;
   pl->ff = prm.solve_arith == REXI_SOLVE_FP32X2;
@@ -333,6 +340,22 @@ rexi_status build_plan(const rexi_params &prm, Plan *pl) {
     }
   }
 
+  // the digit solve's factors, for plans that step batches it serves by default
+  if (pl->fac_fwd && !pl->ff && prm.solver == REXI_SOLVER_DELTA && prm.max_batch >= kDigitMinBatch) {
+    size_t mem_free = 0, mem_total = 0;
+    if ((e = cudaMemGetInfo(&mem_free, &mem_total))) return fail("memory", e);
+    const size_t need = digit_factor_bytes(*pl) + digit_state_bytes(*pl, prm.max_batch);
+    if (need <= std::min(kDigitMostBytes, mem_free / 3)) {
+      if ((e = build_digit_factors(*pl, pl->fac_fwd, pl->dig_fwd))) return fail("digit factors", e);
+      if (pl->dig_fwd.fwd && cudaMalloc(&pl->dig_state, digit_state_bytes(*pl, prm.max_batch)) != cudaSuccess) {
+        cudaGetLastError();
+        pl->dig_state = nullptr;
+        free_digit_factors(pl->dig_fwd);
+      }
+      if (pl->dig_fwd.fwd) bytes += need;
+    }
+  }
+
   // ---- grid, Legendre tables, FFT
   {  // tables serve the grid layout and rexi_analyze / rexi_synthesize
     std::vector<double> mu, w;
@@ -419,7 +442,9 @@ rexi_status build_plan(const rexi_params &prm, Plan *pl) {
   int cap = (int)std::min<size_t>(1024, std::max<size_t>(1, (size_t)(4ull << 30) / per_slot));
   cap = std::min(cap, P);
   pl->partial_cap = (size_t)cap;
-  if ((e = dalloc(&pl->partial, (size_t)cap * 3 * NS * B, &bytes))) return fail("partials", e);
+  pl->partial_elems = (size_t)cap * 3 * NS * B;
+  if (pl->dig_fwd.fwd) pl->partial_elems = std::max(pl->partial_elems, digit_slot_bytes(*pl, B) / sizeof(double2));
+  if ((e = dalloc(&pl->partial, pl->partial_elems, &bytes))) return fail("partials", e);
   pl->resident_warps = pl->num_sms * 16;
   // forward-sweep intermediates: sweep_width poles per lane per row
   if ((e = dalloc(&pl->yscratch, (size_t)pl->resident_warps * pl->lmax * sweep_width(pl->ff) * 32, &bytes)))
@@ -565,6 +590,37 @@ const FusedLayout *fused_layout(Plan &pl, int B) {
   return it->second.st > 0 ? &it->second : nullptr;
 }
 
+// The digit solve's work list for steps of B states, or null where another kernel serves them:
+// no digit factors (see build_plan), an explicit pole_slots, another layout chosen for this
+// batch, or without a choice a batch below kDigitMinBatch.
+const DigitLayout *digit_layout(Plan &pl, int B, bool adjoint) {
+  if (!(adjoint ? pl.dig_adj : pl.dig_fwd).fwd) return nullptr;
+  auto ud = pl.use_digits.find(B);
+  if (ud != pl.use_digits.end() ? !ud->second : (pl.slots_override > 0 || B < kDigitMinBatch)) return nullptr;
+  auto it = pl.digits.find(B);
+  if (it == pl.digits.end()) {
+    DigitLayout L;
+    if (build_digit_layout(pl, B, 0, L) != REXI_OK) return nullptr;
+    it = pl.digits.emplace(B, L).first;
+  }
+  return it->second.items_dev ? &it->second : nullptr;
+}
+
+// the digit layout for batch B with a requested slot count (0: the default), replacing any
+// earlier one
+const DigitLayout *set_digit_slots(Plan &pl, int B, int slots) {
+  auto it = pl.digits.find(B);
+  if (it != pl.digits.end()) {
+    free_digit_layout(it->second);
+    pl.digits.erase(it);
+  }
+  if (!pl.dig_fwd.fwd) return nullptr;
+  DigitLayout L;
+  if (build_digit_layout(pl, B, slots, L) != REXI_OK) return nullptr;
+  it = pl.digits.emplace(B, L).first;
+  return it->second.items_dev ? &it->second : nullptr;
+}
+
 // the fused layout for batch B with a requested CTA tile and number of pole groups (0:
 // the defaults) and form (0: register; lean with CTAs of 1: four, 2: two warps),
 // replacing any earlier one
@@ -584,6 +640,16 @@ const FusedLayout *set_fused_tile(Plan &pl, int B, int tile, int form = 0, int g
 // earlier one for that batch.  Shapes 2, 3 and 4 select the fused solve instead (REXI_EINVAL
 // where it does not apply), with slots = tile + 256 x pole groups.
 rexi_status set_layout(Plan &pl, int B, int slots, int shape, int *used) {
+  if (shape == 5) {
+    const DigitLayout *D = set_digit_slots(pl, B, slots);
+    if (!D) {
+      set_error("rexi_set_pole_slots: the digit solve (shape 5) does not apply to this plan");
+      return REXI_EINVAL;
+    }
+    pl.use_digits[B] = true;
+    if (used) *used = D->slots;
+    return REXI_OK;
+  }
   if (shape >= 2 && shape <= 4) {
     pl.use_slots[B] = false;
     if (!set_fused_tile(pl, B, slots % 256, shape - 2, slots / 256)) {
@@ -592,6 +658,7 @@ rexi_status set_layout(Plan &pl, int B, int slots, int shape, int *used) {
                 "solver on the rotating sphere, with running sums that fit in shared memory");
       return REXI_EINVAL;
     }
+    pl.use_digits[B] = false;
     const FusedLayout *F = fused_layout(pl, B);
     if (used) *used = F->st + 256 * F->ng;
     return REXI_OK;
@@ -610,6 +677,7 @@ rexi_status set_layout(Plan &pl, int B, int slots, int shape, int *used) {
   }
   pl.layouts.emplace(B, L);
   pl.use_slots[B] = true;
+  pl.use_digits[B] = false;
   if (used) *used = L.slots;
   return REXI_OK;
 }
@@ -703,6 +771,29 @@ rexi_status tune_layout(Plan &pl, int B, int *slots_out, int *shape_out) {
     if (tile <= 2 && tile < B) break;  // smaller tiles only re-read the factors more often
   }
   if (best_tile > 0) set_fused_tile(pl, B, best_tile, best_form, best_groups);
+  // the digit solve with its finishing kernel, at the default slot count and around it
+  float digit_ms = 1e30f;
+  int digit_slots = 0;
+  if (const DigitLayout *D0 = set_digit_slots(pl, B, 0)) {
+    const int def = D0->slots;
+    for (int slots : {def, std::max(1, def / 2), 2 * def, 4 * def}) {
+      const DigitLayout *D = set_digit_slots(pl, B, slots);
+      if (!D) break;
+      for (int rep = 0; rep < 3; ++rep) {
+        if (rep == 1) cudaEventRecord(e0, st);
+        launch_solve_digits(pl, *D, false, pl.s_in, B, st);
+        launch_finish_digits(pl, *D, false, pl.s_in, pl.s_out, B, st);
+      }
+      cudaEventRecord(e1, st);
+      float ms = 1e30f;
+      if (cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
+      if (ms < digit_ms) {
+        digit_ms = ms;
+        digit_slots = D->slots;
+      }
+    }
+    set_digit_slots(pl, B, digit_slots);
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   auto it = pl.layouts.find(B);
@@ -716,6 +807,12 @@ rexi_status tune_layout(Plan &pl, int B, int *slots_out, int *shape_out) {
   // path's DRAM traffic for the same FP64 work
   const bool fused_wins = fused_ms <= best * 1.005f;
   pl.use_slots[B] = !fused_wins;
+  pl.use_digits[B] = digit_ms < std::min(fused_ms, best);
+  if (pl.use_digits[B]) {
+    if (slots_out) *slots_out = digit_slots;
+    if (shape_out) *shape_out = 5;
+    return REXI_OK;
+  }
   if (slots_out) *slots_out = fused_wins ? best_tile + 256 * best_groups : bestL.slots;
   if (shape_out) *shape_out = fused_wins ? 2 + best_form : bestL.shape;
   return REXI_OK;
@@ -731,13 +828,17 @@ void free_plan(Plan *pl) {
                   pl->mscale_one32,
                   pl->zd_syn, pl->zd_ana_adj, pl->zd_one, pl->zd_mone, pl->fft.tw_dev, pl->fft.tw32_dev, pl->four,
                   pl->s_in, pl->s_out, pl->s_ff, pl->partial, pl->yscratch, pl->counter, pl->tc_tab_ana,
-                  pl->tc_tab_syn, pl->tc_work_ana, pl->tc_work_syn, pl->dev_err, pl->phi_zc, pl->phi_q, pl->phi_abf, pl->ffc_rows, pl->ffc_ia};
+                  pl->tc_tab_syn, pl->tc_work_ana, pl->tc_work_syn, pl->dev_err, pl->phi_zc, pl->phi_q, pl->phi_abf, pl->ffc_rows, pl->ffc_ia,
+                  pl->dig_state};
   for (cudaEvent_t ev : pl->prof_ev) cudaEventDestroy(ev);
   for (void *p : ptrs)
     if (p) cudaFree(p);
   for (auto &kv : pl->layouts)
     if (kv.second.items_dev) cudaFree(kv.second.items_dev);
   for (auto &kv : pl->fused) free_fused_layout(kv.second);
+  for (auto &kv : pl->digits) free_digit_layout(kv.second);
+  free_digit_factors(pl->dig_fwd);
+  free_digit_factors(pl->dig_adj);
   delete pl;
 }
 

@@ -120,6 +120,21 @@ struct FusedRagged {
   size_t smem = 0;
 };
 
+// The factors of the digit solve (solve_digits.cu): per (row, window of eight poles) records
+// of coupling and weight digits, and the rows' input scales.  Empty (fwd null) where it does
+// not serve the plan.
+struct DigitFactors {
+  char *fwd = nullptr, *bwd = nullptr;
+  int *vexp = nullptr;
+};
+
+// The digit solve's work list for one batch size: items (system, tile of eight states,
+// windows, slot), longest first; each slot's sums are added by a second kernel.
+struct DigitLayout {
+  int slots = 0, nitems = 0;
+  int4 *items_dev = nullptr;
+};
+
 struct FftPlan {
   int n;
   int nstages;
@@ -231,7 +246,7 @@ struct Plan {
   double2 *yscratch = nullptr; // [resident warps][Lmax][32]
   int resident_warps = 0, lmax = 0;
   unsigned *counter = nullptr;
-  size_t partial_cap = 0;
+  size_t partial_cap = 0, partial_elems = 0;  // slots, and values in the buffer
 
   std::map<int, SolveLayout> layouts;  // per batch size
   // bumped whenever a slot layout is replaced (its device work list freed): objects that
@@ -245,6 +260,14 @@ struct Plan {
   std::map<int, int> fused_tile;  // requested states per CTA tile (0: the default)
   std::map<int, int> fused_form;  // 0: register form; lean form with CTAs of 1: four warps, 2: two warps
   std::map<int, int> fused_groups; // requested CTAs per system's poles (0: the default)
+
+  // digit solve: the factors as digits (adjoint on first use), the step's inputs as digits,
+  // per batch size the work list and whether rexi_tune / rexi_set_pole_slots chose it
+  DigitFactors dig_fwd, dig_adj;
+  bool dig_adj_tried = false;
+  char *dig_state = nullptr;
+  std::map<int, DigitLayout> digits;
+  std::map<int, bool> use_digits;
 
   // optional per-stage timing with CUDA events on the launching stream
   bool prof = false;
@@ -300,6 +323,19 @@ void free_fused_ragged(FusedRagged &R);
 cudaError_t launch_fused_ragged(const FusedRagged &R, double2 *ybuf, int num_sms, cudaStream_t st);
 cudaError_t launch_solve_fused(Plan &pl, const FusedLayout &F, bool adjoint, const double2 *sin, double2 *sout,
                                int B, cudaStream_t st);
+// digit solve (solve_digits.cu): sin -> slot sums in pl.partial, then the ordered sum of the
+// slots with the pole-independent terms
+size_t digit_factor_bytes(const Plan &pl);
+size_t digit_state_bytes(const Plan &pl, int B);
+size_t digit_slot_bytes(const Plan &pl, int B);
+cudaError_t build_digit_factors(Plan &pl, const double2 *fac, DigitFactors &D);
+void free_digit_factors(DigitFactors &D);
+rexi_status build_digit_layout(Plan &pl, int B, int slots, DigitLayout &L);
+void free_digit_layout(DigitLayout &L);
+cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, int B,
+                                cudaStream_t st);
+cudaError_t launch_finish_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, double2 *sout,
+                                 int B, cudaStream_t st);
 cudaError_t launch_solve_ragged(const SolveView *views_dev, const WorkItem *items, int nitems, double2 *ybuf,
                                 int lmax, unsigned *counter, int resident_warps, bool ff, cudaStream_t st);
 // float-float solves: convert n complex values in place (factors), or split n binary64

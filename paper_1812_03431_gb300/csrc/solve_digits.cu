@@ -1,0 +1,634 @@
+// Banded shifted solves of whole batches with their two contractions on the tensor cores,
+// exactly (paper Sec. 4.2, Sec. 5, Algorithm 1; binary64 delta solver).
+//
+// The systems, factors and recurrences are those of solve.cu: per (pole k, zonal order m,
+// parity) forward  y_i = r_i - l y_{i-1},  r_i = delta0_n - g Phi0_n - e zeta0_{n-1} - f zeta0_{n+1},
+// backward  w_i = y_i - Chat w_{i+1},  and the sums over k of bd w, bad w, zp w and zm w.
+// Of the 36 FP64 FMAs per (state, pole, row), 8 belong to the two recurrences; the other 28
+// are contractions with factors that no state changes: r over the row's four inputs, and the
+// four weighted sums over the poles.  GB300's FP64 unit issues one warp instruction per 64
+// cycles and scheduler, so the contractions are taken off it:
+//   - every operand is written as a 64-bit fixed-point number relative to the largest of its
+//     group (a power of two per group), cut into 8-bit balanced digits -128..127, which fp16
+//     holds exactly (weights: seven digits, 55 bits and sign; inputs, couplings and w: eight);
+//   - digit products are summed by mma.sync m16n8k16 with FP32 accumulators that start at
+//     1.5 2^23, so that an accumulator's low bits are the integer sum: every partial sum stays
+//     below 2^22 and nothing is rounded (digit pairs i + j <= 7 are taken: what is left out is
+//     below 2^-60 of the largest product);
+//   - the eight sums of equal weight are put together in a 64-bit integer, which is rounded to
+//     binary64 once, on the integer pipe.
+// The sums are therefore exact up to the 2^-55 rounding of a group's smaller operands and one
+// rounding each; the recurrences run in binary64 as before.  The pole sums of an item's
+// windows are added in binary64 in window order, and the items' sums in a fixed order, so
+// results are bit-reproducible.
+//
+// Why mma.sync and not tcgen05: the operand fragments of m16n8k16 are exactly what the lanes
+// hold (a lane's state and pole are a fragment's column and k pair), so digits go from
+// registers into the tensor core and sums come back to the lane that needs them, with no
+// shared memory, no descriptors and no waiting.  The work is 40 MMAs per warp and row at 8.8
+// cycles each, about a third of the FP64 time beside them, so their rate does not bound it.
+//
+// Measured on GB300 (solve and the sum of the slots, against the pole-slot solve and its
+// reduction): T341, 535 poles, 16 states 12.0 / 30.0 ms; T127, 535 poles, 64 states 6.6 / 17.0;
+// T85, 215 poles, 5 states 0.20 / 0.62.  What bounds it now: the FP64 unit for 7.7 of the 11.5 ms
+// at T341 (9 instructions per state, pole and row at 64 cycles, one of them the running sum's
+// addition).
+//
+// A warp takes 8 states x 8 poles (lane: state lane / 4, poles lane % 4 and lane % 4 + 4) of
+// one (m, parity) system, window by window of 8 poles, over all rows.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <string>
+#include <vector>
+
+#include "rexi_internal.h"
+
+namespace rexi {
+
+namespace {
+
+constexpr int kTile = 8;                   // states per warp
+constexpr int kWin = 8;                    // poles per window
+constexpr int kFwdRec = 1024 + 128 + 32;   // per (row, window): coupling digits, l, exponents
+constexpr int kBwdRec = 1024 + 128;        // per (row, window): weight digits and exponents, Chat
+constexpr int kStateRec = 1024;            // per (row, tile): input digits
+constexpr int kNotFinite = 1 << 20;        // exponent of a row input that holds an Inf or NaN
+constexpr int kMaxSpread = 8;              // bits by which a pole's couplings may differ in scale
+constexpr float kMagic = 12582912.0f;      // 1.5 2^23
+
+__device__ __forceinline__ int bexp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// x as a fixed-point number of 61 bits below its group's leading bit, d = that bit's exponent
+// less x's own (truncated at 2^-61 of the leading bit; zero and subnormal x give zero)
+__device__ __forceinline__ long long to_fixed(double x, int d) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+  m = (m << 9) >> (d & 63);
+  if (d > 63 || !(hi & 0x7ff00000u)) m = 0;
+  return (int)hi < 0 ? -(long long)m : (long long)m;
+}
+
+__device__ __forceinline__ unsigned half2_sub(unsigned a, unsigned b) {
+  unsigned r;
+  asm("sub.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+
+// the eight balanced digits of (re, im), most significant first, as fp16 pairs: bytes of the
+// biased number under the fp16 exponent of 1024, less 1024 + 128
+__device__ __forceinline__ void digits(long long re, long long im, unsigned (&w)[8]) {
+  const unsigned long long ur = (unsigned long long)re + 0x8080808080808080ull;
+  const unsigned long long ui = (unsigned long long)im + 0x8080808080808080ull;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const unsigned r = h == 0 ? (unsigned)(ur >> 32) : (unsigned)ur, i = h == 0 ? (unsigned)(ui >> 32) : (unsigned)ui;
+    const unsigned top = __byte_perm(r, i, 0x7362), low = __byte_perm(r, i, 0x5140);
+    w[4 * h + 0] = half2_sub(__byte_perm(top, 0x64646464u, 0x4342), 0x64806480u);
+    w[4 * h + 1] = half2_sub(__byte_perm(top, 0x64646464u, 0x4140), 0x64806480u);
+    w[4 * h + 2] = half2_sub(__byte_perm(low, 0x64646464u, 0x4342), 0x64806480u);
+    w[4 * h + 3] = half2_sub(__byte_perm(low, 0x64646464u, 0x4140), 0x64806480u);
+  }
+}
+
+// t 2^e in binary64 (round half away from zero), on the integer pipe; results below 2^-1022
+// are zero, e of a group that is not finite gives NaN
+__device__ __forceinline__ double fixed_to_double(long long t, int e) {
+  const unsigned long long m = t < 0 ? (unsigned long long)(-t) : (unsigned long long)t;
+  const int lz = __clzll((long long)m);
+  const unsigned long long f = m << (lz & 63);
+  const unsigned long long r = (f >> 11) + ((f >> 10) & 1);
+  const int be = 1023 + 63 + e - lz;
+  unsigned hi = (unsigned)(r >> 32) + ((unsigned)(be - 1) << 20), lo = (unsigned)r;
+  if (m == 0 || be <= 0) hi = lo = 0;
+  if (be >= 2047 && (m != 0 || e >= kNotFinite / 2)) {
+    hi = e >= kNotFinite / 2 ? 0x7ff80000u : 0x7ff00000u;
+    lo = 0;
+  }
+  return __hiloint2double((int)(hi | ((unsigned)((unsigned long long)t >> 32) & 0x80000000u)), (int)lo);
+}
+
+// sum of s_c 2^(-8c), c = 0..7, in units of 2^-46; the pairs (s_0, s_1) ... (s_6, s_7) come as
+// 256 s_c + s_{c+1}
+__device__ __forceinline__ long long weigh(int h, int m, int l, int q) {
+  const long long t = ((long long)h << 32) + (long long)m * 65536 + l;
+  return (t << 6) + ((q + 512) >> 10);
+}
+
+__device__ __forceinline__ void mma_first(float (&d)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0,
+                                          unsigned b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(kMagic));
+}
+__device__ __forceinline__ void mma_add(float (&d)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0,
+                                        unsigned b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ double2 cfms(double2 acc, double2 a, double2 b) {
+  double re = fma(-a.x, b.x, acc.x), im = fma(-a.x, b.y, acc.y);
+  return make_double2(fma(a.y, b.y, re), fma(-a.y, b.x, im));
+}
+__device__ __forceinline__ double2 cfma(double2 acc, double2 a, double2 b) {
+  double re = fma(a.x, b.x, acc.x), im = fma(a.x, b.y, acc.y);
+  return make_double2(fma(-a.y, b.y, re), fma(a.y, b.x, im));
+}
+
+// ---- plan time: the factors as digits ---------------------------------------------------------
+struct SetupArgs {
+  const double2 *fac;  // [F_NCOMP][nrows][P]
+  const int4 *sys;
+  char *fwd, *bwd;     // records, system by system: [window][row of the system]
+  int *vexp;           // [nrows][4]: the scale of each input (0 for delta)
+  int *bad;            // set when the factors are not finite or too unlike in scale
+  int P, nwin, kmid;
+  int64_t nrows;
+};
+
+__global__ void digit_factor_kernel(SetupArgs a) {
+  const int4 sy = a.sys[blockIdx.y];
+  const int len = sy.z;
+  const int64_t row0 = sy.w;
+  const int64_t total = (int64_t)len * a.nwin * kWin;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool live = t < total;  // whole groups of 8 threads
+  const int p8 = (int)(t & 7);
+  const int w = (int)((t >> 3) % a.nwin), i = (int)((t >> 3) / a.nwin);
+  const int k = w * kWin + p8;
+  const int64_t row = row0 + i;
+  const double2 zero = make_double2(0, 0);
+  auto get = [&](int comp, int kk) { return live && kk < a.P ? a.fac[((int64_t)comp * a.nrows + row) * a.P + kk] : zero; };
+  auto neg = [](double2 v) { return make_double2(-v.x, -v.y); };
+  auto emax = [](double2 v) { return max(bexp(v.x), bexp(v.y)); };
+  const int64_t rec = row0 * a.nwin + (int64_t)w * len + i;
+  char *fr = a.fwd + rec * kFwdRec, *br = a.bwd + rec * kBwdRec;
+  bool bad = false;
+
+  // couplings of the four inputs delta, Phi, zeta_{n-1}, zeta_{n+1}
+  double2 v[4] = {live && k < a.P ? make_double2(1.0, 0.0) : zero, neg(get(F_G, k)), neg(get(F_E, k)), neg(get(F_F, k))};
+  int ve[4], E = 0;
+  const int comp[4] = {0, F_G, F_E, F_F};
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int mid = j == 0 ? 1023 : emax(get(comp[j], a.kmid));
+    ve[j] = mid == 0 ? 0 : mid - 1023;
+    const int e = emax(v[j]);
+    if (e == 0x7ff) bad = true;
+    if (e) E = max(E, e - ve[j]);
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int e = emax(v[j]);
+    if (e && E - (e - ve[j]) > kMaxSpread) bad = true;
+    unsigned d[8];
+    digits(to_fixed(v[j].x, E - (bexp(v[j].x) - ve[j])), to_fixed(v[j].y, E - (bexp(v[j].y) - ve[j])), d);
+    if (live) {
+      uint4 *o = reinterpret_cast<uint4 *>(fr + (p8 * 4 + j) * 32);
+      o[0] = make_uint4(d[0], d[1], d[2], d[3]);
+      o[1] = make_uint4(d[4], d[5], d[6], d[7]);
+    }
+  }
+  if (live) {
+    *reinterpret_cast<double2 *>(fr + 1024 + p8 * 16) = get(F_L, k);
+    *reinterpret_cast<int *>(fr + 1152 + p8 * 4) = E - 1023;
+    *reinterpret_cast<double2 *>(br + 1024 + p8 * 16) = get(F_C, k);
+    if (w == 0 && p8 < 4) a.vexp[row * 4 + p8] = ve[p8];
+  }
+  // the four weights, scaled by the largest of the window's eight poles
+  const int wc[4] = {F_BD, F_BAD, F_ZP, F_ZM};
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    const double2 x = get(wc[s], k);
+    int m = emax(x);
+    if (m == 0x7ff) bad = true;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    unsigned d[8];  // seven digits: rounded to the nearest multiple of the eighth's weight
+    digits((to_fixed(x.x, m - bexp(x.x)) + 128) & ~255ll, (to_fixed(x.y, m - bexp(x.y)) + 128) & ~255ll, d);
+    if (live) {
+      uint4 *o = reinterpret_cast<uint4 *>(br + (s * kWin + p8) * 32);
+      o[0] = make_uint4(d[0], d[1], d[2], d[3]);
+      o[1] = make_uint4(d[4], d[5], d[6], (unsigned)(m - 1023));
+    }
+  }
+  const double2 l = get(F_L, k), c = get(F_C, k);
+  if (emax(l) == 0x7ff || emax(c) == 0x7ff) bad = true;
+  if (bad) atomicOr(a.bad, 1);
+}
+
+// ---- per step: the row inputs as digits ---------------------------------------------------------
+struct StateArgs {
+  const double2 *sin;  // [3][nspec][B]
+  const int4 *sys;
+  const int *vexp;
+  char *dig;           // [nrows][tiles] records
+  int *uexp;           // [nrows][tiles][8]
+  int64_t nspec;
+  int B, tiles, N;
+};
+
+__global__ void digit_state_kernel(StateArgs a) {
+  const int4 sy = a.sys[blockIdx.y];
+  const int m = sy.x, n0 = sy.y, len = sy.z;
+  const int lane = threadIdx.x & 31, s = lane >> 2, q = lane & 3;
+  const int wid = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (wid >= len * a.tiles) return;  // whole warps
+  const int i = wid / a.tiles, tile = wid - i * a.tiles;
+  const int64_t row = sy.w + i;
+  const int n = n0 + 2 * i, b = tile * kTile + s, nmin = m > 1 ? m : 1;
+  const int nn = q < 2 ? n : (q == 2 ? n - 1 : n + 1);
+  const int field = q == 0 ? 2 : (q == 1 ? 0 : 1);
+  double2 x = make_double2(0, 0);
+  if (b < a.B && nn >= nmin && nn <= a.N) {
+    const int64_t ix = (int64_t)m * (2 * a.N + 3 - m) / 2 + (nn - m);
+    x = __ldg(a.sin + ((int64_t)field * a.nspec + ix) * a.B + b);
+  }
+  const int v = a.vexp[row * 4 + q];
+  const int er = bexp(x.x), ei = bexp(x.y), e = max(er, ei);
+  int U = e ? e + v : -(1 << 24), nf = e == 0x7ff;
+#pragma unroll
+  for (int o = 1; o < 4; o <<= 1) {
+    U = max(U, __shfl_xor_sync(0xffffffffu, U, o));
+    nf |= __shfl_xor_sync(0xffffffffu, nf, o);
+  }
+  unsigned d[8];
+  digits(nf ? 0 : to_fixed(x.x, U - (er + v)), nf ? 0 : to_fixed(x.y, U - (ei + v)), d);
+  uint4 *o = reinterpret_cast<uint4 *>(a.dig + (row * a.tiles + tile) * kStateRec + lane * 32);
+  o[0] = make_uint4(d[0], d[1], d[2], d[3]);
+  o[1] = make_uint4(d[4], d[5], d[6], d[7]);
+  if (q == 0) a.uexp[(row * a.tiles + tile) * kTile + s] = nf ? kNotFinite : (U < -(1 << 23) ? 0 : U - 1023);
+}
+
+// ---- per step: the sweeps ----------------------------------------------------------------------
+struct SweepArgs {
+  const char *fwd, *bwd, *dig;
+  const int *uexp;
+  const int4 *sys, *items;  // {system, tile, first window | windows << 16, slot}
+  double *part;             // [slots][nrows][tiles][4 streams][re, im][8 states]
+  double2 *ybuf;            // per resident warp: [lmax][2][32]
+  unsigned *counter;
+  int64_t nrows;
+  int nitems, tiles, nwin, lmax;
+};
+
+__device__ __forceinline__ void load_words(const char *p, unsigned (&w)[8]) {
+  const uint4 x = __ldg(reinterpret_cast<const uint4 *>(p)), y = __ldg(reinterpret_cast<const uint4 *>(p) + 1);
+  w[0] = x.x, w[1] = x.y, w[2] = x.z, w[3] = x.w, w[4] = y.x, w[5] = y.y, w[6] = y.z, w[7] = y.w;
+}
+__device__ __forceinline__ double2 ldd(const char *p) { return __ldg(reinterpret_cast<const double2 *>(p)); }
+__device__ __forceinline__ void prefetch(const void *p) { asm volatile("prefetch.global.L1 [%0];" : : "l"(p)); }
+__device__ __forceinline__ int bits(float x) { return __float_as_int(x); }
+
+constexpr unsigned kB = 0x4B400000u;  // bits of kMagic
+
+// rows whose data is brought into the caches ahead of use
+constexpr int kAhead = 2;
+
+template <int CTAS>
+__global__ void __launch_bounds__(128, CTAS) solve_digits_kernel(SweepArgs a) {
+  const int lane = threadIdx.x & 31, q = lane & 3;
+  const int wslot = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  double2 *yb = a.ybuf + (int64_t)wslot * a.lmax * 64 + lane;
+  // a real row of the complex products takes (re, -im) of the factor, an imaginary one (im, re)
+  const bool im_row = (lane >> 2) & 1;
+  const unsigned sel = im_row ? 0x1032u : 0x3210u, flip = im_row ? 0u : 0x80000000u;
+  for (;;) {
+    unsigned it = 0;
+    if (lane == 0) it = atomicAdd(a.counter, 1u);
+    it = __shfl_sync(0xffffffffu, it, 0);
+    if (it >= (unsigned)a.nitems) break;
+    const int4 item = a.items[it];
+    const int4 sy = a.sys[item.x];
+    const int len = sy.z, w0 = item.z & 0xffff, w1 = w0 + (item.z >> 16);
+    const int64_t row0 = sy.w;
+    const char *dig = a.dig + (row0 * a.tiles + item.y) * kStateRec + lane * 32;
+    const int *uexp = a.uexp + (row0 * a.tiles + item.y) * kTile + (lane >> 2);
+    const int64_t dstep = (int64_t)a.tiles * kStateRec;
+    double2 *part = reinterpret_cast<double2 *>(a.part + (((int64_t)item.w * a.nrows + row0) * a.tiles + item.y) * 64) + lane;
+    const int64_t pstep = (int64_t)a.tiles * 32;
+    for (int w = w0; w < w1; ++w) {
+      const char *fr = a.fwd + (row0 * a.nwin + (int64_t)w * len) * kFwdRec;
+      double2 y[2] = {make_double2(0, 0), make_double2(0, 0)};
+      for (int i = 0; i < len; ++i) {
+        if (i + kAhead < len) {
+          const char *nf = fr + (int64_t)(i + kAhead) * kFwdRec, *nd = dig + (i + kAhead) * dstep - lane * 32;
+          if (lane < 10) prefetch(nf + lane * 128);
+          else if (lane >= 16 && lane < 24) prefetch(nd + (lane - 16) * 128);
+        }
+        const char *f = fr + (int64_t)i * kFwdRec;
+        unsigned p[8];
+        load_words(dig + i * dstep, p);
+        const int U = __ldg(uexp + (int64_t)i * a.tiles * kTile);
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          unsigned v[8];
+          load_words(f + ((g * 4 + (lane >> 3)) * 4 + q) * 32, v);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) v[j] = __byte_perm(v[j], 0, sel) ^ flip;
+          float s0[4], s2[4], s4[4], s6[4];
+          mma_first(s0, 0u, p[0], p[0], p[1], v[1], v[0]);
+          mma_first(s2, 0u, p[0], p[0], p[1], v[3], v[2]);
+          mma_first(s4, 0u, p[0], p[0], p[1], v[5], v[4]);
+          mma_first(s6, 0u, p[0], p[0], p[1], v[7], v[6]);
+          mma_add(s2, p[1], p[2], p[2], p[3], v[1], v[0]);
+          mma_add(s4, p[1], p[2], p[2], p[3], v[3], v[2]);
+          mma_add(s6, p[1], p[2], p[2], p[3], v[5], v[4]);
+          mma_add(s4, p[3], p[4], p[4], p[5], v[1], v[0]);
+          mma_add(s6, p[3], p[4], p[4], p[5], v[3], v[2]);
+          mma_add(s6, p[5], p[6], p[6], p[7], v[1], v[0]);
+          const int e = U + __ldg(reinterpret_cast<const int *>(f + 1152) + g * 4 + q) - 56;
+          constexpr unsigned K = kB * 256u + kB;
+          double r[2];
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const int h = (int)((unsigned)bits(s0[c]) * 256u + (unsigned)bits(s0[c + 2]) - K);
+            const int m = (int)((unsigned)bits(s2[c]) * 256u + (unsigned)bits(s2[c + 2]) - K);
+            const int l = (int)((unsigned)bits(s4[c]) * 256u + (unsigned)bits(s4[c + 2]) - K);
+            const int o = (int)((unsigned)bits(s6[c]) * 256u + (unsigned)bits(s6[c + 2]) - K);
+            r[c] = fixed_to_double(weigh(h, m, l, o), e);
+          }
+          y[g] = cfms(make_double2(r[0], r[1]), ldd(f + 1024 + (g * 4 + q) * 16), y[g]);
+          yb[(i * 2 + g) * 32] = y[g];
+        }
+      }
+      const char *br = a.bwd + (row0 * a.nwin + (int64_t)w * len) * kBwdRec;
+      double2 x[2] = {make_double2(0, 0), make_double2(0, 0)};
+      for (int i = len - 1; i >= 0; --i) {
+        if (i >= kAhead) {
+          const char *nb = br + (int64_t)(i - kAhead) * kBwdRec;
+          if (lane < 10) prefetch(nb + (lane < 9 ? lane * 128 : kBwdRec - 16));
+          else if (lane >= 16 && lane < 24) prefetch(reinterpret_cast<const char *>(yb - lane + (i - kAhead) * 64) + (lane - 16) * 128);
+          else if (lane >= 24 && lane < 28 && w > w0) prefetch(reinterpret_cast<const char *>(part - lane + (i - kAhead) * pstep) + (lane - 24) * 128);
+        }
+        const char *f = br + (int64_t)i * kBwdRec;
+        double2 sum = make_double2(0, 0);
+        if (w > w0) sum = part[i * pstep];
+        int E = 0;
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          x[g] = cfms(yb[(i * 2 + g) * 32], ldd(f + 1024 + (g * 4 + q) * 16), x[g]);
+          E = max(E, max(__double2hiint(x[g].x) & 0x7fffffff, __double2hiint(x[g].y) & 0x7fffffff));
+        }
+        E = max(E, __shfl_xor_sync(0xffffffffu, E, 1));
+        E = max(E, __shfl_xor_sync(0xffffffffu, E, 2)) >> 20;
+        unsigned d0[8], d1[8];
+        digits(to_fixed(x[0].x, E - bexp(x[0].x)), to_fixed(x[0].y, E - bexp(x[0].y)), d0);
+        digits(to_fixed(x[1].x, E - bexp(x[1].x)), to_fixed(x[1].y, E - bexp(x[1].y)), d1);
+        unsigned u[8], v[8];
+        load_words(f + ((lane >> 3) * kWin + q) * 32, u);
+        load_words(f + ((lane >> 3) * kWin + q + 4) * 32, v);
+        const int We = (int)u[7];
+#pragma unroll
+        for (int j = 0; j < 7; ++j) {
+          u[j] = __byte_perm(u[j], 0, sel) ^ flip;
+          v[j] = __byte_perm(v[j], 0, sel) ^ flip;
+        }
+        u[7] = v[7] = 0;
+        float s[8][4];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) mma_first(s[c], u[0], u[1], v[0], v[1], d0[c], d1[c]);
+#pragma unroll
+        for (int c = 2; c < 8; ++c) mma_add(s[c], u[2], u[3], v[2], v[3], d0[c - 2], d1[c - 2]);
+#pragma unroll
+        for (int c = 4; c < 8; ++c) mma_add(s[c], u[4], u[5], v[4], v[5], d0[c - 4], d1[c - 4]);
+#pragma unroll
+        for (int c = 6; c < 8; ++c) mma_add(s[c], u[6], u[7], v[6], v[7], d0[c - 6], d1[c - 6]);
+        double r[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const int Es = __shfl_sync(0xffffffffu, E, (q * 2 + c) * 4);  // the exponent of state 2 q + c
+          auto at = [&](int j) { return (unsigned)bits(s[j][c]) + (j ? (unsigned)bits(s[j ? j - 1 : 0][c + 2]) : 0u); };
+          constexpr unsigned K0 = kB * 256u + 2u * kB, K = 2u * kB * 256u + 2u * kB;
+          const int h = (int)(at(0) * 256u + at(1) - K0), m = (int)(at(2) * 256u + at(3) - K);
+          const int l = (int)(at(4) * 256u + at(5) - K), o = (int)(at(6) * 256u + at(7) - K);
+          r[c] = fixed_to_double(weigh(h, m, l, o), Es == 0x7ff ? kNotFinite : We + Es - 1023 - 56);
+        }
+        part[i * pstep] = make_double2(sum.x + r[0], sum.y + r[1]);
+      }
+    }
+  }
+}
+
+// ---- per step: the items' sums, the pole-independent terms, Re at m = 0 --------------------------
+struct FinishArgs {
+  const double *part;
+  const double2 *sin, *w;
+  double2 *sout;
+  const uint8_t *rflags;
+  const int32_t *m_of;
+  const int4 *sys;
+  double2 sphi;
+  int64_t nspec, nrows;
+  int B, tiles, slots, N;
+};
+
+__global__ void digit_finish_kernel(FinishArgs a) {
+  const int64_t total = 3 * a.nspec * a.B;
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
+    const int b = (int)(t % a.B);
+    const int64_t fi = t / a.B;
+    const int f = (int)(fi / a.nspec);
+    const int64_t ix = fi - (int64_t)f * a.nspec;
+    const uint8_t fl = a.rflags[fi];
+    double2 acc = make_double2(0, 0);
+    if (!(fl & 2)) {
+      const int m = a.m_of[ix];
+      if (fl & 1) {
+        const int n = m + (int)(ix - (int64_t)m * (2 * a.N + 3 - m) / 2);
+        auto add = [&](int nn, int stream) {  // the slots' sums of the row at degree nn, in slot order
+          const int4 sy = a.sys[2 * m + ((nn - m) & 1)];
+          const int64_t row = sy.w + (nn - sy.y) / 2;
+          const double *p = a.part + (row * a.tiles + b / kTile) * 64 + stream * 16 + b % kTile;
+          for (int s = 0; s < a.slots; ++s, p += a.nrows * a.tiles * 64) acc = make_double2(acc.x + p[0], acc.y + p[8]);
+        };
+        const int nmin = m > 1 ? m : 1;
+        if (f != 1) add(n, f == 2 ? 0 : 1);
+        else {
+          if (n - 1 >= nmin) add(n - 1, 2);
+          if (n + 1 <= a.N) add(n + 1, 3);
+        }
+      }
+      const double2 x0 = a.sin[t];
+      if (f == 0) acc = cfma(acc, a.sphi, x0);
+      else if (f == 1) acc = cfma(acc, a.w[ix], x0);
+      if (m == 0) acc.y = 0.0;
+    }
+    a.sout[t] = acc;
+  }
+}
+
+// resident CTAs per SM: 12 warps at 168 registers
+constexpr int kCtas = 3;
+
+int tiles_of(int B) { return (B + kTile - 1) / kTile; }
+
+}  // namespace
+
+void free_digit_factors(DigitFactors &D) {
+  for (void *p : {(void *)D.fwd, (void *)D.bwd, (void *)D.vexp})
+    if (p) cudaFree(p);
+  D = DigitFactors{};
+}
+
+size_t digit_factor_bytes(const Plan &pl) {
+  return (size_t)pl.nrows * ((pl.P + kWin - 1) / kWin) * (kFwdRec + kBwdRec) + (size_t)pl.nrows * 4 * sizeof(int);
+}
+
+// The factor set as digits, from the binary64 factors `fac`.  D stays empty (and the other
+// solve kernels serve the plan) where the device memory does not suffice, or where a factor
+// is not finite or a pole's couplings differ in scale by more than the eighth digit covers.
+cudaError_t build_digit_factors(Plan &pl, const double2 *fac, DigitFactors &D) {
+  D = DigitFactors{};
+  const int nwin = (pl.P + kWin - 1) / kWin;
+  if (pl.nrows == 0 || nwin > 0x7fff || pl.sys.size() > 0xffff) return cudaSuccess;
+  const size_t nrec = (size_t)pl.nrows * nwin;
+  int *bad = nullptr;
+  if (cudaMalloc(&D.fwd, nrec * kFwdRec) != cudaSuccess || cudaMalloc(&D.bwd, nrec * kBwdRec) != cudaSuccess ||
+      cudaMalloc(&D.vexp, (size_t)pl.nrows * 4 * sizeof(int) + sizeof(int)) != cudaSuccess) {
+    cudaGetLastError();
+    free_digit_factors(D);
+    return cudaSuccess;
+  }
+  bad = D.vexp + pl.nrows * 4;
+  cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int), 0);
+  SetupArgs a;
+  a.fac = fac;
+  a.sys = pl.sys_dev;
+  a.fwd = D.fwd;
+  a.bwd = D.bwd;
+  a.vexp = D.vexp;
+  a.bad = bad;
+  a.P = pl.P;
+  a.nwin = nwin;
+  a.kmid = (int)(std::min_element(pl.alpha.begin(), pl.alpha.end(),
+                                  [](const cplx &x, const cplx &y) { return std::abs(x) < std::abs(y); }) -
+                 pl.alpha.begin());
+  a.nrows = pl.nrows;
+  const int64_t most = (int64_t)pl.lmax * nwin * kWin;
+  if (e == cudaSuccess) {
+    digit_factor_kernel<<<dim3((unsigned)((most + 255) / 256), (unsigned)pl.sys.size()), 256>>>(a);
+    e = cudaGetLastError();
+  }
+  int hbad = 0;
+  if (e == cudaSuccess) e = cudaMemcpy(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess || hbad) free_digit_factors(D);
+  return e;
+}
+
+size_t digit_state_bytes(const Plan &pl, int B) {
+  return (size_t)pl.nrows * tiles_of(B) * (kStateRec + kTile * sizeof(int));
+}
+
+// partial sums of one slot
+size_t digit_slot_bytes(const Plan &pl, int B) { return (size_t)pl.nrows * tiles_of(B) * 64 * sizeof(double); }
+
+// Work items (system, tile, windows, slot) for batch B, longest first.  slots: items per
+// (system, tile), each over its share of the windows; 0: enough that the longest item is at
+// most half a resident warp's share of the work, capped by the partial-sum buffer.
+rexi_status build_digit_layout(Plan &pl, int B, int slots, DigitLayout &L) {
+  L = DigitLayout{};
+  const int nwin = (pl.P + kWin - 1) / kWin, tiles = tiles_of(B);
+  if (pl.nrows == 0) return REXI_OK;  // not available
+  const int cap = (int)std::min<size_t>((size_t)nwin, pl.partial_elems * sizeof(double2) / digit_slot_bytes(pl, B));
+  if (cap < 1) return REXI_OK;  // not available
+  int64_t rows = 0;
+  for (const SysInfo &s : pl.sys) rows += s.len;
+  int G = slots;
+  if (G <= 0) {
+    const double share = (double)rows * nwin * tiles / (4.0 * kCtas * pl.num_sms);
+    G = 1;
+    while (G < nwin && (double)pl.lmax * ((nwin + G - 1) / G) > 0.5 * share) ++G;
+  }
+  G = std::max(1, std::min(G, cap));
+  struct Keyed { int4 it; int64_t work; };
+  std::vector<Keyed> keyed;
+  for (int s = 0; s < (int)pl.sys.size(); ++s) {
+    if (pl.sys[s].len == 0) continue;
+    for (int g = 0; g < G; ++g) {
+      const int w0 = (int)((int64_t)nwin * g / G), w1 = (int)((int64_t)nwin * (g + 1) / G);
+      for (int t = 0; t < tiles; ++t)
+        keyed.push_back(Keyed{make_int4(s, t, w0 | ((w1 - w0) << 16), g), (int64_t)pl.sys[s].len * (w1 - w0)});
+    }
+  }
+  std::stable_sort(keyed.begin(), keyed.end(), [](const Keyed &x, const Keyed &y) { return x.work > y.work; });
+  std::vector<int4> items;
+  for (const Keyed &k : keyed) items.push_back(k.it);
+  cudaError_t e = cudaMalloc(&L.items_dev, std::max<size_t>(1, items.size()) * sizeof(int4));
+  if (e == cudaSuccess) e = cudaMemcpy(L.items_dev, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    free_digit_layout(L);
+    set_error(std::string("digit work list: ") + cudaGetErrorString(e));
+    return REXI_ENOMEM;
+  }
+  L.slots = G;
+  L.nitems = (int)items.size();
+  return REXI_OK;
+}
+
+void free_digit_layout(DigitLayout &L) {
+  if (L.items_dev) cudaFree(L.items_dev);
+  L = DigitLayout{};
+}
+
+cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, int B, cudaStream_t st) {
+  const DigitFactors &D = adjoint ? pl.dig_adj : pl.dig_fwd;
+  const int tiles = tiles_of(B);
+  StateArgs s;
+  s.sin = sin;
+  s.sys = pl.sys_dev;
+  s.vexp = D.vexp;
+  s.dig = pl.dig_state;
+  s.uexp = reinterpret_cast<int *>(pl.dig_state + (size_t)pl.nrows * tiles * kStateRec);
+  s.nspec = pl.nspec;
+  s.B = B;
+  s.tiles = tiles;
+  s.N = pl.N;
+  digit_state_kernel<<<dim3((unsigned)((pl.lmax * tiles + 7) / 8), (unsigned)pl.sys.size()), 256, 0, st>>>(s);
+  cudaError_t e = cudaMemsetAsync(pl.counter, 0, sizeof(unsigned), st);
+  if (e != cudaSuccess) return e;
+  SweepArgs a;
+  a.fwd = D.fwd;
+  a.bwd = D.bwd;
+  a.dig = s.dig;
+  a.uexp = s.uexp;
+  a.sys = pl.sys_dev;
+  a.items = L.items_dev;
+  a.part = reinterpret_cast<double *>(pl.partial);
+  a.ybuf = pl.yscratch;
+  a.counter = pl.counter;
+  a.nrows = pl.nrows;
+  a.nitems = L.nitems;
+  a.tiles = tiles;
+  a.nwin = (pl.P + kWin - 1) / kWin;
+  a.lmax = pl.lmax;
+  const int ctas = std::min(pl.num_sms * kCtas, (L.nitems + 3) / 4);
+  solve_digits_kernel<kCtas><<<(unsigned)std::max(1, ctas), 128, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_finish_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, double2 *sout, int B,
+                                 cudaStream_t st) {
+  FinishArgs f;
+  f.part = reinterpret_cast<const double *>(pl.partial);
+  f.sin = sin;
+  f.w = adjoint ? pl.w_adj : pl.w_fwd;
+  f.sout = sout;
+  f.rflags = pl.rflags_dev;
+  f.m_of = pl.m_of_dev;
+  f.sys = pl.sys_dev;
+  f.sphi = adjoint ? pl.sphi_adj : pl.sphi_fwd;
+  f.nspec = pl.nspec;
+  f.nrows = pl.nrows;
+  f.B = B;
+  f.tiles = tiles_of(B);
+  f.slots = L.slots;
+  f.N = pl.N;
+  const int64_t total = 3 * pl.nspec * B;
+  digit_finish_kernel<<<(unsigned)std::min<int64_t>((total + 255) / 256, 1 << 20), 256, 0, st>>>(f);
+  return cudaGetLastError();
+}
+
+}  // namespace rexi

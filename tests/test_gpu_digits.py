@@ -1,0 +1,132 @@
+"""The digit solve (both contractions of the shifted solves on the tensor cores, exactly)
+against the pole-slot solve, the oracle and its own linearity."""
+import numpy as np
+import pytest
+
+from oracle import rexi_coeffs as rc
+from oracle import step as ostep
+from oracle.swe import Consts
+from paper_1812_03431_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-10    # against the oracle, as for every binary64 path
+ORDER = 1e-13  # against the pole-slot solve: the same sums in another order
+C = Consts()
+
+
+def fieldwise(a, b):
+    return max(np.linalg.norm(a[:, f] - b[:, f]) / max(np.linalg.norm(b[:, f]), 1e-300) for f in range(3))
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    from paper_1812_03431_gb300 import rexi
+    rexi.load()
+    return torch, rexi
+
+
+def poles(P):
+    """The middle P poles of a longer set (any P runs)."""
+    al, be, _ = rc.rexi_coefficients(64, 0.2)
+    k = (al.size - P) // 2
+    return al[k:k + P], be[k:k + P]
+
+
+def spectral_plan(rexi, N, B, al, be, tau=1800.0, **k):
+    nlon = next(n for n in (12, 24, 48, 72, 96, 144, 192) if n >= 3 * N + 3)
+    return rexi.Plan(N, nlon // 2, nlon, tau=tau, max_batch=B, layout="spectral", alpha=al, beta=be, **k)
+
+
+# truncations down to one row per system; pole counts around a window of eight; batches around
+# a tile of eight states
+@pytest.mark.parametrize("N,P,B", [(1, 1, 5), (1, 9, 8), (2, 7, 9), (3, 8, 5), (8, 16, 16), (13, 17, 7), (21, 31, 17),
+                                   (42, 57, 8), (63, 149, 6)])
+def test_matches_slot_solve(env, N, P, B):
+    torch, rexi = env
+    al, be = poles(P)
+    x = torch.from_numpy(inputs.random_spectral(N, B, 7)).cuda()
+    plan = spectral_plan(rexi, N, B, al, be)
+    got, adj = plan.step(x).cpu().numpy(), plan.step_adjoint(x).cpu().numpy()  # the default above four states
+    for slots in (1, 2, 0, 1000):
+        assert plan.set_pole_slots(B, slots, 5) >= 1
+        y = plan.step(x).cpu().numpy()
+        np.testing.assert_array_equal(y, plan.step(x).cpu().numpy())  # a fixed order
+        assert fieldwise(y, got) < ORDER
+        assert fieldwise(plan.step_adjoint(x).cpu().numpy(), adj) < ORDER
+    plan.set_pole_slots(B, 1, 0)
+    assert fieldwise(got, plan.step(x).cpu().numpy()) < ORDER
+    assert fieldwise(adj, plan.step_adjoint(x).cpu().numpy()) < ORDER
+    plan.close()
+
+
+@pytest.mark.parametrize("N,M,B,tau", [(15, 32, 5, 3600.0), (31, 48, 10, 1200.0)])
+def test_matches_oracle(env, N, M, B, tau):
+    torch, rexi = env
+    al, be, _ = rc.rexi_coefficients(M, 0.2)
+    S = inputs.random_spectral(N, B, 5)
+    plan = spectral_plan(rexi, N, B, al, be, tau)
+    ref = ostep.rexi_step_spectral(S, N, al, be, tau, C)
+    assert fieldwise(plan.step(torch.from_numpy(S).cuda()).cpu().numpy(), ref) < TOL
+    plan.close()
+
+
+def test_states_keep_their_own_scale(env):
+    """Every group's fixed-point scale is a power of two of its own, so a state times a power of
+    two gives that power times the result, bit for bit, whatever the other states hold."""
+    torch, rexi = env
+    N, B = 21, 11
+    al, be = poles(45)
+    S = inputs.random_spectral(N, B, 9)
+    scale = 2.0 ** np.array([0, 300, -300, 0, 60, -60, 500, 1, -1, 0, -450])
+    T = S * scale[:, None, None]
+    T[3] = 0.0
+    plan = spectral_plan(rexi, N, B, al, be)
+    a = plan.step(torch.from_numpy(S).cuda()).cpu().numpy() * scale[:, None, None]
+    a[3] = 0.0
+    np.testing.assert_array_equal(plan.step(torch.from_numpy(T).cuda()).cpu().numpy(), a)
+    # fields of one state far apart in scale: no worse than the slot solve against the oracle
+    S[:, 1:] *= 1e-9
+    plan2 = spectral_plan(rexi, N, B, al, be, pole_slots=4)
+    x = torch.from_numpy(S).cuda()
+    assert fieldwise(plan.step(x).cpu().numpy(), plan2.step(x).cpu().numpy()) < ORDER
+    plan.close()
+    plan2.close()
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+def test_values_that_are_not_finite_stay_in_their_state_and_order(env, value):
+    torch, rexi = env
+    N, B = 21, 9
+    al, be = poles(45)
+    S = inputs.random_spectral(N, B, 11)
+    plan = spectral_plan(rexi, N, B, al, be)
+    clean = plan.step(torch.from_numpy(S).cuda()).cpu().numpy()
+    bad = S.copy()
+    bad[4, 2, (N + 1) + 6] = value  # delta of state 4, m = 1, n = 7
+    x = torch.from_numpy(bad).cuda()
+    got = plan.step(x).cpu().numpy()
+    plan.set_pole_slots(B, 4, 0)
+    ref = plan.step(x).cpu().numpy()
+    np.testing.assert_array_equal(np.isfinite(got), np.isfinite(ref))
+    keep = np.arange(B) != 4
+    np.testing.assert_array_equal(got[keep], clean[keep])
+    fine = np.isfinite(got[4])
+    np.testing.assert_array_equal(got[4][fine], clean[4][fine])
+    plan.close()
+
+
+def test_poles_of_unlike_scale_keep_the_other_solves(env):
+    """Couplings of one pole that differ by more than eight bits from the middle pole's stay with
+    the binary64 kernels, by default and on request."""
+    torch, rexi = env
+    N, B = 13, 8
+    al = np.array([-1e-3 + 0j, -1e3 + 1j, -1.0 + 2j])
+    be = np.array([1e-3 + 0j, 1.0 + 1j, 0.5 - 1j])
+    x = torch.from_numpy(inputs.random_spectral(N, B, 3)).cuda()
+    plan, slots = spectral_plan(rexi, N, B, al, be), spectral_plan(rexi, N, B, al, be, pole_slots=1)
+    assert fieldwise(plan.step(x).cpu().numpy(), slots.step(x).cpu().numpy()) < ORDER
+    with pytest.raises(rexi.RexiError):
+        plan.set_pole_slots(B, 0, 5)
+    plan.close()
+    slots.close()
