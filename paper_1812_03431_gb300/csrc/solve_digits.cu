@@ -29,13 +29,16 @@
 // cycles each, about a third of the FP64 time beside them, so their rate does not bound it.
 //
 // Measured on GB300 (solve and the sum of the slots, against the pole-slot solve and its
-// reduction): T341, 535 poles, 16 states 12.0 / 30.0 ms; T127, 535 poles, 64 states 6.6 / 17.0;
-// T85, 215 poles, 5 states 0.20 / 0.62.  What bounds it now: the FP64 unit for 7.7 of the 11.5 ms
-// at T341 (9 instructions per state, pole and row at 64 cycles, one of them the running sum's
-// addition).
+// reduction): T341, 535 poles, 16 states 10.2 / 30.0 ms; T127, 535 poles, 64 states 5.7 / 17.0;
+// T85, 215 poles, 5 states 0.18 / 0.62.  What bounds it now: the FP64 unit, 78 % busy (ncu, T170 x
+// 16) with 9 instructions per state, pole and row at 64 cycles, one of them the running sum's
+// addition; the rest is waiting that 16 warps per SM do not cover (12 warps: 12.1 ms; 8: 16.0).
 //
-// A warp takes 8 states x 8 poles (lane: state lane / 4, poles lane % 4 and lane % 4 + 4) of
-// one (m, parity) system, window by window of 8 poles, over all rows.
+// A warp takes 8 states x 8 poles (lane: state lane / 4, poles 2 (lane % 4) and the next) of one
+// (m, parity) system, window by window of 8 poles, over all rows.  Real and imaginary rows of
+// a product take their operand as (re, -im) and (im, re): the couplings' products through two
+// forms of the inputs' digits, the weighted sums by keeping the real and the imaginary digits
+// of a pole pair in words of their own, which the two kinds of row load in opposite order.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -55,7 +58,6 @@ constexpr int kBwdRec = 1024 + 128;        // per (row, window): weight digits a
 constexpr int kStateRec = 1024;            // per (row, tile): input digits
 constexpr int kNotFinite = 1 << 20;        // exponent of a row input that holds an Inf or NaN
 constexpr int kMaxSpread = 8;              // bits by which a pole's couplings may differ in scale
-constexpr float kMagic = 12582912.0f;      // 1.5 2^23
 
 __device__ __forceinline__ int bexp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
@@ -94,32 +96,50 @@ __device__ __forceinline__ void digits(long long re, long long im, unsigned (&w)
 // t 2^e in binary64 (round half away from zero), on the integer pipe; results below 2^-1022
 // are zero, e of a group that is not finite gives NaN
 __device__ __forceinline__ double fixed_to_double(long long t, int e) {
-  const unsigned long long m = t < 0 ? (unsigned long long)(-t) : (unsigned long long)t;
-  const int lz = __clzll((long long)m);
-  const unsigned long long f = m << (lz & 63);
-  const unsigned long long r = (f >> 11) + ((f >> 10) & 1);
-  const int be = 1023 + 63 + e - lz;
-  unsigned hi = (unsigned)(r >> 32) + ((unsigned)(be - 1) << 20), lo = (unsigned)r;
-  if (m == 0 || be <= 0) hi = lo = 0;
-  if (be >= 2047 && (m != 0 || e >= kNotFinite / 2)) {
-    hi = e >= kNotFinite / 2 ? 0x7ff80000u : 0x7ff00000u;
+  const int sign = (int)(t >> 63);
+  const unsigned long long m = (unsigned long long)((t ^ (long long)sign) - (long long)sign);
+  unsigned h = (unsigned)(m >> 32), l = (unsigned)m;
+  int be = 1023 + 62 + e;  // the biased exponent less one of a number with bit 63 set
+  if (h == 0) {
+    h = l;
+    l = 0;
+    be -= 32;
+  }
+  const int lz = __clz((int)h);  // 32 where t is zero: the shifts take it as 0
+  const unsigned fh = __funnelshift_l(l, h, lz), fl = l << (lz & 31);
+  be -= lz;
+  const unsigned long long r =
+      ((unsigned long long)(fh >> 11) << 32 | __funnelshift_r(fl, fh, 11)) + ((fl >> 10) & 1);
+  unsigned hi = (unsigned)(r >> 32) + ((unsigned)be << 20), lo = (unsigned)r;
+  if ((unsigned)be >= 2046u || fh == 0) {
+    const bool nan = e >= kNotFinite / 2;
+    hi = nan ? 0x7ff80000u : (be >= 2046 && fh != 0 ? 0x7ff00000u : 0u);
     lo = 0;
   }
-  return __hiloint2double((int)(hi | ((unsigned)((unsigned long long)t >> 32) & 0x80000000u)), (int)lo);
+  return __hiloint2double((int)(hi | ((unsigned)sign & 0x80000000u)), (int)lo);
 }
 
+// An accumulator's bits are kMagicBits + its sum (kEvenBits for those that start at kEven), so
+// that of two neighbouring sums 256 bits(even) + bits(odd) = 256 s_c + s_{c+1} + 2^31.
+constexpr float kMagic = 12582912.0f;  // 1.5 2^23
+constexpr float kEven = 11845632.0f;
+constexpr unsigned kMagicBits = 0x4B400000u, kEvenBits = 0x4B34C000u;
+static_assert(kEvenBits * 256u + kMagicBits == 0x80000000u, "the pair's offset");
+
+__device__ __forceinline__ unsigned bits(float x) { return (unsigned)__float_as_int(x); }
+
 // sum of s_c 2^(-8c), c = 0..7, in units of 2^-46; the pairs (s_0, s_1) ... (s_6, s_7) come as
-// 256 s_c + s_{c+1}
-__device__ __forceinline__ long long weigh(int h, int m, int l, int q) {
-  const long long t = ((long long)h << 32) + (long long)m * 65536 + l;
-  return (t << 6) + ((q + 512) >> 10);
+// 256 s_c + s_{c+1} + 2^31
+__device__ __forceinline__ long long weigh(unsigned h, unsigned m, unsigned l, unsigned q) {
+  const unsigned long long t = ((unsigned long long)h << 32 | l) + (unsigned long long)m * 65536u;
+  return (long long)((t << 6) + (q >> 10) - ((1ull << 53) + (1ull << 37) + (1ull << 21)));
 }
 
 __device__ __forceinline__ void mma_first(float (&d)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0,
-                                          unsigned b1) {
+                                          unsigned b1, float start = kMagic) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
       : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(kMagic));
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(start));
 }
 __device__ __forceinline__ void mma_add(float (&d)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0,
                                         unsigned b1) {
@@ -206,8 +226,12 @@ __global__ void digit_factor_kernel(SetupArgs a) {
     if (m == 0x7ff) bad = true;
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    unsigned d[8];  // seven digits: rounded to the nearest multiple of the eighth's weight
-    digits((to_fixed(x.x, m - bexp(x.x)) + 128) & ~255ll, (to_fixed(x.y, m - bexp(x.y)) + 128) & ~255ll, d);
+    // seven digits (rounded to the nearest multiple of the eighth's weight), the real parts of
+    // poles 2 q and 2 q + 1 by the even thread, their imaginary parts by the odd one
+    const long long re = (to_fixed(x.x, m - bexp(x.x)) + 128) & ~255ll, im = (to_fixed(x.y, m - bexp(x.y)) + 128) & ~255ll;
+    const long long other = __shfl_xor_sync(0xffffffffu, p8 & 1 ? re : im, 1);
+    unsigned d[8];
+    digits(p8 & 1 ? other : re, p8 & 1 ? im : other, d);
     if (live) {
       uint4 *o = reinterpret_cast<uint4 *>(br + (s * kWin + p8) * 32);
       o[0] = make_uint4(d[0], d[1], d[2], d[3]);
@@ -280,21 +304,133 @@ __device__ __forceinline__ void load_words(const char *p, unsigned (&w)[8]) {
 }
 __device__ __forceinline__ double2 ldd(const char *p) { return __ldg(reinterpret_cast<const double2 *>(p)); }
 __device__ __forceinline__ void prefetch(const void *p) { asm volatile("prefetch.global.L1 [%0];" : : "l"(p)); }
-__device__ __forceinline__ int bits(float x) { return __float_as_int(x); }
+__device__ __forceinline__ unsigned half2_fma(unsigned a, unsigned b, unsigned c) {
+  unsigned r;
+  asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+  return r;
+}
 
-constexpr unsigned kB = 0x4B400000u;  // bits of kMagic
+// |x| as to_fixed gives it, E the exponent (biased) of its group's leading bit
+__device__ __forceinline__ unsigned long long magnitude(double x, int E) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int d = min(E - (int)((hi >> 20) & 0x7ff), 63);
+  unsigned h = __funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, 9), l = lo << 9;
+  if (d >= 32) {
+    l = h;
+    h = 0;
+  }
+  return (unsigned long long)(h >> (d & 31)) << 32 | __funnelshift_r(l, h, d & 31);
+}
+
+// the eight digits of two numbers of one group, as fp16 pairs
+__device__ __forceinline__ void digits_of(double a, double b, int E, unsigned (&w)[8]) {
+  const unsigned long long ua = magnitude(a, E) + 0x8080808080808080ull, ub = magnitude(b, E) + 0x8080808080808080ull;
+  const unsigned sign = __byte_perm((unsigned)__double2hiint(a), (unsigned)__double2hiint(b), 0x7632) & 0x80008000u;
+  const unsigned one = sign | 0x3c003c00u, less = sign ^ 0xe480e480u;  // +-1 and -+1152
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const unsigned x = h == 0 ? (unsigned)(ua >> 32) : (unsigned)ua, y = h == 0 ? (unsigned)(ub >> 32) : (unsigned)ub;
+    const unsigned top = __byte_perm(x, y, 0x7362), low = __byte_perm(x, y, 0x5140);
+    w[4 * h + 0] = half2_fma(__byte_perm(top, 0x64646464u, 0x4342), one, less);
+    w[4 * h + 1] = half2_fma(__byte_perm(top, 0x64646464u, 0x4140), one, less);
+    w[4 * h + 2] = half2_fma(__byte_perm(low, 0x64646464u, 0x4342), one, less);
+    w[4 * h + 3] = half2_fma(__byte_perm(low, 0x64646464u, 0x4140), one, less);
+  }
+}
 
 // rows whose data is brought into the caches ahead of use
 constexpr int kAhead = 2;
+
+// The right-hand sides of one row for the lane's two poles: digits of the inputs (rows of the
+// product: states, real rows above imaginary ones) times those of the couplings (columns:
+// poles), one accumulator per sum of digit places, two digit pairs per MMA.
+__device__ __forceinline__ void right_hand_sides(const char *f, const char *dig, const int *uexp, int lane, double2 (&r)[2]) {
+  unsigned p[8], v[8], z[8];
+  load_words(dig, p);
+  load_words(f + lane * 32, v);
+  const int U = __ldg(uexp) - 56;
+  const int2 e = __ldg(reinterpret_cast<const int2 *>(f + 1152) + (lane & 3));
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    z[j] = __byte_perm(p[j], 0, 0x1032);  // (im, re): imaginary rows
+    p[j] ^= 0x80000000u;                  // (re, -im): real rows
+  }
+  unsigned pair[4][4];
+#pragma unroll
+  for (int c = 0; c < 8; c += 2) {
+    float s[2][4];
+#pragma unroll
+    for (int o = 0; o < 2; ++o)
+#pragma unroll
+      for (int i = 0; i <= c + o; i += 2) {
+        const int j = c + o - i;
+        const unsigned a2 = j > 0 ? p[i < 7 ? i + 1 : 7] : 0u, a3 = j > 0 ? z[i < 7 ? i + 1 : 7] : 0u, b1 = j > 0 ? v[j > 0 ? j - 1 : 0] : 0u;
+        if (i == 0) mma_first(s[o], p[i], z[i], a2, a3, v[j], b1, o == 0 ? kEven : kMagic);
+        else mma_add(s[o], p[i], z[i], a2, a3, v[j], b1);
+      }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) pair[c / 2][k] = bits(s[0][k]) * 256u + bits(s[1][k]);
+  }
+#pragma unroll
+  for (int g = 0; g < 2; ++g) {
+    const int ee = U + (g ? e.y : e.x);
+    r[g] = make_double2(fixed_to_double(weigh(pair[0][g], pair[1][g], pair[2][g], pair[3][g]), ee),
+                        fixed_to_double(weigh(pair[0][g + 2], pair[1][g + 2], pair[2][g + 2], pair[3][g + 2]), ee));
+  }
+}
+
+// Adds to the lane's two running sums (states 2 q and 2 q + 1 of one stream's real or
+// imaginary part) the weighted sums over the window's eight poles of x, a row's solutions:
+// digits of the weights (rows: streams) times those of x (columns: states).
+__device__ __forceinline__ double2 weighted_sums(const char *f, const double2 (&x)[2], int lane, double2 sum) {
+  const int q = lane & 3;
+  const bool im_row = (lane >> 2) & 1;
+  // a real row takes (re, -im) of the weights against (re, im) of x, an imaginary one (im, re)
+  unsigned lo[8], hi[8];
+  const char *wr = f + ((lane >> 3) * 4 + q) * 64;
+  load_words(wr + (im_row ? 32 : 0), lo);
+  load_words(wr + (im_row ? 0 : 32), hi);
+  const int We = (int)lo[7];
+  const unsigned flip = im_row ? 0u : 0x80008000u;
+#pragma unroll
+  for (int j = 0; j < 7; ++j) hi[j] ^= flip;
+  lo[7] = hi[7] = 0;
+  int E = 0;
+#pragma unroll
+  for (int g = 0; g < 2; ++g) E = max(E, max(__double2hiint(x[g].x) & 0x7fffffff, __double2hiint(x[g].y) & 0x7fffffff));
+  E = max(E, __shfl_xor_sync(0xffffffffu, E, 1));
+  E = max(E, __shfl_xor_sync(0xffffffffu, E, 2)) >> 20;
+  if (E < 64) E += 4096;  // groups below 2^-959 are taken as zero
+  unsigned re[8], im[8];
+  digits_of(x[0].x, x[1].x, E, re);
+  digits_of(x[0].y, x[1].y, E, im);
+  float s[8][4];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) mma_first(s[c], lo[0], lo[1], hi[0], hi[1], re[c], im[c]);
+#pragma unroll
+  for (int i = 2; i < 8; i += 2)
+#pragma unroll
+    for (int c = i; c < 8; ++c) mma_add(s[c], lo[i], lo[i + 1], hi[i], hi[i + 1], re[c - i], im[c - i]);
+  double r[2];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const int Es = __shfl_sync(0xffffffffu, E, (q * 2 + c) * 4);  // the exponent of state 2 q + c
+    // digit places j come from the upper rows of accumulator j and the lower ones of j - 1
+    unsigned at[8];
+    at[0] = bits(s[0][c]) + (0x00800000u - kMagicBits);
+#pragma unroll
+    for (int j = 1; j < 8; ++j) at[j] = bits(s[j][c]) + bits(s[j - 1][c + 2]) + ((j & 1 ? 0u : 0x00800000u) - 2u * kMagicBits);
+    r[c] = fixed_to_double(weigh(at[0] * 256u + at[1], at[2] * 256u + at[3], at[4] * 256u + at[5], at[6] * 256u + at[7]),
+                           (Es & 4095) == 0x7ff ? kNotFinite : We + (Es & 4095) - 1023 - 56);
+  }
+  return make_double2(sum.x + r[0], sum.y + r[1]);
+}
 
 template <int CTAS>
 __global__ void __launch_bounds__(128, CTAS) solve_digits_kernel(SweepArgs a) {
   const int lane = threadIdx.x & 31, q = lane & 3;
   const int wslot = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   double2 *yb = a.ybuf + (int64_t)wslot * a.lmax * 64 + lane;
-  // a real row of the complex products takes (re, -im) of the factor, an imaginary one (im, re)
-  const bool im_row = (lane >> 2) & 1;
-  const unsigned sel = im_row ? 0x1032u : 0x3210u, flip = im_row ? 0u : 0x80000000u;
   for (;;) {
     unsigned it = 0;
     if (lane == 0) it = atomicAdd(a.counter, 1u);
@@ -304,109 +440,62 @@ __global__ void __launch_bounds__(128, CTAS) solve_digits_kernel(SweepArgs a) {
     const int4 sy = a.sys[item.x];
     const int len = sy.z, w0 = item.z & 0xffff, w1 = w0 + (item.z >> 16);
     const int64_t row0 = sy.w;
-    const char *dig = a.dig + (row0 * a.tiles + item.y) * kStateRec + lane * 32;
-    const int *uexp = a.uexp + (row0 * a.tiles + item.y) * kTile + (lane >> 2);
-    const int64_t dstep = (int64_t)a.tiles * kStateRec;
-    double2 *part = reinterpret_cast<double2 *>(a.part + (((int64_t)item.w * a.nrows + row0) * a.tiles + item.y) * 64) + lane;
-    const int64_t pstep = (int64_t)a.tiles * 32;
+    const char *dig0 = a.dig + (row0 * a.tiles + item.y) * kStateRec + lane * 32;
+    const int *uexp0 = a.uexp + (row0 * a.tiles + item.y) * kTile + (lane >> 2);
+    const int dstep = a.tiles * kStateRec, ustep = a.tiles * kTile;
+    double2 *part0 = reinterpret_cast<double2 *>(a.part + (((int64_t)item.w * a.nrows + row0) * a.tiles + item.y) * 64) + lane;
+    const int pstep = a.tiles * 32;
     for (int w = w0; w < w1; ++w) {
-      const char *fr = a.fwd + (row0 * a.nwin + (int64_t)w * len) * kFwdRec;
-      double2 y[2] = {make_double2(0, 0), make_double2(0, 0)};
-      for (int i = 0; i < len; ++i) {
-        if (i + kAhead < len) {
-          const char *nf = fr + (int64_t)(i + kAhead) * kFwdRec, *nd = dig + (i + kAhead) * dstep - lane * 32;
-          if (lane < 10) prefetch(nf + lane * 128);
-          else if (lane >= 16 && lane < 24) prefetch(nd + (lane - 16) * 128);
-        }
-        const char *f = fr + (int64_t)i * kFwdRec;
-        unsigned p[8];
-        load_words(dig + i * dstep, p);
-        const int U = __ldg(uexp + (int64_t)i * a.tiles * kTile);
-#pragma unroll
-        for (int g = 0; g < 2; ++g) {
-          unsigned v[8];
-          load_words(f + ((g * 4 + (lane >> 3)) * 4 + q) * 32, v);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) v[j] = __byte_perm(v[j], 0, sel) ^ flip;
-          float s0[4], s2[4], s4[4], s6[4];
-          mma_first(s0, 0u, p[0], p[0], p[1], v[1], v[0]);
-          mma_first(s2, 0u, p[0], p[0], p[1], v[3], v[2]);
-          mma_first(s4, 0u, p[0], p[0], p[1], v[5], v[4]);
-          mma_first(s6, 0u, p[0], p[0], p[1], v[7], v[6]);
-          mma_add(s2, p[1], p[2], p[2], p[3], v[1], v[0]);
-          mma_add(s4, p[1], p[2], p[2], p[3], v[3], v[2]);
-          mma_add(s6, p[1], p[2], p[2], p[3], v[5], v[4]);
-          mma_add(s4, p[3], p[4], p[4], p[5], v[1], v[0]);
-          mma_add(s6, p[3], p[4], p[4], p[5], v[3], v[2]);
-          mma_add(s6, p[5], p[6], p[6], p[7], v[1], v[0]);
-          const int e = U + __ldg(reinterpret_cast<const int *>(f + 1152) + g * 4 + q) - 56;
-          constexpr unsigned K = kB * 256u + kB;
-          double r[2];
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            const int h = (int)((unsigned)bits(s0[c]) * 256u + (unsigned)bits(s0[c + 2]) - K);
-            const int m = (int)((unsigned)bits(s2[c]) * 256u + (unsigned)bits(s2[c + 2]) - K);
-            const int l = (int)((unsigned)bits(s4[c]) * 256u + (unsigned)bits(s4[c + 2]) - K);
-            const int o = (int)((unsigned)bits(s6[c]) * 256u + (unsigned)bits(s6[c + 2]) - K);
-            r[c] = fixed_to_double(weigh(h, m, l, o), e);
+      {  // forward: y_i = r_i - l y_{i-1}; the next row's r is formed beside the FMAs of this one
+        const char *f = a.fwd + (row0 * a.nwin + (int64_t)w * len) * kFwdRec, *dig = dig0;
+        const int *uexp = uexp0;
+        double2 *yp = yb;
+        double2 y[2] = {make_double2(0, 0), make_double2(0, 0)}, r[2];
+        right_hand_sides(f, dig, uexp, lane, r);
+        for (int i = 0; i < len; ++i) {
+          const double2 l0 = ldd(f + 1024 + q * 32), l1 = ldd(f + 1040 + q * 32);
+          if (i + kAhead < len) {
+            if (lane < 10) prefetch(f + kAhead * kFwdRec + lane * 128);
+            else if (lane >= 16 && lane < 24) prefetch(dig + kAhead * dstep + (lane - 16) * 128 - lane * 32);
           }
-          y[g] = cfms(make_double2(r[0], r[1]), ldd(f + 1024 + (g * 4 + q) * 16), y[g]);
-          yb[(i * 2 + g) * 32] = y[g];
+          y[0] = cfms(r[0], l0, y[0]);
+          y[1] = cfms(r[1], l1, y[1]);
+          f += kFwdRec;
+          dig += dstep;
+          uexp += ustep;
+          if (i + 1 < len) right_hand_sides(f, dig, uexp, lane, r);
+          yp[0] = y[0];
+          yp[32] = y[1];
+          yp += 64;
         }
       }
-      const char *br = a.bwd + (row0 * a.nwin + (int64_t)w * len) * kBwdRec;
-      double2 x[2] = {make_double2(0, 0), make_double2(0, 0)};
-      for (int i = len - 1; i >= 0; --i) {
-        if (i >= kAhead) {
-          const char *nb = br + (int64_t)(i - kAhead) * kBwdRec;
-          if (lane < 10) prefetch(nb + (lane < 9 ? lane * 128 : kBwdRec - 16));
-          else if (lane >= 16 && lane < 24) prefetch(reinterpret_cast<const char *>(yb - lane + (i - kAhead) * 64) + (lane - 16) * 128);
-          else if (lane >= 24 && lane < 28 && w > w0) prefetch(reinterpret_cast<const char *>(part - lane + (i - kAhead) * pstep) + (lane - 24) * 128);
+      {  // backward: x_i = y_i - Chat x_{i+1}; the sums of row i + 1 beside the FMAs of row i
+        const char *f = a.bwd + (row0 * a.nwin + (int64_t)(w + 1) * len - 1) * kBwdRec;
+        const double2 *yp = yb + (len - 1) * 64;
+        double2 *part = part0 + (int64_t)(len - 1) * pstep;
+        double2 x[2] = {yp[0], yp[32]};  // Chat is zero in the last row
+        for (int i = len - 1; i >= 0; --i) {
+          if (i >= kAhead) {
+            if (lane < 10) prefetch(f - kAhead * kBwdRec + (lane < 9 ? lane * 128 : kBwdRec - 16));
+            else if (lane >= 16 && lane < 24) prefetch(reinterpret_cast<const char *>(yp - lane - kAhead * 64) + (lane - 16) * 128);
+            else if (lane >= 24 && lane < 28 && w > w0)
+              prefetch(reinterpret_cast<const char *>(part - lane - (int64_t)kAhead * pstep) + (lane - 24) * 128);
+          }
+          double2 sum = make_double2(0, 0);
+          if (w > w0) sum = *part;
+          double2 xn[2] = {x[0], x[1]};
+          const char *g = f;
+          f -= kBwdRec;
+          yp -= 64;
+          if (i > 0) {
+            xn[0] = cfms(yp[0], ldd(f + 1024 + q * 32), x[0]);
+            xn[1] = cfms(yp[32], ldd(f + 1040 + q * 32), x[1]);
+          }
+          *part = weighted_sums(g, x, lane, sum);
+          part -= pstep;
+          x[0] = xn[0];
+          x[1] = xn[1];
         }
-        const char *f = br + (int64_t)i * kBwdRec;
-        double2 sum = make_double2(0, 0);
-        if (w > w0) sum = part[i * pstep];
-        int E = 0;
-#pragma unroll
-        for (int g = 0; g < 2; ++g) {
-          x[g] = cfms(yb[(i * 2 + g) * 32], ldd(f + 1024 + (g * 4 + q) * 16), x[g]);
-          E = max(E, max(__double2hiint(x[g].x) & 0x7fffffff, __double2hiint(x[g].y) & 0x7fffffff));
-        }
-        E = max(E, __shfl_xor_sync(0xffffffffu, E, 1));
-        E = max(E, __shfl_xor_sync(0xffffffffu, E, 2)) >> 20;
-        unsigned d0[8], d1[8];
-        digits(to_fixed(x[0].x, E - bexp(x[0].x)), to_fixed(x[0].y, E - bexp(x[0].y)), d0);
-        digits(to_fixed(x[1].x, E - bexp(x[1].x)), to_fixed(x[1].y, E - bexp(x[1].y)), d1);
-        unsigned u[8], v[8];
-        load_words(f + ((lane >> 3) * kWin + q) * 32, u);
-        load_words(f + ((lane >> 3) * kWin + q + 4) * 32, v);
-        const int We = (int)u[7];
-#pragma unroll
-        for (int j = 0; j < 7; ++j) {
-          u[j] = __byte_perm(u[j], 0, sel) ^ flip;
-          v[j] = __byte_perm(v[j], 0, sel) ^ flip;
-        }
-        u[7] = v[7] = 0;
-        float s[8][4];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) mma_first(s[c], u[0], u[1], v[0], v[1], d0[c], d1[c]);
-#pragma unroll
-        for (int c = 2; c < 8; ++c) mma_add(s[c], u[2], u[3], v[2], v[3], d0[c - 2], d1[c - 2]);
-#pragma unroll
-        for (int c = 4; c < 8; ++c) mma_add(s[c], u[4], u[5], v[4], v[5], d0[c - 4], d1[c - 4]);
-#pragma unroll
-        for (int c = 6; c < 8; ++c) mma_add(s[c], u[6], u[7], v[6], v[7], d0[c - 6], d1[c - 6]);
-        double r[2];
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const int Es = __shfl_sync(0xffffffffu, E, (q * 2 + c) * 4);  // the exponent of state 2 q + c
-          auto at = [&](int j) { return (unsigned)bits(s[j][c]) + (j ? (unsigned)bits(s[j ? j - 1 : 0][c + 2]) : 0u); };
-          constexpr unsigned K0 = kB * 256u + 2u * kB, K = 2u * kB * 256u + 2u * kB;
-          const int h = (int)(at(0) * 256u + at(1) - K0), m = (int)(at(2) * 256u + at(3) - K);
-          const int l = (int)(at(4) * 256u + at(5) - K), o = (int)(at(6) * 256u + at(7) - K);
-          r[c] = fixed_to_double(weigh(h, m, l, o), Es == 0x7ff ? kNotFinite : We + Es - 1023 - 56);
-        }
-        part[i * pstep] = make_double2(sum.x + r[0], sum.y + r[1]);
       }
     }
   }
@@ -460,8 +549,8 @@ __global__ void digit_finish_kernel(FinishArgs a) {
   }
 }
 
-// resident CTAs per SM: 12 warps at 168 registers
-constexpr int kCtas = 3;
+// resident CTAs per SM: 16 warps at 128 registers
+constexpr int kCtas = 4;
 
 int tiles_of(int B) { return (B + kTile - 1) / kTile; }
 
