@@ -126,7 +126,7 @@ typedef struct {
                            fused solve that keeps the pole sum on chip (one kernel, every
                            output written once), for larger ones the digit solve (the
                            contractions exactly on the tensor cores; needs device memory
-                           for 292 B per row and pole and poles of like scale), else the
+                           for 164 B per row and pole and poles of like scale), else the
                            pole-slot solve (rexi_tune picks per batch); > 0: the pole-slot solve with this many pole groups
                            summed separately, then reduced in slot order (a deterministic
                            tuning knob, any >= 1) */

@@ -103,8 +103,8 @@ void free_plan(Plan *pl);
 
 // The smallest batch the digit solve takes by default: its warps carry tiles of eight states;
 // five of them still take a third of the pole-slot solve's time (T85: 0.20 / 0.62 ms); up to
-// four the fused solve is the default.  Then the most device memory its factors may take: 2336 B per
-// row and eight poles, twice the binary64 factors.
+// four the fused solve is the default.  Then the most device memory its factors may take: 1312 B per
+// row and eight poles, 1.14 times the binary64 factors.
 constexpr int kDigitMinBatch = 5;
 constexpr size_t kDigitMostBytes = (size_t)32 << 30;
 

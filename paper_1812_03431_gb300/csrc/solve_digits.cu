@@ -53,8 +53,8 @@ namespace {
 
 constexpr int kTile = 8;                   // states per warp
 constexpr int kWin = 8;                    // poles per window
-constexpr int kFwdRec = 1024 + 128 + 32;   // per (row, window): coupling digits, l, exponents
-constexpr int kBwdRec = 1024 + 128;        // per (row, window): weight digits and exponents, Chat
+constexpr int kLOff = 512, kEOff = 640, kFwdRec = 672;  // per (row, window): coupling digits, l, exponents
+constexpr int kCOff = 512, kBwdRec = 640;  // per (row, window): weight digits and exponents, Chat
 constexpr int kStateRec = 1024;            // per (row, tile): input digits
 constexpr int kNotFinite = 1 << 20;        // exponent of a row input that holds an Inf or NaN
 constexpr int kMaxSpread = 8;              // bits by which a pole's couplings may differ in scale
@@ -91,6 +91,16 @@ __device__ __forceinline__ void digits(long long re, long long im, unsigned (&w)
     w[4 * h + 2] = half2_sub(__byte_perm(low, 0x64646464u, 0x4342), 0x64806480u);
     w[4 * h + 3] = half2_sub(__byte_perm(low, 0x64646464u, 0x4140), 0x64806480u);
   }
+}
+
+// the same digits as stored: biased bytes, each place's pair (re, im) side by side, most
+// significant first
+__device__ __forceinline__ uint4 packed_digits(long long re, long long im) {
+  const unsigned long long ur = (unsigned long long)re + 0x8080808080808080ull;
+  const unsigned long long ui = (unsigned long long)im + 0x8080808080808080ull;
+  const unsigned rh = (unsigned)(ur >> 32), rl = (unsigned)ur, ih = (unsigned)(ui >> 32), il = (unsigned)ui;
+  return make_uint4(__byte_perm(rh, ih, 0x6273), __byte_perm(rh, ih, 0x4051), __byte_perm(rl, il, 0x6273),
+                    __byte_perm(rl, il, 0x4051));
 }
 
 // t 2^e in binary64 (round half away from zero), on the integer pipe; results below 2^-1022
@@ -203,18 +213,14 @@ __global__ void digit_factor_kernel(SetupArgs a) {
   for (int j = 0; j < 4; ++j) {
     const int e = emax(v[j]);
     if (e && E - (e - ve[j]) > kMaxSpread) bad = true;
-    unsigned d[8];
-    digits(to_fixed(v[j].x, E - (bexp(v[j].x) - ve[j])), to_fixed(v[j].y, E - (bexp(v[j].y) - ve[j])), d);
-    if (live) {
-      uint4 *o = reinterpret_cast<uint4 *>(fr + (p8 * 4 + j) * 32);
-      o[0] = make_uint4(d[0], d[1], d[2], d[3]);
-      o[1] = make_uint4(d[4], d[5], d[6], d[7]);
-    }
+    if (live)
+      reinterpret_cast<uint4 *>(fr)[p8 * 4 + j] =
+          packed_digits(to_fixed(v[j].x, E - (bexp(v[j].x) - ve[j])), to_fixed(v[j].y, E - (bexp(v[j].y) - ve[j])));
   }
   if (live) {
-    *reinterpret_cast<double2 *>(fr + 1024 + p8 * 16) = get(F_L, k);
-    *reinterpret_cast<int *>(fr + 1152 + p8 * 4) = E - 1023;
-    *reinterpret_cast<double2 *>(br + 1024 + p8 * 16) = get(F_C, k);
+    *reinterpret_cast<double2 *>(fr + kLOff + p8 * 16) = get(F_L, k);
+    *reinterpret_cast<int *>(fr + kEOff + p8 * 4) = E - 1023;
+    *reinterpret_cast<double2 *>(br + kCOff + p8 * 16) = get(F_C, k);
     if (w == 0 && p8 < 4) a.vexp[row * 4 + p8] = ve[p8];
   }
   // the four weights, scaled by the largest of the window's eight poles
@@ -230,13 +236,9 @@ __global__ void digit_factor_kernel(SetupArgs a) {
     // poles 2 q and 2 q + 1 by the even thread, their imaginary parts by the odd one
     const long long re = (to_fixed(x.x, m - bexp(x.x)) + 128) & ~255ll, im = (to_fixed(x.y, m - bexp(x.y)) + 128) & ~255ll;
     const long long other = __shfl_xor_sync(0xffffffffu, p8 & 1 ? re : im, 1);
-    unsigned d[8];
-    digits(p8 & 1 ? other : re, p8 & 1 ? im : other, d);
-    if (live) {
-      uint4 *o = reinterpret_cast<uint4 *>(br + (s * kWin + p8) * 32);
-      o[0] = make_uint4(d[0], d[1], d[2], d[3]);
-      o[1] = make_uint4(d[4], d[5], d[6], (unsigned)(m - 1023));
-    }
+    uint4 d = packed_digits(p8 & 1 ? other : re, p8 & 1 ? im : other);
+    d.w = (d.w & 0xffffu) | (unsigned)(m - 1023) << 16;  // the exponent in the eighth digits' place
+    if (live) reinterpret_cast<uint4 *>(br)[s * kWin + p8] = d;
   }
   const double2 l = get(F_L, k), c = get(F_C, k);
   if (emax(l) == 0x7ff || emax(c) == 0x7ff) bad = true;
@@ -338,6 +340,16 @@ __device__ __forceinline__ void digits_of(double a, double b, int E, unsigned (&
   }
 }
 
+// stored digits as fp16 pairs, times `one` (+-1 each, less = -+1152)
+__device__ __forceinline__ void unpack(uint4 d, unsigned one, unsigned less, unsigned (&w)[8]) {
+  const unsigned v[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    w[2 * j] = half2_fma(__byte_perm(v[j], 0x64646464u, 0x4140), one, less);
+    w[2 * j + 1] = half2_fma(__byte_perm(v[j], 0x64646464u, 0x4342), one, less);
+  }
+}
+
 // rows whose data is brought into the caches ahead of use
 constexpr int kAhead = 2;
 
@@ -347,9 +359,9 @@ constexpr int kAhead = 2;
 __device__ __forceinline__ void right_hand_sides(const char *f, const char *dig, const int *uexp, int lane, double2 (&r)[2]) {
   unsigned p[8], v[8], z[8];
   load_words(dig, p);
-  load_words(f + lane * 32, v);
+  unpack(__ldg(reinterpret_cast<const uint4 *>(f) + lane), 0x3c003c00u, 0xe480e480u, v);
   const int U = __ldg(uexp) - 56;
-  const int2 e = __ldg(reinterpret_cast<const int2 *>(f + 1152) + (lane & 3));
+  const int2 e = __ldg(reinterpret_cast<const int2 *>(f + kEOff) + (lane & 3));
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     z[j] = __byte_perm(p[j], 0, 0x1032);  // (im, re): imaginary rows
@@ -387,13 +399,11 @@ __device__ __forceinline__ double2 weighted_sums(const char *f, const double2 (&
   const bool im_row = (lane >> 2) & 1;
   // a real row takes (re, -im) of the weights against (re, im) of x, an imaginary one (im, re)
   unsigned lo[8], hi[8];
-  const char *wr = f + ((lane >> 3) * 4 + q) * 64;
-  load_words(wr + (im_row ? 32 : 0), lo);
-  load_words(wr + (im_row ? 0 : 32), hi);
-  const int We = (int)lo[7];
-  const unsigned flip = im_row ? 0u : 0x80008000u;
-#pragma unroll
-  for (int j = 0; j < 7; ++j) hi[j] ^= flip;
+  const uint4 *wr = reinterpret_cast<const uint4 *>(f) + ((lane >> 3) * 4 + q) * 2;
+  const uint4 dl = __ldg(wr + (im_row ? 1 : 0)), dh = __ldg(wr + (im_row ? 0 : 1));
+  const int We = (int)dl.w >> 16;
+  unpack(dl, 0x3c003c00u, 0xe480e480u, lo);
+  unpack(dh, im_row ? 0x3c003c00u : 0xbc00bc00u, im_row ? 0xe480e480u : 0x64806480u, hi);
   lo[7] = hi[7] = 0;
   int E = 0;
 #pragma unroll
@@ -453,9 +463,9 @@ __global__ void __launch_bounds__(128, CTAS) solve_digits_kernel(SweepArgs a) {
         double2 y[2] = {make_double2(0, 0), make_double2(0, 0)}, r[2];
         right_hand_sides(f, dig, uexp, lane, r);
         for (int i = 0; i < len; ++i) {
-          const double2 l0 = ldd(f + 1024 + q * 32), l1 = ldd(f + 1040 + q * 32);
+          const double2 l0 = ldd(f + kLOff + q * 32), l1 = ldd(f + kLOff + q * 32 + 16);
           if (i + kAhead < len) {
-            if (lane < 10) prefetch(f + kAhead * kFwdRec + lane * 128);
+            if (lane < 6) prefetch(f + kAhead * kFwdRec + lane * 128);
             else if (lane >= 16 && lane < 24) prefetch(dig + kAhead * dstep + (lane - 16) * 128 - lane * 32);
           }
           y[0] = cfms(r[0], l0, y[0]);
@@ -476,7 +486,7 @@ __global__ void __launch_bounds__(128, CTAS) solve_digits_kernel(SweepArgs a) {
         double2 x[2] = {yp[0], yp[32]};  // Chat is zero in the last row
         for (int i = len - 1; i >= 0; --i) {
           if (i >= kAhead) {
-            if (lane < 10) prefetch(f - kAhead * kBwdRec + (lane < 9 ? lane * 128 : kBwdRec - 16));
+            if (lane < 6) prefetch(f - kAhead * kBwdRec + (lane < 5 ? lane * 128 : kBwdRec - 16));
             else if (lane >= 16 && lane < 24) prefetch(reinterpret_cast<const char *>(yp - lane - kAhead * 64) + (lane - 16) * 128);
             else if (lane >= 24 && lane < 28 && w > w0)
               prefetch(reinterpret_cast<const char *>(part - lane - (int64_t)kAhead * pstep) + (lane - 24) * 128);
@@ -488,8 +498,8 @@ __global__ void __launch_bounds__(128, CTAS) solve_digits_kernel(SweepArgs a) {
           f -= kBwdRec;
           yp -= 64;
           if (i > 0) {
-            xn[0] = cfms(yp[0], ldd(f + 1024 + q * 32), x[0]);
-            xn[1] = cfms(yp[32], ldd(f + 1040 + q * 32), x[1]);
+            xn[0] = cfms(yp[0], ldd(f + kCOff + q * 32), x[0]);
+            xn[1] = cfms(yp[32], ldd(f + kCOff + q * 32 + 16), x[1]);
           }
           *part = weighted_sums(g, x, lane, sum);
           part -= pstep;
