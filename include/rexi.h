@@ -121,15 +121,17 @@ typedef struct {
   int32_t strict_range; /* 1: plan creation fails with REXI_ERANGE when tau * max|omega|
                            exceeds h (M - 10), the range where Re of the REXI symbol
                            matches cos to the fit level */
-  int32_t pole_slots;   /* 0: the default solve -- for batches of up to four states with
-                           binary64 solves of the delta solver on the rotating sphere, the
-                           fused solve that keeps the pole sum on chip (one kernel, every
-                           output written once), for larger ones the digit solve (the
-                           contractions exactly on the tensor cores; needs device memory
-                           for 164 B per row and pole and poles of like scale), else the
-                           pole-slot solve (rexi_tune picks per batch); > 0: the pole-slot solve with this many pole groups
-                           summed separately, then reduced in slot order (a deterministic
-                           tuning knob, any >= 1) */
+  int32_t pole_slots;   /* 0: the default solve -- with binary64 solves of the delta solver on
+                           the rotating sphere the fixed-point solve (shape 5 of
+                           rexi_set_pole_slots) where its factors fit (148 to 164 B of device
+                           memory per row and pole, at most 32 GiB and a third of what is
+                           free) and the poles are of like scale, except for batches of up to
+                           four states in plans with max_batch >= 5; else for up to four
+                           states the fused solve that keeps the pole sum on chip (one
+                           kernel, every output written once), else the pole-slot solve
+                           (rexi_tune picks per batch); > 0: the pole-slot solve with this
+                           many pole groups summed separately, then reduced in slot order (a
+                           deterministic tuning knob, any >= 1) */
   const double *alpha;  /* optional: P complex poles (re, im interleaved); NULL -> computed */
   const double *beta;   /* optional: P complex weights, used as given (no renormalisation) */
   int32_t npoles;       /* P when alpha/beta are given */
@@ -283,10 +285,11 @@ rexi_status rexi_tune(rexi_plan *plan, int32_t batch, int32_t *slots, int32_t *s
  * split over `groups` CTAs in whole passes of the CTA's pole lanes (0: the default, more
  * than one only when a batch is too small to fill the GPU; a request is capped at the
  * passes), the last CTA of a tile to finish adding the groups' partial sums in group
- * order, or shape 5 for the digit solve (binary64 delta solver on the rotating sphere, plans
- * with max_batch >= 5: the right-hand sides and the pole sums as exact fixed-point products
- * on the tensor cores; slots: the items each system's poles are split over, 0: the default;
- * the default solve above four states), or shape 3 for its lean form (three or four CTAs of four warps per SM, fewer
+ * order, or shape 5 for the fixed-point solve (binary64 delta solver on the rotating sphere:
+ * the right-hand sides and the pole sums as exact fixed-point products, on the tensor cores in
+ * plans with max_batch >= 5, for batches of five and more by default, and in integer limbs in
+ * plans of up to four states, by default; slots: the items each system's poles are split over,
+ * plus 65536 x the poles per lane for the limbs, 0: the defaults), or shape 3 for its lean form (three or four CTAs of four warps per SM, fewer
  * registers, the next rows prefetched into the caches; tiles of up to 8 states), or shape
  * 4 for the lean form on CTAs of two warps (seven or eight per SM; tiles of up to 4
  * states; a tile of 2 states puts each state on a warp of its own, so no CTA splits its
@@ -329,7 +332,8 @@ void rexi_ragged_destroy(rexi_ragged *rg);
 /* Optional per-stage timing (no counterpart in the paper): with max_calls > 0 the next max_calls calls of
  * rexi_step / rexi_step_adjoint record CUDA events on their stream around each
  * stage (0 FFT forward, 1 Legendre analysis, 2 banded solve + pole sum,
- * 3 slot reduction (zero with the fused solve, which has none), 4 Legendre
+ * 3 slot reduction (zero with the fused solve, which has none, and in plans of up to four
+ * states, which count it with the solve), 4 Legendre
  * synthesis, 5 FFT inverse, 6/7 layout transposes).  max_calls = 0 turns it off.  rexi_profile_read waits for the
  * recorded events, writes the summed milliseconds per stage to stage_ms[0..n)
  * and the number of timed calls to *calls, and restarts the count. */

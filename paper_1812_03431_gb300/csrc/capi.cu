@@ -146,7 +146,7 @@ rexi_status core(Plan &pl, int B, bool adjoint, cudaStream_t st, Marks &mk) {
     mk.mark(ST_SOLVE);
     cudaError_t e = launch_solve_digits(pl, *dl, adjoint, pl.s_in, B, st);
     if (e != cudaSuccess) return cuda_fail("digit solve", e);
-    mk.mark(ST_REDUCE);
+    if (!pl.limbs) mk.mark(ST_REDUCE);  // small batches count it with the solve
     e = launch_finish_digits(pl, *dl, adjoint, pl.s_in, pl.s_out, B, st);
     return e == cudaSuccess ? REXI_OK : cuda_fail("digit sums", e);
   }

@@ -341,7 +341,8 @@ rexi_status build_plan(const rexi_params &prm, Plan *pl) {
   }
 
   // the digit solve's factors, for plans that step batches it serves by default
-  if (pl->fac_fwd && !pl->ff && prm.solver == REXI_SOLVER_DELTA && prm.max_batch >= kDigitMinBatch) {
+  pl->limbs = prm.max_batch < kDigitMinBatch;
+  if (pl->fac_fwd && !pl->ff && prm.solver == REXI_SOLVER_DELTA) {
     size_t mem_free = 0, mem_total = 0;
     if ((e = cudaMemGetInfo(&mem_free, &mem_total))) return fail("memory", e);
     const size_t need = digit_factor_bytes(*pl) + digit_state_bytes(*pl, prm.max_batch);
@@ -596,7 +597,7 @@ const FusedLayout *fused_layout(Plan &pl, int B) {
 const DigitLayout *digit_layout(Plan &pl, int B, bool adjoint) {
   if (!(adjoint ? pl.dig_adj : pl.dig_fwd).fwd) return nullptr;
   auto ud = pl.use_digits.find(B);
-  if (ud != pl.use_digits.end() ? !ud->second : (pl.slots_override > 0 || B < kDigitMinBatch)) return nullptr;
+  if (ud != pl.use_digits.end() ? !ud->second : (pl.slots_override > 0 || (B < kDigitMinBatch && !pl.limbs))) return nullptr;
   auto it = pl.digits.find(B);
   if (it == pl.digits.end()) {
     DigitLayout L;
@@ -605,6 +606,9 @@ const DigitLayout *digit_layout(Plan &pl, int B, bool adjoint) {
   }
   return it->second.items_dev ? &it->second : nullptr;
 }
+
+// a digit layout's slot count as rexi_set_pole_slots takes it
+int digit_slots_used(const Plan &pl, const DigitLayout &L) { return L.slots + (pl.limbs ? 65536 * L.kc : 0); }
 
 // the digit layout for batch B with a requested slot count (0: the default), replacing any
 // earlier one
@@ -647,7 +651,7 @@ rexi_status set_layout(Plan &pl, int B, int slots, int shape, int *used) {
       return REXI_EINVAL;
     }
     pl.use_digits[B] = true;
-    if (used) *used = D->slots;
+    if (used) *used = digit_slots_used(pl, *D);
     return REXI_OK;
   }
   if (shape >= 2 && shape <= 4) {
@@ -776,7 +780,9 @@ rexi_status tune_layout(Plan &pl, int B, int *slots_out, int *shape_out) {
   int digit_slots = 0;
   if (const DigitLayout *D0 = set_digit_slots(pl, B, 0)) {
     const int def = D0->slots;
-    for (int slots : {def, std::max(1, def / 2), 2 * def, 4 * def}) {
+    std::vector<int> tries = {def, std::max(1, def / 2), 2 * def, 4 * def};
+    if (pl.limbs) tries = {65536, 2 * 65536};
+    for (int slots : tries) {
       const DigitLayout *D = set_digit_slots(pl, B, slots);
       if (!D) break;
       for (int rep = 0; rep < 3; ++rep) {
@@ -789,7 +795,7 @@ rexi_status tune_layout(Plan &pl, int B, int *slots_out, int *shape_out) {
       if (cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
       if (ms < digit_ms) {
         digit_ms = ms;
-        digit_slots = D->slots;
+        digit_slots = digit_slots_used(pl, *D);
       }
     }
     set_digit_slots(pl, B, digit_slots);

@@ -132,6 +132,7 @@ struct DigitFactors {
 // windows, slot), longest first; each slot's sums are added by a second kernel.
 struct DigitLayout {
   int slots = 0, nitems = 0;
+  int kc = 2;  // poles per lane
   int4 *items_dev = nullptr;
 };
 
@@ -265,6 +266,7 @@ struct Plan {
   // per batch size the work list and whether rexi_tune / rexi_set_pole_slots chose it
   DigitFactors dig_fwd, dig_adj;
   bool dig_adj_tried = false;
+  bool limbs = false;  // small batches: the factors are limbs (solve_limbs.cu) instead
   char *dig_state = nullptr;
   std::map<int, DigitLayout> digits;
   std::map<int, bool> use_digits;
@@ -330,6 +332,14 @@ size_t digit_state_bytes(const Plan &pl, int B);
 size_t digit_slot_bytes(const Plan &pl, int B);
 cudaError_t build_digit_factors(Plan &pl, const double2 *fac, DigitFactors &D);
 void free_digit_factors(DigitFactors &D);
+int limb_tile(int B);
+int limb_window(int B, int kc);
+size_t limb_factor_bytes(const Plan &pl);
+size_t limb_state_bytes(const Plan &pl, int B);
+cudaError_t limb_configure(int B);
+void limb_record_bytes(size_t *fwd, size_t *bwd, int *block);
+cudaError_t launch_limb_factors(Plan &pl, const double2 *fac, DigitFactors &D, int kmid, int *bad);
+cudaError_t launch_solve_limbs(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, int B, cudaStream_t st);
 rexi_status build_digit_layout(Plan &pl, int B, int slots, DigitLayout &L);
 void free_digit_layout(DigitLayout &L);
 cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, int B,

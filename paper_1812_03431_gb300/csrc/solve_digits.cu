@@ -45,9 +45,12 @@
 #include <string>
 #include <vector>
 
+#include "fixed.h"
 #include "rexi_internal.h"
 
 namespace rexi {
+
+using namespace fixed;
 
 namespace {
 
@@ -56,20 +59,6 @@ constexpr int kWin = 8;                    // poles per window
 constexpr int kLOff = 512, kEOff = 640, kFwdRec = 672;  // per (row, window): coupling digits, l, exponents
 constexpr int kCOff = 512, kBwdRec = 640;  // per (row, window): weight digits and exponents, Chat
 constexpr int kStateRec = 1024;            // per (row, tile): input digits
-constexpr int kNotFinite = 1 << 20;        // exponent of a row input that holds an Inf or NaN
-constexpr int kMaxSpread = 8;              // bits by which a pole's couplings may differ in scale
-
-__device__ __forceinline__ int bexp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-
-// x as a fixed-point number of 61 bits below its group's leading bit, d = that bit's exponent
-// less x's own (truncated at 2^-61 of the leading bit; zero and subnormal x give zero)
-__device__ __forceinline__ long long to_fixed(double x, int d) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
-  m = (m << 9) >> (d & 63);
-  if (d > 63 || !(hi & 0x7ff00000u)) m = 0;
-  return (int)hi < 0 ? -(long long)m : (long long)m;
-}
 
 __device__ __forceinline__ unsigned half2_sub(unsigned a, unsigned b) {
   unsigned r;
@@ -103,32 +92,6 @@ __device__ __forceinline__ uint4 packed_digits(long long re, long long im) {
                     __byte_perm(rl, il, 0x4051));
 }
 
-// t 2^e in binary64 (round half away from zero), on the integer pipe; results below 2^-1022
-// are zero, e of a group that is not finite gives NaN
-__device__ __forceinline__ double fixed_to_double(long long t, int e) {
-  const int sign = (int)(t >> 63);
-  const unsigned long long m = (unsigned long long)((t ^ (long long)sign) - (long long)sign);
-  unsigned h = (unsigned)(m >> 32), l = (unsigned)m;
-  int be = 1023 + 62 + e;  // the biased exponent less one of a number with bit 63 set
-  if (h == 0) {
-    h = l;
-    l = 0;
-    be -= 32;
-  }
-  const int lz = __clz((int)h);  // 32 where t is zero: the shifts take it as 0
-  const unsigned fh = __funnelshift_l(l, h, lz), fl = l << (lz & 31);
-  be -= lz;
-  const unsigned long long r =
-      ((unsigned long long)(fh >> 11) << 32 | __funnelshift_r(fl, fh, 11)) + ((fl >> 10) & 1);
-  unsigned hi = (unsigned)(r >> 32) + ((unsigned)be << 20), lo = (unsigned)r;
-  if ((unsigned)be >= 2046u || fh == 0) {
-    const bool nan = e >= kNotFinite / 2;
-    hi = nan ? 0x7ff80000u : (be >= 2046 && fh != 0 ? 0x7ff00000u : 0u);
-    lo = 0;
-  }
-  return __hiloint2double((int)(hi | ((unsigned)sign & 0x80000000u)), (int)lo);
-}
-
 // An accumulator's bits are kMagicBits + its sum (kEvenBits for those that start at kEven), so
 // that of two neighbouring sums 256 bits(even) + bits(odd) = 256 s_c + s_{c+1} + 2^31.
 constexpr float kMagic = 12582912.0f;  // 1.5 2^23
@@ -141,7 +104,8 @@ __device__ __forceinline__ unsigned bits(float x) { return (unsigned)__float_as_
 // sum of s_c 2^(-8c), c = 0..7, in units of 2^-46; the pairs (s_0, s_1) ... (s_6, s_7) come as
 // 256 s_c + s_{c+1} + 2^31
 __device__ __forceinline__ long long weigh(unsigned h, unsigned m, unsigned l, unsigned q) {
-  const unsigned long long t = ((unsigned long long)h << 32 | l) + (unsigned long long)m * 65536u;
+  unsigned long long t = (unsigned long long)h << 32 | l;
+  asm("mad.wide.u32 %0, %1, 65536, %0;" : "+l"(t) : "r"(m));
   return (long long)((t << 6) + (q >> 10) - ((1ull << 53) + (1ull << 37) + (1ull << 21)));
 }
 
@@ -156,15 +120,6 @@ __device__ __forceinline__ void mma_add(float (&d)[4], unsigned a0, unsigned a1,
   asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-__device__ __forceinline__ double2 cfms(double2 acc, double2 a, double2 b) {
-  double re = fma(-a.x, b.x, acc.x), im = fma(-a.x, b.y, acc.y);
-  return make_double2(fma(a.y, b.y, re), fma(-a.y, b.x, im));
-}
-__device__ __forceinline__ double2 cfma(double2 acc, double2 a, double2 b) {
-  double re = fma(a.x, b.x, acc.x), im = fma(a.x, b.y, acc.y);
-  return make_double2(fma(-a.y, b.y, re), fma(a.y, b.x, im));
 }
 
 // ---- plan time: the factors as digits ---------------------------------------------------------
@@ -513,7 +468,7 @@ __global__ void __launch_bounds__(128, CTAS) solve_digits_kernel(SweepArgs a) {
 
 // ---- per step: the items' sums, the pole-independent terms, Re at m = 0 --------------------------
 struct FinishArgs {
-  const double *part;
+  const double *part;  // per (slot, row, tile): `unit` values, [4 streams][re, im][states] or [states][4 streams][re, im]
   const double2 *sin, *w;
   double2 *sout;
   const uint8_t *rflags;
@@ -521,11 +476,11 @@ struct FinishArgs {
   const int4 *sys;
   double2 sphi;
   int64_t nspec, nrows;
-  int B, tiles, slots, N;
+  int B, tile, tiles, unit, sstr, pstr, slots, N;
 };
 
 __global__ void digit_finish_kernel(FinishArgs a) {
-  const int64_t total = 3 * a.nspec * a.B;
+  const int64_t total = 3 * a.nspec * a.B, slot = a.nrows * a.tiles * a.unit;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
     const int b = (int)(t % a.B);
     const int64_t fi = t / a.B;
@@ -540,8 +495,19 @@ __global__ void digit_finish_kernel(FinishArgs a) {
         auto add = [&](int nn, int stream) {  // the slots' sums of the row at degree nn, in slot order
           const int4 sy = a.sys[2 * m + ((nn - m) & 1)];
           const int64_t row = sy.w + (nn - sy.y) / 2;
-          const double *p = a.part + (row * a.tiles + b / kTile) * 64 + stream * 16 + b % kTile;
-          for (int s = 0; s < a.slots; ++s, p += a.nrows * a.tiles * 64) acc = make_double2(acc.x + p[0], acc.y + p[8]);
+          const double *p = a.part + (row * a.tiles + b / a.tile) * a.unit + b % a.tile + stream * a.sstr;
+          int s = 0;
+          for (; s + 4 <= a.slots; s += 4, p += 4 * slot) {
+            double re[4], im[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              re[u] = __ldcs(p + u * slot);
+              im[u] = __ldcs(p + u * slot + a.pstr);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc = make_double2(acc.x + re[u], acc.y + im[u]);
+          }
+          for (; s < a.slots; ++s, p += slot) acc = make_double2(acc.x + p[0], acc.y + p[a.pstr]);
         };
         const int nmin = m > 1 ? m : 1;
         if (f != 1) add(n, f == 2 ? 0 : 1);
@@ -562,7 +528,13 @@ __global__ void digit_finish_kernel(FinishArgs a) {
 // resident CTAs per SM: 16 warps at 128 registers
 constexpr int kCtas = 4;
 
-int tiles_of(int B) { return (B + kTile - 1) / kTile; }
+// states per tile and poles per window of this plan's windowed solve
+int tile_of(const Plan &pl, int B) { return pl.limbs ? limb_tile(B) : kTile; }
+int tiles_of(const Plan &pl, int B) { return (B + tile_of(pl, B) - 1) / tile_of(pl, B); }
+int windows_of(const Plan &pl, int B, int kc) {
+  const int w = pl.limbs ? limb_window(B, kc) : kWin;
+  return (pl.P + w - 1) / w;
+}
 
 }  // namespace
 
@@ -573,41 +545,48 @@ void free_digit_factors(DigitFactors &D) {
 }
 
 size_t digit_factor_bytes(const Plan &pl) {
+  if (pl.limbs) return limb_factor_bytes(pl);
   return (size_t)pl.nrows * ((pl.P + kWin - 1) / kWin) * (kFwdRec + kBwdRec) + (size_t)pl.nrows * 4 * sizeof(int);
 }
 
-// The factor set as digits, from the binary64 factors `fac`.  D stays empty (and the other
-// solve kernels serve the plan) where the device memory does not suffice, or where a factor
-// is not finite or a pole's couplings differ in scale by more than the eighth digit covers.
+// The factor set as digits or limbs (pl.limbs), from the binary64 factors `fac`.  D stays empty
+// (and the other solve kernels serve the plan) where the device memory does not suffice, or
+// where a factor is not finite or a pole's couplings differ in scale by more than the
+// fixed-point forms cover.
 cudaError_t build_digit_factors(Plan &pl, const double2 *fac, DigitFactors &D) {
   D = DigitFactors{};
-  const int nwin = (pl.P + kWin - 1) / kWin;
-  if (pl.nrows == 0 || nwin > 0x7fff || pl.sys.size() > 0xffff) return cudaSuccess;
+  size_t fwd = kFwdRec, bwd = kBwdRec;
+  int block = kWin;
+  if (pl.limbs) limb_record_bytes(&fwd, &bwd, &block);
+  const int nwin = (pl.P + block - 1) / block;
+  if (pl.nrows == 0 || (pl.P + kWin - 1) / kWin > 0x7fff || pl.sys.size() > 0xffff) return cudaSuccess;
   const size_t nrec = (size_t)pl.nrows * nwin;
-  int *bad = nullptr;
-  if (cudaMalloc(&D.fwd, nrec * kFwdRec) != cudaSuccess || cudaMalloc(&D.bwd, nrec * kBwdRec) != cudaSuccess ||
+  if (cudaMalloc(&D.fwd, nrec * fwd) != cudaSuccess || cudaMalloc(&D.bwd, nrec * bwd) != cudaSuccess ||
       cudaMalloc(&D.vexp, (size_t)pl.nrows * 4 * sizeof(int) + sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
     free_digit_factors(D);
     return cudaSuccess;
   }
-  bad = D.vexp + pl.nrows * 4;
+  int *bad = D.vexp + pl.nrows * 4;
   cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int), 0);
-  SetupArgs a;
-  a.fac = fac;
-  a.sys = pl.sys_dev;
-  a.fwd = D.fwd;
-  a.bwd = D.bwd;
-  a.vexp = D.vexp;
-  a.bad = bad;
-  a.P = pl.P;
-  a.nwin = nwin;
-  a.kmid = (int)(std::min_element(pl.alpha.begin(), pl.alpha.end(),
-                                  [](const cplx &x, const cplx &y) { return std::abs(x) < std::abs(y); }) -
-                 pl.alpha.begin());
-  a.nrows = pl.nrows;
-  const int64_t most = (int64_t)pl.lmax * nwin * kWin;
-  if (e == cudaSuccess) {
+  const int kmid = (int)(std::min_element(pl.alpha.begin(), pl.alpha.end(),
+                                          [](const cplx &x, const cplx &y) { return std::abs(x) < std::abs(y); }) -
+                         pl.alpha.begin());
+  if (e == cudaSuccess && pl.limbs) {
+    e = launch_limb_factors(pl, fac, D, kmid, bad);
+  } else if (e == cudaSuccess) {
+    SetupArgs a;
+    a.fac = fac;
+    a.sys = pl.sys_dev;
+    a.fwd = D.fwd;
+    a.bwd = D.bwd;
+    a.vexp = D.vexp;
+    a.bad = bad;
+    a.P = pl.P;
+    a.nwin = nwin;
+    a.kmid = kmid;
+    a.nrows = pl.nrows;
+    const int64_t most = (int64_t)pl.lmax * nwin * kWin;
     digit_factor_kernel<<<dim3((unsigned)((most + 255) / 256), (unsigned)pl.sys.size()), 256>>>(a);
     e = cudaGetLastError();
   }
@@ -618,21 +597,38 @@ cudaError_t build_digit_factors(Plan &pl, const double2 *fac, DigitFactors &D) {
 }
 
 size_t digit_state_bytes(const Plan &pl, int B) {
-  return (size_t)pl.nrows * tiles_of(B) * (kStateRec + kTile * sizeof(int));
+  if (pl.limbs) return limb_state_bytes(pl, B);
+  return (size_t)pl.nrows * tiles_of(pl, B) * (kStateRec + kTile * sizeof(int));
 }
 
 // partial sums of one slot
-size_t digit_slot_bytes(const Plan &pl, int B) { return (size_t)pl.nrows * tiles_of(B) * 64 * sizeof(double); }
+size_t digit_slot_bytes(const Plan &pl, int B) {
+  return (size_t)pl.nrows * (pl.limbs ? B : tiles_of(pl, B) * kTile) * 8 * sizeof(double);
+}
 
 // Work items (system, tile, windows, slot) for batch B, longest first.  slots: items per
 // (system, tile), each over its share of the windows; 0: enough that the longest item is at
-// most half a resident warp's share of the work, capped by the partial-sum buffer.
+// most half a resident warp's share of the work, capped by the partial-sum buffer.  For limbs
+// slots carries 65536 x the poles per lane (1 or 2; 0: the default).  One pole per lane halves
+// a warp's chain of FP64 FMAs per row at 0.7 of the whole row's instructions, which pays where
+// items of two are fewer than 1.6 per resident warp (26 per SM): T63 x 1 0.073 / 0.085 ms, T170 x
+// 1 0.275 / 0.348 (20 per SM); T128 x 1 with 1047 poles 0.296 / 0.291 (29), T341 x 1 1.14 / 1.09 (40).
 rexi_status build_digit_layout(Plan &pl, int B, int slots, DigitLayout &L) {
   L = DigitLayout{};
-  const int nwin = (pl.P + kWin - 1) / kWin, tiles = tiles_of(B);
   if (pl.nrows == 0) return REXI_OK;  // not available
+  const int tiles = tiles_of(pl, B);
+  if (pl.limbs) {
+    L.kc = std::min(2, slots >> 16);
+    if (L.kc == 0) L.kc = (int64_t)pl.sys.size() * windows_of(pl, B, 2) * tiles < 26 * (int64_t)pl.num_sms ? 1 : 2;
+  }
+  slots &= 0xffff;
+  const int nwin = windows_of(pl, B, L.kc);
   const int cap = (int)std::min<size_t>((size_t)nwin, pl.partial_elems * sizeof(double2) / digit_slot_bytes(pl, B));
   if (cap < 1) return REXI_OK;  // not available
+  if (pl.limbs && limb_configure(B) != cudaSuccess) {
+    cudaGetLastError();
+    return REXI_OK;
+  }
   int64_t rows = 0;
   for (const SysInfo &s : pl.sys) rows += s.len;
   int G = slots;
@@ -673,8 +669,9 @@ void free_digit_layout(DigitLayout &L) {
 }
 
 cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, int B, cudaStream_t st) {
+  if (pl.limbs) return launch_solve_limbs(pl, L, adjoint, sin, B, st);
   const DigitFactors &D = adjoint ? pl.dig_adj : pl.dig_fwd;
-  const int tiles = tiles_of(B);
+  const int tiles = tiles_of(pl, B);
   StateArgs s;
   s.sin = sin;
   s.sys = pl.sys_dev;
@@ -701,7 +698,7 @@ cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, co
   a.nrows = pl.nrows;
   a.nitems = L.nitems;
   a.tiles = tiles;
-  a.nwin = (pl.P + kWin - 1) / kWin;
+  a.nwin = windows_of(pl, B, 2);
   a.lmax = pl.lmax;
   const int ctas = std::min(pl.num_sms * kCtas, (L.nitems + 3) / 4);
   solve_digits_kernel<kCtas><<<(unsigned)std::max(1, ctas), 128, 0, st>>>(a);
@@ -722,7 +719,11 @@ cudaError_t launch_finish_digits(Plan &pl, const DigitLayout &L, bool adjoint, c
   f.nspec = pl.nspec;
   f.nrows = pl.nrows;
   f.B = B;
-  f.tiles = tiles_of(B);
+  f.tile = pl.limbs ? 1 : kTile;
+  f.tiles = pl.limbs ? B : tiles_of(pl, B);
+  f.unit = 8 * f.tile;
+  f.sstr = 2 * f.tile;
+  f.pstr = f.tile;
   f.slots = L.slots;
   f.N = pl.N;
   const int64_t total = 3 * pl.nspec * B;

@@ -1,5 +1,5 @@
-"""The digit solve (both contractions of the shifted solves on the tensor cores, exactly)
-against the pole-slot solve, the oracle and its own linearity."""
+"""The fixed-point solves (both contractions of the shifted solves exactly: on the tensor cores
+above four states, in integer limbs up to four) against the pole-slot solve, the oracle and its own linearity."""
 import numpy as np
 import pytest
 
@@ -38,10 +38,13 @@ def spectral_plan(rexi, N, B, al, be, tau=1800.0, **k):
     return rexi.Plan(N, nlon // 2, nlon, tau=tau, max_batch=B, layout="spectral", alpha=al, beta=be, **k)
 
 
-# truncations down to one row per system; pole counts around a window of eight; batches around
-# a tile of eight states
+# truncations down to one row per system; pole counts around a window of eight (above four
+# states) and around 16, 32 and 64 (up to four); batches around a tile of eight states
 @pytest.mark.parametrize("N,P,B", [(1, 1, 5), (1, 9, 8), (2, 7, 9), (3, 8, 5), (8, 16, 16), (13, 17, 7), (21, 31, 17),
-                                   (42, 57, 8), (63, 149, 6)])
+                                   (42, 57, 8), (63, 149, 6),
+                                   (1, 1, 1), (2, 31, 1), (8, 32, 1), (13, 33, 1), (21, 64, 1), (42, 65, 1), (63, 149, 1),
+                                   (3, 15, 2), (13, 17, 2), (21, 33, 2), (31, 100, 2), (5, 8, 3), (21, 9, 3), (31, 57, 4),
+                                   (42, 149, 4)])
 def test_matches_slot_solve(env, N, P, B):
     torch, rexi = env
     al, be = poles(P)
@@ -60,7 +63,7 @@ def test_matches_slot_solve(env, N, P, B):
     plan.close()
 
 
-@pytest.mark.parametrize("N,M,B,tau", [(15, 32, 5, 3600.0), (31, 48, 10, 1200.0)])
+@pytest.mark.parametrize("N,M,B,tau", [(15, 32, 5, 3600.0), (31, 48, 10, 1200.0), (15, 32, 1, 3600.0), (31, 48, 3, 1200.0)])
 def test_matches_oracle(env, N, M, B, tau):
     torch, rexi = env
     al, be, _ = rc.rexi_coefficients(M, 0.2)
@@ -71,14 +74,15 @@ def test_matches_oracle(env, N, M, B, tau):
     plan.close()
 
 
-def test_states_keep_their_own_scale(env):
+@pytest.mark.parametrize("B", [11, 4])
+def test_states_keep_their_own_scale(env, B):
     """Every group's fixed-point scale is a power of two of its own, so a state times a power of
     two gives that power times the result, bit for bit, whatever the other states hold."""
     torch, rexi = env
-    N, B = 21, 11
+    N = 21
     al, be = poles(45)
     S = inputs.random_spectral(N, B, 9)
-    scale = 2.0 ** np.array([0, 300, -300, 0, 60, -60, 500, 1, -1, 0, -450])
+    scale = 2.0 ** np.array([0, 300, -300, 0, 60, -60, 500, 1, -1, 0, -450])[:B]
     T = S * scale[:, None, None]
     T[3] = 0.0
     plan = spectral_plan(rexi, N, B, al, be)
@@ -94,33 +98,35 @@ def test_states_keep_their_own_scale(env):
     plan2.close()
 
 
-@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
-def test_values_that_are_not_finite_stay_in_their_state_and_order(env, value):
+@pytest.mark.parametrize("value,B,s", [(np.nan, 9, 4), (np.inf, 9, 8), (-np.inf, 9, 0), (np.nan, 1, 0), (np.inf, 2, 1),
+                                       (-np.inf, 3, 2)])
+def test_values_that_are_not_finite_stay_in_their_state_and_order(env, value, B, s):
     torch, rexi = env
-    N, B = 21, 9
+    N = 21
     al, be = poles(45)
     S = inputs.random_spectral(N, B, 11)
     plan = spectral_plan(rexi, N, B, al, be)
     clean = plan.step(torch.from_numpy(S).cuda()).cpu().numpy()
     bad = S.copy()
-    bad[4, 2, (N + 1) + 6] = value  # delta of state 4, m = 1, n = 7
+    bad[s, 2, (N + 1) + 6] = value  # delta at m = 1, n = 7
     x = torch.from_numpy(bad).cuda()
     got = plan.step(x).cpu().numpy()
     plan.set_pole_slots(B, 4, 0)
     ref = plan.step(x).cpu().numpy()
     np.testing.assert_array_equal(np.isfinite(got), np.isfinite(ref))
-    keep = np.arange(B) != 4
+    keep = np.arange(B) != s
     np.testing.assert_array_equal(got[keep], clean[keep])
-    fine = np.isfinite(got[4])
-    np.testing.assert_array_equal(got[4][fine], clean[4][fine])
+    fine = np.isfinite(got[s])
+    np.testing.assert_array_equal(got[s][fine], clean[s][fine])
     plan.close()
 
 
-def test_poles_of_unlike_scale_keep_the_other_solves(env):
+@pytest.mark.parametrize("B", [8, 2])
+def test_poles_of_unlike_scale_keep_the_other_solves(env, B):
     """Couplings of one pole that differ by more than eight bits from the middle pole's stay with
     the binary64 kernels, by default and on request."""
     torch, rexi = env
-    N, B = 13, 8
+    N = 13
     al = np.array([-1e-3 + 0j, -1e3 + 1j, -1.0 + 2j])
     be = np.array([1e-3 + 0j, 1.0 + 1j, 0.5 - 1j])
     x = torch.from_numpy(inputs.random_spectral(N, B, 3)).cuda()
