@@ -208,6 +208,7 @@ void tiles(int B, int *TB, int *TN) {
 
 cudaError_t launch_leg_ana(Plan &pl, const double2 *four, double2 *sint, int B, const double *zd,
                            cudaStream_t st) {
+  if (pl.leg_ana.dig) return launch_leg_ana_digits(pl, four, sint, B, zd, st);
   LegArgs a{pl.tabP, pl.tabH, const_cast<double2 *>(four), sint, zd, pl.N, pl.nlat, pl.J, B, 0, 0, pl.nspec};
   tiles(B, &a.TB, &a.TN);
   dim3 g((unsigned)((pl.N + 1 + a.TN - 1) / a.TN), (unsigned)(pl.N + 1), (unsigned)((B + a.TB - 1) / a.TB));
@@ -218,6 +219,7 @@ cudaError_t launch_leg_ana(Plan &pl, const double2 *four, double2 *sint, int B, 
 
 cudaError_t launch_leg_syn(Plan &pl, const double2 *sint, double2 *four, int B, const double *zd,
                            cudaStream_t st) {
+  if (pl.leg_syn.dig) return launch_leg_syn_digits(pl, sint, four, B, zd, st);
   LegArgs a{pl.tabP, pl.tabH, four, const_cast<double2 *>(sint), zd, pl.N, pl.nlat, pl.J, B, 0, 0, pl.nspec};
   tiles(B, &a.TB, &a.TN);
   dim3 g((unsigned)((pl.J + a.TN - 1) / a.TN), (unsigned)(pl.N + 1), (unsigned)((B + a.TB - 1) / a.TB));

@@ -429,6 +429,19 @@ rexi_status build_plan(const rexi_params &prm, Plan *pl) {
 
   if (prm.precision == REXI_MIXED) {
     if ((e = tc_setup(*pl))) return fail("tensor-core tables", e);
+  } else {
+    // the tables as digits, in place of the binary64 ones where both directions fit
+    if ((e = build_legendre_digits(*pl, false, pl->leg_ana))) return fail("Legendre digits", e);
+    if (pl->leg_ana.dig && (e = build_legendre_digits(*pl, true, pl->leg_syn))) return fail("Legendre digits", e);
+    if (pl->leg_syn.dig) {
+      if ((e = cudaDeviceSynchronize())) return fail("Legendre digits", e);
+      cudaFree(pl->tabP);
+      cudaFree(pl->tabH);
+      pl->tabP = pl->tabH = nullptr;
+      bytes += pl->leg_ana.bytes + pl->leg_syn.bytes - 2 * (size_t)NS * pl->J * sizeof(double);
+    } else {
+      free_legendre_digits(pl->leg_ana);
+    }
   }
 
   // ---- workspaces
@@ -843,6 +856,8 @@ void free_plan(Plan *pl) {
     if (kv.second.items_dev) cudaFree(kv.second.items_dev);
   for (auto &kv : pl->fused) free_fused_layout(kv.second);
   for (auto &kv : pl->digits) free_digit_layout(kv.second);
+  free_legendre_digits(pl->leg_ana);
+  free_legendre_digits(pl->leg_syn);
   free_digit_factors(pl->dig_fwd);
   free_digit_factors(pl->dig_adj);
   delete pl;

@@ -136,6 +136,15 @@ struct DigitLayout {
   int4 *items_dev = nullptr;
 };
 
+// The FP64 form's Legendre tables as digits in fragment order, for one direction
+// (legendre_digits.cu).  Empty (dig null) where the FP64 kernels serve the plan.
+struct LegendreDigits {
+  uint4 *dig = nullptr;
+  int *exps = nullptr;
+  int4 *sys = nullptr;  // per 2 m + class: {rows, first fragment, first exponent group, 0}
+  size_t bytes = 0;
+};
+
 struct FftPlan {
   int n;
   int nstages;
@@ -210,6 +219,7 @@ struct Plan {
   double *zd_one = nullptr;         // [nspec]: 1
   double *zd_mone = nullptr;        // [nspec]: -1
   FftPlan fft{};
+  LegendreDigits leg_ana, leg_syn;  // FP64 form: tables as digits
   // mixed precision: packed TF32 hi/lo tables and per-CTA work lists of the tensor-core kernels
   uint32_t *tc_tab_ana = nullptr, *tc_tab_syn = nullptr;
   int4 *tc_work_ana = nullptr, *tc_work_syn = nullptr;
@@ -369,6 +379,12 @@ cudaError_t launch_leg_ana(Plan &pl, const double2 *four, double2 *sint, int B,
                            const double *zdscale, cudaStream_t st);
 cudaError_t launch_leg_syn(Plan &pl, const double2 *sint, double2 *four, int B,
                            const double *zdscale, cudaStream_t st);
+cudaError_t build_legendre_digits(Plan &pl, bool synthesis, LegendreDigits &t);
+void free_legendre_digits(LegendreDigits &t);
+cudaError_t launch_leg_ana_digits(Plan &pl, const double2 *four, double2 *sint, int B, const double *zd,
+                                  cudaStream_t st);
+cudaError_t launch_leg_syn_digits(Plan &pl, const double2 *sint, double2 *four, int B, const double *zd,
+                                  cudaStream_t st);
 cudaError_t launch_leg_ana_tc(Plan &pl, const double2 *four, double2 *sint, int B,
                               const double *zdscale, cudaStream_t st);
 cudaError_t launch_leg_syn_tc(Plan &pl, const double2 *sint, double2 *four, int B,

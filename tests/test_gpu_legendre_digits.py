@@ -1,0 +1,77 @@
+"""The FP64 form's transforms (Legendre sums as exact fixed-point products on the tensor cores)
+against the oracle's, at the edges of their tiles: 16 degrees or latitudes, groups of 64 terms,
+four states."""
+import numpy as np
+import pytest
+
+from oracle import sphere
+from paper_1812_03431_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+A, G = inputs.EARTH["radius"], inputs.EARTH["gravity"]
+TOL = 1e-11  # sums of up to 130 terms with weights up to 1 / (1 - mu^2) ~ 3e3: 130 x 3e3 x 2^-53 = 4e-11 at worst
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    from paper_1812_03431_gb300 import rexi
+    rexi.load()
+    return torch, rexi
+
+
+def oracle_analysis(g, x):
+    cos = g.coslat[:, None]
+    zeta, delta = g.uv_to_vortdiv(x[:, 1] * cos, x[:, 2] * cos, A)
+    return np.stack([G * g.analysis(x[:, 0]), zeta, delta], axis=1)
+
+
+def oracle_synthesis(g, S):
+    u, v = g.vortdiv_to_uv(S[:, 1], S[:, 2], A)
+    return np.stack([g.synthesis(S[:, 0]) / G, u / g.coslat[:, None], v / g.coslat[:, None]], axis=1)
+
+
+# (N, nlat, nlon, states): one to 66 degrees per class, 2 to 65 latitude pairs
+@pytest.mark.parametrize("N,nlat,nlon,B", [(1, 4, 8, 1), (2, 6, 12, 2), (15, 32, 48, 4), (16, 34, 48, 5), (30, 64, 96, 3),
+                                           (31, 66, 96, 8), (33, 128, 108, 9), (63, 130, 192, 1), (64, 96, 200, 2),
+                                           (130, 132, 400, 1)])
+def test_transforms_match_oracle(env, N, nlat, nlon, B):
+    torch, rexi = env
+    plan = rexi.Plan(N, nlat, nlon, M=8, max_batch=B)
+    g = sphere.Grid(N, nlat, nlon)
+    x = inputs.random_grid(B, nlat, nlon, 3)  # white noise: every latitude counts
+    got = plan.analyze(torch.from_numpy(x).cuda()).cpu().numpy()
+    ref = oracle_analysis(g, x)
+    ref[:, 1:, 0] = got[:, 1:, 0]  # zeta_0^0 and delta_0^0 are not state
+    S = inputs.random_spectral(N, B, 5, slope=0.0)  # white spectrum: every degree counts
+    grid = plan.synthesize(torch.from_numpy(S).cuda()).cpu().numpy()
+    want = oracle_synthesis(g, S)
+    for f in range(3):
+        assert np.linalg.norm(got[:, f] - ref[:, f]) < TOL * np.linalg.norm(ref[:, f])
+        assert np.linalg.norm(grid[:, f] - want[:, f]) < TOL * np.linalg.norm(want[:, f])
+    plan.close()
+
+
+def test_scales_and_values_that_are_not_finite_stay_in_their_state(env):
+    """Groups are scaled per state and order by powers of two: a power of two times a state gives
+    that power times its result, bit for bit, and a NaN reaches no other state."""
+    torch, rexi = env
+    N, nlat, nlon, B = 20, 40, 64, 6
+    plan = rexi.Plan(N, nlat, nlon, M=8, max_batch=B)
+    x = inputs.random_grid(B, nlat, nlon, 3)
+    S = inputs.random_spectral(N, B, 5)
+    scale = 2.0 ** np.array([0, 200, -200, 3, 0, -1])
+    run = lambda a: plan.analyze(torch.from_numpy(a).cuda()).cpu().numpy()  # noqa: E731
+    syn = lambda a: plan.synthesize(torch.from_numpy(a).cuda()).cpu().numpy()  # noqa: E731
+    a, s = run(x), syn(S)
+    np.testing.assert_array_equal(run(x * scale[:, None, None, None]), a * scale[:, None, None])
+    np.testing.assert_array_equal(syn(S * scale[:, None, None]), s * scale[:, None, None, None])
+    x[3, 0, 7, 9] = np.nan
+    S[3, 1, 30] = np.inf
+    b, t = run(x), syn(S)
+    keep = np.arange(B) != 3
+    np.testing.assert_array_equal(b[keep], a[keep])
+    np.testing.assert_array_equal(t[keep], s[keep])
+    assert not np.isfinite(b[3, 0]).any() and np.isfinite(b[3, 1:]).all()  # h' reaches Phi only
+    assert not np.isfinite(t[3, 1]).all() and np.isfinite(t[3, 0]).all()   # zeta reaches the wind only
+    plan.close()
