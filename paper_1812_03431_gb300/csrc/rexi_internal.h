@@ -349,7 +349,26 @@ size_t limb_state_bytes(const Plan &pl, int B);
 cudaError_t limb_configure(int B);
 void limb_record_bytes(size_t *fwd, size_t *bwd, int *block);
 cudaError_t launch_limb_factors(Plan &pl, const double2 *fac, DigitFactors &D, int kmid, int *bad);
-cudaError_t launch_solve_limbs(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, int B, cudaStream_t st);
+cudaError_t launch_limb_state(Plan &pl, bool adjoint, const double2 *sin, int B, cudaStream_t st);
+cudaError_t launch_solve_limbs(Plan &pl, const DigitLayout &L, bool adjoint, int B, cudaStream_t st);
+cudaError_t launch_digit_state(Plan &pl, bool adjoint, const double2 *sin, int B, cudaStream_t st);
+struct DigitItem {
+  int4 it;       // system, tile, first window | windows << 16, slot
+  int64_t work;  // rows x windows
+};
+bool digit_items(const Plan &pl, int B, int slots, double longest, DigitLayout &L, std::vector<DigitItem> &items);
+int64_t digit_work(const Plan &pl, int B, int kc);
+// the fixed-point solves of several plans in one launch (ragged_fixed.cu)
+struct FixedRagged {
+  void *views_dev = nullptr;        // per plan
+  int4 *items_dev = nullptr;        // items, then their plans (int each)
+  int nitems = 0, lmax = 0;
+  std::vector<DigitLayout> layouts; // per plan (slots and poles per lane; no work list of its own)
+};
+bool build_fixed_ragged(const std::vector<Plan *> &plans, const std::vector<int> &counts, FixedRagged &R);
+void free_fixed_ragged(FixedRagged &R);
+cudaError_t launch_fixed_ragged(const std::vector<Plan *> &plans, const std::vector<int> &counts, const FixedRagged &R,
+                                double2 *ybuf, unsigned *counter, cudaStream_t st);
 rexi_status build_digit_layout(Plan &pl, int B, int slots, DigitLayout &L);
 void free_digit_layout(DigitLayout &L);
 cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, int B,

@@ -29,10 +29,11 @@
 // cycles each, about a third of the FP64 time beside them, so their rate does not bound it.
 //
 // Measured on GB300 (solve and the sum of the slots, against the pole-slot solve and its
-// reduction): T341, 535 poles, 16 states 10.2 / 30.0 ms; T127, 535 poles, 64 states 5.7 / 17.0;
-// T85, 215 poles, 5 states 0.18 / 0.62.  What bounds it now: the FP64 unit, 78 % busy (ncu, T170 x
+// reduction): T341, 535 poles, 16 states 9.1 / 30.0 ms; T127, 535 poles, 64 states 5.1 / 17.0;
+// T85, 215 poles, 5 states 0.17 / 0.62.  What bounds it now: the FP64 unit, 86 % busy (ncu, T170 x
 // 16) with 9 instructions per state, pole and row at 64 cycles, one of them the running sum's
-// addition; the rest is waiting that 16 warps per SM do not cover (12 warps: 12.1 ms; 8: 16.0).
+// addition, at 16 warps per SM (12 warps: 10.2 ms at T341).  Rows staged ahead in shared memory
+// with asynchronous copies took it there from 78 % (9.9 ms with prefetches into the caches).
 //
 // A warp takes 8 states x 8 poles (lane: state lane / 4, poles 2 (lane % 4) and the next) of one
 // (m, parity) system, window by window of 8 poles, over all rows.  Real and imaginary rows of
@@ -45,21 +46,15 @@
 #include <string>
 #include <vector>
 
-#include "fixed.h"
-#include "mma_digits.h"
+#include "digit_sweep.h"
 #include "rexi_internal.h"
 
 namespace rexi {
 
 using namespace fixed;
+using namespace digit_solve;
 
 namespace {
-
-constexpr int kTile = 8;                   // states per warp
-constexpr int kWin = 8;                    // poles per window
-constexpr int kLOff = 512, kEOff = 640, kFwdRec = 672;  // per (row, window): coupling digits, l, exponents
-constexpr int kCOff = 512, kBwdRec = 640;  // per (row, window): weight digits and exponents, Chat
-constexpr int kStateRec = 1024;            // per (row, tile): input digits
 
 // ---- plan time: the factors as digits ---------------------------------------------------------
 struct SetupArgs {
@@ -114,7 +109,8 @@ __global__ void digit_factor_kernel(SetupArgs a) {
   if (live) {
     *reinterpret_cast<double2 *>(fr + kLOff + p8 * 16) = get(F_L, k);
     *reinterpret_cast<int *>(fr + kEOff + p8 * 4) = E - 1023;
-    *reinterpret_cast<double2 *>(br + kCOff + p8 * 16) = get(F_C, k);
+    *reinterpret_cast<double2 *>(br + kCOff + p8 * 16) =
+        i > 0 && k < a.P ? a.fac[((int64_t)F_C * a.nrows + row - 1) * a.P + k] : zero;
     if (w == 0 && p8 < 4) a.vexp[row * 4 + p8] = ve[p8];
   }
   // the four weights, scaled by the largest of the window's eight poles
@@ -182,210 +178,20 @@ __global__ void digit_state_kernel(StateArgs a) {
   if (q == 0) a.uexp[(row * a.tiles + tile) * kTile + s] = nf ? kNotFinite : (U < -(1 << 23) ? 0 : U - 1023);
 }
 
-// ---- per step: the sweeps ----------------------------------------------------------------------
-struct SweepArgs {
-  const char *fwd, *bwd, *dig;
-  const int *uexp;
-  const int4 *sys, *items;  // {system, tile, first window | windows << 16, slot}
-  double *part;             // [slots][nrows][tiles][4 streams][re, im][8 states]
-  double2 *ybuf;            // per resident warp: [lmax][2][32]
-  unsigned *counter;
-  int64_t nrows;
-  int nitems, tiles, nwin, lmax;
-};
-
-__device__ __forceinline__ void load_words(const char *p, unsigned (&w)[8]) {
-  const uint4 x = __ldg(reinterpret_cast<const uint4 *>(p)), y = __ldg(reinterpret_cast<const uint4 *>(p) + 1);
-  w[0] = x.x, w[1] = x.y, w[2] = x.z, w[3] = x.w, w[4] = y.x, w[5] = y.y, w[6] = y.z, w[7] = y.w;
-}
-__device__ __forceinline__ double2 ldd(const char *p) { return __ldg(reinterpret_cast<const double2 *>(p)); }
-__device__ __forceinline__ void prefetch(const void *p) { asm volatile("prefetch.global.L1 [%0];" : : "l"(p)); }
-// |x| as to_fixed gives it, E the exponent (biased) of its group's leading bit
-__device__ __forceinline__ unsigned long long magnitude(double x, int E) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const int d = min(E - (int)((hi >> 20) & 0x7ff), 63);
-  unsigned h = __funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, 9), l = lo << 9;
-  if (d >= 32) {
-    l = h;
-    h = 0;
-  }
-  return (unsigned long long)(h >> (d & 31)) << 32 | __funnelshift_r(l, h, d & 31);
-}
-
-// the eight digits of two numbers of one group, as fp16 pairs
-__device__ __forceinline__ void digits_of(double a, double b, int E, unsigned (&w)[8]) {
-  const unsigned long long ua = magnitude(a, E) + 0x8080808080808080ull, ub = magnitude(b, E) + 0x8080808080808080ull;
-  const unsigned sign = __byte_perm((unsigned)__double2hiint(a), (unsigned)__double2hiint(b), 0x7632) & 0x80008000u;
-  const unsigned one = sign | 0x3c003c00u, less = sign ^ 0xe480e480u;  // +-1 and -+1152
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const unsigned x = h == 0 ? (unsigned)(ua >> 32) : (unsigned)ua, y = h == 0 ? (unsigned)(ub >> 32) : (unsigned)ub;
-    const unsigned top = __byte_perm(x, y, 0x7362), low = __byte_perm(x, y, 0x5140);
-    w[4 * h + 0] = half2_fma(__byte_perm(top, 0x64646464u, 0x4342), one, less);
-    w[4 * h + 1] = half2_fma(__byte_perm(top, 0x64646464u, 0x4140), one, less);
-    w[4 * h + 2] = half2_fma(__byte_perm(low, 0x64646464u, 0x4342), one, less);
-    w[4 * h + 3] = half2_fma(__byte_perm(low, 0x64646464u, 0x4140), one, less);
-  }
-}
-
-// rows whose data is brought into the caches ahead of use
-constexpr int kAhead = 2;
-
-// The right-hand sides of one row for the lane's two poles: digits of the inputs (rows of the
-// product: states, real rows above imaginary ones) times those of the couplings (columns:
-// poles), one accumulator per sum of digit places, two digit pairs per MMA.
-__device__ __forceinline__ void right_hand_sides(const char *f, const char *dig, const int *uexp, int lane, double2 (&r)[2]) {
-  unsigned p[8], v[8], z[8];
-  load_words(dig, p);
-  unpack(__ldg(reinterpret_cast<const uint4 *>(f) + lane), 0x3c003c00u, 0xe480e480u, v);
-  const int U = __ldg(uexp) - 56;
-  const int2 e = __ldg(reinterpret_cast<const int2 *>(f + kEOff) + (lane & 3));
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    z[j] = __byte_perm(p[j], 0, 0x1032);  // (im, re): imaginary rows
-    p[j] ^= 0x80000000u;                  // (re, -im): real rows
-  }
-  unsigned pair[4][4];
-#pragma unroll
-  for (int c = 0; c < 8; c += 2) {
-    float s[2][4];
-#pragma unroll
-    for (int o = 0; o < 2; ++o)
-#pragma unroll
-      for (int i = 0; i <= c + o; i += 2) {
-        const int j = c + o - i;
-        const unsigned a2 = j > 0 ? p[i < 7 ? i + 1 : 7] : 0u, a3 = j > 0 ? z[i < 7 ? i + 1 : 7] : 0u, b1 = j > 0 ? v[j > 0 ? j - 1 : 0] : 0u;
-        if (i == 0) mma_first(s[o], p[i], z[i], a2, a3, v[j], b1, o == 0 ? kEven : kMagic);
-        else mma_add(s[o], p[i], z[i], a2, a3, v[j], b1);
-      }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) pair[c / 2][k] = bits(s[0][k]) * 256u + bits(s[1][k]);
-  }
-#pragma unroll
-  for (int g = 0; g < 2; ++g) {
-    const int ee = U + (g ? e.y : e.x);
-    r[g] = make_double2(fixed_to_double(weigh(pair[0][g], pair[1][g], pair[2][g], pair[3][g]), ee),
-                        fixed_to_double(weigh(pair[0][g + 2], pair[1][g + 2], pair[2][g + 2], pair[3][g + 2]), ee));
-  }
-}
-
-// Adds to the lane's two running sums (states 2 q and 2 q + 1 of one stream's real or
-// imaginary part) the weighted sums over the window's eight poles of x, a row's solutions:
-// digits of the weights (rows: streams) times those of x (columns: states).
-__device__ __forceinline__ double2 weighted_sums(const char *f, const double2 (&x)[2], int lane, double2 sum) {
-  const int q = lane & 3;
-  const bool im_row = (lane >> 2) & 1;
-  // a real row takes (re, -im) of the weights against (re, im) of x, an imaginary one (im, re)
-  unsigned lo[8], hi[8];
-  const uint4 *wr = reinterpret_cast<const uint4 *>(f) + ((lane >> 3) * 4 + q) * 2;
-  const uint4 dl = __ldg(wr + (im_row ? 1 : 0)), dh = __ldg(wr + (im_row ? 0 : 1));
-  const int We = (int)dl.w >> 16;
-  unpack(dl, 0x3c003c00u, 0xe480e480u, lo);
-  unpack(dh, im_row ? 0x3c003c00u : 0xbc00bc00u, im_row ? 0xe480e480u : 0x64806480u, hi);
-  lo[7] = hi[7] = 0;
-  int E = 0;
-#pragma unroll
-  for (int g = 0; g < 2; ++g) E = max(E, max(__double2hiint(x[g].x) & 0x7fffffff, __double2hiint(x[g].y) & 0x7fffffff));
-  E = max(E, __shfl_xor_sync(0xffffffffu, E, 1));
-  E = max(E, __shfl_xor_sync(0xffffffffu, E, 2)) >> 20;
-  if (E < 64) E += 4096;  // groups below 2^-959 are taken as zero
-  unsigned re[8], im[8];
-  digits_of(x[0].x, x[1].x, E, re);
-  digits_of(x[0].y, x[1].y, E, im);
-  float s[8][4];
-#pragma unroll
-  for (int c = 0; c < 8; ++c) mma_first(s[c], lo[0], lo[1], hi[0], hi[1], re[c], im[c]);
-#pragma unroll
-  for (int i = 2; i < 8; i += 2)
-#pragma unroll
-    for (int c = i; c < 8; ++c) mma_add(s[c], lo[i], lo[i + 1], hi[i], hi[i + 1], re[c - i], im[c - i]);
-  double r[2];
-#pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    const int Es = __shfl_sync(0xffffffffu, E, (q * 2 + c) * 4);  // the exponent of state 2 q + c
-    // digit places j come from the upper rows of accumulator j and the lower ones of j - 1
-    unsigned at[8];
-    at[0] = bits(s[0][c]) + (0x00800000u - kMagicBits);
-#pragma unroll
-    for (int j = 1; j < 8; ++j) at[j] = bits(s[j][c]) + bits(s[j - 1][c + 2]) + ((j & 1 ? 0u : 0x00800000u) - 2u * kMagicBits);
-    r[c] = fixed_to_double(weigh(at[0] * 256u + at[1], at[2] * 256u + at[3], at[4] * 256u + at[5], at[6] * 256u + at[7]),
-                           (Es & 4095) == 0x7ff ? kNotFinite : We + (Es & 4095) - 1023 - 56);
-  }
-  return make_double2(sum.x + r[0], sum.y + r[1]);
-}
-
+// ---- per step: the sweeps (digit_sweep.h) ---------------------------------------------------------
 template <int CTAS>
-__global__ void __launch_bounds__(128, CTAS) solve_digits_kernel(SweepArgs a) {
-  const int lane = threadIdx.x & 31, q = lane & 3;
+__global__ void __launch_bounds__(128, CTAS) solve_digits_kernel(DigitSweep a) {
+  const int lane = threadIdx.x & 31;
   const int wslot = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   double2 *yb = a.ybuf + (int64_t)wslot * a.lmax * 64 + lane;
+  extern __shared__ __align__(16) char stages[];
+  char *smem = stages + (threadIdx.x >> 5) * kSmemWarp;
   for (;;) {
     unsigned it = 0;
     if (lane == 0) it = atomicAdd(a.counter, 1u);
     it = __shfl_sync(0xffffffffu, it, 0);
     if (it >= (unsigned)a.nitems) break;
-    const int4 item = a.items[it];
-    const int4 sy = a.sys[item.x];
-    const int len = sy.z, w0 = item.z & 0xffff, w1 = w0 + (item.z >> 16);
-    const int64_t row0 = sy.w;
-    const char *dig0 = a.dig + (row0 * a.tiles + item.y) * kStateRec + lane * 32;
-    const int *uexp0 = a.uexp + (row0 * a.tiles + item.y) * kTile + (lane >> 2);
-    const int dstep = a.tiles * kStateRec, ustep = a.tiles * kTile;
-    double2 *part0 = reinterpret_cast<double2 *>(a.part + (((int64_t)item.w * a.nrows + row0) * a.tiles + item.y) * 64) + lane;
-    const int pstep = a.tiles * 32;
-    for (int w = w0; w < w1; ++w) {
-      {  // forward: y_i = r_i - l y_{i-1}; the next row's r is formed beside the FMAs of this one
-        const char *f = a.fwd + (row0 * a.nwin + (int64_t)w * len) * kFwdRec, *dig = dig0;
-        const int *uexp = uexp0;
-        double2 *yp = yb;
-        double2 y[2] = {make_double2(0, 0), make_double2(0, 0)}, r[2];
-        right_hand_sides(f, dig, uexp, lane, r);
-        for (int i = 0; i < len; ++i) {
-          const double2 l0 = ldd(f + kLOff + q * 32), l1 = ldd(f + kLOff + q * 32 + 16);
-          if (i + kAhead < len) {
-            if (lane < 6) prefetch(f + kAhead * kFwdRec + lane * 128);
-            else if (lane >= 16 && lane < 24) prefetch(dig + kAhead * dstep + (lane - 16) * 128 - lane * 32);
-          }
-          y[0] = cfms(r[0], l0, y[0]);
-          y[1] = cfms(r[1], l1, y[1]);
-          f += kFwdRec;
-          dig += dstep;
-          uexp += ustep;
-          if (i + 1 < len) right_hand_sides(f, dig, uexp, lane, r);
-          yp[0] = y[0];
-          yp[32] = y[1];
-          yp += 64;
-        }
-      }
-      {  // backward: x_i = y_i - Chat x_{i+1}; the sums of row i + 1 beside the FMAs of row i
-        const char *f = a.bwd + (row0 * a.nwin + (int64_t)(w + 1) * len - 1) * kBwdRec;
-        const double2 *yp = yb + (len - 1) * 64;
-        double2 *part = part0 + (int64_t)(len - 1) * pstep;
-        double2 x[2] = {yp[0], yp[32]};  // Chat is zero in the last row
-        for (int i = len - 1; i >= 0; --i) {
-          if (i >= kAhead) {
-            if (lane < 6) prefetch(f - kAhead * kBwdRec + (lane < 5 ? lane * 128 : kBwdRec - 16));
-            else if (lane >= 16 && lane < 24) prefetch(reinterpret_cast<const char *>(yp - lane - kAhead * 64) + (lane - 16) * 128);
-            else if (lane >= 24 && lane < 28 && w > w0)
-              prefetch(reinterpret_cast<const char *>(part - lane - (int64_t)kAhead * pstep) + (lane - 24) * 128);
-          }
-          double2 sum = make_double2(0, 0);
-          if (w > w0) sum = *part;
-          double2 xn[2] = {x[0], x[1]};
-          const char *g = f;
-          f -= kBwdRec;
-          yp -= 64;
-          if (i > 0) {
-            xn[0] = cfms(yp[0], ldd(f + kCOff + q * 32), x[0]);
-            xn[1] = cfms(yp[32], ldd(f + kCOff + q * 32 + 16), x[1]);
-          }
-          *part = weighted_sums(g, x, lane, sum);
-          part -= pstep;
-          x[0] = xn[0];
-          x[1] = xn[1];
-        }
-      }
-    }
+    digit_item(a, a.items[it], lane, yb, smem);
   }
 }
 
@@ -419,18 +225,7 @@ __global__ void digit_finish_kernel(FinishArgs a) {
           const int4 sy = a.sys[2 * m + ((nn - m) & 1)];
           const int64_t row = sy.w + (nn - sy.y) / 2;
           const double *p = a.part + (row * a.tiles + b / a.tile) * a.unit + b % a.tile + stream * a.sstr;
-          int s = 0;
-          for (; s + 4 <= a.slots; s += 4, p += 4 * slot) {
-            double re[4], im[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              re[u] = __ldcs(p + u * slot);
-              im[u] = __ldcs(p + u * slot + a.pstr);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) acc = make_double2(acc.x + re[u], acc.y + im[u]);
-          }
-          for (; s < a.slots; ++s, p += slot) acc = make_double2(acc.x + p[0], acc.y + p[a.pstr]);
+          for (int s = 0; s < a.slots; ++s, p += slot) acc = make_double2(acc.x + p[0], acc.y + p[a.pstr]);
         };
         const int nmin = m > 1 ? m : 1;
         if (f != 1) add(n, f == 2 ? 0 : 1);
@@ -529,6 +324,36 @@ size_t digit_slot_bytes(const Plan &pl, int B) {
   return (size_t)pl.nrows * (pl.limbs ? B : tiles_of(pl, B) * kTile) * 8 * sizeof(double);
 }
 
+// The items of one plan's batch: `slots` per (system, tile), each over its share of the windows
+// (0: enough that the longest item's rows x windows are at most `longest`), capped by the
+// partial-sum buffer.  False where the buffer holds no slot.
+bool digit_items(const Plan &pl, int B, int slots, double longest, DigitLayout &L, std::vector<DigitItem> &items) {
+  const int tiles = tiles_of(pl, B), nwin = windows_of(pl, B, L.kc);
+  const int cap = (int)std::min<size_t>((size_t)nwin, pl.partial_elems * sizeof(double2) / digit_slot_bytes(pl, B));
+  if (cap < 1) return false;
+  int G = slots;
+  if (G <= 0) {
+    G = 1;
+    while (G < nwin && (double)pl.lmax * ((nwin + G - 1) / G) > longest) ++G;
+  }
+  G = std::max(1, std::min(G, cap));
+  for (int s = 0; s < (int)pl.sys.size(); ++s) {
+    if (pl.sys[s].len == 0) continue;
+    for (int g = 0; g < G; ++g) {
+      const int w0 = (int)((int64_t)nwin * g / G), w1 = (int)((int64_t)nwin * (g + 1) / G);
+      for (int t = 0; t < tiles; ++t)
+        items.push_back(DigitItem{make_int4(s, t, w0 | ((w1 - w0) << 16), g), (int64_t)pl.sys[s].len * (w1 - w0)});
+    }
+  }
+  L.slots = G;
+  return true;
+}
+
+// rows x windows x tiles of a batch
+int64_t digit_work(const Plan &pl, int B, int kc) {
+  return pl.nrows * windows_of(pl, B, kc) * tiles_of(pl, B);
+}
+
 // Work items (system, tile, windows, slot) for batch B, longest first.  slots: items per
 // (system, tile), each over its share of the windows; 0: enough that the longest item is at
 // most half a resident warp's share of the work, capped by the partial-sum buffer.  For limbs
@@ -539,41 +364,21 @@ size_t digit_slot_bytes(const Plan &pl, int B) {
 rexi_status build_digit_layout(Plan &pl, int B, int slots, DigitLayout &L) {
   L = DigitLayout{};
   if (pl.nrows == 0) return REXI_OK;  // not available
-  const int tiles = tiles_of(pl, B);
   if (pl.limbs) {
     L.kc = std::min(2, slots >> 16);
-    if (L.kc == 0) L.kc = (int64_t)pl.sys.size() * windows_of(pl, B, 2) * tiles < 26 * (int64_t)pl.num_sms ? 1 : 2;
-  }
-  slots &= 0xffff;
-  const int nwin = windows_of(pl, B, L.kc);
-  const int cap = (int)std::min<size_t>((size_t)nwin, pl.partial_elems * sizeof(double2) / digit_slot_bytes(pl, B));
-  if (cap < 1) return REXI_OK;  // not available
-  if (pl.limbs && limb_configure(B) != cudaSuccess) {
-    cudaGetLastError();
-    return REXI_OK;
-  }
-  int64_t rows = 0;
-  for (const SysInfo &s : pl.sys) rows += s.len;
-  int G = slots;
-  if (G <= 0) {
-    const double share = (double)rows * nwin * tiles / (4.0 * kCtas * pl.num_sms);
-    G = 1;
-    while (G < nwin && (double)pl.lmax * ((nwin + G - 1) / G) > 0.5 * share) ++G;
-  }
-  G = std::max(1, std::min(G, cap));
-  struct Keyed { int4 it; int64_t work; };
-  std::vector<Keyed> keyed;
-  for (int s = 0; s < (int)pl.sys.size(); ++s) {
-    if (pl.sys[s].len == 0) continue;
-    for (int g = 0; g < G; ++g) {
-      const int w0 = (int)((int64_t)nwin * g / G), w1 = (int)((int64_t)nwin * (g + 1) / G);
-      for (int t = 0; t < tiles; ++t)
-        keyed.push_back(Keyed{make_int4(s, t, w0 | ((w1 - w0) << 16), g), (int64_t)pl.sys[s].len * (w1 - w0)});
+    if (L.kc == 0)
+      L.kc = (int64_t)pl.sys.size() * windows_of(pl, B, 2) * tiles_of(pl, B) < 26 * (int64_t)pl.num_sms ? 1 : 2;
+    if (limb_configure(B) != cudaSuccess) {
+      cudaGetLastError();
+      return REXI_OK;
     }
   }
-  std::stable_sort(keyed.begin(), keyed.end(), [](const Keyed &x, const Keyed &y) { return x.work > y.work; });
+  std::vector<DigitItem> keyed;
+  if (!digit_items(pl, B, slots & 0xffff, 0.5 * digit_work(pl, B, L.kc) / (4.0 * kCtas * pl.num_sms), L, keyed))
+    return REXI_OK;
+  std::stable_sort(keyed.begin(), keyed.end(), [](const DigitItem &x, const DigitItem &y) { return x.work > y.work; });
   std::vector<int4> items;
-  for (const Keyed &k : keyed) items.push_back(k.it);
+  for (const DigitItem &k : keyed) items.push_back(k.it);
   cudaError_t e = cudaMalloc(&L.items_dev, std::max<size_t>(1, items.size()) * sizeof(int4));
   if (e == cudaSuccess) e = cudaMemcpy(L.items_dev, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
@@ -581,7 +386,6 @@ rexi_status build_digit_layout(Plan &pl, int B, int slots, DigitLayout &L) {
     set_error(std::string("digit work list: ") + cudaGetErrorString(e));
     return REXI_ENOMEM;
   }
-  L.slots = G;
   L.nitems = (int)items.size();
   return REXI_OK;
 }
@@ -591,14 +395,14 @@ void free_digit_layout(DigitLayout &L) {
   L = DigitLayout{};
 }
 
-cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, int B, cudaStream_t st) {
-  if (pl.limbs) return launch_solve_limbs(pl, L, adjoint, sin, B, st);
-  const DigitFactors &D = adjoint ? pl.dig_adj : pl.dig_fwd;
+// the batch's inputs in fixed point
+cudaError_t launch_digit_state(Plan &pl, bool adjoint, const double2 *sin, int B, cudaStream_t st) {
+  if (pl.limbs) return launch_limb_state(pl, adjoint, sin, B, st);
   const int tiles = tiles_of(pl, B);
   StateArgs s;
   s.sin = sin;
   s.sys = pl.sys_dev;
-  s.vexp = D.vexp;
+  s.vexp = (adjoint ? pl.dig_adj : pl.dig_fwd).vexp;
   s.dig = pl.dig_state;
   s.uexp = reinterpret_cast<int *>(pl.dig_state + (size_t)pl.nrows * tiles * kStateRec);
   s.nspec = pl.nspec;
@@ -606,13 +410,17 @@ cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, co
   s.tiles = tiles;
   s.N = pl.N;
   digit_state_kernel<<<dim3((unsigned)((pl.lmax * tiles + 7) / 8), (unsigned)pl.sys.size()), 256, 0, st>>>(s);
-  cudaError_t e = cudaMemsetAsync(pl.counter, 0, sizeof(unsigned), st);
-  if (e != cudaSuccess) return e;
-  SweepArgs a;
+  return cudaGetLastError();
+}
+
+DigitSweep digit_sweep(Plan &pl, const DigitLayout &L, bool adjoint, int B) {
+  const DigitFactors &D = adjoint ? pl.dig_adj : pl.dig_fwd;
+  const int tiles = tiles_of(pl, B);
+  DigitSweep a;
   a.fwd = D.fwd;
   a.bwd = D.bwd;
-  a.dig = s.dig;
-  a.uexp = s.uexp;
+  a.dig = pl.dig_state;
+  a.uexp = reinterpret_cast<const int *>(pl.dig_state + (size_t)pl.nrows * tiles * kStateRec);
   a.sys = pl.sys_dev;
   a.items = L.items_dev;
   a.part = reinterpret_cast<double *>(pl.partial);
@@ -623,8 +431,16 @@ cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, co
   a.tiles = tiles;
   a.nwin = windows_of(pl, B, 2);
   a.lmax = pl.lmax;
+  return a;
+}
+
+cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, int B, cudaStream_t st) {
+  cudaError_t e = launch_digit_state(pl, adjoint, sin, B, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(pl.counter, 0, sizeof(unsigned), st);
+  if (e != cudaSuccess) return e;
+  if (pl.limbs) return launch_solve_limbs(pl, L, adjoint, B, st);
   const int ctas = std::min(pl.num_sms * kCtas, (L.nitems + 3) / 4);
-  solve_digits_kernel<kCtas><<<(unsigned)std::max(1, ctas), 128, 0, st>>>(a);
+  solve_digits_kernel<kCtas><<<(unsigned)std::max(1, ctas), 128, 4 * kSmemWarp, st>>>(digit_sweep(pl, L, adjoint, B));
   return cudaGetLastError();
 }
 
