@@ -34,6 +34,8 @@ struct rexi_ragged {
     std::vector<uint64_t> gens;  // the plans' layout generations the views were built from
     bool fused = false;          // binary64 plans: the fused solve over every plan's items
     rexi::FusedRagged fr;
+    bool fixed = false;          // the fixed-point solves over every plan's items
+    rexi::FixedRagged xr;
   };
   std::map<std::vector<int>, Cfg> cfgs;
 };
@@ -161,18 +163,17 @@ rexi_status rexi_ragged_step(rexi_ragged *rg, const void *const *in_dev, void *c
       set_error("rexi_ragged_step: more states for plan " + std::to_string(p) + " than its max_batch");
       return REXI_EINVAL;
     }
-  // binary64 plans: one fused launch over every plan's items (the pole sum on chip, no
-  // reductions); else the slot kernel over the merged work list, then per-plan reductions.
+  // binary64 plans: one launch of the fixed-point solves over every plan's items, or where
+  // that does not apply one fused launch (the pole sum on chip, no reductions); else the slot kernel over the merged work list, then per-plan reductions.
   // Either work list is cached per count vector.
   auto it = rg->cfgs.find(counts);
   if (it == rg->cfgs.end() && !rg->plans[0]->ff) {
     rexi_ragged::Cfg cfg;
-    if (build_fused_ragged(rg->plans, counts, cfg.fr)) {
-      cfg.fused = true;
-      it = rg->cfgs.emplace(counts, cfg).first;
-    }
+    cfg.fixed = build_fixed_ragged(rg->plans, counts, cfg.xr);
+    cfg.fused = !cfg.fixed && build_fused_ragged(rg->plans, counts, cfg.fr);
+    if (cfg.fixed || cfg.fused) it = rg->cfgs.emplace(counts, cfg).first;
   }
-  const bool fused = it != rg->cfgs.end() && it->second.fused;
+  const bool fused = it != rg->cfgs.end() && (it->second.fused || it->second.fixed);  // no slot layouts
   std::vector<SolveLayout *> lays(np, nullptr);
   for (int p = 0; p < np && !fused; ++p)
     if (counts[p] > 0) {
@@ -225,7 +226,9 @@ rexi_status rexi_ragged_step(rexi_ragged *rg, const void *const *in_dev, void *c
   const rexi_ragged::Cfg &cfg = it->second;
   cudaError_t e = move_states(rg->plans, in_dev, state_plan, nstates, counts, rank, true, st);
   const bool ff = rg->plans[0]->ff;
-  if (cfg.fused) {
+  if (cfg.fixed) {
+    if (e == cudaSuccess) e = launch_fixed_ragged(rg->plans, counts, cfg.xr, rg->ybuf, rg->counter, st);
+  } else if (cfg.fused) {
     if (e == cudaSuccess) e = launch_fused_ragged(cfg.fr, rg->ybuf, rg->plans[0]->num_sms, st);
   } else {
     for (int p = 0; p < np && e == cudaSuccess; ++p)  // float-float solves read split states
@@ -253,6 +256,7 @@ void rexi_ragged_destroy(rexi_ragged *rg) {
     if (kv.second.views_dev) cudaFree(kv.second.views_dev);
     if (kv.second.items_dev) cudaFree(kv.second.items_dev);
     free_fused_ragged(kv.second.fr);
+    free_fixed_ragged(kv.second.xr);
   }
   if (rg->ybuf) cudaFree(rg->ybuf);
   if (rg->counter) cudaFree(rg->counter);
