@@ -13,16 +13,17 @@
 // Z'_m = E'_m + i O'_m from the Hermitian spectrum and evaluates
 // conj(FFT(conj Z')).
 //
+// The kernels here are those of the mixed form, whose transform is FP32; the FP64 form's
+// (fft_fixed.cu) compute the same sums in block fixed point.
+//
 // Layouts: grid [B][3][nlat][nlon] float64; Fourier [nlat][N+1][3B] complex (FP64 in
-// the FP64 form, FP32 in the mixed form, where the transform itself is FP32), column
-// c = 3 b + field, so that for each latitude the Legendre kernels read contiguous
-// columns.  The mixed form scales in FP32 (scales rounded to binary32 once, at plan time)
+// the FP64 form, FP32 in the mixed form), column c = 3 b + field, so that for each latitude
+// the Legendre kernels read contiguous columns.  The mixed form scales in FP32 (scales rounded to binary32 once, at plan time)
 // and converts the data between FP64 and FP32 on the integer pipe (f64_to_f32 /
 // f32_to_f64): no FP64 instruction is left in its kernels.
 #include <cuda_runtime.h>
 
 #include <cmath>
-#include <type_traits>
 
 #include "rexi_internal.h"
 
@@ -30,13 +31,11 @@ namespace rexi {
 
 namespace {
 
-template <typename T> struct V2;
-template <> struct V2<double> { using t = double2; };
-template <> struct V2<float> { using t = float2; };
-template <typename T> __device__ __forceinline__ typename V2<T>::t mk(T x, T y) { return {x, y}; }
+using T = float;
+using C = float2;
 
 struct FftArgs {
-  const void *tw;  // n twiddles e^{-2 pi i k / n} (n = nlon), double2 or float2
+  const C *tw;  // n twiddles e^{-2 pi i k / n} (n = nlon)
   int n, h, nstages, N, nlat, ncol, np;  // h = n / 2 complex points per row; np rows per CTA
   int radix[24];
   // division by run-time sizes as a multiply-high: x / d = umulhi(x, mag) for x, d < 2^16
@@ -50,16 +49,15 @@ __device__ __forceinline__ int fdiv(int x, uint32_t mag, int d) {
   return d == 1 ? x : (int)__umulhi((uint32_t)x, mag);
 }
 
-template <typename C> __device__ __forceinline__ C cmulz(C a, C b) { return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x}; }
-template <typename C> __device__ __forceinline__ C addz(C a, C b) { return {a.x + b.x, a.y + b.y}; }
-template <typename C> __device__ __forceinline__ C subz(C a, C b) { return {a.x - b.x, a.y - b.y}; }
-template <typename C> __device__ __forceinline__ C mulmi(C a) { return {a.y, -a.x}; }  // -i a
+__device__ __forceinline__ C cmulz(C a, C b) { return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x}; }
+__device__ __forceinline__ C addz(C a, C b) { return {a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ C subz(C a, C b) { return {a.x - b.x, a.y - b.y}; }
+__device__ __forceinline__ C mulmi(C a) { return {a.y, -a.x}; }  // -i a
 
 // In-register DFT of R points (forward, e^{-2 pi i jk/R}); R is a compile-time constant
 // so v[] stays in registers and the loops unroll.
-template <typename T, int R>
-__device__ __forceinline__ void dft_small(typename V2<T>::t *v, const FftArgs &a) {
-  using C = typename V2<T>::t;
+template <int R>
+__device__ __forceinline__ void dft_small(C *v, const FftArgs &a) {
   if constexpr (R == 2) {
     C t = v[0];
     v[0] = addz(t, v[1]);
@@ -117,11 +115,10 @@ __device__ __forceinline__ void dft_small(typename V2<T>::t *v, const FftArgs &a
 }
 
 // One Stockham pass of radix R over np rows of n points: src -> dst.
-template <typename T, int R>
-__device__ __forceinline__ void stockham_pass(const typename V2<T>::t *src, typename V2<T>::t *dst, int n, int Ns,
+template <int R>
+__device__ __forceinline__ void stockham_pass(const C *src, C *dst, int n, int Ns,
                                               uint32_t mnb, uint32_t mns, const FftArgs &a) {
-  using C = typename V2<T>::t;
-  const C *tw = static_cast<const C *>(a.tw);
+  const C *tw = a.tw;
   const int nb = n / R;
   const int tstep = 2 * (n / (Ns * R));  // twiddle e^{-2 pi i jm r / (Ns R)} = tw[r jm tstep]
   for (int t = threadIdx.x; t < a.np * nb; t += blockDim.x) {
@@ -133,7 +130,7 @@ __device__ __forceinline__ void stockham_pass(const typename V2<T>::t *src, type
     v[0] = in[jb];
 #pragma unroll
     for (int r = 1; r < R; ++r) v[r] = cmulz(in[jb + r * nb], tw[r * jm * tstep]);  // tw[0] = 1 exactly
-    dft_small<T, R>(v, a);
+    dft_small<R>(v, a);
     const int od = jd * Ns * R + jm;
 #pragma unroll
     for (int r = 0; r < R; ++r) out[od + r * Ns] = v[r];
@@ -142,9 +139,7 @@ __device__ __forceinline__ void stockham_pass(const typename V2<T>::t *src, type
 
 // In-shared-memory forward FFT of np rows of h points; returns the buffer holding
 // the result (buf0 or buf1).
-template <typename T>
-__device__ typename V2<T>::t *fft_smem(typename V2<T>::t *buf0, typename V2<T>::t *buf1, const FftArgs &a) {
-  using C = typename V2<T>::t;
+__device__ C *fft_smem(C *buf0, C *buf1, const FftArgs &a) {
   const int n = a.h;
   C *src = buf0, *dst = buf1;
   int Ns = 1;
@@ -152,11 +147,11 @@ __device__ typename V2<T>::t *fft_smem(typename V2<T>::t *buf0, typename V2<T>::
     const int R = a.radix[s];
     const uint32_t mnb = a.mag_nb[s], mns = a.mag_ns[s];
     switch (R) {  // uniform across the block
-      case 8: stockham_pass<T, 8>(src, dst, n, Ns, mnb, mns, a); break;
-      case 4: stockham_pass<T, 4>(src, dst, n, Ns, mnb, mns, a); break;
-      case 2: stockham_pass<T, 2>(src, dst, n, Ns, mnb, mns, a); break;
-      case 3: stockham_pass<T, 3>(src, dst, n, Ns, mnb, mns, a); break;
-      default: stockham_pass<T, 5>(src, dst, n, Ns, mnb, mns, a); break;
+      case 8: stockham_pass<8>(src, dst, n, Ns, mnb, mns, a); break;
+      case 4: stockham_pass<4>(src, dst, n, Ns, mnb, mns, a); break;
+      case 2: stockham_pass<2>(src, dst, n, Ns, mnb, mns, a); break;
+      case 3: stockham_pass<3>(src, dst, n, Ns, mnb, mns, a); break;
+      default: stockham_pass<5>(src, dst, n, Ns, mnb, mns, a); break;
     }
     __syncthreads();
     C *tmp = src;
@@ -167,15 +162,11 @@ __device__ typename V2<T>::t *fft_smem(typename V2<T>::t *buf0, typename V2<T>::
   return src;
 }
 
-// T: arithmetic type inside the transform (double, or float in the mixed form, whose
-// Fourier array is FP32); the grid stays FP64 either way, and the scales come in type T.
-template <typename T>
+// The transform and the Fourier array are FP32, the grid is FP64, the scales come in FP32.
 __global__ void fft_fwd_kernel(FftArgs a, const double *grid, void *four_v, const T *in_scale, const T *m_scale) {
-  using C = typename V2<T>::t;
-  constexpr bool F32 = std::is_same<T, float>::value;
   extern __shared__ __align__(16) unsigned char smraw[];
   C *sm = reinterpret_cast<C *>(smraw);
-  const C *tw = static_cast<const C *>(a.tw);
+  const C *tw = a.tw;
   C *four = static_cast<C *>(four_v);
   const int h = a.h;
   C *buf0 = sm, *buf1 = sm + a.np * h;
@@ -205,17 +196,13 @@ __global__ void fft_fwd_kernel(FftArgs a, const double *grid, void *four_v, cons
       if (t >= a.np * h) break;
       C v = {0, 0};
       if (ok[i]) {
-        if constexpr (F32) {
-          v = C{sv[i] * f64_to_f32(x[i].x), sv[i] * f64_to_f32(x[i].y)};
-        } else {
-          v = C{sv[i] * x[i].x, sv[i] * x[i].y};
-        }
+        v = C{sv[i] * f64_to_f32(x[i].x), sv[i] * f64_to_f32(x[i].y)};
       }
       buf0[t] = v;
     }
   }
   __syncthreads();
-  const C *Z = fft_smem<T>(buf0, buf1, a);
+  const C *Z = fft_smem(buf0, buf1, a);
   const int M1 = a.N + 1;
   for (int t = threadIdx.x; t < a.np * M1; t += blockDim.x) {
     const int m = fdiv(t, a.mag_np, a.np), q = t - m * a.np;
@@ -232,13 +219,10 @@ __global__ void fft_fwd_kernel(FftArgs a, const double *grid, void *four_v, cons
   }
 }
 
-template <typename T>
 __global__ void fft_inv_kernel(FftArgs a, const void *four_v, double *grid, const T *m_scale, const T *out_scale) {
-  using C = typename V2<T>::t;
-  constexpr bool F32 = std::is_same<T, float>::value;
   extern __shared__ __align__(16) unsigned char smraw[];
   C *sm = reinterpret_cast<C *>(smraw);
-  const C *tw = static_cast<const C *>(a.tw);
+  const C *tw = a.tw;
   const C *four = static_cast<const C *>(four_v);
   const int h = a.h;
   C *buf0 = sm, *buf1 = sm + a.np * h;
@@ -285,7 +269,7 @@ __global__ void fft_inv_kernel(FftArgs a, const void *four_v, double *grid, cons
     }
   }
   __syncthreads();
-  const C *r = fft_smem<T>(buf0, buf1, a);
+  const C *r = fft_smem(buf0, buf1, a);
   double2 *g2 = reinterpret_cast<double2 *>(grid);
   for (int t = threadIdx.x; t < a.np * h; t += blockDim.x) {
     const int q = fdiv(t, a.mag_h, h), k = t - q * h;
@@ -293,17 +277,13 @@ __global__ void fft_inv_kernel(FftArgs a, const void *four_v, double *grid, cons
     if (c >= a.ncol) continue;
     const T s = out_scale[(c % 3) * a.nlat + j];
     const C v = r[t];  // conj of z_k = x_{2k} + i x_{2k+1}
-    if constexpr (F32) {
-      g2[((int64_t)c * a.nlat + j) * h + k] = make_double2(f32_to_f64(s * v.x), f32_to_f64(-s * v.y));
-    } else {
-      g2[((int64_t)c * a.nlat + j) * h + k] = make_double2(s * v.x, -s * v.y);
-    }
+    g2[((int64_t)c * a.nlat + j) * h + k] = make_double2(f32_to_f64(s * v.x), f32_to_f64(-s * v.y));
   }
 }
 
 FftArgs make_args(const Plan &pl, int B) {
   FftArgs a;
-  a.tw = pl.prm.precision == REXI_MIXED ? pl.fft.tw32_dev : pl.fft.tw_dev;
+  a.tw = static_cast<const C *>(pl.fft.tw32_dev);
   a.n = pl.fft.n;
   a.h = pl.fft.n / 2;
   a.nstages = pl.fft.nstages;
@@ -353,47 +333,38 @@ bool fft_factor(int n, int *radix, int *nstages) {
 }
 
 bool fft32(const Plan &pl) { return pl.prm.precision == REXI_MIXED; }
-size_t fft_smem_bytes(const Plan &pl) {
-  return (size_t)pl.fft.nsplit * pl.fft.n * (fft32(pl) ? sizeof(float2) : sizeof(double2));
-}
+size_t fft_smem_bytes(const Plan &pl) { return (size_t)pl.fft.nsplit * pl.fft.n * sizeof(float2); }
 
 cudaError_t launch_fft_fwd(Plan &pl, const double *grid, double2 *four, int B, const void *in_scale,
                            const void *m_scale, cudaStream_t st) {
+  if (!fft32(pl))
+    return launch_fft_fixed_fwd(pl, grid, four, B, static_cast<const double *>(in_scale),
+                                static_cast<const double *>(m_scale), st);
   FftArgs a = make_args(pl, B);
   dim3 g((unsigned)((a.ncol + a.np - 1) / a.np), (unsigned)pl.nlat);
-  size_t sm = fft_smem_bytes(pl);
-  if (fft32(pl))
-    fft_fwd_kernel<float><<<g, 256, sm, st>>>(a, grid, four, static_cast<const float *>(in_scale),
-                                              static_cast<const float *>(m_scale));
-  else
-    fft_fwd_kernel<double><<<g, 256, sm, st>>>(a, grid, four, static_cast<const double *>(in_scale),
-                                               static_cast<const double *>(m_scale));
+  fft_fwd_kernel<<<g, 256, fft_smem_bytes(pl), st>>>(a, grid, four, static_cast<const float *>(in_scale),
+                                                     static_cast<const float *>(m_scale));
   return cudaGetLastError();
 }
 
 cudaError_t launch_fft_inv(Plan &pl, const double2 *four, double *grid, int B, const void *m_scale,
                            const void *out_scale, cudaStream_t st) {
+  if (!fft32(pl))
+    return launch_fft_fixed_inv(pl, four, grid, B, static_cast<const double *>(m_scale),
+                                static_cast<const double *>(out_scale), st);
   FftArgs a = make_args(pl, B);
   dim3 g((unsigned)((a.ncol + a.np - 1) / a.np), (unsigned)pl.nlat);
-  size_t sm = fft_smem_bytes(pl);
-  if (fft32(pl))
-    fft_inv_kernel<float><<<g, 256, sm, st>>>(a, four, grid, static_cast<const float *>(m_scale),
-                                              static_cast<const float *>(out_scale));
-  else
-    fft_inv_kernel<double><<<g, 256, sm, st>>>(a, four, grid, static_cast<const double *>(m_scale),
-                                               static_cast<const double *>(out_scale));
+  fft_inv_kernel<<<g, 256, fft_smem_bytes(pl), st>>>(a, four, grid, static_cast<const float *>(m_scale),
+                                                     static_cast<const float *>(out_scale));
   return cudaGetLastError();
 }
 
 cudaError_t fft_configure(Plan &pl) {
+  if (!fft32(pl)) return fft_fixed_configure(pl);
   const int bytes = (int)fft_smem_bytes(pl);
-  cudaError_t e;
-  if (fft32(pl)) {
-    if ((e = cudaFuncSetAttribute(fft_fwd_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
-    return cudaFuncSetAttribute(fft_inv_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  }
-  if ((e = cudaFuncSetAttribute(fft_fwd_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes))) return e;
-  return cudaFuncSetAttribute(fft_inv_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaError_t e = cudaFuncSetAttribute(fft_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(fft_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 }  // namespace rexi

@@ -415,14 +415,19 @@ rexi_status build_plan(const rexi_params &prm, Plan *pl) {
       const double th = 2.0 * M_PI * k / f.n;
       tw[k] = make_double2(std::cos(th), -std::sin(th));
     }
-    double2 *twd = nullptr;
-    if ((e = upload(&twd, tw, &bytes))) return fail("twiddles", e);
-    f.tw_dev = twd;
-    std::vector<float2> tw32(f.n);
-    for (int k = 0; k < f.n; ++k) tw32[k] = make_float2((float)tw[k].x, (float)tw[k].y);
-    float2 *tw32d = nullptr;
-    if ((e = upload(&tw32d, tw32, &bytes))) return fail("twiddles", e);
-    f.tw32_dev = tw32d;
+    if (prm.precision == REXI_MIXED) {
+      std::vector<float2> tw32(f.n);
+      for (int k = 0; k < f.n; ++k) tw32[k] = make_float2((float)tw[k].x, (float)tw[k].y);
+      float2 *tw32d = nullptr;
+      if ((e = upload(&tw32d, tw32, &bytes))) return fail("twiddles", e);
+      f.tw32_dev = tw32d;
+    } else {
+      std::vector<int4> limbs;
+      fft_fixed_twiddles(tw, limbs);
+      int4 *twd = nullptr;
+      if ((e = upload(&twd, limbs, &bytes))) return fail("twiddles", e);
+      f.tw_dev = twd;
+    }
     if ((e = fft_configure(*pl))) return fail("fft configure", e);
     if ((e = legendre_configure())) return fail("legendre configure", e);
   }

@@ -150,8 +150,8 @@ struct FftPlan {
   int nstages;
   int radix[24];
   int nsplit;     // rows per CTA (pairs of real rows packed as one complex row)
-  void *tw_dev;   // n twiddles e^{-2 pi i k/n}, double2
-  void *tw32_dev; // the same as float2 (mixed form)
+  void *tw_dev = nullptr;    // FP64 form: n twiddles e^{-2 pi i k/n} as limbs (fft_fixed.cu)
+  void *tw32_dev = nullptr;  // mixed form: the same as float2
 };
 
 enum FacComp { F_L = 0, F_G, F_E, F_F, F_C, F_BD, F_BAD, F_ZP, F_ZM, F_NCOMP };
@@ -394,6 +394,13 @@ cudaError_t launch_fft_fwd(Plan &pl, const double *grid, double2 *four, int B,
                            const void *in_scale, const void *m_scale, cudaStream_t st);
 cudaError_t launch_fft_inv(Plan &pl, const double2 *four, double *grid, int B,
                            const void *m_scale, const void *out_scale, cudaStream_t st);
+// the FP64 form's, in block fixed point (fft_fixed.cu)
+void fft_fixed_twiddles(const std::vector<double2> &tw, std::vector<int4> &limbs);
+cudaError_t fft_fixed_configure(Plan &pl);
+cudaError_t launch_fft_fixed_fwd(Plan &pl, const double *grid, double2 *four, int B, const double *in_scale,
+                                 const double *m_scale, cudaStream_t st);
+cudaError_t launch_fft_fixed_inv(Plan &pl, const double2 *four, double *grid, int B, const double *m_scale,
+                                 const double *out_scale, cudaStream_t st);
 cudaError_t launch_leg_ana(Plan &pl, const double2 *four, double2 *sint, int B,
                            const double *zdscale, cudaStream_t st);
 cudaError_t launch_leg_syn(Plan &pl, const double2 *sint, double2 *four, int B,

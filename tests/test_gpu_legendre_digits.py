@@ -75,3 +75,30 @@ def test_scales_and_values_that_are_not_finite_stay_in_their_state(env):
     assert not np.isfinite(b[3, 0]).any() and np.isfinite(b[3, 1:]).all()  # h' reaches Phi only
     assert not np.isfinite(t[3, 1]).all() and np.isfinite(t[3, 0]).all()   # zeta reaches the wind only
     plan.close()
+
+
+@pytest.mark.parametrize("nlon", [8, 10, 16, 18, 24, 30, 64, 90, 100, 250, 486, 1024, 2000])
+def test_longitude_transforms(env, nlon):
+    """Every radix and row length against the oracle, for rows that a common scale suits least: one
+    point among zeros, one field 1e-9 of the others, a constant row."""
+    torch, rexi = env
+    N, nlat, B = min(3, nlon // 2 - 1), 6, 3
+    plan = rexi.Plan(N, nlat, nlon, M=8, max_batch=B)
+    g = sphere.Grid(N, nlat, nlon)
+    x = inputs.random_grid(B, nlat, nlon, 8)
+    x[0] = 0.0
+    x[0, :, 2, nlon // 3] = 1.0
+    x[1, 0] *= 1e-9
+    x[2, 1] = 7.0
+    got = plan.analyze(torch.from_numpy(x).cuda()).cpu().numpy()
+    ref = oracle_analysis(g, x)
+    ref[:, 1:, 0] = got[:, 1:, 0]
+    S = got.copy()
+    grid = plan.synthesize(torch.from_numpy(S).cuda()).cpu().numpy()
+    want = oracle_synthesis(g, S)
+    for b in range(B):
+        assert np.linalg.norm(got[b, 0] - ref[b, 0]) < TOL * np.linalg.norm(ref[b, 0])
+        assert np.linalg.norm(got[b, 1:] - ref[b, 1:]) < TOL * np.linalg.norm(ref[b, 1:])
+        assert np.linalg.norm(grid[b, 0] - want[b, 0]) < TOL * np.linalg.norm(want[b, 0])
+        assert np.linalg.norm(grid[b, 1:] - want[b, 1:]) < TOL * np.linalg.norm(want[b, 1:])
+    plan.close()
