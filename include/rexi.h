@@ -123,7 +123,7 @@ typedef struct {
                            matches cos to the fit level */
   int32_t pole_slots;   /* 0: the default solve -- with binary64 solves of the delta solver on
                            the rotating sphere the fixed-point solve (shape 5 of
-                           rexi_set_pole_slots) where its factors fit (148 to 164 B of device
+                           rexi_set_pole_slots) where its factors fit (64 to 164 B of device
                            memory per row and pole, at most 32 GiB and a third of what is
                            free) and the poles are of like scale, except for batches of up to
                            four states in plans with max_batch >= 5; else for up to four

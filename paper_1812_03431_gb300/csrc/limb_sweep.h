@@ -11,12 +11,15 @@ namespace limb_solve {
 
 using namespace fixed;
 
-constexpr int kBlock = 64;  // poles per record
-// per (row, block of 64 poles): [g][e][f] limbs, l, exponents (kNoPole past the last pole)
-constexpr int kFL = 3 * 1024, kFE = 4 * 1024, kFwd = 4 * 1024 + 256;
-constexpr int kNoPole = 1000;
-// per (row, block): Chat of the row before, [bd][bad][zp][zm] limbs, the four exponents
-constexpr int kBW = 1024, kBE = 5 * 1024, kBwd = 5 * 1024 + 16;
+// Poles per record.  Every factor of a row is a product of one of four complex numbers per pole
+// with a real number per row (row_scale) or 1: 1/s_{n-1} and 1/s_{n+1}, s_n = alpha + i tau sigma_n
+// (shared by neighbouring rows), 1/alpha (per pole only), and beta/d'; and the recurrences'
+// l and Chat.  Records are [pole] arrays of 16 B: `inv` one per (system, block, j = 0..len) of
+// 1/s at degree n0 - 1 + 2 j, `fwd` one per (row, block) of l, `bwd` of Chat of the row before
+// and beta/d', with the latter's exponent behind.
+constexpr int kBlock = 64;
+constexpr int kRec = kBlock * 16;
+constexpr int kBE = 2 * kRec, kBwd = 2 * kRec + 16;
 
 // v as limbs: v = x 2^30 + y, -2^29 <= y < 2^29
 __device__ __forceinline__ int2 limbs(long long v) {
@@ -29,7 +32,8 @@ __device__ __forceinline__ int4 limbs2(long long re, long long im) {
 }
 
 struct LimbSweep {
-  const char *fwd, *bwd;
+  const char *fwd, *bwd, *inv;
+  const int4 *inv_alpha;    // [P padded]
   const int4 *dig;
   const int *uexp;
   const int4 *sys, *items;  // {system, tile, first window | windows << 16, slot}
@@ -38,15 +42,16 @@ struct LimbSweep {
   unsigned *counter;
   int64_t nrows;
   int nitems, B, P, nblk, lmax, kc;
+  int e0;                   // exponent of the limbs of 1/s and 1/alpha
 };
 
 // Staging: each lane copies the factors of its poles for the rows ahead into shared memory
-// (three forward stages, two backward), and the row's inputs are copied once per warp.  Bytes
-// of a forward stage: (g, e, f, l) per pole of the lane, exponents, inputs and their exponents.
-constexpr int kSE = 2 * 4 * 512, kSIn = kSE + 256, kSU = kSIn + 256, kStage = kSU + 64;
-constexpr int kFwdStages = 3;
-constexpr int kSmemWarp = kFwdStages * kStage;
-static_assert(kSmemWarp >= 2 * 2 * 5 * 512, "two backward stages");
+// (rings of four stages), and the row's inputs are copied once per warp.  Bytes of a forward
+// stage: (1/s, l) per pole of the lane, inputs and their exponents; of a backward one: (1/s,
+// Chat, beta/d').  Behind the ring: 1/alpha per pole of the lane.
+constexpr int kSIn = 2 * 2 * 512, kSU = kSIn + 256, kStage = 2 * 3 * 512;
+constexpr int kInvAlpha = 4 * kStage, kSmemWarp = kInvAlpha + 2 * 512;
+static_assert(kSU + 64 <= kStage, "forward stage");
 
 template <int BYTES>
 __device__ __forceinline__ void copy_async(unsigned to, const void *from) {
@@ -81,41 +86,47 @@ __device__ __forceinline__ long long fixed59(double x, int E) {
   return (long long)(((unsigned long long)(h >> (d & 31)) << 32 | __funnelshift_r(l, h, d & 31)) ^ (unsigned long long)s) - s;
 }
 
-// r = delta0 - g Phi0 - e zeta0_{n-1} - f zeta0_{n+1} at one row for the lane's KC poles, and l,
-// from a forward stage; s: the lane's state
+// acc += v w for complex limb pairs (re hi, re lo, im hi, im lo)
+__device__ __forceinline__ void cmad(long long &rh, long long &rl, long long &ih, long long &il, int4 v, int4 w) {
+  mad(rh, rl, v.x, v.y, w.x, w.y);
+  mad(rh, rl, -v.z, -v.w, w.z, w.w);
+  mad(ih, il, v.x, v.y, w.z, w.w);
+  mad(ih, il, v.z, v.w, w.x, w.y);
+}
+
+// r = delta0 + Phi'/alpha + zeta'_{n-1}/s_{n-1} + zeta'_{n+1}/s_{n+1} at one row for the lane's KC
+// poles (the inputs carry the row's real factors), and l, from the row's stage and the next;
+// s: the lane's state
 template <int KC>
-__device__ __forceinline__ void right_hand_sides(const char *stage, int s, int lane, double2 (&r)[2], double2 (&l)[2]) {
+__device__ __forceinline__ void right_hand_sides(const char *stage, const char *next, const char *inv_alpha, int e0,
+                                                 const int (&one)[2], int s, int lane, double2 (&r)[2], double2 (&l)[2]) {
   int4 in[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) in[j] = reinterpret_cast<const int4 *>(stage + kSIn)[s * 4 + j];
-  const int U = reinterpret_cast<const int *>(stage + kSU)[s] - 57;
+  const int e = reinterpret_cast<const int *>(stage + kSU)[s] + e0 - 57;
 #pragma unroll
   for (int c = 0; c < KC; ++c) {
-    const int e = reinterpret_cast<const int *>(stage + kSE)[c * 32 + lane];
-    // delta: its weight is a power of two, one limb
-    const int one = e > 28 ? 0 : 1 << (28 - e);
+    // delta: its weight 1 is one limb (0 past the last pole)
     long long rh = 0, rl = 1 << 28, ih = 0, il = 1 << 28;  // the middle sums are rounded at bit 29
-    mad_wide(rh, one, in[0].x);
-    mad_wide(rl, one, in[0].y);
-    mad_wide(ih, one, in[0].z);
-    mad_wide(il, one, in[0].w);
-#pragma unroll
-    for (int j = 1; j < 4; ++j) {
-      const int4 v = reinterpret_cast<const int4 *>(stage)[(c * 4 + j - 1) * 32 + lane];
-      mad(rh, rl, v.x, v.y, in[j].x, in[j].y);
-      mad(rh, rl, -v.z, -v.w, in[j].z, in[j].w);
-      mad(ih, il, v.x, v.y, in[j].z, in[j].w);
-      mad(ih, il, v.z, v.w, in[j].x, in[j].y);
-    }
-    l[c] = reinterpret_cast<const double2 *>(stage)[(c * 4 + 3) * 32 + lane];
-    r[c] = make_double2(fixed_to_double((rh << 1) + (rl >> 29), U + e), fixed_to_double((ih << 1) + (il >> 29), U + e));
+    mad_wide(rh, one[c], in[0].x);
+    mad_wide(rl, one[c], in[0].y);
+    mad_wide(ih, one[c], in[0].z);
+    mad_wide(il, one[c], in[0].w);
+    cmad(rh, rl, ih, il, reinterpret_cast<const int4 *>(inv_alpha)[c * 32 + lane], in[1]);
+    cmad(rh, rl, ih, il, reinterpret_cast<const int4 *>(stage)[c * 32 + lane], in[2]);
+    cmad(rh, rl, ih, il, reinterpret_cast<const int4 *>(next)[c * 32 + lane], in[3]);
+    l[c] = reinterpret_cast<const double2 *>(stage)[(2 + c) * 32 + lane];
+    r[c] = make_double2(fixed_to_double((rh << 1) + (rl >> 29), e), fixed_to_double((ih << 1) + (il >> 29), e));
   }
 }
 
-// The window's weighted sums of a row's solutions x, over the lanes of each state: returns the
-// one of the eight (stream, part) values that this lane ends up with (index: see sum_index).
+// The window's sums over the lanes of each state of u = (beta/d') x, u/alpha, u/s_{n+1} and
+// u/s_{n-1}, x a row's solutions: returns the one of the eight (stream, part) values that this lane
+// ends up with (index: see sum_index).  prev: the stage of the row before (n + 2); wexp: the
+// exponent of beta/d' and the stream's.
 template <int SB, int KC>
-__device__ __forceinline__ double weighted_sums(const char *stage, int wexp, const double2 (&x)[2], int lane) {
+__device__ __forceinline__ double weighted_sums(const char *stage, const char *prev, const char *inv_alpha, int wexp,
+                                                const double2 (&x)[2], int lane) {
   constexpr int LPS = 32 / SB;  // lanes per state
   int E = 0;
 #pragma unroll
@@ -124,26 +135,28 @@ __device__ __forceinline__ double weighted_sums(const char *stage, int wexp, con
   for (int o = 1; o < LPS; o <<= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
   E >>= 20;
   const bool finite = E != 0x7ff;
-  const int Ew = E - 1023 - 53;
+  const int Ew = E - 1023;
   if (E < 64) E += 4096;  // groups below 2^-959 are taken as zero
-  long long hh[8], hl[8];
+  // sums over up to 64 poles of numbers below 2^59: kept in units of 2^3
+  long long hh[8], hl[8], t[8];
+  t[0] = t[1] = 4;
 #pragma unroll
-  for (int j = 0; j < 8; ++j) hh[j] = 0, hl[j] = 1 << 29;  // rounded at bit 30
+  for (int j = 2; j < 8; ++j) hh[j] = 4, hl[j] = 1 << 29;  // rounded at bit 30, then at bit 3
 #pragma unroll
   for (int c = 0; c < KC; ++c) {
-    const int2 re = limbs(fixed59(x[c].x, E)), im = limbs(fixed59(x[c].y, E));
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      const int4 v = reinterpret_cast<const int4 *>(stage)[(c * 5 + 1 + s) * 32 + lane];
-      mad(hh[2 * s], hl[2 * s], v.x, v.y, re.x, re.y);
-      mad(hh[2 * s], hl[2 * s], v.z, v.w, -im.x, -im.y);
-      mad(hh[2 * s + 1], hl[2 * s + 1], v.x, v.y, im.x, im.y);
-      mad(hh[2 * s + 1], hl[2 * s + 1], v.z, v.w, re.x, re.y);
-    }
+    long long rh = 0, rl = 1 << 29, ih = 0, il = 1 << 29;
+    cmad(rh, rl, ih, il, reinterpret_cast<const int4 *>(stage)[(2 * KC + c) * 32 + lane],
+         limbs2(fixed59(x[c].x, E), fixed59(x[c].y, E)));
+    const long long ur = rh + (rl >> 30), ui = ih + (il >> 30);
+    t[0] += ur;
+    t[1] += ui;
+    const int4 u = limbs2(ur, ui);
+    cmad(hh[2], hl[2], hh[3], hl[3], reinterpret_cast<const int4 *>(inv_alpha)[c * 32 + lane], u);
+    cmad(hh[4], hl[4], hh[5], hl[5], reinterpret_cast<const int4 *>(prev)[c * 32 + lane], u);
+    cmad(hh[6], hl[6], hh[7], hl[7], reinterpret_cast<const int4 *>(stage)[c * 32 + lane], u);
   }
-  long long t[8];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) t[j] = hh[j] + (hl[j] >> 30);
+  for (int j = 0; j < 8; ++j) t[j] = (j < 2 ? t[j] : hh[j] + (hl[j] >> 30)) >> 3;
   int n = 8;
 #pragma unroll
   for (int o = LPS / 2; o > 0; o >>= 1) {
@@ -172,43 +185,48 @@ __device__ __forceinline__ int sum_index(int lane) {
 }
 
 template <int SB, int KC>
-__device__ void sweep_window(const LimbSweep &a, int64_t row0, int len, int p0, int b0, int idx, double *part, bool first,
-                             double2 *yb, char *smem, int lane) {
+__device__ void sweep_window(const LimbSweep &a, int sysid, int64_t row0, int len, int p0, int b0, int idx, double *part,
+                             bool first, double2 *yb, char *smem, int lane) {
   constexpr int LPS = 32 / SB;
   const int k = lane & (LPS - 1), s = lane / LPS, blk = p0 / kBlock, pk = p0 % kBlock + k;
   const int64_t rec = row0 * a.nblk + (int64_t)blk * len;
+  const char *inv0 = a.inv + ((row0 + sysid) * a.nblk + (int64_t)blk * (len + 1)) * kRec + pk * 16;
   const unsigned sm = (unsigned)__cvta_generic_to_shared(smem);
+  const char *ia = smem + kInvAlpha;
   {  // forward: y_i = r_i - l y_{i-1}; row i + 1's r is formed beside the FMAs of row i
-    const char *f = a.fwd + rec * kFwd;
+    const char *f = a.fwd + rec * kRec + pk * 16, *inv = inv0;
     const int4 *dig = a.dig + (row0 * a.B + b0) * 4;
     const int *uexp = a.uexp + row0 * a.B + b0;
     const int ns = min(SB, a.B - b0);  // states with inputs of their own
-    int todo = len;                    // rows not copied yet
-    unsigned to = sm;
+    int j = 0;                         // next stage to copy, 0..len
     auto issue = [&]() {
-      if (todo > 0) {
+      if (j <= len) {
+        const unsigned to = sm + (j & 3) * kStage;
 #pragma unroll
-        for (int c = 0; c < KC; ++c) {
+        for (int c = 0; c < KC; ++c) copy_async<16>(to + (c * 32 + lane) * 16, inv + c * LPS * 16);
+        if (j < len) {
 #pragma unroll
-          for (int j = 0; j < 4; ++j) copy_async<16>(to + (c * 4 + j) * 512 + lane * 16, f + j * 1024 + (pk + c * LPS) * 16);
-          copy_async<4>(to + kSE + (c * 32 + lane) * 4, f + kFE + (pk + c * LPS) * 4);
+          for (int c = 0; c < KC; ++c) copy_async<16>(to + ((2 + c) * 32 + lane) * 16, f + c * LPS * 16);
+          if (lane < 4 * ns) copy_async<16>(to + kSIn + lane * 16, dig + lane);
+          else if (lane >= 16 && lane < 16 + ns) copy_async<4>(to + kSU + (lane - 16) * 4, uexp + lane - 16);
         }
-        if (lane < 4 * ns) copy_async<16>(to + kSIn + lane * 16, dig + lane);
-        else if (lane >= 16 && lane < 16 + ns) copy_async<4>(to + kSU + (lane - 16) * 4, uexp + lane - 16);
-        f += kFwd;
+        inv += kRec;
+        f += kRec;
         dig += a.B * 4;
         uexp += a.B;
-        --todo;
-        to = to == sm + (kFwdStages - 1) * kStage ? sm : to + kStage;
+        ++j;
       }
       copy_commit();
     };
     __syncwarp();  // every lane has read the stages of the window before
+#pragma unroll
+    for (int c = 0; c < KC; ++c) copy_async<16>(sm + kInvAlpha + (c * 32 + lane) * 16, a.inv_alpha + p0 + k + c * LPS);
+    issue();
     issue();
     issue();
     const int mine = min(s, ns - 1);
+    const int one[2] = {p0 + k < a.P ? 1 << (28 - a.e0) : 0, p0 + k + LPS < a.P ? 1 << (28 - a.e0) : 0};
     double2 *yp = yb;
-    const char *stage = smem;
     double2 y[2] = {make_double2(0, 0), make_double2(0, 0)}, r[2], l[2];
     for (int i = 0; i <= len; ++i) {
       if (i > 0) {
@@ -217,10 +235,9 @@ __device__ void sweep_window(const LimbSweep &a, int64_t row0, int len, int p0, 
       }
       if (i < len) {
         copy_wait<1>();
-        __syncwarp();  // row i has landed for every lane; the stage of row i - 1 has been read
+        __syncwarp();  // stages i and i + 1 have landed for every lane; i - 1 has been read
         issue();
-        right_hand_sides<KC>(stage, mine, lane, r, l);
-        stage = stage == smem + (kFwdStages - 1) * kStage ? smem : stage + kStage;
+        right_hand_sides<KC>(smem + (i & 3) * kStage, smem + ((i + 1) & 3) * kStage, ia, a.e0, one, mine, lane, r, l);
       }
       if (i > 0) {
 #pragma unroll
@@ -230,25 +247,32 @@ __device__ void sweep_window(const LimbSweep &a, int64_t row0, int len, int p0, 
     }
   }
   {  // backward: x_i = y_i - Chat x_{i+1}; the sums of row i + 1 beside the FMAs of row i
-    const char *f = a.bwd + (rec + len - 1) * kBwd;
-    int todo = len;
-    unsigned odd = 0;
-    auto issue = [&]() {  // the lane's own copies only
-      if (todo > 0) {
-        const unsigned to = sm + odd * (KC * 5 * 512) + lane * 16;
+    const char *f = a.bwd + (rec + len - 1) * kBwd + pk * 16, *inv = inv0 + (int64_t)len * kRec;
+    const int *we = reinterpret_cast<const int *>(a.bwd + (rec + len - 1) * kBwd + kBE);
+    const int se = idx > 1 ? a.e0 - 51 : -53;
+    int j = len;  // next stage to copy, len..0; the lane's own copies only
+    auto issue = [&]() {
+      if (j >= 0) {
+        const unsigned to = sm + (j & 3) * kStage + lane * 16;
 #pragma unroll
-        for (int c = 0; c < KC; ++c)
+        for (int c = 0; c < KC; ++c) copy_async<16>(to + c * 512, inv + c * LPS * 16);
+        if (j < len) {
 #pragma unroll
-          for (int j = 0; j < 5; ++j) copy_async<16>(to + (c * 5 + j) * 512, f + j * 1024 + (pk + c * LPS) * 16);
-        f -= kBwd;
-        --todo;
-        odd ^= 1;
+          for (int c = 0; c < KC; ++c) {
+            copy_async<16>(to + (KC + c) * 512, f + c * LPS * 16);
+            copy_async<16>(to + (2 * KC + c) * 512, f + kRec + c * LPS * 16);
+          }
+          f -= kBwd;
+        }
+        inv -= kRec;
+        --j;
       }
       copy_commit();
     };
-    const int *we = reinterpret_cast<const int *>(f + kBE) + (idx >= 0 ? idx >> 1 : 0);
     copy_wait<0>();
     __syncwarp();
+    issue();
+    issue();
     issue();
     const double2 *yp = yb + (len - 1) * 64;
     part += (int64_t)(len - 1) * a.B * 8 + (idx > 0 ? idx : 0);
@@ -259,20 +283,20 @@ __device__ void sweep_window(const LimbSweep &a, int64_t row0, int len, int p0, 
       y[c] = len > 1 ? yp[c * 32 - 64] : x[c];
     }
     for (int i = len - 1; i >= 0; --i) {
-      const char *stage = smem + (odd ^ 1) * (KC * 5 * 512);
-      const int wexp = __ldg(we);
+      const char *stage = smem + (i & 3) * kStage;
+      const int wexp = __ldg(we) + se;
       double sum = 0;
       if (!first && idx >= 0) sum = *part;
-      copy_wait<0>();
-      issue();
+      copy_wait<1>();  // stages i + 1 and i
+      issue();         // stage i - 2, in the place of i + 2
       double2 xn[2];
 #pragma unroll
       for (int c = 0; c < KC; ++c) {
         // Chat of row i - 1 is stored with row i (zero with row 0, whose xn is not used)
-        xn[c] = cfms(y[c], reinterpret_cast<const double2 *>(stage)[(c * 5) * 32 + lane], x[c]);
+        xn[c] = cfms(y[c], reinterpret_cast<const double2 *>(stage)[(KC + c) * 32 + lane], x[c]);
         if (i > 1) y[c] = yp[c * 32 - 128];
       }
-      const double v = weighted_sums<SB, KC>(stage, wexp, x, lane);
+      const double v = weighted_sums<SB, KC>(stage, smem + ((i + 1) & 3) * kStage, ia, wexp, x, lane);
       if (idx >= 0) *part = sum + v;
       part -= a.B * 8;
       we = reinterpret_cast<const int *>(reinterpret_cast<const char *>(we) - kBwd);
@@ -296,8 +320,8 @@ __device__ __forceinline__ void limb_item(const LimbSweep &a, int4 item, int lan
   double *part = a.part + (((int64_t)item.w * a.nrows + sy.w) * a.B + min(state, a.B - 1)) * 8;
   for (int w = w0; w < w1; ++w) {
     const int p0 = w * per;
-    if (a.kc == 2 && p0 + LPS < a.P) sweep_window<SB, 2>(a, sy.w, sy.z, p0, b0, idx, part, w == w0, yb, smem, lane);
-    else sweep_window<SB, 1>(a, sy.w, sy.z, p0, b0, idx, part, w == w0, yb, smem, lane);
+    if (a.kc == 2 && p0 + LPS < a.P) sweep_window<SB, 2>(a, item.x, sy.w, sy.z, p0, b0, idx, part, w == w0, yb, smem, lane);
+    else sweep_window<SB, 1>(a, item.x, sy.w, sy.z, p0, b0, idx, part, w == w0, yb, smem, lane);
   }
 }
 

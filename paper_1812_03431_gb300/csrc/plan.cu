@@ -102,9 +102,10 @@ __global__ void alp_tables_kernel(const double *mu_all, int N, int J, double *ta
 void free_plan(Plan *pl);
 
 // The smallest batch the digit solve takes by default: its warps carry tiles of eight states;
-// five of them still take a third of the pole-slot solve's time (T85: 0.20 / 0.62 ms); up to
-// four the fused solve is the default.  Then the most device memory its factors may take: 1312 B per
-// row and eight poles, 1.14 times the binary64 factors.
+// five of them still take a third of the pole-slot solve's time (T85: 0.18 / 0.62 ms).  Plans of
+// up to four states use the limb solve (T170, four states: 0.80 ms against 2.08 fused).  Then the
+// most device memory either's factors may take: 164 and 64 B per row and pole beside the
+// binary64 factors' 144.
 constexpr int kDigitMinBatch = 5;
 constexpr size_t kDigitMostBytes = (size_t)32 << 30;
 
@@ -347,7 +348,7 @@ rexi_status build_plan(const rexi_params &prm, Plan *pl) {
     if ((e = cudaMemGetInfo(&mem_free, &mem_total))) return fail("memory", e);
     const size_t need = digit_factor_bytes(*pl) + digit_state_bytes(*pl, prm.max_batch);
     if (need <= std::min(kDigitMostBytes, mem_free / 3)) {
-      if ((e = build_digit_factors(*pl, pl->fac_fwd, pl->dig_fwd))) return fail("digit factors", e);
+      if ((e = build_digit_factors(*pl, false, pl->fac_fwd, pl->dig_fwd))) return fail("digit factors", e);
       if (pl->dig_fwd.fwd && cudaMalloc(&pl->dig_state, digit_state_bytes(*pl, prm.max_batch)) != cudaSuccess) {
         cudaGetLastError();
         pl->dig_state = nullptr;

@@ -126,6 +126,11 @@ struct FusedRagged {
 struct DigitFactors {
   char *fwd = nullptr, *bwd = nullptr;
   int *vexp = nullptr;
+  // limbs only: reciprocals of the shifts, of the poles, their exponent, the rows' real factors
+  char *inv = nullptr;
+  int4 *inv_alpha = nullptr;
+  int e0 = 0;
+  double *scale = nullptr;
 };
 
 // The digit solve's work list for one batch size: items (system, tile of eight states,
@@ -340,15 +345,14 @@ cudaError_t launch_solve_fused(Plan &pl, const FusedLayout &F, bool adjoint, con
 size_t digit_factor_bytes(const Plan &pl);
 size_t digit_state_bytes(const Plan &pl, int B);
 size_t digit_slot_bytes(const Plan &pl, int B);
-cudaError_t build_digit_factors(Plan &pl, const double2 *fac, DigitFactors &D);
+cudaError_t build_digit_factors(Plan &pl, bool adjoint, const double2 *fac, DigitFactors &D);
 void free_digit_factors(DigitFactors &D);
 int limb_tile(int B);
 int limb_window(int B, int kc);
 size_t limb_factor_bytes(const Plan &pl);
 size_t limb_state_bytes(const Plan &pl, int B);
 cudaError_t limb_configure(int B);
-void limb_record_bytes(size_t *fwd, size_t *bwd, int *block);
-cudaError_t launch_limb_factors(Plan &pl, const double2 *fac, DigitFactors &D, int kmid, int *bad);
+cudaError_t launch_limb_factors(Plan &pl, bool adjoint, const double2 *fac, DigitFactors &D, int *bad);
 cudaError_t launch_limb_state(Plan &pl, bool adjoint, const double2 *sin, int B, cudaStream_t st);
 cudaError_t launch_solve_limbs(Plan &pl, const DigitLayout &L, bool adjoint, int B, cudaStream_t st);
 cudaError_t launch_digit_state(Plan &pl, bool adjoint, const double2 *sin, int B, cudaStream_t st);

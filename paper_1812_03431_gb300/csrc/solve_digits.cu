@@ -205,6 +205,7 @@ struct FinishArgs {
   const int4 *sys;
   double2 sphi;
   int64_t nspec, nrows;
+  const double *scale;  // limbs: per row the sums' real factors at 3..5 (see solve_limbs.cu), else null
   int B, tile, tiles, unit, sstr, pstr, slots, N;
 };
 
@@ -225,7 +226,12 @@ __global__ void digit_finish_kernel(FinishArgs a) {
           const int4 sy = a.sys[2 * m + ((nn - m) & 1)];
           const int64_t row = sy.w + (nn - sy.y) / 2;
           const double *p = a.part + (row * a.tiles + b / a.tile) * a.unit + b % a.tile + stream * a.sstr;
-          for (int s = 0; s < a.slots; ++s, p += slot) acc = make_double2(acc.x + p[0], acc.y + p[a.pstr]);
+          if (a.scale && stream > 0) {
+            const double c = a.scale[row * 6 + 2 + stream];
+            for (int s = 0; s < a.slots; ++s, p += slot) acc = make_double2(fma(c, p[0], acc.x), fma(c, p[a.pstr], acc.y));
+          } else {
+            for (int s = 0; s < a.slots; ++s, p += slot) acc = make_double2(acc.x + p[0], acc.y + p[a.pstr]);
+          }
         };
         const int nmin = m > 1 ? m : 1;
         if (f != 1) add(n, f == 2 ? 0 : 1);
@@ -257,7 +263,7 @@ int windows_of(const Plan &pl, int B, int kc) {
 }  // namespace
 
 void free_digit_factors(DigitFactors &D) {
-  for (void *p : {(void *)D.fwd, (void *)D.bwd, (void *)D.vexp})
+  for (void *p : {(void *)D.fwd, (void *)D.bwd, (void *)D.vexp, (void *)D.inv, (void *)D.inv_alpha, (void *)D.scale})
     if (p) cudaFree(p);
   D = DigitFactors{};
 }
@@ -267,50 +273,51 @@ size_t digit_factor_bytes(const Plan &pl) {
   return (size_t)pl.nrows * ((pl.P + kWin - 1) / kWin) * (kFwdRec + kBwdRec) + (size_t)pl.nrows * 4 * sizeof(int);
 }
 
+namespace {
+cudaError_t launch_digit_factors(Plan &pl, const double2 *fac, DigitFactors &D, int *bad) {
+  const int nwin = (pl.P + kWin - 1) / kWin;
+  const size_t nrec = (size_t)pl.nrows * nwin;
+  cudaError_t e = cudaMalloc(&D.fwd, nrec * kFwdRec);
+  if (e == cudaSuccess) e = cudaMalloc(&D.bwd, nrec * kBwdRec);
+  if (e == cudaSuccess) e = cudaMalloc(&D.vexp, (size_t)pl.nrows * 4 * sizeof(int));
+  if (e != cudaSuccess) return e;
+  SetupArgs a;
+  a.fac = fac;
+  a.sys = pl.sys_dev;
+  a.fwd = D.fwd;
+  a.bwd = D.bwd;
+  a.vexp = D.vexp;
+  a.bad = bad;
+  a.P = pl.P;
+  a.nwin = nwin;
+  a.kmid = (int)(std::min_element(pl.alpha.begin(), pl.alpha.end(),
+                                  [](const cplx &x, const cplx &y) { return std::abs(x) < std::abs(y); }) -
+                 pl.alpha.begin());
+  a.nrows = pl.nrows;
+  const int64_t most = (int64_t)pl.lmax * nwin * kWin;
+  digit_factor_kernel<<<dim3((unsigned)((most + 255) / 256), (unsigned)pl.sys.size()), 256>>>(a);
+  return cudaGetLastError();
+}
+}  // namespace
+
 // The factor set as digits or limbs (pl.limbs), from the binary64 factors `fac`.  D stays empty
 // (and the other solve kernels serve the plan) where the device memory does not suffice, or
 // where a factor is not finite or a pole's couplings differ in scale by more than the
 // fixed-point forms cover.
-cudaError_t build_digit_factors(Plan &pl, const double2 *fac, DigitFactors &D) {
+cudaError_t build_digit_factors(Plan &pl, bool adjoint, const double2 *fac, DigitFactors &D) {
   D = DigitFactors{};
-  size_t fwd = kFwdRec, bwd = kBwdRec;
-  int block = kWin;
-  if (pl.limbs) limb_record_bytes(&fwd, &bwd, &block);
-  const int nwin = (pl.P + block - 1) / block;
   if (pl.nrows == 0 || (pl.P + kWin - 1) / kWin > 0x7fff || pl.sys.size() > 0xffff) return cudaSuccess;
-  const size_t nrec = (size_t)pl.nrows * nwin;
-  if (cudaMalloc(&D.fwd, nrec * fwd) != cudaSuccess || cudaMalloc(&D.bwd, nrec * bwd) != cudaSuccess ||
-      cudaMalloc(&D.vexp, (size_t)pl.nrows * 4 * sizeof(int) + sizeof(int)) != cudaSuccess) {
+  int *bad = nullptr, hbad = 0;
+  cudaError_t e = cudaMalloc(&bad, sizeof(int));
+  if (e == cudaSuccess) e = cudaMemsetAsync(bad, 0, sizeof(int), 0);
+  if (e == cudaSuccess) e = pl.limbs ? launch_limb_factors(pl, adjoint, fac, D, bad) : launch_digit_factors(pl, fac, D, bad);
+  if (e == cudaSuccess) e = cudaMemcpy(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost);
+  if (bad) cudaFree(bad);
+  if (e != cudaSuccess || hbad) free_digit_factors(D);
+  if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
-    free_digit_factors(D);
     return cudaSuccess;
   }
-  int *bad = D.vexp + pl.nrows * 4;
-  cudaError_t e = cudaMemsetAsync(bad, 0, sizeof(int), 0);
-  const int kmid = (int)(std::min_element(pl.alpha.begin(), pl.alpha.end(),
-                                          [](const cplx &x, const cplx &y) { return std::abs(x) < std::abs(y); }) -
-                         pl.alpha.begin());
-  if (e == cudaSuccess && pl.limbs) {
-    e = launch_limb_factors(pl, fac, D, kmid, bad);
-  } else if (e == cudaSuccess) {
-    SetupArgs a;
-    a.fac = fac;
-    a.sys = pl.sys_dev;
-    a.fwd = D.fwd;
-    a.bwd = D.bwd;
-    a.vexp = D.vexp;
-    a.bad = bad;
-    a.P = pl.P;
-    a.nwin = nwin;
-    a.kmid = kmid;
-    a.nrows = pl.nrows;
-    const int64_t most = (int64_t)pl.lmax * nwin * kWin;
-    digit_factor_kernel<<<dim3((unsigned)((most + 255) / 256), (unsigned)pl.sys.size()), 256>>>(a);
-    e = cudaGetLastError();
-  }
-  int hbad = 0;
-  if (e == cudaSuccess) e = cudaMemcpy(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess || hbad) free_digit_factors(D);
   return e;
 }
 
@@ -464,6 +471,7 @@ cudaError_t launch_finish_digits(Plan &pl, const DigitLayout &L, bool adjoint, c
   f.sstr = 2 * f.tile;
   f.pstr = f.tile;
   f.slots = L.slots;
+  f.scale = (adjoint ? pl.dig_adj : pl.dig_fwd).scale;
   f.N = pl.N;
   const int64_t total = 3 * pl.nspec * B;
   digit_finish_kernel<<<(unsigned)std::min<int64_t>((total + 255) / 256, 1 << 20), 256, 0, st>>>(f);

@@ -5,26 +5,31 @@
 // on the FP64 unit (one warp instruction per 64 cycles and scheduler); the right-hand sides
 // and the beta-weighted sums, 28 of the 36, are fixed-point products.  With one state a factor is
 // used once, so the tensor cores would multiply mostly padding: here each operand is a 59-bit
-// integer (weights: 56) relative to the largest of its group, held as two signed limbs of radix
-// 2^30, and a product is three 32 x 32 -> 64 bit multiply-adds into a high and a middle 64-bit
-// sum, 40 for the four inputs of a right-hand side and 48 for the four weighted sums of a pole.
-// The product of the low limbs, below 2^-60 of the largest product, is left out; nothing else
-// is rounded until a sum is put together (59 bits below the largest product) and rounded to
-// binary64 once.  A window's sums over the lanes are 64-bit integer additions.
+// integer relative to the largest of its group, held as two signed limbs of radix 2^30, and a
+// product is three 32 x 32 -> 64 bit multiply-adds into a high and a middle 64-bit sum.  The
+// product of the low limbs, below 2^-60 of the largest product, is left out.
+//
+// A row's couplings and weights are not stored one by one: each is a real number of the row
+// times 1/alpha, 1/s_{n-1}, 1/s_{n+1} (s_n = alpha + i tau sigma_n, shared by neighbouring rows), and
+// for the weights beta/d'.  The real numbers go into the inputs before the sweep and into the
+// sums after it; the sweep forms u = (beta/d') w once and sums u, u/alpha, u/s_{n+1} and u/s_{n-1}:
+// 40 multiply-adds for a right-hand side and 48 for the sums as with stored factors, at 64 B per
+// row and pole instead of 148.  Roundings: u at 2^-59 of the window's largest, a lane's sums at
+// 2^-56, the total once to binary64; sums over the lanes are 64-bit integer additions.
 //
 // Measured on GB300 (solve with its sums, against the fused FP64 solve): T341, 535 poles, one state
-// 0.91 / 2.10 ms, four states 3.04 / 8.12; T170 x 1 0.27 / 0.56, T128 x 1 with 1047 poles 0.29 / 0.61,
-// T639 x 1 3.05 / 7.87 (slot solve), T63 x 1 with 279 poles 0.073 / 0.089.  With one state the factors
-// bound it (T639: 16.3 GB per step, 5.3 TB/s), with four the FP64 unit and the instruction issue
-// share it; small truncations wait on the row-to-row chain of their few warps.
+// 0.81 / 2.10 ms, four states 3.04 / 8.12; T170 x 1 0.27 / 0.56, T128 x 1 with 1047 poles 0.27 / 0.61,
+// T639 x 1 2.72 / 7.87 (slot solve), T63 x 1 with 279 poles 0.066 / 0.089.  With every factor of a
+// row stored (148 B per row and pole) one state waited on HBM: T639 3.05 ms, T341 0.91.  Now the
+// integer pipe is 59 % and the FP64 unit 57 % busy (ncu, T341 x 1) and the rest is latency; small
+// truncations wait on the row-to-row chain of their few warps.
 //
 // Lanes of a warp are (state, pole): SB states x 32 / SB poles, two poles per lane where the
-// window is full (poles k and k + 32 / SB), one for a short last window.  The factors are as
-// large as the binary64 set (148 B per row and pole) and each is read once per tile of states.
+// window is full (poles k and k + 32 / SB), one for a short last window.
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <string>
+#include <cmath>
 #include <vector>
 
 #include "limb_sweep.h"
@@ -40,77 +45,80 @@ namespace {
 // ---- plan time ----------------------------------------------------------------------------------
 struct SetupArgs {
   const double2 *fac;  // [F_NCOMP][nrows][P]
+  const double2 *alpha;
+  const double *coef;  // [nspec][4]: sigma, ct, dt, G
   const int4 *sys;
-  char *fwd, *bwd;     // records, system by system: [block][row of the system]
-  int *vexp;           // [nrows][4]: the scale of each input (0 for delta)
+  char *fwd, *bwd, *inv;
+  int4 *inv_alpha;
+  double *scale;       // [nrows][6]: inputs Phi, zeta_{n-1}, zeta_{n+1}; sums Phi, zeta_{n+1}, zeta_{n-1}
   int *bad;            // set when the factors are not finite or too unlike in scale
-  int P, nblk, kmid;
+  int P, nblk, N, e0, adjoint;
   int64_t nrows;
+  double tau, q, phibar;  // q = 2 Omega tau
 };
 
+// One block of threads per (system, block of poles, j = 0..len): 1/s at degree n0 - 1 + 2 j and,
+// for j < len, the row's l, Chat and beta/d' and its real factors.
 __global__ void __launch_bounds__(kBlock) limb_factor_kernel(SetupArgs a) {
-  __shared__ int emx[2][4];
+  __shared__ int emx[2];
   const int4 sy = a.sys[blockIdx.y];
-  const int len = sy.z, i = blockIdx.x / a.nblk, blk = blockIdx.x - i * a.nblk;
-  if (i >= len) return;
-  const int64_t row0 = sy.w, row = row0 + i;
-  const int p = threadIdx.x, k = blk * kBlock + p;
+  const int m = sy.x, n0 = sy.y, len = sy.z, j = blockIdx.x / a.nblk, blk = blockIdx.x - j * a.nblk;
+  if (len == 0 || j > len) return;
+  const int64_t row0 = sy.w, row = row0 + j;
+  const int p = threadIdx.x, k = blk * kBlock + p, nmin = m > 1 ? m : 1;
   const bool live = k < a.P;
-  auto get = [&](int comp, int kk) {
-    return kk < a.P ? a.fac[((int64_t)comp * a.nrows + row) * a.P + kk] : make_double2(0, 0);
+  const double2 zero = make_double2(0, 0);
+  auto C4 = [&](int n, int c) {
+    return n < nmin || n > a.N ? 0.0 : a.coef[4 * ((int64_t)m * (2 * a.N + 3 - m) / 2 + (n - m)) + c];
   };
   auto emax = [](double2 v) { return max(bexp(v.x), bexp(v.y)); };
-  const int64_t rec = row0 * a.nblk + (int64_t)blk * len + i;
-  char *fr = a.fwd + rec * kFwd, *br = a.bwd + rec * kBwd;
   bool bad = false;
-
-  // couplings of Phi, zeta_{n-1}, zeta_{n+1} (delta's is 1), negated; 59 bits below the pole's largest
-  const int comp[3] = {F_G, F_E, F_F};
-  double2 v[3];
-  int ve[3], E = live ? 1023 : 0;
+  // the reciprocal of s as 59 bits below 2^(e0 + 1); the poles' may differ by kMaxSpread bits
+  auto inverse = [&](double2 s) {
+    if (!live) return make_int4(0, 0, 0, 0);
+    const double d = s.x * s.x + s.y * s.y;
+    const double2 v = make_double2(s.x / d, -s.y / d);
+    const int e = emax(v), top = a.e0 + 1023;
+    if (e > top || e + kMaxSpread < top) {  // also what is not finite
+      bad = true;
+      return make_int4(0, 0, 0, 0);
+    }
+    return limbs2((to_fixed(v.x, top - bexp(v.x)) + 4) >> 3, (to_fixed(v.y, top - bexp(v.y)) + 4) >> 3);
+  };
+  double2 al = live ? a.alpha[k] : make_double2(1, 0);
+  if (a.adjoint) al.y = -al.y;
+  const double sg = a.tau * C4(n0 - 1 + 2 * j, 0);
+  reinterpret_cast<int4 *>(a.inv + ((row0 + blockIdx.y) * a.nblk + (int64_t)blk * (len + 1) + j) * kRec)[p] =
+      inverse(make_double2(al.x, a.adjoint ? al.y - sg : al.y + sg));
+  if (row == 0 && j == 0) a.inv_alpha[k] = inverse(al);
+  if (j < len) {
+    auto get = [&](int comp, int64_t r) { return live ? a.fac[((int64_t)comp * a.nrows + r) * a.P + k] : zero; };
+    const int64_t rec = row0 * a.nblk + (int64_t)blk * len + j;
+    const double2 l = get(F_L, row), c = j > 0 ? get(F_C, row - 1) : zero, b = get(F_BD, row);
+    if (emax(l) == 0x7ff || emax(c) == 0x7ff || emax(b) == 0x7ff) bad = true;
+    char *br = a.bwd + rec * kBwd;
+    reinterpret_cast<double2 *>(a.fwd + rec * kRec)[p] = l;
+    reinterpret_cast<double2 *>(br)[p] = c;
+    // beta/d': 59 bits below the block's largest
+    int top = emax(b);
 #pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    v[j] = get(comp[j], k);
-    v[j] = make_double2(-v[j].x, -v[j].y);
-    const int mid = emax(get(comp[j], a.kmid)), e = emax(v[j]);
-    ve[j] = mid == 0 ? 0 : mid - 1023;
-    if (e == 0x7ff) bad = true;
-    if (e) E = max(E, e - ve[j]);
-  }
-  if (live && E - 1023 > kMaxSpread) bad = true;
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    const int e = emax(v[j]);
-    if (e && E - (e - ve[j]) > kMaxSpread) bad = true;
-    reinterpret_cast<int4 *>(fr)[j * kBlock + p] = limbs2((to_fixed(v[j].x, E - (bexp(v[j].x) - ve[j])) + 4) >> 3,
-                                                          (to_fixed(v[j].y, E - (bexp(v[j].y) - ve[j])) + 4) >> 3);
-  }
-  const double2 l = get(F_L, k), c = get(F_C, k);
-  if (emax(l) == 0x7ff || emax(c) == 0x7ff) bad = true;
-  reinterpret_cast<double2 *>(fr + kFL)[p] = l;
-  reinterpret_cast<int *>(fr + kFE)[p] = live ? E - 1023 : kNoPole;
-  reinterpret_cast<double2 *>(br)[p] =
-      i > 0 && k < a.P ? a.fac[((int64_t)F_C * a.nrows + row - 1) * a.P + k] : make_double2(0, 0);
-  if (blk == 0 && p < 4) a.vexp[row * 4 + p] = p == 0 ? 0 : ve[p - 1];
-
-  // the four weights, 56 bits below the block's largest
-  const int wc[4] = {F_BD, F_BAD, F_ZP, F_ZM};
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    int m = emax(get(wc[s], k));
-    if (m == 0x7ff) bad = true;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((p & 31) == 0) emx[p >> 5][s] = m;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const double2 x = get(wc[s], k);
-    const int m = max(emx[0][s], emx[1][s]);
-    reinterpret_cast<int4 *>(br + kBW)[s * kBlock + p] =
-        limbs2((to_fixed(x.x, m - bexp(x.x)) + 32) >> 6, (to_fixed(x.y, m - bexp(x.y)) + 32) >> 6);
-    if (p == s) reinterpret_cast<int *>(br + kBE)[s] = m - 1023;
+    for (int o = 1; o < 32; o <<= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+    if ((p & 31) == 0) emx[p >> 5] = top;
+    __syncthreads();
+    top = max(emx[0], emx[1]);
+    reinterpret_cast<int4 *>(br + kRec)[p] =
+        limbs2((to_fixed(b.x, top - bexp(b.x)) + 4) >> 3, (to_fixed(b.y, top - bexp(b.y)) + 4) >> 3);
+    if (p == 0) *reinterpret_cast<int *>(br + kBE) = top - 1023;
+    if (blk == 0 && p == 0) {
+      const int n = n0 + 2 * j;
+      double *s = a.scale + row * 6;
+      s[0] = a.adjoint ? a.tau * a.phibar : -a.tau * C4(n, 3);
+      s[1] = a.adjoint ? a.q * C4(n - 1, 2) : -a.q * C4(n, 1);
+      s[2] = a.adjoint ? a.q * C4(n + 1, 1) : -a.q * C4(n, 2);
+      s[3] = a.adjoint ? -a.tau * C4(n, 3) : a.tau * a.phibar;
+      s[4] = a.adjoint ? -a.q * C4(n, 2) : a.q * C4(n + 1, 1);
+      s[5] = a.adjoint ? -a.q * C4(n, 1) : a.q * C4(n - 1, 2);
+    }
   }
   if (bad) atomicOr(a.bad, 1);
 }
@@ -119,7 +127,7 @@ __global__ void __launch_bounds__(kBlock) limb_factor_kernel(SetupArgs a) {
 struct StateArgs {
   const double2 *sin;  // [3][nspec][B]
   const int4 *sys;
-  const int *vexp;
+  const double *scale;
   int4 *dig;           // [nrows][B][4 inputs]
   int *uexp;           // [nrows][B]
   int64_t nspec;
@@ -139,9 +147,12 @@ __global__ void limb_state_kernel(StateArgs a) {
     const int64_t ix = (int64_t)m * (2 * a.N + 3 - m) / 2 + (nn - m);
     x = __ldg(a.sin + ((int64_t)field * a.nspec + ix) * a.B + b);
   }
-  const int v = live ? a.vexp[((int64_t)sy.w + i) * 4 + q] : 0;
+  if (live && q > 0) {
+    const double v = a.scale[((int64_t)sy.w + i) * 6 + q - 1];
+    x = make_double2(v * x.x, v * x.y);
+  }
   const int er = bexp(x.x), ei = bexp(x.y), e = max(er, ei);
-  int U = e ? e + v : -(1 << 24), nf = e == 0x7ff;
+  int U = e, nf = e == 0x7ff;
 #pragma unroll
   for (int o = 1; o < 4; o <<= 1) {
     U = max(U, __shfl_xor_sync(0xffffffffu, U, o));
@@ -149,8 +160,8 @@ __global__ void limb_state_kernel(StateArgs a) {
   }
   if (!live) return;
   a.dig[at * 4 + q] = nf ? make_int4(0, 0, 0, 0)
-                         : limbs2((to_fixed(x.x, U - (er + v)) + 4) >> 3, (to_fixed(x.y, U - (ei + v)) + 4) >> 3);
-  if (q == 0) a.uexp[at] = nf ? kNotFinite : (U < -(1 << 23) ? 0 : U - 1023);
+                         : limbs2((to_fixed(x.x, U - er) + 4) >> 3, (to_fixed(x.y, U - ei) + 4) >> 3);
+  if (q == 0) a.uexp[at] = nf ? kNotFinite : U - 1023;
 }
 
 // ---- per step: the sweeps (limb_sweep.h) ----------------------------------------------------------
@@ -193,39 +204,65 @@ cudaError_t limb_configure(int B) {
 }
 
 int limb_window(int B, int kc) { return kc * 32 / limb_tile(B); }  // poles per window, kc per lane
+namespace {
+int blocks_of(const Plan &pl) { return (pl.P + kBlock - 1) / kBlock; }
+size_t inv_bytes(const Plan &pl) { return (size_t)(pl.nrows + (int64_t)pl.sys.size()) * blocks_of(pl) * kRec; }
+size_t scale_bytes(const Plan &pl) { return (size_t)pl.nrows * 6 * sizeof(double); }
+}  // namespace
 size_t limb_factor_bytes(const Plan &pl) {
-  return (size_t)pl.nrows * ((pl.P + kBlock - 1) / kBlock) * (kFwd + kBwd) + (size_t)pl.nrows * 4 * sizeof(int);
+  return (size_t)pl.nrows * blocks_of(pl) * (kRec + kBwd) + inv_bytes(pl) + scale_bytes(pl) +
+         (size_t)blocks_of(pl) * kBlock * sizeof(int4);
 }
 size_t limb_state_bytes(const Plan &pl, int B) { return (size_t)pl.nrows * B * (4 * sizeof(int4) + sizeof(int)); }
 
-// The factor set as limbs; D's buffers are allocated, D.vexp with one more int for `bad`.
-cudaError_t launch_limb_factors(Plan &pl, const double2 *fac, DigitFactors &D, int kmid, int *bad) {
+// The exponent of the reciprocals' limbs: |1/s| <= 1/|Re alpha| < 2^(e0 + 1), and 1 (delta's weight)
+// below it as well.
+int limb_exponent(const Plan &pl) {
+  double least = 1.0;
+  for (const cplx &a : pl.alpha) least = std::min(least, std::fabs(a.real()));
+  return least > 0.0 ? std::max(0, std::ilogb(1.0 / least)) : kMaxSpread + 1;
+}
+
+// The factor set as limbs; `bad` set where it does not serve.  cudaErrorMemoryAllocation where
+// it does not fit.
+cudaError_t launch_limb_factors(Plan &pl, bool adjoint, const double2 *fac, DigitFactors &D, int *bad) {
+  const size_t nrec = (size_t)pl.nrows * blocks_of(pl);
+  cudaError_t e = cudaMalloc(&D.fwd, nrec * kRec);
+  if (e == cudaSuccess) e = cudaMalloc(&D.bwd, nrec * kBwd);
+  if (e == cudaSuccess) e = cudaMalloc(&D.inv, inv_bytes(pl));
+  if (e == cudaSuccess) e = cudaMalloc(&D.inv_alpha, (size_t)blocks_of(pl) * kBlock * sizeof(int4));
+  if (e == cudaSuccess) e = cudaMalloc(&D.scale, scale_bytes(pl));
+  if (e != cudaSuccess) return e;
   SetupArgs a;
   a.fac = fac;
+  a.alpha = pl.alpha_dev;
+  a.coef = pl.coef_dev;
   a.sys = pl.sys_dev;
   a.fwd = D.fwd;
   a.bwd = D.bwd;
-  a.vexp = D.vexp;
+  a.inv = D.inv;
+  a.inv_alpha = D.inv_alpha;
+  a.scale = D.scale;
   a.bad = bad;
   a.P = pl.P;
-  a.nblk = (pl.P + kBlock - 1) / kBlock;
-  a.kmid = kmid;
+  a.nblk = blocks_of(pl);
+  a.N = pl.N;
+  a.e0 = D.e0 = limb_exponent(pl);
+  a.adjoint = adjoint;
   a.nrows = pl.nrows;
-  limb_factor_kernel<<<dim3((unsigned)(pl.lmax * a.nblk), (unsigned)pl.sys.size()), kBlock>>>(a);
+  a.tau = pl.prm.tau;
+  a.q = 2.0 * pl.prm.omega * pl.prm.tau;
+  a.phibar = pl.prm.gravity * pl.prm.mean_depth;
+  if (a.e0 > kMaxSpread) return cudaMemset(bad, 1, 1);
+  limb_factor_kernel<<<dim3((unsigned)((pl.lmax + 1) * a.nblk), (unsigned)pl.sys.size()), kBlock>>>(a);
   return cudaGetLastError();
-}
-
-void limb_record_bytes(size_t *fwd, size_t *bwd, int *block) {
-  *fwd = kFwd;
-  *bwd = kBwd;
-  *block = kBlock;
 }
 
 cudaError_t launch_limb_state(Plan &pl, bool adjoint, const double2 *sin, int B, cudaStream_t st) {
   StateArgs s;
   s.sin = sin;
   s.sys = pl.sys_dev;
-  s.vexp = (adjoint ? pl.dig_adj : pl.dig_fwd).vexp;
+  s.scale = (adjoint ? pl.dig_adj : pl.dig_fwd).scale;
   s.dig = reinterpret_cast<int4 *>(pl.dig_state);
   s.uexp = reinterpret_cast<int *>(pl.dig_state + (size_t)pl.nrows * B * 4 * sizeof(int4));
   s.nspec = pl.nspec;
@@ -240,6 +277,9 @@ LimbSweep limb_sweep(Plan &pl, const DigitLayout &L, bool adjoint, int B) {
   LimbSweep a;
   a.fwd = D.fwd;
   a.bwd = D.bwd;
+  a.inv = D.inv;
+  a.inv_alpha = D.inv_alpha;
+  a.e0 = D.e0;
   a.dig = reinterpret_cast<const int4 *>(pl.dig_state);
   a.uexp = reinterpret_cast<const int *>(pl.dig_state + (size_t)pl.nrows * B * 4 * sizeof(int4));
   a.sys = pl.sys_dev;
@@ -251,7 +291,7 @@ LimbSweep limb_sweep(Plan &pl, const DigitLayout &L, bool adjoint, int B) {
   a.nitems = L.nitems;
   a.B = B;
   a.P = pl.P;
-  a.nblk = (pl.P + kBlock - 1) / kBlock;
+  a.nblk = blocks_of(pl);
   a.lmax = pl.lmax;
   a.kc = L.kc;
   return a;
