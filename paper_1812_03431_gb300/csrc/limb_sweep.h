@@ -16,10 +16,10 @@ using namespace fixed;
 // (shared by neighbouring rows), 1/alpha (per pole only), and beta/d'; and the recurrences'
 // l and Chat.  Records are [pole] arrays of 16 B: `inv` one per (system, block, j = 0..len) of
 // 1/s at degree n0 - 1 + 2 j, `fwd` one per (row, block) of l, `bwd` of Chat of the row before
-// and beta/d', with the latter's exponent behind.
+// and beta/d', with the latter's exponents (per pole) behind.
 constexpr int kBlock = 64;
 constexpr int kRec = kBlock * 16;
-constexpr int kBE = 2 * kRec, kBwd = 2 * kRec + 16;
+constexpr int kBE = 2 * kRec, kBwd = 2 * kRec + kBlock * 4;
 
 // v as limbs: v = x 2^30 + y, -2^29 <= y < 2^29
 __device__ __forceinline__ int2 limbs(long long v) {
@@ -42,6 +42,7 @@ struct LimbSweep {
   unsigned *counter;
   int64_t nrows;
   int nitems, B, P, nblk, lmax, kc;
+  const int *eblk;          // per block of poles: the exponent of its largest 1/s or 1/alpha
   int e0;                   // exponent of the limbs of 1/s and 1/alpha
 };
 
@@ -122,41 +123,51 @@ __device__ __forceinline__ void right_hand_sides(const char *stage, const char *
 
 // The window's sums over the lanes of each state of u = (beta/d') x, u/alpha, u/s_{n+1} and
 // u/s_{n-1}, x a row's solutions: returns the one of the eight (stream, part) values that this lane
-// ends up with (index: see sum_index).  prev: the stage of the row before (n + 2); wexp: the
-// exponent of beta/d' and the stream's.
+// ends up with (index: see sum_index).  prev: the stage of the row before (n + 2); be: the
+// exponents of beta/d'; fine: the bits by which the block's reciprocals are below 2^e0; sexp: the
+// exponent of the lane's stream.  beta, 1/d' and x vary over the poles by some bits each and not
+// together, so each pole's u has an exponent of its own and the window's unit is that of its
+// largest u.
 template <int SB, int KC>
-__device__ __forceinline__ double weighted_sums(const char *stage, const char *prev, const char *inv_alpha, int wexp,
-                                                const double2 (&x)[2], int lane) {
+__device__ __forceinline__ double weighted_sums(const char *stage, const char *prev, const char *inv_alpha,
+                                                const int (&be)[2], int fine, int sexp, const double2 (&x)[2], int lane) {
   constexpr int LPS = 32 / SB;  // lanes per state
-  int E = 0;
+  long long ur[2], ui[2];
+  int eu[2], E = -(1 << 20);
 #pragma unroll
-  for (int c = 0; c < KC; ++c) E = max(E, max(__double2hiint(x[c].x) & 0x7fffffff, __double2hiint(x[c].y) & 0x7fffffff));
+  for (int c = 0; c < KC; ++c) {
+    int e = max(__double2hiint(x[c].x) & 0x7fffffff, __double2hiint(x[c].y) & 0x7fffffff) >> 20;
+    eu[c] = e == 0x7ff ? kNotFinite : e - 1023 + be[c];
+    E = max(E, eu[c]);
+    if (e < 64) e += 4096;  // below 2^-959: taken as zero
+    long long rh = 0, rl = 1 << 29, ih = 0, il = 1 << 29;
+    cmad(rh, rl, ih, il, reinterpret_cast<const int4 *>(stage)[(2 * KC + c) * 32 + lane],
+         limbs2(fixed59(x[c].x, e), fixed59(x[c].y, e)));
+    ur[c] = rh + (rl >> 30);
+    ui[c] = ih + (il >> 30);
+  }
 #pragma unroll
   for (int o = 1; o < LPS; o <<= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
-  E >>= 20;
-  const bool finite = E != 0x7ff;
-  const int Ew = E - 1023;
-  if (E < 64) E += 4096;  // groups below 2^-959 are taken as zero
   // sums over up to 64 poles of numbers below 2^59: kept in units of 2^3
   long long hh[8], hl[8], t[8];
   t[0] = t[1] = 4;
 #pragma unroll
-  for (int j = 2; j < 8; ++j) hh[j] = 4, hl[j] = 1 << 29;  // rounded at bit 30, then at bit 3
+  for (int j = 2; j < 8; ++j) hh[j] = hl[j] = 0;
 #pragma unroll
   for (int c = 0; c < KC; ++c) {
-    long long rh = 0, rl = 1 << 29, ih = 0, il = 1 << 29;
-    cmad(rh, rl, ih, il, reinterpret_cast<const int4 *>(stage)[(2 * KC + c) * 32 + lane],
-         limbs2(fixed59(x[c].x, E), fixed59(x[c].y, E)));
-    const long long ur = rh + (rl >> 30), ui = ih + (il >> 30);
-    t[0] += ur;
-    t[1] += ui;
-    const int4 u = limbs2(ur, ui);
+    const int d = min(E - eu[c], 62);
+    const long long half = (1ll << d) >> 1;
+    ur[c] = (ur[c] + half) >> d;
+    ui[c] = (ui[c] + half) >> d;
+    t[0] += ur[c];
+    t[1] += ui[c];
+    const int4 u = limbs2(ur[c], ui[c]);
     cmad(hh[2], hl[2], hh[3], hl[3], reinterpret_cast<const int4 *>(inv_alpha)[c * 32 + lane], u);
     cmad(hh[4], hl[4], hh[5], hl[5], reinterpret_cast<const int4 *>(prev)[c * 32 + lane], u);
     cmad(hh[6], hl[6], hh[7], hl[7], reinterpret_cast<const int4 *>(stage)[c * 32 + lane], u);
   }
 #pragma unroll
-  for (int j = 0; j < 8; ++j) t[j] = (j < 2 ? t[j] : hh[j] + (hl[j] >> 30)) >> 3;
+  for (int j = 0; j < 8; ++j) t[j] = (j < 2 ? t[j] : (hh[j] << fine) + (hl[j] >> (30 - fine)) + 4) >> 3;
   int n = 8;
 #pragma unroll
   for (int o = LPS / 2; o > 0; o >>= 1) {
@@ -173,7 +184,7 @@ __device__ __forceinline__ double weighted_sums(const char *stage, const char *p
       t[0] += __shfl_xor_sync(0xffffffffu, t[0], o);
     }
   }
-  return fixed_to_double(t[0], finite ? Ew + wexp : kNotFinite);
+  return fixed_to_double(t[0], E >= kNotFinite / 2 ? kNotFinite : E + sexp);
 }
 
 // the value a lane holds after weighted_sums (2 stream + part), -1 for lanes that repeat another's
@@ -248,8 +259,11 @@ __device__ void sweep_window(const LimbSweep &a, int sysid, int64_t row0, int le
   }
   {  // backward: x_i = y_i - Chat x_{i+1}; the sums of row i + 1 beside the FMAs of row i
     const char *f = a.bwd + (rec + len - 1) * kBwd + pk * 16, *inv = inv0 + (int64_t)len * kRec;
-    const int *we = reinterpret_cast<const int *>(a.bwd + (rec + len - 1) * kBwd + kBE);
-    const int se = idx > 1 ? a.e0 - 51 : -53;
+    const int *we = reinterpret_cast<const int *>(a.bwd + (rec + len - 1) * kBwd + kBE) + pk;
+    const int fine = min(a.e0 - __ldg(a.eblk + blk), 8), sexp = idx > 1 ? a.e0 - fine - 51 : -53;
+    int be[2], bn[2];
+#pragma unroll
+    for (int c = 0; c < KC; ++c) be[c] = bn[c] = __ldg(we + c * LPS);
     int j = len;  // next stage to copy, len..0; the lane's own copies only
     auto issue = [&]() {
       if (j >= 0) {
@@ -284,9 +298,13 @@ __device__ void sweep_window(const LimbSweep &a, int sysid, int64_t row0, int le
     }
     for (int i = len - 1; i >= 0; --i) {
       const char *stage = smem + (i & 3) * kStage;
-      const int wexp = __ldg(we) + se;
       double sum = 0;
       if (!first && idx >= 0) sum = *part;
+      we = reinterpret_cast<const int *>(reinterpret_cast<const char *>(we) - kBwd);
+      if (i > 0) {
+#pragma unroll
+        for (int c = 0; c < KC; ++c) bn[c] = __ldg(we + c * LPS);
+      }
       copy_wait<1>();  // stages i + 1 and i
       issue();         // stage i - 2, in the place of i + 2
       double2 xn[2];
@@ -296,13 +314,15 @@ __device__ void sweep_window(const LimbSweep &a, int sysid, int64_t row0, int le
         xn[c] = cfms(y[c], reinterpret_cast<const double2 *>(stage)[(KC + c) * 32 + lane], x[c]);
         if (i > 1) y[c] = yp[c * 32 - 128];
       }
-      const double v = weighted_sums<SB, KC>(stage, smem + ((i + 1) & 3) * kStage, ia, wexp, x, lane);
+      const double v = weighted_sums<SB, KC>(stage, smem + ((i + 1) & 3) * kStage, ia, be, fine, sexp, x, lane);
       if (idx >= 0) *part = sum + v;
       part -= a.B * 8;
-      we = reinterpret_cast<const int *>(reinterpret_cast<const char *>(we) - kBwd);
       yp -= 64;
 #pragma unroll
-      for (int c = 0; c < KC; ++c) x[c] = xn[c];
+      for (int c = 0; c < KC; ++c) {
+        x[c] = xn[c];
+        be[c] = bn[c];
+      }
     }
   }
 }

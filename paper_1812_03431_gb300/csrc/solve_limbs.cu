@@ -13,13 +13,16 @@
 // times 1/alpha, 1/s_{n-1}, 1/s_{n+1} (s_n = alpha + i tau sigma_n, shared by neighbouring rows), and
 // for the weights beta/d'.  The real numbers go into the inputs before the sweep and into the
 // sums after it; the sweep forms u = (beta/d') w once and sums u, u/alpha, u/s_{n+1} and u/s_{n-1}:
-// 40 multiply-adds for a right-hand side and 48 for the sums as with stored factors, at 64 B per
-// row and pole instead of 148.  Roundings: u at 2^-59 of the window's largest, a lane's sums at
-// 2^-56, the total once to binary64; sums over the lanes are 64-bit integer additions.
+// 40 multiply-adds for a right-hand side and 48 for the sums as with stored factors, at 68 B per
+// row and pole instead of 148.  Roundings: u at 2^-59 of the window's largest u, a lane's sums at
+// 2^-56, the total once to binary64; sums over the lanes are 64-bit integer additions.  beta, 1/d'
+// and w differ over the poles by several bits and not together: with one exponent of beta/d' per
+// block of poles and one of w per window, the outputs lost 1e-15 on white noise; with an exponent
+// per pole they agree with the tensor-core solve's to 3e-16, for 4 B per row and pole more.
 //
 // Measured on GB300 (solve with its sums, against the fused FP64 solve): T341, 535 poles, one state
-// 0.81 / 2.10 ms, four states 3.04 / 8.12; T170 x 1 0.27 / 0.56, T128 x 1 with 1047 poles 0.27 / 0.61,
-// T639 x 1 2.72 / 7.87 (slot solve), T63 x 1 with 279 poles 0.066 / 0.089.  With every factor of a
+// 0.82 / 2.10 ms, four states 3.15 / 8.12; T170 x 1 0.27 / 0.56, T128 x 1 with 1047 poles 0.29 / 0.61,
+// T639 x 1 2.77 / 7.87 (slot solve), T63 x 1 with 279 poles 0.066 / 0.089.  With every factor of a
 // row stored (148 B per row and pole) one state waited on HBM: T639 3.05 ms, T341 0.91.  Now the
 // integer pipe is 59 % and the FP64 unit 57 % busy (ncu, T341 x 1) and the rest is latency; small
 // truncations wait on the row-to-row chain of their few warps.
@@ -50,6 +53,7 @@ struct SetupArgs {
   const int4 *sys;
   char *fwd, *bwd, *inv;
   int4 *inv_alpha;
+  int *eblk;           // [nblk]
   double *scale;       // [nrows][6]: inputs Phi, zeta_{n-1}, zeta_{n+1}; sums Phi, zeta_{n+1}, zeta_{n-1}
   int *bad;            // set when the factors are not finite or too unlike in scale
   int P, nblk, N, e0, adjoint;
@@ -60,7 +64,6 @@ struct SetupArgs {
 // One block of threads per (system, block of poles, j = 0..len): 1/s at degree n0 - 1 + 2 j and,
 // for j < len, the row's l, Chat and beta/d' and its real factors.
 __global__ void __launch_bounds__(kBlock) limb_factor_kernel(SetupArgs a) {
-  __shared__ int emx[2];
   const int4 sy = a.sys[blockIdx.y];
   const int m = sy.x, n0 = sy.y, len = sy.z, j = blockIdx.x / a.nblk, blk = blockIdx.x - j * a.nblk;
   if (len == 0 || j > len) return;
@@ -73,12 +76,14 @@ __global__ void __launch_bounds__(kBlock) limb_factor_kernel(SetupArgs a) {
   };
   auto emax = [](double2 v) { return max(bexp(v.x), bexp(v.y)); };
   bool bad = false;
+  int largest = -1023;
   // the reciprocal of s as 59 bits below 2^(e0 + 1); the poles' may differ by kMaxSpread bits
   auto inverse = [&](double2 s) {
     if (!live) return make_int4(0, 0, 0, 0);
     const double d = s.x * s.x + s.y * s.y;
     const double2 v = make_double2(s.x / d, -s.y / d);
     const int e = emax(v), top = a.e0 + 1023;
+    largest = max(largest, e - 1023);
     if (e > top || e + kMaxSpread < top) {  // also what is not finite
       bad = true;
       return make_int4(0, 0, 0, 0);
@@ -99,16 +104,11 @@ __global__ void __launch_bounds__(kBlock) limb_factor_kernel(SetupArgs a) {
     char *br = a.bwd + rec * kBwd;
     reinterpret_cast<double2 *>(a.fwd + rec * kRec)[p] = l;
     reinterpret_cast<double2 *>(br)[p] = c;
-    // beta/d': 59 bits below the block's largest
-    int top = emax(b);
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
-    if ((p & 31) == 0) emx[p >> 5] = top;
-    __syncthreads();
-    top = max(emx[0], emx[1]);
+    // beta/d': 59 bits, each with its exponent
+    const int top = emax(b);
     reinterpret_cast<int4 *>(br + kRec)[p] =
         limbs2((to_fixed(b.x, top - bexp(b.x)) + 4) >> 3, (to_fixed(b.y, top - bexp(b.y)) + 4) >> 3);
-    if (p == 0) *reinterpret_cast<int *>(br + kBE) = top - 1023;
+    reinterpret_cast<int *>(br + kBE)[p] = top - 1023;
     if (blk == 0 && p == 0) {
       const int n = n0 + 2 * j;
       double *s = a.scale + row * 6;
@@ -120,6 +120,8 @@ __global__ void __launch_bounds__(kBlock) limb_factor_kernel(SetupArgs a) {
       s[5] = a.adjoint ? -a.q * C4(n, 1) : a.q * C4(n - 1, 2);
     }
   }
+  largest = (int)__reduce_max_sync(0xffffffffu, (unsigned)(largest + 2048)) - 2048;
+  if ((p & 31) == 0) atomicMax(a.eblk + blk, largest);
   if (bad) atomicOr(a.bad, 1);
 }
 
@@ -211,7 +213,7 @@ size_t scale_bytes(const Plan &pl) { return (size_t)pl.nrows * 6 * sizeof(double
 }  // namespace
 size_t limb_factor_bytes(const Plan &pl) {
   return (size_t)pl.nrows * blocks_of(pl) * (kRec + kBwd) + inv_bytes(pl) + scale_bytes(pl) +
-         (size_t)blocks_of(pl) * kBlock * sizeof(int4);
+         (size_t)blocks_of(pl) * (kBlock * sizeof(int4) + sizeof(int));
 }
 size_t limb_state_bytes(const Plan &pl, int B) { return (size_t)pl.nrows * B * (4 * sizeof(int4) + sizeof(int)); }
 
@@ -230,7 +232,7 @@ cudaError_t launch_limb_factors(Plan &pl, bool adjoint, const double2 *fac, Digi
   cudaError_t e = cudaMalloc(&D.fwd, nrec * kRec);
   if (e == cudaSuccess) e = cudaMalloc(&D.bwd, nrec * kBwd);
   if (e == cudaSuccess) e = cudaMalloc(&D.inv, inv_bytes(pl));
-  if (e == cudaSuccess) e = cudaMalloc(&D.inv_alpha, (size_t)blocks_of(pl) * kBlock * sizeof(int4));
+  if (e == cudaSuccess) e = cudaMalloc(&D.inv_alpha, (size_t)blocks_of(pl) * (kBlock * sizeof(int4) + sizeof(int)));
   if (e == cudaSuccess) e = cudaMalloc(&D.scale, scale_bytes(pl));
   if (e != cudaSuccess) return e;
   SetupArgs a;
@@ -242,6 +244,7 @@ cudaError_t launch_limb_factors(Plan &pl, bool adjoint, const double2 *fac, Digi
   a.bwd = D.bwd;
   a.inv = D.inv;
   a.inv_alpha = D.inv_alpha;
+  a.eblk = reinterpret_cast<int *>(D.inv_alpha + (size_t)blocks_of(pl) * kBlock);
   a.scale = D.scale;
   a.bad = bad;
   a.P = pl.P;
@@ -254,6 +257,8 @@ cudaError_t launch_limb_factors(Plan &pl, bool adjoint, const double2 *fac, Digi
   a.q = 2.0 * pl.prm.omega * pl.prm.tau;
   a.phibar = pl.prm.gravity * pl.prm.mean_depth;
   if (a.e0 > kMaxSpread) return cudaMemset(bad, 1, 1);
+  e = cudaMemset(a.eblk, 0x80, blocks_of(pl) * sizeof(int));  // a very negative number
+  if (e != cudaSuccess) return e;
   limb_factor_kernel<<<dim3((unsigned)((pl.lmax + 1) * a.nblk), (unsigned)pl.sys.size()), kBlock>>>(a);
   return cudaGetLastError();
 }
@@ -280,6 +285,7 @@ LimbSweep limb_sweep(Plan &pl, const DigitLayout &L, bool adjoint, int B) {
   a.inv = D.inv;
   a.inv_alpha = D.inv_alpha;
   a.e0 = D.e0;
+  a.eblk = reinterpret_cast<const int *>(D.inv_alpha + (size_t)blocks_of(pl) * kBlock);
   a.dig = reinterpret_cast<const int4 *>(pl.dig_state);
   a.uexp = reinterpret_cast<const int *>(pl.dig_state + (size_t)pl.nrows * B * 4 * sizeof(int4));
   a.sys = pl.sys_dev;

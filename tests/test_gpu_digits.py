@@ -63,6 +63,24 @@ def test_matches_slot_solve(env, N, P, B):
     plan.close()
 
 
+@pytest.mark.parametrize("B", [1, 2, 4, 8])
+@pytest.mark.parametrize("field", [0, 1, 2])
+def test_single_inputs_keep_the_rounding_of_binary64(env, B, field):
+    """White noise in one input field, all poles of a set (their weights differ by 2^5): each output
+    within six roundings of the pole-slot solve's.  Either side rounds right-hand side, two
+    recurrences, sum and row scale, some 2^-53 rms each: two roundings of 2^-52, times three."""
+    torch, rexi = env
+    N = 42
+    al, be, _ = rc.rexi_coefficients(64, 0.2)
+    x = torch.zeros((B, 3, (N + 1) * (N + 2) // 2), dtype=torch.complex128)
+    x[:, field] = torch.from_numpy(np.random.default_rng(field).standard_normal((2, B, x.shape[2]))[0] * (10.0, 1e-5, 1e-5)[field])
+    x = x.cuda()
+    plan, slots = spectral_plan(rexi, N, B, al, be), spectral_plan(rexi, N, B, al, be, pole_slots=8)
+    assert fieldwise(plan.step(x).cpu().numpy(), slots.step(x).cpu().numpy()) < 6 * 2.0**-52
+    plan.close()
+    slots.close()
+
+
 @pytest.mark.parametrize("N,M,B,tau", [(15, 32, 5, 3600.0), (31, 48, 10, 1200.0), (15, 32, 1, 3600.0), (31, 48, 3, 1200.0)])
 def test_matches_oracle(env, N, M, B, tau):
     torch, rexi = env
