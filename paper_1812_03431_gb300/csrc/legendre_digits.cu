@@ -12,16 +12,23 @@
 // one 64-bit integer, rounded once to binary64 and added to the running sum.  So each output
 // carries one rounding per 64 terms in place of 64.
 //
-// A CTA of eight warps takes one zonal order and four states (blockIdx: m, states, rows); it
-// folds and cuts a group's data into digits in shared memory, each warp then forms the five
-// products of a row tile of 16 degrees or latitudes.  A tile of the product's columns is one
-// field of the four states (re, im), so that a lane ends up with all fields of one state and
-// combines them in registers.  Tables: 8 B per value as in the FP64 form, in fragment order.
+// A CTA of eight warps takes one zonal order and four states (blockIdx: states, rows, m; the states'
+// CTAs of an order side by side, so that its tables come from HBM once); it cuts a group's data
+// into digits in shared memory, each warp then forms the five products of a row tile of 16
+// degrees or latitudes.  A tile of the product's columns is one field of the four states (re,
+// im), so that a lane ends up with all fields of one state and combines them in registers.  With
+// one state that tile would be three quarters padding: there the three fields share one, and two
+// products (P and H times all fields) do for the five.  Tables: 8 B per value as in the FP64 form,
+// in fragment order.  Everything is copied ahead with cp.async: a warp's next table fragment, also
+// across products and barriers, and the next group's inputs while the products run.
 //
-// Measured on GB300 (analysis, synthesis; against the FP64 kernels): T341 x 16 0.92, 0.79 / 4.37, 4.07
-// ms; T255 x 8 0.234, 0.204 / 1.01, 0.86; T170 x 1 0.058, 0.076 / 0.114, 0.169; T63 x 1 0.020, 0.027 /
-// 0.037, 0.065.  The tensor pipe is a third busy (ncu, T255 x 8), the rest is waiting for table
-// fragments and at the groups' barriers; two CTAs per SM (one: 1.39, 1.11 ms at T341).
+// Measured on GB300 (analysis, synthesis; against the FP64 kernels): T341 x 16 0.84, 0.70 / 4.37, 4.07
+// ms; T255 x 8 0.212, 0.193 / 1.01, 0.86; T639 x 1 0.52, 0.48; T170 x 1 0.031, 0.033 / 0.114, 0.169;
+// T63 x 1 0.012, 0.014 / 0.037, 0.065.  Without the copies ahead and the shared tile: 0.92, 0.79;
+// 0.234, 0.204; T170 x 1 0.058, 0.076; T63 x 1 0.020, 0.027.  At T255 x 8 the tensor pipe is 35 %, the
+// issue slots 45 % busy (ncu): four warps per scheduler, which wait for each other at the groups'
+// barriers and within the chains of a product; registers allow no more warps.  Fewer instructions
+// (sums read off the accumulators' bits per 32 terms) gave nothing.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -39,11 +46,16 @@ namespace {
 
 constexpr int kGroup = 64;       // contraction length of a group
 constexpr int kWarps = 8;
-constexpr int kColPitch = kGroup + 1;
-constexpr int kBuf = 48 * kColPitch * 8;             // two classes of 24 real columns, binary64
-constexpr int kTileDig = (kGroup / 16) * 2 * 2 * 512;  // digits of one column tile
-constexpr int kSmem = kBuf + 6 * kTileDig + 48 * 4;
 constexpr int kFrag = 2048;      // bytes of a 16 x 16 table fragment
+constexpr int kTileDig = (kGroup / 16) * 2 * 2 * 512;  // digits of one column tile
+// Shared memory: a group's inputs as they come (two halves -- hemispheres, or degrees of either
+// class -- of 64 x 12 complex numbers; even and odd places apart and 13 to a row, so that lanes
+// reading every second place meet no bank twice), their zeta/delta scale (synthesis), their digits,
+// the columns' exponents, and per warp two table fragments.
+constexpr int kPitch = 13;
+constexpr int kZd = 2 * 2 * (kGroup / 2) * kPitch * 16, kDig = kZd + 2 * kGroup * 8, kExp = kDig + 6 * kTileDig;
+constexpr int kRing = kExp + 48 * 4, kSmem = kRing + kWarps * 2 * kFrag;
+static_assert(2 * (kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
 
 struct TabArgs {
   const double *tab[2];          // Pbar, H: [nspec][J]
@@ -108,28 +120,53 @@ struct LegArgs {
   int64_t nspec;
 };
 
-// The columns in `buf` ([48][kColPitch] binary64, `n` values each, zero up to a multiple of 16)
-// as digits in fragment order in `dig`, their exponents in `cexp`.  Column 8 t + c of six
-// tiles; each warp takes six columns.
-__device__ __forceinline__ void cut_columns(const double *buf, uint4 *dig, int *cexp, int warp, int lane) {
-#pragma unroll 2
-  for (int u = 0; u < 6; ++u) {
-    const int col = warp * 6 + u, t = col >> 3, c = col & 7;
-    const double x = buf[col * kColPitch + 2 * lane], y = buf[col * kColPitch + 2 * lane + 1];
-    const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(bexp(x), bexp(y)));
-    if (lane == 0) cexp[col] = e == 0x7ff ? kNotFinite : e - 1023;
+__device__ __forceinline__ int raw_at(int half, int k, int c) {
+  return ((half * 2 + (k & 1)) * (kGroup / 2) + (k >> 1)) * kPitch + c;
+}
+
+template <int BYTES>
+__device__ __forceinline__ void copy_or_zero(unsigned to, const void *from, bool ok) {
+  if constexpr (BYTES == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" : : "r"(to), "l"(from), "r"(ok ? 16 : 0) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" : : "r"(to), "l"(from), "r"(ok ? 8 : 0) : "memory");
+}
+__device__ __forceinline__ void copy_all() { asm volatile("cp.async.wait_all;" : : : "memory"); }
+
+// Two real columns (a complex number's parts, x and y at this lane's places 2 lane and 2 lane + 1)
+// as digits in fragment order, columns `col` and `col` + 1 of tile t, with their exponents.
+__device__ __forceinline__ void cut_pair(double2 x, double2 y, uint4 *dig, int *cexp, int t, int col, int lane) {
+  uint4 *o = dig + t * (kTileDig / 16) + (((lane >> 3) * 2 + ((lane >> 2) & 1)) * 2) * 32 + col * 4 + (lane & 3);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const double u = h ? x.y : x.x, v = h ? y.y : y.x;
+    const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(bexp(u), bexp(v)));
+    if (lane == 0) cexp[t * 8 + col + h] = e == 0x7ff ? kNotFinite : e - 1023;
     unsigned w[8];
-    digits(to_fixed(x, e - bexp(x)), to_fixed(y, e - bexp(y)), w);
-    uint4 *o = dig + t * (kTileDig / 16) + (((lane >> 3) * 2 + ((lane >> 2) & 1)) * 2) * 32 + c * 4 + (lane & 3);
-    o[0] = make_uint4(w[0], w[1], w[2], w[3]);
-    o[32] = make_uint4(w[4], w[5], w[6], w[7]);
+    digits(to_fixed(u, e - bexp(u)), to_fixed(v, e - bexp(v)), w);
+    o[h * 4] = make_uint4(w[0], w[1], w[2], w[3]);
+    o[h * 4 + 32] = make_uint4(w[4], w[5], w[6], w[7]);
   }
 }
 
-// One product of a row tile: `steps` fragments of the table (`stride` uint4 apart) times one
-// column tile's digits.  r: rows g and g + 8, columns 2 q and 2 q + 1.
-__device__ __forceinline__ void product(const uint4 *a, int64_t stride, const uint4 *b, int steps, int lane, int ea0, int ea1,
-                                        int eb0, int eb1, double (&r)[4]) {
+// A warp's table fragments, one step ahead in two places of shared memory; a lane reads only what
+// it copied.
+struct Ring {
+  char *at;
+  int lane, slot;
+  __device__ __forceinline__ void copy(int s, const uint4 *from) const {
+    const unsigned to = (unsigned)__cvta_generic_to_shared(at + s * kFrag + lane * 16);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) copy_or_zero<16>(to + i * 512, from + i * 32 + lane, true);
+  }
+};
+
+// One product of a row tile: `steps` fragments of the table (`stride` uint4 apart, the first
+// already on its way) times one column tile's digits; `next`: the fragment after these, if any.
+// r: rows g and g + 8, columns 2 q and 2 q + 1.
+__device__ __forceinline__ void product(Ring &ring, const uint4 *a, int64_t stride, const uint4 *next, const uint4 *b, int steps,
+                                        int ea0, int ea1, int eb0, int eb1, double (&r)[4]) {
+  const int lane = ring.lane;
   float s[8][4];
 #pragma unroll
   for (int c = 0; c < 8; ++c)
@@ -137,9 +174,14 @@ __device__ __forceinline__ void product(const uint4 *a, int64_t stride, const ui
     for (int k = 0; k < 4; ++k) s[c][k] = 0.0f;
 #pragma unroll 1
   for (int k = 0; k < steps; ++k) {
+    a = k + 1 < steps ? a + stride : next;
+    if (a) ring.copy(ring.slot ^ 1, a);
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 1;" : : : "memory");
+    const uint4 *f = reinterpret_cast<const uint4 *>(ring.at + ring.slot * kFrag) + lane;
+    ring.slot ^= 1;
     unsigned w[4][8], v[2][8];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) unpack(__ldg(a + i * 32 + lane), 0x3c003c00u, 0xe480e480u, w[i]);
+    for (int i = 0; i < 4; ++i) unpack(f[i * 32], 0x3c003c00u, 0xe480e480u, w[i]);
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const uint4 x = b[(2 * i) * 32 + lane], y = b[(2 * i + 1) * 32 + lane];
@@ -150,7 +192,6 @@ __device__ __forceinline__ void product(const uint4 *a, int64_t stride, const ui
     for (int i = 0; i < 8; ++i)
 #pragma unroll
       for (int j = 0; j < 8 - i; ++j) mma_add(s[i + j], w[0][i], w[1][i], w[2][i], w[3][i], v[0][j], v[1][j]);
-    a += stride;
     b += 4 * 32;
   }
 #pragma unroll
@@ -165,160 +206,259 @@ __device__ __forceinline__ void product(const uint4 *a, int64_t stride, const ui
   }
 }
 
-// Analysis: out[n] = sum_j; blockIdx.x: m, .y: states, .z: row tiles (eight per CTA, classes 0, 1)
+__device__ __forceinline__ void add(double2 &s, double x, double y) { s = make_double2(s.x + x, s.y + y); }
+__device__ __forceinline__ void add_im(double2 &s, double fm, double x, double y) {  // += i fm (x + i y)
+  s = make_double2(fma(-fm, y, s.x), fma(fm, x, s.y));
+}
+__device__ __forceinline__ double2 of_field(double2 v, int lane, int f) {
+  const int from = (lane & ~3) + f;
+  return make_double2(__shfl_sync(0xffffffffu, v.x, from), __shfl_sync(0xffffffffu, v.y, from));
+}
+
+// Analysis: out[n] = sum_j; blockIdx.x: states, .y: row tiles (eight per CTA, classes 0, 1), .z: m.
+// ONE: a batch of one state.  Its three fields share a column tile (lane q holds field q), which
+// makes two products, P and H times all fields, of the five.
+template <bool ONE>
 __global__ void __launch_bounds__(256, 2) legendre_digits_analysis(LegArgs a) {
   extern __shared__ __align__(16) char smem[];
-  double *buf = reinterpret_cast<double *>(smem);
-  uint4 *dig = reinterpret_cast<uint4 *>(smem + kBuf);
-  int *cexp = reinterpret_cast<int *>(smem + kBuf + 6 * kTileDig);
-  const int m = blockIdx.x, b0 = blockIdx.y * 4, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int NC = ONE ? 3 : 12, CT = ONE ? 1 : 3;  // complex columns, column tiles of a class
+  const double2 *raw = reinterpret_cast<const double2 *>(smem);
+  uint4 *dig = reinterpret_cast<uint4 *>(smem + kDig);
+  int *cexp = reinterpret_cast<int *>(smem + kExp);
+  const int m = blockIdx.z, b0 = blockIdx.x * 4, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int4 s0 = a.sys[2 * m], s1 = a.sys[2 * m + 1];
   const int t0 = (s0.x + 15) / 16, t1 = (s1.x + 15) / 16;
-  if ((int)blockIdx.z * kWarps >= t0 + t1) return;
-  const int unit = blockIdx.z * kWarps + warp, cls = unit >= t0, tile = cls ? unit - t0 : unit;
+  if ((int)blockIdx.y * kWarps >= t0 + t1) return;
+  const int unit = blockIdx.y * kWarps + warp, cls = unit >= t0, tile = cls ? unit - t0 : unit;
   const bool live = unit < t0 + t1;
   const int4 sy = cls ? s1 : s0;
   const int tiles = cls ? t1 : t0, q = lane & 3, row = lane >> 2;
   const int M1 = a.N + 1, ncol = 3 * a.B;
   const double fm = (double)m;
-  double2 phi[2], zeta[2], delta[2];  // rows row, row + 8
+  const int64_t stride = (int64_t)tiles * 2 * (kFrag / 16);
+  const uint4 *fr = a.dig + ((int64_t)sy.y * tiles + tile) * 2 * (kFrag / 16);
+  const int *ex = a.exps + ((int64_t)sy.z * tiles + tile) * 32 + row;
+  Ring ring{smem + kRing + warp * 2 * kFrag, lane, 0};
+  auto fetch = [&](int j0) {
+    const unsigned to = (unsigned)__cvta_generic_to_shared(smem);
+    for (int t = tid; t < 2 * kGroup * NC; t += 256) {
+      const int c = t % NC, u = t / NC, half = u >> 6, jj = u & (kGroup - 1), j = j0 + jj;
+      const bool ok = j < a.J && 3 * b0 + c < ncol;
+      copy_or_zero<16>(to + raw_at(half, jj, c) * 16,
+                       ok ? a.four + ((int64_t)(half ? a.nlat - 1 - j : j) * M1 + m) * ncol + 3 * b0 + c : a.four, ok);
+    }
+  };
+  double2 phi[2], zeta[2], delta[2];  // rows row, row + 8; ONE: of this lane's field, P and H times it
 #pragma unroll
   for (int i = 0; i < 2; ++i) phi[i] = zeta[i] = delta[i] = make_double2(0, 0);
-  for (int j0 = 0, g = 0; j0 < a.J; j0 += kGroup, ++g) {
-    const int jn = min(kGroup, a.J - j0);
-    __syncthreads();  // the digits of the group before have been used
-    for (int t = tid; t < kGroup * 12; t += 256) {
-      const int jj = t / 12, c = t - jj * 12, f = c % 3, st = c / 3, cg = 3 * b0 + c;
-      double2 n = make_double2(0, 0), s = n;
-      if (jj < jn && cg < ncol) {
-        n = a.four[((int64_t)(j0 + jj) * M1 + m) * ncol + cg];
-        s = a.four[((int64_t)(a.nlat - 1 - j0 - jj) * M1 + m) * ncol + cg];
+  fetch(0);
+  if (live) ring.copy(0, fr);
+  for (int j0 = 0; j0 < a.J; j0 += kGroup) {
+    copy_all();
+    __syncthreads();  // the group's inputs are there, the digits of the group before have been used
+    for (int u = warp; u < (ONE ? 8 : 24); u += kWarps) {
+      const int odd = u & 1, f = ONE ? u >> 1 : (u >> 1) % 3, st = ONE ? 0 : (u >> 1) / 3;
+      double2 v[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        v[h] = make_double2(0, 0);
+        if (ONE && f == 3) continue;
+        const double2 n = raw[raw_at(0, 2 * lane + h, 3 * st + f)], s = raw[raw_at(1, 2 * lane + h, 3 * st + f)];
+        v[h] = odd ? make_double2(n.x - s.x, n.y - s.y) : make_double2(n.x + s.x, n.y + s.y);
       }
-      double *e = buf + (f * 8 + 2 * st) * kColPitch + jj, *o = e + 24 * kColPitch;
-      e[0] = n.x + s.x;
-      e[kColPitch] = n.y + s.y;
-      o[0] = n.x - s.x;
-      o[kColPitch] = n.y - s.y;
+      cut_pair(v[0], v[1], dig, cexp, odd * CT + (ONE ? 0 : f), 2 * (ONE ? f : st), lane);
     }
     __syncthreads();
-    cut_columns(buf, dig, cexp, warp, lane);
-    __syncthreads();
+    const bool more = j0 + kGroup < a.J;
+    if (more) fetch(j0 + kGroup);
     if (!live) continue;
-    const int steps = (jn + 15) / 16;
-    const int64_t stride = (int64_t)tiles * 2 * (kFrag / 16);
-    const uint4 *fr = a.dig + (((int64_t)sy.y + g * 4) * tiles + tile) * 2 * (kFrag / 16);
-    const int *ex = a.exps + (((int64_t)sy.z + g) * tiles + tile) * 32 + row;
-    // Pbar has the rows' own symmetry, H the other
-    auto run = [&](int x, int f, double (&r)[4]) {
-      const int t = (x ? 1 - cls : cls) * 3 + f;
-      product(fr + x * (kFrag / 16), stride, dig + t * (kTileDig / 16), steps, lane, __ldg(ex + x * 16), __ldg(ex + x * 16 + 8),
-              cexp[t * 8 + 2 * q], cexp[t * 8 + 2 * q + 1], r);
+    const int steps = (min(kGroup, a.J - j0) + 15) / 16;
+    const uint4 *after = more ? fr + 4 * stride : nullptr;
+    // Pbar has the rows' own symmetry, H the other; xn: the table of the product after this one
+    auto run = [&](int x, int f, int xn, double (&r)[4]) {
+      const int t = (x ? 1 - cls : cls) * CT + f;
+      product(ring, fr + x * (kFrag / 16), stride, xn < 0 ? after : fr + xn * (kFrag / 16), dig + t * (kTileDig / 16), steps,
+              __ldg(ex + x * 16), __ldg(ex + x * 16 + 8), cexp[t * 8 + 2 * q], cexp[t * 8 + 2 * q + 1], r);
     };
     double r[4];
-    run(0, 0, r);
+    if constexpr (ONE) {
+      run(0, 0, 1, r);
 #pragma unroll
-    for (int i = 0; i < 2; ++i) phi[i] = make_double2(phi[i].x + r[2 * i], phi[i].y + r[2 * i + 1]);
-    run(0, 2, r);  // i m P V
+      for (int i = 0; i < 2; ++i) add(phi[i], r[2 * i], r[2 * i + 1]);
+      run(1, 0, -1, r);
 #pragma unroll
-    for (int i = 0; i < 2; ++i) zeta[i] = make_double2(fma(-fm, r[2 * i + 1], zeta[i].x), fma(fm, r[2 * i], zeta[i].y));
-    run(1, 1, r);  // H U
+      for (int i = 0; i < 2; ++i) add(zeta[i], r[2 * i], r[2 * i + 1]);
+    } else {
+      run(0, 0, 0, r);
 #pragma unroll
-    for (int i = 0; i < 2; ++i) zeta[i] = make_double2(zeta[i].x + r[2 * i], zeta[i].y + r[2 * i + 1]);
-    run(0, 1, r);  // i m P U
+      for (int i = 0; i < 2; ++i) add(phi[i], r[2 * i], r[2 * i + 1]);
+      run(0, 2, 1, r);  // i m P V
 #pragma unroll
-    for (int i = 0; i < 2; ++i) delta[i] = make_double2(fma(-fm, r[2 * i + 1], delta[i].x), fma(fm, r[2 * i], delta[i].y));
-    run(1, 2, r);  // -H V
+      for (int i = 0; i < 2; ++i) add_im(zeta[i], fm, r[2 * i], r[2 * i + 1]);
+      run(1, 1, 0, r);  // H U
 #pragma unroll
-    for (int i = 0; i < 2; ++i) delta[i] = make_double2(delta[i].x - r[2 * i], delta[i].y - r[2 * i + 1]);
+      for (int i = 0; i < 2; ++i) add(zeta[i], r[2 * i], r[2 * i + 1]);
+      run(0, 1, 1, r);  // i m P U
+#pragma unroll
+      for (int i = 0; i < 2; ++i) add_im(delta[i], fm, r[2 * i], r[2 * i + 1]);
+      run(1, 2, -1, r);  // -H V
+#pragma unroll
+      for (int i = 0; i < 2; ++i) add(delta[i], -r[2 * i], -r[2 * i + 1]);
+    }
+    fr += 4 * stride;
+    ex += tiles * 32;
   }
-  const int b = b0 + q;
-  if (!live || b >= a.B) return;
+  if (!live) return;
+  if constexpr (ONE) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const double2 pu = of_field(phi[i], lane, 1), pv = of_field(phi[i], lane, 2);
+      const double2 hu = of_field(zeta[i], lane, 1), hv = of_field(zeta[i], lane, 2);
+      zeta[i] = hu;
+      add_im(zeta[i], fm, pv.x, pv.y);
+      delta[i] = make_double2(-hv.x, -hv.y);
+      add_im(delta[i], fm, pu.x, pu.y);
+    }
+  }
+  const int b = ONE ? 0 : b0 + q;
+  if (b >= a.B) return;
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     const int r = tile * 16 + row + 8 * i;
     if (r >= sy.x) continue;
     const int64_t ix = (int64_t)m * (2 * a.N + 3 - m) / 2 + cls + 2 * r;
     const double s = a.zd[ix];
-    a.spec[ix * a.B + b] = phi[i];
-    a.spec[(a.nspec + ix) * a.B + b] = make_double2(s * zeta[i].x, s * zeta[i].y);
-    a.spec[(2 * a.nspec + ix) * a.B + b] = make_double2(s * delta[i].x, s * delta[i].y);
+    if (!ONE || q == 0) a.spec[ix * a.B + b] = phi[i];
+    if (!ONE || q == 1) a.spec[(a.nspec + ix) * a.B + b] = make_double2(s * zeta[i].x, s * zeta[i].y);
+    if (!ONE || q == 2) a.spec[(2 * a.nspec + ix) * a.B + b] = make_double2(s * delta[i].x, s * delta[i].y);
   }
 }
 
-// Synthesis: F[j] = sum_n; blockIdx.x: m, .y: states, .z: latitude tiles (eight per CTA)
+// Synthesis: F[j] = sum_n; blockIdx.x: states, .y: latitude tiles (eight per CTA), .z: m.  ONE: as above.
+template <bool ONE>
 __global__ void __launch_bounds__(256, 2) legendre_digits_synthesis(LegArgs a) {
   extern __shared__ __align__(16) char smem[];
-  double *buf = reinterpret_cast<double *>(smem);
-  uint4 *dig = reinterpret_cast<uint4 *>(smem + kBuf);
-  int *cexp = reinterpret_cast<int *>(smem + kBuf + 6 * kTileDig);
-  const int m = blockIdx.x, b0 = blockIdx.y * 4, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int tiles = (a.J + 15) / 16, tile = blockIdx.z * kWarps + warp, q = lane & 3, row = lane >> 2;
+  constexpr int NC = ONE ? 3 : 12, CT = ONE ? 1 : 3, NS = ONE ? 1 : 4;
+  const double2 *raw = reinterpret_cast<const double2 *>(smem);
+  const double *zds = reinterpret_cast<const double *>(smem + kZd);
+  uint4 *dig = reinterpret_cast<uint4 *>(smem + kDig);
+  int *cexp = reinterpret_cast<int *>(smem + kExp);
+  const int m = blockIdx.z, b0 = blockIdx.x * 4, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tiles = (a.J + 15) / 16, tile = blockIdx.y * kWarps + warp, q = lane & 3, row = lane >> 2;
   const bool live = tile < tiles;
   const int64_t idx0 = (int64_t)m * (2 * a.N + 3 - m) / 2;
   const int deg = a.N - m + 1;
   const double fm = (double)m;
-  double2 F[2][3][2];  // symmetry class, field, rows row and row + 8
+  const int64_t stride = (int64_t)tiles * 2 * (kFrag / 16);
+  const int4 s0 = a.sys[2 * m], s1 = a.sys[2 * m + 1];
+  const uint4 *fr[2] = {a.dig + ((int64_t)s0.y * tiles + tile) * 2 * (kFrag / 16),
+                        a.dig + ((int64_t)s1.y * tiles + tile) * 2 * (kFrag / 16)};
+  const int *ex[2] = {a.exps + ((int64_t)s0.z * tiles + tile) * 32 + row, a.exps + ((int64_t)s1.z * tiles + tile) * 32 + row};
+  Ring ring{smem + kRing + warp * 2 * kFrag, lane, 0};
+  auto fetch = [&](int r0) {  // degrees of both classes, three fields, the states
+    const unsigned to = (unsigned)__cvta_generic_to_shared(smem);
+    for (int t = tid; t < 2 * kGroup * NC; t += 256) {
+      const int st = ONE ? 0 : t & 3, f = (ONE ? t : t >> 2) % 3, d = t / NC, n = 2 * r0 + d;
+      const bool ok = n < deg && b0 + st < a.B;
+      copy_or_zero<16>(to + raw_at(d & 1, d >> 1, f * NS + st) * 16,
+                       ok ? a.spec + ((int64_t)f * a.nspec + idx0 + n) * a.B + b0 + st : a.spec, ok);
+    }
+    if (tid < 2 * kGroup) {
+      const bool ok = 2 * r0 + tid < deg;
+      copy_or_zero<8>(to + kZd + tid * 8, ok ? a.zd + idx0 + 2 * r0 + tid : a.zd, ok);
+    }
+  };
+  double2 F[2][3][2];  // symmetry class, field, rows row and row + 8; ONE: P and H times this lane's field
 #pragma unroll
   for (int c = 0; c < 2; ++c)
 #pragma unroll
     for (int f = 0; f < 3; ++f) F[c][f][0] = F[c][f][1] = make_double2(0, 0);
-  for (int r0 = 0, g = 0; r0 * 2 < deg; r0 += kGroup, ++g) {
+  fetch(0);
+  if (live) ring.copy(0, fr[0]);
+  for (int r0 = 0; r0 * 2 < deg; r0 += kGroup) {
+    copy_all();
     __syncthreads();
-    for (int t = tid; t < 2 * kGroup * 12; t += 256) {  // degrees of both classes, three fields, four states
-      const int d = t / 12, c = t - d * 12, st = c & 3, f = c >> 2, b = b0 + st, n = 2 * r0 + d;
-      double2 v = make_double2(0, 0);
-      if (n < deg && b < a.B) {
-        v = a.spec[((int64_t)f * a.nspec + idx0 + n) * a.B + b];
+    for (int u = warp; u < (ONE ? 8 : 24); u += kWarps) {
+      const int odd = u & 1, f = ONE ? u >> 1 : (u >> 1) % 3, st = ONE ? 0 : (u >> 1) / 3;
+      double2 v[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        v[h] = make_double2(0, 0);
+        if (ONE && f == 3) continue;
+        v[h] = raw[raw_at(odd, 2 * lane + h, f * NS + st)];
         if (f > 0) {
-          const double s = a.zd[idx0 + n];
-          v = make_double2(s * v.x, s * v.y);
+          const double s = zds[2 * (2 * lane + h) + odd];
+          v[h] = make_double2(s * v[h].x, s * v[h].y);
         }
       }
-      double *o = buf + ((d & 1) * 24 + f * 8 + 2 * st) * kColPitch + (d >> 1);
-      o[0] = v.x;
-      o[kColPitch] = v.y;
+      cut_pair(v[0], v[1], dig, cexp, odd * CT + (ONE ? 0 : f), 2 * (ONE ? f : st), lane);
     }
     __syncthreads();
-    cut_columns(buf, dig, cexp, warp, lane);
-    __syncthreads();
+    const bool more = (r0 + kGroup) * 2 < deg;
+    if (more) fetch(r0 + kGroup);
     if (!live) continue;
 #pragma unroll
     for (int cls = 0; cls < 2; ++cls) {
-      const int4 sy = a.sys[2 * m + cls];
-      const int left = sy.x - r0;
-      if (left <= 0) continue;
+      const int left = (cls ? s1.x : s0.x) - r0;
+      if (left <= 0) continue;  // class 1 of the last group only
       const int steps = (min(left, kGroup) + 15) / 16;
-      const int64_t stride = (int64_t)tiles * 2 * (kFrag / 16);
-      const uint4 *fr = a.dig + (((int64_t)sy.y + g * 4) * tiles + tile) * 2 * (kFrag / 16);
-      const int *ex = a.exps + (((int64_t)sy.z + g) * tiles + tile) * 32 + row;
-      auto run = [&](int x, int f, double (&r)[4]) {
-        const int t = cls * 3 + f;
-        product(fr + x * (kFrag / 16), stride, dig + t * (kTileDig / 16), steps, lane, __ldg(ex + x * 16),
-                __ldg(ex + x * 16 + 8), cexp[t * 8 + 2 * q], cexp[t * 8 + 2 * q + 1], r);
+      const uint4 *after = cls == 0 ? (s1.x > r0 ? fr[1] : nullptr) : (more ? fr[0] + 4 * stride : nullptr);
+      auto run = [&](int x, int f, int xn, double (&r)[4]) {
+        const int t = cls * CT + f;
+        product(ring, fr[cls] + x * (kFrag / 16), stride, xn < 0 ? after : fr[cls] + xn * (kFrag / 16),
+                dig + t * (kTileDig / 16), steps, __ldg(ex[cls] + x * 16), __ldg(ex[cls] + x * 16 + 8), cexp[t * 8 + 2 * q],
+                cexp[t * 8 + 2 * q + 1], r);
       };
-      auto add = [](double2 &s, double x, double y) { s = make_double2(s.x + x, s.y + y); };
       double r[4];
-      run(0, 0, r);  // P Phi
+      if constexpr (ONE) {
+        run(0, 0, 1, r);
 #pragma unroll
-      for (int i = 0; i < 2; ++i) add(F[cls][0][i], r[2 * i], r[2 * i + 1]);
-      run(0, 2, r);  // U: i m P chi'
+        for (int i = 0; i < 2; ++i) add(F[cls][0][i], r[2 * i], r[2 * i + 1]);
+        run(1, 0, -1, r);
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
-        F[cls][1][i] = make_double2(fma(-fm, r[2 * i + 1], F[cls][1][i].x), fma(fm, r[2 * i], F[cls][1][i].y));
-      run(0, 1, r);  // V: i m P psi'
+        for (int i = 0; i < 2; ++i) add(F[cls][1][i], r[2 * i], r[2 * i + 1]);
+      } else {
+        run(0, 0, 0, r);  // P Phi
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
-        F[cls][2][i] = make_double2(fma(-fm, r[2 * i + 1], F[cls][2][i].x), fma(fm, r[2 * i], F[cls][2][i].y));
-      run(1, 1, r);  // U: -H psi', of the other symmetry
+        for (int i = 0; i < 2; ++i) add(F[cls][0][i], r[2 * i], r[2 * i + 1]);
+        run(0, 2, 0, r);  // U: i m P chi'
 #pragma unroll
-      for (int i = 0; i < 2; ++i) add(F[1 - cls][1][i], -r[2 * i], -r[2 * i + 1]);
-      run(1, 2, r);  // V: H chi'
+        for (int i = 0; i < 2; ++i) add_im(F[cls][1][i], fm, r[2 * i], r[2 * i + 1]);
+        run(0, 1, 1, r);  // V: i m P psi'
 #pragma unroll
-      for (int i = 0; i < 2; ++i) add(F[1 - cls][2][i], r[2 * i], r[2 * i + 1]);
+        for (int i = 0; i < 2; ++i) add_im(F[cls][2][i], fm, r[2 * i], r[2 * i + 1]);
+        run(1, 1, 1, r);  // U: -H psi', of the other symmetry
+#pragma unroll
+        for (int i = 0; i < 2; ++i) add(F[1 - cls][1][i], -r[2 * i], -r[2 * i + 1]);
+        run(1, 2, -1, r);  // V: H chi'
+#pragma unroll
+        for (int i = 0; i < 2; ++i) add(F[1 - cls][2][i], r[2 * i], r[2 * i + 1]);
+      }
+    }
+#pragma unroll
+    for (int cls = 0; cls < 2; ++cls) {
+      fr[cls] += 4 * stride;
+      ex[cls] += tiles * 32;
     }
   }
-  const int b = b0 + q, M1 = a.N + 1, ncol = 3 * a.B;
-  if (!live || b >= a.B) return;
+  if (!live) return;
+  const int b = ONE ? 0 : b0 + q, M1 = a.N + 1, ncol = 3 * a.B;
+  if constexpr (ONE) {  // lane q takes field q: Phi; U = i m P chi' - H psi'; V = i m P psi' + H chi'
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      double2 o[2];
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const double2 p = of_field(F[c][0][i], lane, q == 1 ? 2 : (q == 2 ? 1 : 0)), h = of_field(F[1 - c][1][i], lane, q);
+        const double sg = q == 1 ? -1.0 : 1.0;
+        o[c] = q == 0 ? p : make_double2(sg * h.x, sg * h.y);
+        if (q > 0) add_im(o[c], fm, p.x, p.y);
+      }
+      F[0][0][i] = o[0];
+      F[1][0][i] = o[1];
+    }
+  }
+  if (b >= a.B || (ONE && q == 3)) return;
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     const int j = tile * 16 + row + 8 * i;
@@ -326,10 +466,10 @@ __global__ void __launch_bounds__(256, 2) legendre_digits_synthesis(LegArgs a) {
     double2 *north = a.four + ((int64_t)j * M1 + m) * ncol + 3 * b;
     double2 *south = a.four + ((int64_t)(a.nlat - 1 - j) * M1 + m) * ncol + 3 * b;
 #pragma unroll
-    for (int f = 0; f < 3; ++f) {
+    for (int f = 0; f < (ONE ? 1 : 3); ++f) {
       const double2 x = F[0][f][i], y = F[1][f][i];
-      north[f] = make_double2(x.x + y.x, x.y + y.y);
-      south[f] = make_double2(x.x - y.x, x.y - y.y);
+      north[ONE ? q : f] = make_double2(x.x + y.x, x.y + y.y);
+      south[ONE ? q : f] = make_double2(x.x - y.x, x.y - y.y);
     }
   }
 }
@@ -402,7 +542,8 @@ cudaError_t build_legendre_digits(Plan &pl, bool synthesis, LegendreDigits &t) {
     legendre_digits_setup<<<dim3((unsigned)most, (unsigned)sys.size()), 32>>>(a);
     e = cudaGetLastError();
   }
-  for (auto k : {legendre_digits_analysis, legendre_digits_synthesis})
+  for (auto k : {legendre_digits_analysis<true>, legendre_digits_analysis<false>, legendre_digits_synthesis<true>,
+                 legendre_digits_synthesis<false>})
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   if (e != cudaSuccess) free_legendre_digits(t);
   t.bytes = (size_t)nfrag * 2 * kFrag + (size_t)nexp * 32 * sizeof(int);
@@ -411,14 +552,16 @@ cudaError_t build_legendre_digits(Plan &pl, bool synthesis, LegendreDigits &t) {
 
 cudaError_t launch_leg_ana_digits(Plan &pl, const double2 *four, double2 *sint, int B, const double *zd, cudaStream_t st) {
   const int tiles = (pl.N / 2 + 1 + 15) / 16 + ((pl.N + 1) / 2 + 15) / 16;
-  const dim3 g((unsigned)(pl.N + 1), (unsigned)((B + 3) / 4), (unsigned)((tiles + kWarps - 1) / kWarps));
-  legendre_digits_analysis<<<g, 32 * kWarps, kSmem, st>>>(leg_args(pl, pl.leg_ana, four, sint, B, zd));
+  const dim3 g((unsigned)((B + 3) / 4), (unsigned)((tiles + kWarps - 1) / kWarps), (unsigned)(pl.N + 1));
+  (B == 1 ? legendre_digits_analysis<true> : legendre_digits_analysis<false>)<<<g, 32 * kWarps, kSmem, st>>>(
+      leg_args(pl, pl.leg_ana, four, sint, B, zd));
   return cudaGetLastError();
 }
 
 cudaError_t launch_leg_syn_digits(Plan &pl, const double2 *sint, double2 *four, int B, const double *zd, cudaStream_t st) {
-  const dim3 g((unsigned)(pl.N + 1), (unsigned)((B + 3) / 4), (unsigned)(((pl.J + 15) / 16 + kWarps - 1) / kWarps));
-  legendre_digits_synthesis<<<g, 32 * kWarps, kSmem, st>>>(leg_args(pl, pl.leg_syn, four, sint, B, zd));
+  const dim3 g((unsigned)((B + 3) / 4), (unsigned)(((pl.J + 15) / 16 + kWarps - 1) / kWarps), (unsigned)(pl.N + 1));
+  (B == 1 ? legendre_digits_synthesis<true> : legendre_digits_synthesis<false>)<<<g, 32 * kWarps, kSmem, st>>>(
+      leg_args(pl, pl.leg_syn, four, sint, B, zd));
   return cudaGetLastError();
 }
 

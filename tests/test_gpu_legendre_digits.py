@@ -52,6 +52,22 @@ def test_transforms_match_oracle(env, N, nlat, nlon, B):
     plan.close()
 
 
+@pytest.mark.parametrize("N,nlat,nlon", [(1, 2, 4), (2, 4, 8), (15, 32, 48), (16, 36, 48), (31, 64, 96), (33, 128, 108),
+                                         (66, 132, 200), (127, 192, 384)])
+def test_one_state_alone_as_in_a_batch(env, N, nlat, nlon):
+    """A single state's fields share a column tile; each product is exact up to 2^-59 of its group and
+    is rounded as in a batch, the sums over groups in another order (up to four of them)."""
+    torch, rexi = env
+    plan = rexi.Plan(N, nlat, nlon, M=8, max_batch=2)
+    x = torch.from_numpy(inputs.random_grid(2, nlat, nlon, 7)).cuda()
+    S = torch.from_numpy(inputs.random_spectral(N, 2, 8, slope=0.0)).cuda()
+    for f, v in ((plan.analyze, x), (plan.synthesize, S)):
+        one, two = f(v[1:].contiguous()).cpu().numpy()[0], f(v).cpu().numpy()[1]
+        for k in range(3):
+            assert np.linalg.norm(one[k] - two[k]) <= 4 * 2.0**-52 * np.linalg.norm(two[k])
+    plan.close()
+
+
 def test_scales_and_values_that_are_not_finite_stay_in_their_state(env):
     """Groups are scaled per state and order by powers of two: a power of two times a state gives
     that power times its result, bit for bit, and a NaN reaches no other state."""
