@@ -41,7 +41,9 @@ struct LimbSweep {
   double2 *ybuf;            // per resident warp: [lmax][2][32]
   unsigned *counter;
   int64_t nrows;
-  int nitems, B, P, nblk, lmax, kc;
+  int nitems, B, P, nblk, lmax;
+  int kc;                   // poles per lane; 3: one, by a CTA per window
+  int sms;
   const int *eblk;          // per block of poles: the exponent of its largest 1/s or 1/alpha
   int e0;                   // exponent of the limbs of 1/s and 1/alpha
 };
@@ -343,6 +345,155 @@ __device__ __forceinline__ void limb_item(const LimbSweep &a, int4 item, int lan
     if (a.kc == 2 && p0 + LPS < a.P) sweep_window<SB, 2>(a, item.x, sy.w, sy.z, p0, b0, idx, part, w == w0, yb, smem, lane);
     else sweep_window<SB, 1>(a, item.x, sy.w, sy.z, p0, b0, idx, part, w == w0, yb, smem, lane);
   }
+}
+
+// A window of one pole per lane by a CTA of four warps, for launches whose warps are too few to
+// hide a row's chain (1800 cycles where one warp does all of it): one warp carries the two
+// recurrences, 4 FP64 FMAs per row, the others form the right-hand sides and the sums of three
+// rows at a time beside it, both through shared memory.  The arithmetic and the order of the
+// sums are those of sweep_window.  role: 0 for the recurrences; smem: the CTA's stages; mine: this
+// warp's among them; rows: the recurrences' warp's, [2][3 rows][32].
+constexpr int kRowsAhead = 3;
+template <int SB>
+__device__ void sweep_window_split(const LimbSweep &a, int sysid, int64_t row0, int len, int p0, int b0, int idx, double *part,
+                                   bool first, double2 *yb, char *ring, double2 *rows, int role, int lane) {
+  constexpr int LPS = 32 / SB;
+  const int k = lane & (LPS - 1), s = lane / LPS, blk = p0 / kBlock, pk = p0 % kBlock + k;
+  const int64_t rec = row0 * a.nblk + (int64_t)blk * len;
+  const char *inv = a.inv + ((row0 + sysid) * a.nblk + (int64_t)blk * (len + 1)) * kRec + pk * 16;
+  const int chunks = (len + kRowsAhead - 1) / kRowsAhead;
+  auto at = [&](int t, int c) { return rows + ((t & 1) * kRowsAhead + c) * 32 + lane; };
+  if (role == 0) {
+    const double2 zero = make_double2(0, 0);
+    const char *f = a.fwd + rec * kRec + pk * 16;
+    double2 v = zero, l[kRowsAhead], ln[kRowsAhead];
+#pragma unroll
+    for (int c = 0; c < kRowsAhead; ++c) l[c] = c < len ? __ldg(reinterpret_cast<const double2 *>(f + (int64_t)c * kRec)) : zero;
+    for (int t = 0; t < chunks; ++t) {
+#pragma unroll
+      for (int c = 0; c < kRowsAhead; ++c) {
+        const int i = kRowsAhead * (t + 1) + c;
+        ln[c] = i < len ? __ldg(reinterpret_cast<const double2 *>(f + (int64_t)i * kRec)) : zero;
+      }
+      __syncthreads();  // the chunk's right-hand sides are there
+#pragma unroll
+      for (int c = 0; c < kRowsAhead; ++c) {
+        const int i = kRowsAhead * t + c;
+        if (i < len) {
+          v = cfms(*at(t, c), l[c], v);
+          yb[i * 64] = v;
+        }
+        l[c] = ln[c];
+      }
+    }
+    // backward: x_i = y_i - Chat x_{i+1}, Chat of row i stored with row i + 1
+    const char *g = a.bwd + rec * kBwd + pk * 16;
+    double2 y[kRowsAhead], yn[kRowsAhead], h[kRowsAhead], hn[kRowsAhead];
+    auto load = [&](int t, double2 (&yy)[kRowsAhead], double2 (&hh)[kRowsAhead]) {
+#pragma unroll
+      for (int c = 0; c < kRowsAhead; ++c) {
+        const int i = len - 1 - kRowsAhead * t - c;
+        yy[c] = i >= 0 ? yb[i * 64] : zero;
+        hh[c] = i >= 0 && i + 1 < len ? __ldg(reinterpret_cast<const double2 *>(g + (int64_t)(i + 1) * kBwd)) : zero;
+      }
+    };
+    load(0, y, h);
+    v = zero;
+    for (int t = 0; t < chunks; ++t) {
+      load(t + 1, yn, hn);
+#pragma unroll
+      for (int c = 0; c < kRowsAhead; ++c) {
+        v = t + c > 0 ? cfms(y[c], h[c], v) : y[c];
+        *at(t, c) = v;
+        y[c] = yn[c];
+        h[c] = hn[c];
+      }
+      __syncthreads();  // the chunk's solutions are there
+    }
+    return;
+  }
+  const unsigned sm = (unsigned)__cvta_generic_to_shared(ring);
+  const char *ia = ring + kInvAlpha;
+  const int ns = min(SB, a.B - b0), mine = min(s, ns - 1), c0 = role - 1;
+  // two stages per row (its own factors, and 1/s of the row after), the next row's being copied
+  auto issue = [&](int i, int set) {
+    if (i >= 0 && i < len) {
+      const unsigned to = sm + 2 * set * kStage;
+      copy_async<16>(to + lane * 16, inv + (int64_t)i * kRec);
+      copy_async<16>(to + kStage + lane * 16, inv + (int64_t)(i + 1) * kRec);
+    }
+  };
+  auto issue_inputs = [&](int i, int set) {
+    issue(i, set);
+    if (i < len) {
+      const unsigned to = sm + 2 * set * kStage;
+      const int64_t st = (row0 + i) * a.B + b0;
+      if (lane < 4 * ns) copy_async<16>(to + kSIn + lane * 16, a.dig + st * 4 + lane);
+      else if (lane >= 16 && lane < 16 + ns) copy_async<4>(to + kSU + (lane - 16) * 4, a.uexp + st + lane - 16);
+    }
+    copy_commit();
+  };
+  const int one[2] = {p0 + k < a.P ? 1 << (28 - a.e0) : 0, 0};
+  __syncwarp();  // every lane has read the stages of the window before
+  copy_async<16>(sm + kInvAlpha + lane * 16, a.inv_alpha + p0 + k);
+  issue_inputs(c0, 0);
+  for (int t = 0; t < chunks; ++t) {
+    const int i = kRowsAhead * t + c0;
+    issue_inputs(i + kRowsAhead, (t + 1) & 1);
+    copy_wait<1>();
+    __syncwarp();
+    if (i < len) {
+      double2 r[2], l[2];
+      const char *stage = ring + 2 * (t & 1) * kStage;
+      right_hand_sides<1>(stage, stage + kStage, ia, a.e0, one, mine, lane, r, l);
+      *at(t, c0) = r[0];
+    }
+    __syncthreads();
+  }
+  copy_wait<0>();
+  const char *g = a.bwd + rec * kBwd;
+  const int fine = min(a.e0 - __ldg(a.eblk + blk), 8), sexp = idx > 1 ? a.e0 - fine - 51 : -53;
+  int be[2] = {0, 0}, bn = 0;
+  auto issue_weights = [&](int i, int set) {
+    issue(i, set);
+    if (i >= 0) {
+      copy_async<16>(sm + 2 * set * kStage + (64 + lane) * 16, g + (int64_t)i * kBwd + kRec + pk * 16);
+      bn = __ldg(reinterpret_cast<const int *>(g + (int64_t)i * kBwd + kBE) + pk);
+    }
+    copy_commit();
+  };
+  issue_weights(len - 1 - c0, 0);
+  for (int t = 0; t < chunks; ++t) {
+    const int i = len - 1 - kRowsAhead * t - c0;
+    be[0] = bn;
+    issue_weights(i - kRowsAhead, (t + 1) & 1);
+    double *p = part + (int64_t)i * a.B * 8 + (idx > 0 ? idx : 0);
+    double sum = 0;
+    if (!first && idx >= 0 && i >= 0) sum = *p;
+    copy_wait<1>();
+    __syncthreads();
+    if (i >= 0) {
+      const double2 x[2] = {*at(t, c0), make_double2(0, 0)};
+      const char *stage = ring + 2 * (t & 1) * kStage;
+      const double v = weighted_sums<SB, 1>(stage, stage + kStage, ia, be, fine, sexp, x, lane);
+      if (idx >= 0) *p = sum + v;
+    }
+  }
+  copy_wait<0>();
+}
+
+// One item by a CTA of four warps (kc 3); smem: the CTA's stages
+template <int SB>
+__device__ __forceinline__ void limb_item_split(const LimbSweep &a, int4 item, int lane, int warp, int lead, double2 *yb,
+                                                char *smem) {
+  constexpr int LPS = 32 / SB;
+  const int4 sy = a.sys[item.x];
+  const int w0 = item.z & 0xffff, w1 = w0 + (item.z >> 16);
+  const int b0 = item.y * SB, state = b0 + lane / LPS, idx = state < a.B ? sum_index<SB>(lane) : -1;
+  double *part = a.part + (((int64_t)item.w * a.nrows + sy.w) * a.B + min(state, a.B - 1)) * 8;
+  for (int w = w0; w < w1; ++w)
+    sweep_window_split<SB>(a, item.x, sy.w, sy.z, w * LPS, b0, idx, part, w == w0, yb, smem + warp * kSmemWarp,
+                           reinterpret_cast<double2 *>(smem + lead * kSmemWarp), (warp - lead) & 3, lane);
 }
 
 }  // namespace limb_solve

@@ -156,7 +156,7 @@ cudaError_t launch_fixed_ragged(const std::vector<Plan *> &plans, const std::vec
   int num_sms = 1;
   for (size_t p = 0; p < plans.size() && e == cudaSuccess; ++p) {
     num_sms = std::max(num_sms, plans[p]->num_sms);
-    if (counts[p] > 0) e = launch_digit_state(*plans[p], false, plans[p]->s_in, counts[p], st);
+    if (counts[p] > 0) e = launch_digit_state(*plans[p], false, plans[p]->s_in, counts[p], nullptr, st);
   }
   if (e != cudaSuccess) return e;
   const int ctas = std::max(1, std::min(num_sms * kCtas, (R.nitems + 3) / 4));

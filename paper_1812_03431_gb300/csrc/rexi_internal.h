@@ -351,11 +351,11 @@ int limb_tile(int B);
 int limb_window(int B, int kc);
 size_t limb_factor_bytes(const Plan &pl);
 size_t limb_state_bytes(const Plan &pl, int B);
-cudaError_t limb_configure(int B);
+cudaError_t limb_configure(int B, int kc);
 cudaError_t launch_limb_factors(Plan &pl, bool adjoint, const double2 *fac, DigitFactors &D, int *bad);
-cudaError_t launch_limb_state(Plan &pl, bool adjoint, const double2 *sin, int B, cudaStream_t st);
+cudaError_t launch_limb_state(Plan &pl, bool adjoint, const double2 *sin, int B, unsigned *counter, cudaStream_t st);
 cudaError_t launch_solve_limbs(Plan &pl, const DigitLayout &L, bool adjoint, int B, cudaStream_t st);
-cudaError_t launch_digit_state(Plan &pl, bool adjoint, const double2 *sin, int B, cudaStream_t st);
+cudaError_t launch_digit_state(Plan &pl, bool adjoint, const double2 *sin, int B, unsigned *counter, cudaStream_t st);
 struct DigitItem {
   int4 it;       // system, tile, first window | windows << 16, slot
   int64_t work;  // rows x windows

@@ -142,11 +142,13 @@ struct StateArgs {
   const int *vexp;
   char *dig;           // [nrows][tiles] records
   int *uexp;           // [nrows][tiles][8]
+  unsigned *counter;   // the sweep's next item, set to zero here (null: not)
   int64_t nspec;
   int B, tiles, N;
 };
 
 __global__ void digit_state_kernel(StateArgs a) {
+  if (a.counter && blockIdx.x + blockIdx.y + threadIdx.x == 0) *a.counter = 0;
   const int4 sy = a.sys[blockIdx.y];
   const int m = sy.x, n0 = sy.y, len = sy.z;
   const int lane = threadIdx.x & 31, s = lane >> 2, q = lane & 3;
@@ -364,24 +366,30 @@ int64_t digit_work(const Plan &pl, int B, int kc) {
 // Work items (system, tile, windows, slot) for batch B, longest first.  slots: items per
 // (system, tile), each over its share of the windows; 0: enough that the longest item is at
 // most half a resident warp's share of the work, capped by the partial-sum buffer.  For limbs
-// slots carries 65536 x the poles per lane (1 or 2; 0: the default).  One pole per lane halves
-// a warp's chain of FP64 FMAs per row at 0.7 of the whole row's instructions, which pays where
-// items of two are fewer than 1.6 per resident warp (26 per SM): T63 x 1 0.073 / 0.085 ms, T170 x
-// 1 0.275 / 0.348 (20 per SM); T128 x 1 with 1047 poles 0.296 / 0.291 (29), T341 x 1 1.14 / 1.09 (40).
+// slots carries 65536 x the packing (1 or 2 poles per lane; 3: one, by a CTA per window; 0: the
+// default).  A CTA's warps share a window's rows where the windows are fewer than 22 per SM, 5.5 per
+// resident CTA (its barriers cost more than the shorter chains give beyond that): T63 x 1 with 71
+// poles 0.038 against 0.056 ms for one warp, with 279 poles (7.6 windows per SM) 0.047 / 0.068; T127 x
+// 1 with 151 poles (8.4) 0.078 / 0.134, T255 x 1 (17) 0.226 / 0.328; T127 x 1 with 535 poles (29) 0.208 /
+// 0.183, T63 x 4 with 279 (29) 0.135 / 0.115.  Otherwise one pole per lane halves a warp's chain of
+// FP64 FMAs per row at 0.7 of the whole row's instructions, which pays where items of two are
+// fewer than 1.6 per resident warp (26 per SM): T170 x 1 with 535 poles 0.266 / 0.360 ms (20 per SM);
+// T128 x 1 with 1047 poles 0.293 / 0.288 (29), T341 x 1 1.14 / 1.09 (40).
 rexi_status build_digit_layout(Plan &pl, int B, int slots, DigitLayout &L) {
   L = DigitLayout{};
   if (pl.nrows == 0) return REXI_OK;  // not available
   if (pl.limbs) {
-    L.kc = std::min(2, slots >> 16);
-    if (L.kc == 0)
-      L.kc = (int64_t)pl.sys.size() * windows_of(pl, B, 2) * tiles_of(pl, B) < 26 * (int64_t)pl.num_sms ? 1 : 2;
-    if (limb_configure(B) != cudaSuccess) {
+    L.kc = std::min(3, slots >> 16);
+    auto windows = [&](int kc) { return (int64_t)pl.sys.size() * windows_of(pl, B, kc) * tiles_of(pl, B); };
+    if (L.kc == 0) L.kc = windows(3) < 22 * (int64_t)pl.num_sms ? 3 : windows(2) < 26 * (int64_t)pl.num_sms ? 1 : 2;
+    if (limb_configure(B, L.kc) != cudaSuccess) {
       cudaGetLastError();
       return REXI_OK;
     }
   }
   std::vector<DigitItem> keyed;
-  if (!digit_items(pl, B, slots & 0xffff, 0.5 * digit_work(pl, B, L.kc) / (4.0 * kCtas * pl.num_sms), L, keyed))
+  const double teams = (double)kCtas * pl.num_sms * (L.kc == 3 ? 1 : 4);
+  if (!digit_items(pl, B, slots & 0xffff, 0.5 * digit_work(pl, B, L.kc) / teams, L, keyed))
     return REXI_OK;
   std::stable_sort(keyed.begin(), keyed.end(), [](const DigitItem &x, const DigitItem &y) { return x.work > y.work; });
   std::vector<int4> items;
@@ -402,9 +410,9 @@ void free_digit_layout(DigitLayout &L) {
   L = DigitLayout{};
 }
 
-// the batch's inputs in fixed point
-cudaError_t launch_digit_state(Plan &pl, bool adjoint, const double2 *sin, int B, cudaStream_t st) {
-  if (pl.limbs) return launch_limb_state(pl, adjoint, sin, B, st);
+// the batch's inputs in fixed point, and *counter = 0
+cudaError_t launch_digit_state(Plan &pl, bool adjoint, const double2 *sin, int B, unsigned *counter, cudaStream_t st) {
+  if (pl.limbs) return launch_limb_state(pl, adjoint, sin, B, counter, st);
   const int tiles = tiles_of(pl, B);
   StateArgs s;
   s.sin = sin;
@@ -412,6 +420,7 @@ cudaError_t launch_digit_state(Plan &pl, bool adjoint, const double2 *sin, int B
   s.vexp = (adjoint ? pl.dig_adj : pl.dig_fwd).vexp;
   s.dig = pl.dig_state;
   s.uexp = reinterpret_cast<int *>(pl.dig_state + (size_t)pl.nrows * tiles * kStateRec);
+  s.counter = counter;
   s.nspec = pl.nspec;
   s.B = B;
   s.tiles = tiles;
@@ -442,8 +451,7 @@ DigitSweep digit_sweep(Plan &pl, const DigitLayout &L, bool adjoint, int B) {
 }
 
 cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, int B, cudaStream_t st) {
-  cudaError_t e = launch_digit_state(pl, adjoint, sin, B, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(pl.counter, 0, sizeof(unsigned), st);
+  cudaError_t e = launch_digit_state(pl, adjoint, sin, B, pl.counter, st);
   if (e != cudaSuccess) return e;
   if (pl.limbs) return launch_solve_limbs(pl, L, adjoint, B, st);
   const int ctas = std::min(pl.num_sms * kCtas, (L.nitems + 3) / 4);

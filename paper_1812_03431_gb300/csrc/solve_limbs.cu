@@ -22,10 +22,11 @@
 //
 // Measured on GB300 (solve with its sums, against the fused FP64 solve): T341, 535 poles, one state
 // 0.82 / 2.10 ms, four states 3.15 / 8.12; T170 x 1 0.27 / 0.56, T128 x 1 with 1047 poles 0.29 / 0.61,
-// T639 x 1 2.77 / 7.87 (slot solve), T63 x 1 with 279 poles 0.066 / 0.089.  With every factor of a
+// T639 x 1 2.77 / 7.87 (slot solve), T63 x 1 with 279 poles 0.047 / 0.089.  With every factor of a
 // row stored (148 B per row and pole) one state waited on HBM: T639 3.05 ms, T341 0.91.  Now the
-// integer pipe is 59 % and the FP64 unit 57 % busy (ncu, T341 x 1) and the rest is latency; small
-// truncations wait on the row-to-row chain of their few warps.
+// integer pipe is 59 % and the FP64 unit 57 % busy (ncu, T341 x 1) and the rest is latency.  Small
+// truncations waited on the row-to-row chain of their few warps (T63 0.066 ms): there a CTA's four
+// warps share a window (sweep_window_split).
 //
 // Lanes of a warp are (state, pole): SB states x 32 / SB poles, two poles per lane where the
 // window is full (poles k and k + 32 / SB), one for a short last window.
@@ -132,11 +133,13 @@ struct StateArgs {
   const double *scale;
   int4 *dig;           // [nrows][B][4 inputs]
   int *uexp;           // [nrows][B]
+  unsigned *counter;   // the sweep's next item, set to zero here (null: not)
   int64_t nspec;
   int B, N;
 };
 
 __global__ void limb_state_kernel(StateArgs a) {
+  if (a.counter && blockIdx.x + blockIdx.y + threadIdx.x == 0) *a.counter = 0;
   const int4 sy = a.sys[blockIdx.y];
   const int m = sy.x, n0 = sy.y, len = sy.z, nmin = m > 1 ? m : 1;
   const int t = blockIdx.x * blockDim.x + threadIdx.x, q = t & 3, rb = t >> 2;
@@ -186,26 +189,44 @@ __global__ void __launch_bounds__(128, CTAS) solve_limbs_kernel(LimbSweep a) {
 // resident CTAs of four warps per SM
 constexpr int kCtas = 4;
 
+// The recurrences' warp differs between an SM's CTAs (blocks fill the SMs in turn), so that
+// each scheduler's FP64 unit gets one of the four.
+template <int SB>
+__global__ void __launch_bounds__(128, kCtas) solve_limbs_split_kernel(LimbSweep a) {
+  __shared__ unsigned next;
+  extern __shared__ __align__(16) char stages[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lead = (blockIdx.x / a.sms) & 3;
+  double2 *yb = a.ybuf + (int64_t)(blockIdx.x * 4 + warp) * a.lmax * 64 + lane;
+  for (;;) {
+    if (threadIdx.x == 0) next = atomicAdd(a.counter, 1u);
+    __syncthreads();
+    const unsigned it = next;
+    if (it >= (unsigned)a.nitems) break;
+    limb_item_split<SB>(a, a.items[it], lane, warp, lead, yb, stages);
+  }
+}
+
 }  // namespace
 
 int limb_tile(int B) { return B >= 3 ? 4 : B; }                    // states per warp
 
 namespace {
-void (*kernel_for(int B))(LimbSweep) {
+void (*kernel_for(int B, bool split))(LimbSweep) {
   switch (limb_tile(B)) {
-    case 1: return solve_limbs_kernel<1, kCtas>;
-    case 2: return solve_limbs_kernel<2, kCtas>;
-    default: return solve_limbs_kernel<4, kCtas>;
+    case 1: return split ? solve_limbs_split_kernel<1> : solve_limbs_kernel<1, kCtas>;
+    case 2: return split ? solve_limbs_split_kernel<2> : solve_limbs_kernel<2, kCtas>;
+    default: return split ? solve_limbs_split_kernel<4> : solve_limbs_kernel<4, kCtas>;
   }
 }
 }  // namespace
 
 // raises the kernel's shared-memory limit, when a layout is built
-cudaError_t limb_configure(int B) {
-  return cudaFuncSetAttribute(kernel_for(B), cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * kSmemWarp);
+cudaError_t limb_configure(int B, int kc) {
+  return cudaFuncSetAttribute(kernel_for(B, kc == 3), cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * kSmemWarp);
 }
 
-int limb_window(int B, int kc) { return kc * 32 / limb_tile(B); }  // poles per window, kc per lane
+// poles per window: kc per lane; 3: one per lane, a CTA per window
+int limb_window(int B, int kc) { return (kc == 2 ? 2 : 1) * 32 / limb_tile(B); }
 namespace {
 int blocks_of(const Plan &pl) { return (pl.P + kBlock - 1) / kBlock; }
 size_t inv_bytes(const Plan &pl) { return (size_t)(pl.nrows + (int64_t)pl.sys.size()) * blocks_of(pl) * kRec; }
@@ -263,13 +284,14 @@ cudaError_t launch_limb_factors(Plan &pl, bool adjoint, const double2 *fac, Digi
   return cudaGetLastError();
 }
 
-cudaError_t launch_limb_state(Plan &pl, bool adjoint, const double2 *sin, int B, cudaStream_t st) {
+cudaError_t launch_limb_state(Plan &pl, bool adjoint, const double2 *sin, int B, unsigned *counter, cudaStream_t st) {
   StateArgs s;
   s.sin = sin;
   s.sys = pl.sys_dev;
   s.scale = (adjoint ? pl.dig_adj : pl.dig_fwd).scale;
   s.dig = reinterpret_cast<int4 *>(pl.dig_state);
   s.uexp = reinterpret_cast<int *>(pl.dig_state + (size_t)pl.nrows * B * 4 * sizeof(int4));
+  s.counter = counter;
   s.nspec = pl.nspec;
   s.B = B;
   s.N = pl.N;
@@ -300,12 +322,14 @@ LimbSweep limb_sweep(Plan &pl, const DigitLayout &L, bool adjoint, int B) {
   a.nblk = blocks_of(pl);
   a.lmax = pl.lmax;
   a.kc = L.kc;
+  a.sms = pl.num_sms;
   return a;
 }
 
 cudaError_t launch_solve_limbs(Plan &pl, const DigitLayout &L, bool adjoint, int B, cudaStream_t st) {
-  const unsigned ctas = (unsigned)std::max(1, std::min(pl.num_sms * kCtas, (L.nitems + 3) / 4));
-  kernel_for(B)<<<ctas, 128, 4 * kSmemWarp, st>>>(limb_sweep(pl, L, adjoint, B));
+  const bool split = L.kc == 3;
+  const unsigned ctas = (unsigned)std::max(1, std::min(pl.num_sms * kCtas, split ? L.nitems : (L.nitems + 3) / 4));
+  kernel_for(B, split)<<<ctas, 128, 4 * kSmemWarp, st>>>(limb_sweep(pl, L, adjoint, B));
   return cudaGetLastError();
 }
 

@@ -139,6 +139,25 @@ def test_values_that_are_not_finite_stay_in_their_state_and_order(env, value, B,
     plan.close()
 
 
+# rows around chunks of three, poles around windows of 32, 16 and 8, a part-filled state tile
+@pytest.mark.parametrize("N,P,B", [(1, 1, 1), (2, 32, 1), (3, 33, 1), (5, 64, 1), (7, 65, 1), (13, 100, 1), (63, 149, 1),
+                                   (5, 16, 2), (13, 33, 2), (5, 9, 3), (21, 31, 4), (31, 57, 3)])
+def test_windows_shared_by_a_block(env, N, P, B):
+    """Packing 3 (a block's warps share a window's rows) does the arithmetic of packing 1 in its order."""
+    torch, rexi = env
+    al, be = poles(P)
+    plan = spectral_plan(rexi, N, B, al, be)
+    x = torch.from_numpy(inputs.random_spectral(N, B, 11)).cuda()
+    for slots in (1, 2):
+        out = []
+        for packing in (1, 3):
+            assert plan.set_pole_slots(B, 65536 * packing + slots, 5) >> 16 == packing
+            out.append((plan.step(x).cpu().numpy(), plan.step_adjoint(x).cpu().numpy()))
+        np.testing.assert_array_equal(out[0][0], out[1][0])
+        np.testing.assert_array_equal(out[0][1], out[1][1])
+    plan.close()
+
+
 @pytest.mark.parametrize("B", [8, 2])
 def test_poles_of_unlike_scale_keep_the_other_solves(env, B):
     """Couplings of one pole that differ by more than eight bits from the middle pole's stay with
