@@ -15,7 +15,7 @@ using namespace fixed;
 constexpr int kTile = 8;                   // states per warp
 constexpr int kWin = 8;                    // poles per window
 constexpr int kLOff = 512, kEOff = 640, kFwdRec = 672;  // per (row, window): coupling digits, l, exponents
-constexpr int kCOff = 512, kBwdRec = 640;  // per (row, window): weight digits and exponents, Chat of the row before
+constexpr int kCOff = 512, kBwdRec = 576;  // per (row, window): weight digits and exponents, |Chat| of the row before
 constexpr int kStateRec = 1024;            // per (row, tile): input digits
 
 struct DigitSweep {
@@ -219,7 +219,7 @@ __device__ __forceinline__ void digit_item(const DigitSweep &a, int4 item, int l
         }
       }
     }
-    {  // backward: x_i = y_i - Chat x_{i+1}; the sums of row i + 1 beside the FMAs of row i
+    {  // backward: x_i = y_i - |Chat| x_{i+1}; the sums of row i + 1 beside the FMAs of row i
       const char *f = a.bwd + (row0 * a.nwin + (int64_t)(w + 1) * len - 1) * kBwdRec + lane * 16;
       int todo = len;
       unsigned odd = 0;
@@ -227,7 +227,7 @@ __device__ __forceinline__ void digit_item(const DigitSweep &a, int4 item, int l
         if (todo > 0) {
           const unsigned to = sm + odd * kBwdRec + lane * 16;
           copy_async(to, f);
-          if (lane < 8) copy_async(to + 512, f + 512);
+          if (lane < 4) copy_async(to + 512, f + 512);
           f -= kBwdRec;
           --todo;
           odd ^= 1;
@@ -253,8 +253,9 @@ __device__ __forceinline__ void digit_item(const DigitSweep &a, int4 item, int l
         __syncwarp();  // row i has landed for every lane; the stage of row i + 1 has been read
         issue();
         // Chat of row i - 1 is stored with row i (zero with row 0, whose xn is not used)
-        const double2 xn[2] = {cfms(y[0], reinterpret_cast<const double2 *>(stage + kCOff)[2 * q], x[0]),
-                               cfms(y[1], reinterpret_cast<const double2 *>(stage + kCOff)[2 * q + 1], x[1])};
+        const double2 c = reinterpret_cast<const double2 *>(stage + kCOff)[q];
+        const double2 xn[2] = {make_double2(fma(-c.x, x[0].x, y[0].x), fma(-c.x, x[0].y, y[0].y)),
+                               make_double2(fma(-c.y, x[1].x, y[1].x), fma(-c.y, x[1].y, y[1].y))};
         if (i > 1) {
           y[0] = yp[-128];
           y[1] = yp[-96];

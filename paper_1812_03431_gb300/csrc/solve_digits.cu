@@ -4,7 +4,8 @@
 // The systems, factors and recurrences are those of solve.cu: per (pole k, zonal order m,
 // parity) forward  y_i = r_i - l y_{i-1},  r_i = delta0_n - g Phi0_n - e zeta0_{n-1} - f zeta0_{n+1},
 // backward  w_i = y_i - Chat w_{i+1},  and the sums over k of bd w, bad w, zp w and zm w.
-// Of the 36 FP64 FMAs per (state, pole, row), 8 belong to the two recurrences; the other 28
+// Of the 36 FP64 FMAs per (state, pole, row), 8 belong to the two recurrences (6 here: see below);
+// the other 28
 // are contractions with factors that no state changes: r over the row's four inputs, and the
 // four weighted sums over the poles.  GB300's FP64 unit issues one warp instruction per 64
 // cycles and scheduler, so the contractions are taken off it:
@@ -17,6 +18,10 @@
 //     below 2^-60 of the largest product);
 //   - the eight sums of equal weight are put together in a 64-bit integer, which is rounded to
 //     binary64 once, on the integer pipe.
+// The recurrences take 6: with y_i = p_i y~_i, w_i = p_i w~_i and unit complex p_i such that
+// Chat_i p_{i+1} / p_i = |Chat_i|, the backward one multiplies by a real number.  1/p_i goes into the
+// couplings and p_i into the weights before they are cut into digits (p is kept to 2^-60), and l
+// turns into l p_{i-1} / p_i; nothing else changes.
 // The sums are therefore exact up to the 2^-55 rounding of a group's smaller operands and one
 // rounding each; the recurrences run in binary64 as before.  The pole sums of an item's
 // windows are added in binary64 in window order, and the items' sums in a fixed order, so
@@ -29,11 +34,11 @@
 // cycles each, about a third of the FP64 time beside them, so their rate does not bound it.
 //
 // Measured on GB300 (solve and the sum of the slots, against the pole-slot solve and its
-// reduction): T341, 535 poles, 16 states 9.1 / 30.0 ms; T127, 535 poles, 64 states 5.1 / 17.0;
-// T85, 215 poles, 5 states 0.17 / 0.62.  What bounds it now: the FP64 unit, 86 % busy (ncu, T170 x
-// 16) with 9 instructions per state, pole and row at 64 cycles, one of them the running sum's
-// addition, at 16 warps per SM (12 warps: 10.2 ms at T341).  Rows staged ahead in shared memory
-// with asynchronous copies took it there from 78 % (9.9 ms with prefetches into the caches).
+// reduction): T341, 535 poles, 16 states 8.3 / 30.0 ms; T127, 535 poles, 64 states 4.6 / 17.0;
+// T85, 215 poles, 5 states 0.17 / 0.62.  The FP64 unit takes 7 instructions per state, pole and
+// row at 64 cycles, one of them the running sum's addition, at 16 warps per SM (12 warps: 10.2 ms
+// at T341); with the complex Chat it was 9, 86 % busy, and 9.1 ms.  Rows staged ahead in shared
+// memory with asynchronous copies took it there from 78 % (9.9 ms with prefetches into the caches).
 //
 // A warp takes 8 states x 8 poles (lane: state lane / 4, poles 2 (lane % 4) and the next) of one
 // (m, parity) system, window by window of 8 poles, over all rows.  Real and imaginary rows of
@@ -59,6 +64,7 @@ namespace {
 // ---- plan time: the factors as digits ---------------------------------------------------------
 struct SetupArgs {
   const double2 *fac;  // [F_NCOMP][nrows][P]
+  longlong2 *phase;    // [nrows][P]: p
   const int4 *sys;
   char *fwd, *bwd;     // records, system by system: [window][row of the system]
   int *vexp;           // [nrows][4]: the scale of each input (0 for delta)
@@ -66,6 +72,53 @@ struct SetupArgs {
   int P, nwin, kmid;
   int64_t nrows;
 };
+
+// Unit complex numbers as pairs of integers in units of 2^-62.  v q, rounded:
+__device__ __forceinline__ long long times(long long v, long long q) {
+  const unsigned long long l = (unsigned long long)v * (unsigned long long)q;
+  return (long long)((unsigned long long)__mul64hi(v, q) << 2 | l >> 62) + (long long)(l >> 61 & 1);
+}
+__device__ __forceinline__ longlong2 times(longlong2 v, longlong2 q) {
+  return longlong2{times(v.x, q.x) - times(v.y, q.y), times(v.x, q.y) + times(v.y, q.x)};
+}
+__device__ __forceinline__ longlong2 conj(longlong2 q) { return longlong2{q.x, -q.y}; }
+
+// c / |c| (1 where c is zero): in binary64, then its phase and length corrected to first order
+__device__ longlong2 unit_of(double2 c) {
+  const int e = max(bexp(c.x), bexp(c.y));
+  if (e == 0 || e > 2040) return longlong2{1ll << 62, 0};
+  const double s = __longlong_as_double((long long)(2046 - e) << 52);
+  const double x = c.x * s, y = c.y * s, r = rsqrt(x * x + y * y), ux = x * r, uy = y * r;
+  const double w = x * uy, phase = (fma(y, ux, -w) + fma(-x, uy, w)) * r;
+  const double big = fmax(fabs(ux), fabs(uy)), small = fmin(fabs(ux), fabs(uy)), b2 = big * big, s2 = small * small;
+  const double half = 0.5 * (((1.0 - b2) - s2) - (fma(big, big, -b2) + fma(small, small, -s2)));
+  auto q62 = [](double hi, double lo) {
+    return __double2ll_rn(hi * 4611686018427387904.0) + __double2ll_rn(lo * 4611686018427387904.0);
+  };
+  return longlong2{q62(ux, ux * half - uy * phase), q62(uy, uy * half + ux * phase)};
+}
+
+// p of every row, one thread per (pole, system): p_0 = 1, p_{i+1} = p_i |Chat_i| / Chat_i
+__global__ void digit_phase_kernel(SetupArgs a) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  const int4 sy = a.sys[blockIdx.y];
+  if (k >= a.P) return;
+  longlong2 p{1ll << 62, 0};
+  for (int i = 0; i < sy.z; ++i) {
+    const int64_t row = (int64_t)sy.w + i;
+    a.phase[row * a.P + k] = p;
+    if (i + 1 < sy.z) p = times(p, conj(unit_of(a.fac[((int64_t)F_C * a.nrows + row) * a.P + k])));
+  }
+}
+
+// v's parts as to_fixed gives them, E the exponent (biased) of their group's leading bit
+__device__ __forceinline__ longlong2 fixed_of(double2 v, int E) {
+  return longlong2{to_fixed(v.x, E - bexp(v.x)), to_fixed(v.y, E - bexp(v.y))};
+}
+__device__ __forceinline__ bool reaches_62(longlong2 v) {
+  return v.x >= 1ll << 62 || v.x <= -(1ll << 62) || v.y >= 1ll << 62 || v.y <= -(1ll << 62);
+}
+__device__ __forceinline__ longlong2 halve(longlong2 v) { return longlong2{(v.x + 1) >> 1, (v.y + 1) >> 1}; }
 
 __global__ void digit_factor_kernel(SetupArgs a) {
   const int4 sy = a.sys[blockIdx.y];
@@ -98,19 +151,30 @@ __global__ void digit_factor_kernel(SetupArgs a) {
     if (e == 0x7ff) bad = true;
     if (e) E = max(E, e - ve[j]);
   }
+  // rotated by 1/p, which can take a part of one past the leading bit
+  const longlong2 p = live && k < a.P ? a.phase[row * a.P + k] : longlong2{1ll << 62, 0};
+  longlong2 fv[4];
+  bool past = false;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const int e = emax(v[j]);
     if (e && E - (e - ve[j]) > kMaxSpread) bad = true;
-    if (live)
-      reinterpret_cast<uint4 *>(fr)[p8 * 4 + j] =
-          packed_digits(to_fixed(v[j].x, E - (bexp(v[j].x) - ve[j])), to_fixed(v[j].y, E - (bexp(v[j].y) - ve[j])));
+    fv[j] = times(fixed_of(v[j], E + ve[j]), conj(p));
+    past |= reaches_62(fv[j]);
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (past) fv[j] = halve(fv[j]);
+    if (live) reinterpret_cast<uint4 *>(fr)[p8 * 4 + j] = packed_digits(fv[j].x, fv[j].y);
   }
   if (live) {
-    *reinterpret_cast<double2 *>(fr + kLOff + p8 * 16) = get(F_L, k);
-    *reinterpret_cast<int *>(fr + kEOff + p8 * 4) = E - 1023;
-    *reinterpret_cast<double2 *>(br + kCOff + p8 * 16) =
-        i > 0 && k < a.P ? a.fac[((int64_t)F_C * a.nrows + row - 1) * a.P + k] : zero;
+    // l p_{i-1} / p_i and |Chat| of the row before, u = Chat / |Chat| of that row
+    const double2 l = get(F_L, k), c = i > 0 && k < a.P ? a.fac[((int64_t)F_C * a.nrows + row - 1) * a.P + k] : zero;
+    const longlong2 u = unit_of(c), fl = times(fixed_of(l, emax(l)), u), fc = times(fixed_of(c, emax(c)), conj(u));
+    const int le = emax(l) - 1023 - 61;
+    reinterpret_cast<double2 *>(fr + kLOff)[p8] = make_double2(fixed_to_double(fl.x, le), fixed_to_double(fl.y, le));
+    reinterpret_cast<int *>(fr + kEOff)[p8] = E - 1023 + past;
+    reinterpret_cast<double *>(br + kCOff)[p8] = fixed_to_double(fc.x, emax(c) - 1023 - 61);
     if (w == 0 && p8 < 4) a.vexp[row * 4 + p8] = ve[p8];
   }
   // the four weights, scaled by the largest of the window's eight poles
@@ -122,16 +186,24 @@ __global__ void digit_factor_kernel(SetupArgs a) {
     if (m == 0x7ff) bad = true;
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    longlong2 f = times(fixed_of(x, m), p);
+    int over = reaches_62(f);
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) over |= __shfl_xor_sync(0xffffffffu, over, o);
+    if (over) {
+      f = halve(f);
+      ++m;
+    }
     // seven digits (rounded to the nearest multiple of the eighth's weight), the real parts of
     // poles 2 q and 2 q + 1 by the even thread, their imaginary parts by the odd one
-    const long long re = (to_fixed(x.x, m - bexp(x.x)) + 128) & ~255ll, im = (to_fixed(x.y, m - bexp(x.y)) + 128) & ~255ll;
+    const long long re = (f.x + 128) & ~255ll, im = (f.y + 128) & ~255ll;
     const long long other = __shfl_xor_sync(0xffffffffu, p8 & 1 ? re : im, 1);
     uint4 d = packed_digits(p8 & 1 ? other : re, p8 & 1 ? im : other);
     d.w = (d.w & 0xffffu) | (unsigned)(m - 1023) << 16;  // the exponent in the eighth digits' place
     if (live) reinterpret_cast<uint4 *>(br)[s * kWin + p8] = d;
   }
   const double2 l = get(F_L, k), c = get(F_C, k);
-  if (emax(l) == 0x7ff || emax(c) == 0x7ff) bad = true;
+  if (emax(l) == 0x7ff || emax(c) > 2040) bad = true;  // unit_of goes up to there
   if (bad) atomicOr(a.bad, 1);
 }
 
@@ -282,8 +354,9 @@ cudaError_t launch_digit_factors(Plan &pl, const double2 *fac, DigitFactors &D, 
   cudaError_t e = cudaMalloc(&D.fwd, nrec * kFwdRec);
   if (e == cudaSuccess) e = cudaMalloc(&D.bwd, nrec * kBwdRec);
   if (e == cudaSuccess) e = cudaMalloc(&D.vexp, (size_t)pl.nrows * 4 * sizeof(int));
-  if (e != cudaSuccess) return e;
   SetupArgs a;
+  if (e == cudaSuccess) e = cudaMalloc(&a.phase, (size_t)pl.nrows * pl.P * sizeof(longlong2));
+  if (e != cudaSuccess) return e;
   a.fac = fac;
   a.sys = pl.sys_dev;
   a.fwd = D.fwd;
@@ -297,8 +370,11 @@ cudaError_t launch_digit_factors(Plan &pl, const double2 *fac, DigitFactors &D, 
                  pl.alpha.begin());
   a.nrows = pl.nrows;
   const int64_t most = (int64_t)pl.lmax * nwin * kWin;
+  digit_phase_kernel<<<dim3((unsigned)((pl.P + 63) / 64), (unsigned)pl.sys.size()), 64>>>(a);
   digit_factor_kernel<<<dim3((unsigned)((most + 255) / 256), (unsigned)pl.sys.size()), 256>>>(a);
-  return cudaGetLastError();
+  e = cudaGetLastError();
+  cudaFree(a.phase);  // waits for the kernels
+  return e;
 }
 }  // namespace
 
