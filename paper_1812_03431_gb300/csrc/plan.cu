@@ -9,6 +9,7 @@
 #include <numeric>
 #include <string>
 
+#include "recip.h"
 #include "rexi_internal.h"
 
 namespace rexi {
@@ -50,24 +51,16 @@ __global__ void zeta_weights_kernel(const double *coef, const int32_t *m_of, con
   if (ix >= NS) return;
   const double sig = coef[4 * ix + 0];
   const double G = coef[4 * ix + 3];  // n (n + 1) / a^2, zero only at n = 0
-  double2 sf = make_double2(0, 0), sa = make_double2(0, 0);
+  double2 sf = make_double2(0, 0);
   if (G > 0.0 || m_of[ix] > 0) {
     for (int k = 0; k < P; ++k) {
       const double2 al = alpha[k], be = beta[k];
-      // beta / (alpha + i tau sigma)
-      double dr = al.x, di = al.y + tau * sig, d = dr * dr + di * di;
-      sf.x += (be.x * dr + be.y * di) / d;
-      sf.y += (be.y * dr - be.x * di) / d;
-      // conj(beta) / (conj(alpha) - i tau sigma)
-      dr = al.x;
-      di = -al.y - tau * sig;
-      d = dr * dr + di * di;
-      sa.x += (be.x * dr - be.y * di) / d;
-      sa.y += (-be.y * dr - be.x * di) / d;
+      const double2 v = ComplexRecip(make_double2(al.x, al.y + tau * sig)).of(be);  // beta / (alpha + i tau sigma)
+      sf = make_double2(sf.x + v.x, sf.y + v.y);
     }
   }
   wf[ix] = sf;
-  wa[ix] = sa;
+  wa[ix] = make_double2(sf.x, -sf.y);  // conj(beta) / (conj(alpha) - i tau sigma) is its conjugate, bit for bit
 }
 
 // Orthonormal Pbar_n^m(mu_j) and H_n^m(mu_j) for the northern latitudes j < J, one

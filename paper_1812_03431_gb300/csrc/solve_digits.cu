@@ -64,7 +64,6 @@ namespace {
 // ---- plan time: the factors as digits ---------------------------------------------------------
 struct SetupArgs {
   const double2 *fac;  // [F_NCOMP][nrows][P]
-  longlong2 *phase;    // [nrows][P]: p
   const int4 *sys;
   char *fwd, *bwd;     // records, system by system: [window][row of the system]
   int *vexp;           // [nrows][4]: the scale of each input (0 for delta)
@@ -98,16 +97,21 @@ __device__ longlong2 unit_of(double2 c) {
   return longlong2{q62(ux, ux * half - uy * phase), q62(uy, uy * half + ux * phase)};
 }
 
-// p of every row, one thread per (pole, system): p_0 = 1, p_{i+1} = p_i |Chat_i| / Chat_i
+// p of every row and u = Chat / |Chat| of the row before, one thread per (pole, system): p_0 = 1,
+// p_{i+1} = p_i / u_i.  They go where the pole's coupling digits will be, which the thread that
+// reads them writes.
 __global__ void digit_phase_kernel(SetupArgs a) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   const int4 sy = a.sys[blockIdx.y];
   if (k >= a.P) return;
-  longlong2 p{1ll << 62, 0};
-  for (int i = 0; i < sy.z; ++i) {
-    const int64_t row = (int64_t)sy.w + i;
-    a.phase[row * a.P + k] = p;
-    if (i + 1 < sy.z) p = times(p, conj(unit_of(a.fac[((int64_t)F_C * a.nrows + row) * a.P + k])));
+  char *to = a.fwd + ((int64_t)sy.w * a.nwin + (int64_t)(k / kWin) * sy.z) * kFwdRec + (k % kWin) * 64;
+  longlong2 p{1ll << 62, 0}, u = p;
+  for (int i = 0; i < sy.z; ++i, to += kFwdRec) {
+    reinterpret_cast<longlong2 *>(to)[0] = p;
+    reinterpret_cast<longlong2 *>(to)[1] = u;
+    if (i + 1 == sy.z) break;
+    u = unit_of(a.fac[((int64_t)F_C * a.nrows + sy.w + i) * a.P + k]);
+    p = times(p, conj(u));
   }
 }
 
@@ -152,7 +156,8 @@ __global__ void digit_factor_kernel(SetupArgs a) {
     if (e) E = max(E, e - ve[j]);
   }
   // rotated by 1/p, which can take a part of one past the leading bit
-  const longlong2 p = live && k < a.P ? a.phase[row * a.P + k] : longlong2{1ll << 62, 0};
+  const longlong2 one{1ll << 62, 0}, *pu = reinterpret_cast<const longlong2 *>(fr + p8 * 64);
+  const longlong2 p = live && k < a.P ? pu[0] : one, u = live && k < a.P ? pu[1] : one;
   longlong2 fv[4];
   bool past = false;
 #pragma unroll
@@ -168,9 +173,9 @@ __global__ void digit_factor_kernel(SetupArgs a) {
     if (live) reinterpret_cast<uint4 *>(fr)[p8 * 4 + j] = packed_digits(fv[j].x, fv[j].y);
   }
   if (live) {
-    // l p_{i-1} / p_i and |Chat| of the row before, u = Chat / |Chat| of that row
+    // l p_{i-1} / p_i and |Chat| of the row before
     const double2 l = get(F_L, k), c = i > 0 && k < a.P ? a.fac[((int64_t)F_C * a.nrows + row - 1) * a.P + k] : zero;
-    const longlong2 u = unit_of(c), fl = times(fixed_of(l, emax(l)), u), fc = times(fixed_of(c, emax(c)), conj(u));
+    const longlong2 fl = times(fixed_of(l, emax(l)), u), fc = times(fixed_of(c, emax(c)), conj(u));
     const int le = emax(l) - 1023 - 61;
     reinterpret_cast<double2 *>(fr + kLOff)[p8] = make_double2(fixed_to_double(fl.x, le), fixed_to_double(fl.y, le));
     reinterpret_cast<int *>(fr + kEOff)[p8] = E - 1023 + past;
@@ -354,9 +359,8 @@ cudaError_t launch_digit_factors(Plan &pl, const double2 *fac, DigitFactors &D, 
   cudaError_t e = cudaMalloc(&D.fwd, nrec * kFwdRec);
   if (e == cudaSuccess) e = cudaMalloc(&D.bwd, nrec * kBwdRec);
   if (e == cudaSuccess) e = cudaMalloc(&D.vexp, (size_t)pl.nrows * 4 * sizeof(int));
-  SetupArgs a;
-  if (e == cudaSuccess) e = cudaMalloc(&a.phase, (size_t)pl.nrows * pl.P * sizeof(longlong2));
   if (e != cudaSuccess) return e;
+  SetupArgs a;
   a.fac = fac;
   a.sys = pl.sys_dev;
   a.fwd = D.fwd;
@@ -372,9 +376,7 @@ cudaError_t launch_digit_factors(Plan &pl, const double2 *fac, DigitFactors &D, 
   const int64_t most = (int64_t)pl.lmax * nwin * kWin;
   digit_phase_kernel<<<dim3((unsigned)((pl.P + 63) / 64), (unsigned)pl.sys.size()), 64>>>(a);
   digit_factor_kernel<<<dim3((unsigned)((most + 255) / 256), (unsigned)pl.sys.size()), 256>>>(a);
-  e = cudaGetLastError();
-  cudaFree(a.phase);  // waits for the kernels
-  return e;
+  return cudaGetLastError();
 }
 }  // namespace
 
