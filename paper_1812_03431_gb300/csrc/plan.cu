@@ -100,6 +100,12 @@ void free_plan(Plan *pl);
 // most device memory either's factors may take: 156 and 68 B per row and pole beside the
 // binary64 factors' 144.
 constexpr int kDigitMinBatch = 5;
+// Larger plans' batches of three and four: the digit solve, its tiles padded, from this many rows
+// times poles (T63, 279 poles, 0.58 million: three states 0.144 / 0.159 ms, four 0.144 / 0.199; T170 x
+// 3 1.17 / 1.59; T341 x 3 4.4 / 6.3), else the fused solve (T42, 151 poles, 0.14 million: 0.082 /
+// 0.067).  Two states: 4.4 / 4.1 ms at T341.
+constexpr int kDigitMinBatchLarge = 3;
+constexpr int64_t kDigitLarge = 400000;
 constexpr size_t kDigitMostBytes = (size_t)32 << 30;
 
 rexi_status build_plan(const rexi_params &prm, Plan *pl) {
@@ -605,11 +611,12 @@ const FusedLayout *fused_layout(Plan &pl, int B) {
 
 // The digit solve's work list for steps of B states, or null where another kernel serves them:
 // no digit factors (see build_plan), an explicit pole_slots, another layout chosen for this
-// batch, or without a choice a batch below kDigitMinBatch.
+// batch, or without a choice a batch below kDigitMinBatch (kDigitMinBatchLarge).
 const DigitLayout *digit_layout(Plan &pl, int B, bool adjoint) {
   if (!(adjoint ? pl.dig_adj : pl.dig_fwd).fwd) return nullptr;
   auto ud = pl.use_digits.find(B);
-  if (ud != pl.use_digits.end() ? !ud->second : (pl.slots_override > 0 || (B < kDigitMinBatch && !pl.limbs))) return nullptr;
+  const int least = pl.limbs ? 1 : (pl.nrows * pl.P >= kDigitLarge ? kDigitMinBatchLarge : kDigitMinBatch);
+  if (ud != pl.use_digits.end() ? !ud->second : (pl.slots_override > 0 || B < least)) return nullptr;
   auto it = pl.digits.find(B);
   if (it == pl.digits.end()) {
     DigitLayout L;

@@ -173,3 +173,17 @@ def test_poles_of_unlike_scale_keep_the_other_solves(env, B):
         plan.set_pole_slots(B, 0, 5)
     plan.close()
     slots.close()
+
+
+@pytest.mark.parametrize("B", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("N,M", [(42, 64), (63, 128)])
+def test_small_batches_of_a_larger_plan(env, N, M, B):
+    """Batches below the tile of eight, on both sides of the rule's line, against the pole-slot solve."""
+    torch, rexi = env
+    al, be, _ = rc.rexi_coefficients(M, 0.2)
+    x = torch.from_numpy(inputs.random_spectral(N, B, 13)).cuda()
+    plan, slots = spectral_plan(rexi, N, 6, al, be), spectral_plan(rexi, N, 6, al, be, pole_slots=8)
+    assert fieldwise(plan.step(x).cpu().numpy(), slots.step(x).cpu().numpy()) < ORDER
+    assert fieldwise(plan.step_adjoint(x).cpu().numpy(), slots.step_adjoint(x).cpu().numpy()) < ORDER
+    plan.close()
+    slots.close()
