@@ -288,9 +288,15 @@ struct FinishArgs {
   int B, tile, tiles, unit, sstr, pstr, slots, N;
 };
 
+// SPLIT threads per output, each over every SPLIT-th slot: one where the outputs fill the chip (HBM
+// bounds it: T341 x 16 with 8 slots 0.123 to 0.131 ms, 0.137 without four slots' loads in flight), four where
+// they are few and the slots many (T85 x 5 with 27 20 / 31 us, T42 x 8 with 19 12 / 16 us).
+template <int SPLIT>
 __global__ void digit_finish_kernel(FinishArgs a) {
-  const int64_t total = 3 * a.nspec * a.B, slot = a.nrows * a.tiles * a.unit;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t total = 3 * a.nspec * a.B, slot = a.nrows * a.tiles * a.unit, step = slot * SPLIT;
+  const int first = threadIdx.x % SPLIT;
+  for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / SPLIT; t < total;
+       t += (int64_t)gridDim.x * blockDim.x / SPLIT) {
     const int b = (int)(t % a.B);
     const int64_t fi = t / a.B;
     const int f = (int)(fi / a.nspec);
@@ -304,13 +310,17 @@ __global__ void digit_finish_kernel(FinishArgs a) {
         auto add = [&](int nn, int stream) {  // the slots' sums of the row at degree nn, in slot order
           const int4 sy = a.sys[2 * m + ((nn - m) & 1)];
           const int64_t row = sy.w + (nn - sy.y) / 2;
-          const double *p = a.part + (row * a.tiles + b / a.tile) * a.unit + b % a.tile + stream * a.sstr;
-          if (a.scale && stream > 0) {
-            const double c = a.scale[row * 6 + 2 + stream];
-            for (int s = 0; s < a.slots; ++s, p += slot) acc = make_double2(fma(c, p[0], acc.x), fma(c, p[a.pstr], acc.y));
-          } else {
-            for (int s = 0; s < a.slots; ++s, p += slot) acc = make_double2(acc.x + p[0], acc.y + p[a.pstr]);
+          const double *p = a.part + (row * a.tiles + b / a.tile) * a.unit + b % a.tile + stream * a.sstr + first * slot;
+          const double c = a.scale && stream > 0 ? a.scale[row * 6 + 2 + stream] : 1.0;
+          int s = first;
+          for (; s + 3 * SPLIT < a.slots; s += 4 * SPLIT) {  // loads of four slots in flight
+            double2 v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k, p += step) v[k] = make_double2(p[0], p[a.pstr]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc = make_double2(fma(c, v[k].x, acc.x), fma(c, v[k].y, acc.y));
           }
+          for (; s < a.slots; s += SPLIT, p += step) acc = make_double2(fma(c, p[0], acc.x), fma(c, p[a.pstr], acc.y));
         };
         const int nmin = m > 1 ? m : 1;
         if (f != 1) add(n, f == 2 ? 0 : 1);
@@ -318,13 +328,19 @@ __global__ void digit_finish_kernel(FinishArgs a) {
           if (n - 1 >= nmin) add(n - 1, 2);
           if (n + 1 <= a.N) add(n + 1, 3);
         }
+#pragma unroll
+        for (int o = 1; o < SPLIT; o <<= 1) {  // an output's threads are neighbours and take the same branches
+          const unsigned group = ((1u << SPLIT) - 1) << (threadIdx.x & 31 & -SPLIT);
+          const double re = __shfl_xor_sync(group, acc.x, o), im = __shfl_xor_sync(group, acc.y, o);
+          acc = make_double2(acc.x + re, acc.y + im);
+        }
       }
       const double2 x0 = a.sin[t];
       if (f == 0) acc = cfma(acc, a.sphi, x0);
       else if (f == 1) acc = cfma(acc, a.w[ix], x0);
       if (m == 0) acc.y = 0.0;
     }
-    a.sout[t] = acc;
+    if (first == 0) a.sout[t] = acc;
   }
 }
 
@@ -560,7 +576,9 @@ cudaError_t launch_finish_digits(Plan &pl, const DigitLayout &L, bool adjoint, c
   f.scale = (adjoint ? pl.dig_adj : pl.dig_fwd).scale;
   f.N = pl.N;
   const int64_t total = 3 * pl.nspec * B;
-  digit_finish_kernel<<<(unsigned)std::min<int64_t>((total + 255) / 256, 1 << 20), 256, 0, st>>>(f);
+  const int split = L.slots >= 8 && total <= 2048 * (int64_t)pl.num_sms ? 4 : 1;
+  (split > 1 ? digit_finish_kernel<4> : digit_finish_kernel<1>)<<<
+      (unsigned)std::min<int64_t>((total * split + 255) / 256, 1 << 20), 256, 0, st>>>(f);
   return cudaGetLastError();
 }
 
