@@ -56,6 +56,12 @@ METRIC = "REXI steps/s at T341, K=256 poles: chosen vs plain FP64 form at stated
 # comparison only: it does not keep the solves in binary64.
 FORMS = [("mixed", "mixed", "fp64"), ("fp64", "fp64", "fp64"), ("ff_solve", "mixed", "fp32x2")]
 FLOPS_PER_ROW = 72  # FP64 flops per (state, pole, row) of the fused solve: 36 FMAs
+# The fixed-point solve (layout shape 5) keeps the two recurrences and one addition on the FP64
+# unit: 7 instructions per (state, pole, row) on its tensor-core form (6 FMAs, counted as 2
+# each like the addition), 8 FMAs and no addition per pole on the limb form of small batches
+DIGIT_FLOPS_PER_ROW, LIMB_FLOPS_PER_ROW = 14, 16
+# its Legendre transforms: 36 digit products per multiply-add, on the tensor cores
+DIGIT_PRODUCTS = 36
 # FP32 operations per (state, pole, row) of the float-float solve: the same 36 real
 # multiply-adds, each an error-free product and sum of 12 FP32 operations (1 mul, 3 FMA,
 # 8 add); stored values stay unnormalised pairs, so there is no renormalisation
@@ -107,7 +113,14 @@ def solve_layout(r):
     return {"pole_slots": r["slots"], "layout_shape": r["shape"]}
 
 
-def kernel_rooflines(form, stages, slots, sm_mhz, solve_arith="fp64", fp64_peak=None):
+def solve_flops_per_row(shape, batch):
+    """FP64 work per (state, pole, row) of a binary64 solve layout."""
+    if shape != 5:
+        return FLOPS_PER_ROW
+    return DIGIT_FLOPS_PER_ROW if batch > 4 else LIMB_FLOPS_PER_ROW
+
+
+def kernel_rooflines(form, stages, slots, sm_mhz, solve_arith="fp64", fp64_peak=None, shape=None):
     """Every stage of the grid step against its own bound: algorithmic bytes (HBM-bound
     stages) or flops (ALU-bound stages) per launch / its live CUDA-event time.
     fp64_peak: the measured FP64 FMA rate in TFLOP/s (else derived from the clock)."""
@@ -141,26 +154,27 @@ def kernel_rooflines(form, stages, slots, sm_mhz, solve_arith="fp64", fp64_peak=
         put("leg_ana", "hbm", leg_b, "GB/s", hbm, src + " HBM copy")
         put("leg_syn", "hbm", leg_b, "GB/s", hbm, src + " HBM copy")
     else:
-        # FP64 FFT: 5 n log2 n flops per half-length complex transform of each real row
-        import math
-        half = nlon // 2
-        fl = 5.0 * half * math.log2(half) * B * 3 * nlat
-        put("fft_fwd", "alu", fl, "TFLOP/s", fp64, fp64_src)
-        put("fft_inv", "alu", fl, "TFLOP/s", fp64, fp64_src)
-        # FP64 Legendre: 10 FMAs per (n, lat pair, state) each way
-        fl = 20.0 * ns * (nlat // 2) * B
-        put("leg_ana", "alu", fl, "TFLOP/s", fp64, fp64_src)
-        put("leg_syn", "alu", fl, "TFLOP/s", fp64, fp64_src)
+        # the FP64 form's transforms run in block fixed point: the FFTs on the integer pipe (bytes
+        # moved are their floor), the Legendre sums as digit products, 10 multiply-adds per (n, lat
+        # pair, state) each way, against the library GEMM's rate
+        put("fft_fwd", "hbm", grid_b + four_b, "GB/s", hbm, src + " HBM copy")
+        put("fft_inv", "hbm", grid_b + four_b, "GB/s", hbm, src + " HBM copy")
+        fl = 20.0 * DIGIT_PRODUCTS * ns * (nlat // 2) * B
+        put("leg_ana", "alu", fl, "TFLOP/s", bf16, src + " bf16 GEMM")
+        put("leg_syn", "alu", fl, "TFLOP/s", bf16, src + " bf16 GEMM")
     if solve_arith == "fp32x2":
         put("solve", "alu", FF_OPS_PER_ROW * B * P * rows_of(N), "Tops/s", fp32_peak_tops(sm_mhz),
             "derived FP32 (ops = adds, multiplies and FMAs)")
         # float-float reduction: reads every slot's partials once, writes the result
         put("reduce", "hbm", (slots + 2) * 3 * ns * B * 16, "GB/s", hbm, src + " HBM copy")
     else:
-        put("solve", "alu", FLOPS_PER_ROW * B * P * rows_of(N), "TFLOP/s", fp64, fp64_src)
+        put("solve", "alu", solve_flops_per_row(shape, B) * B * P * rows_of(N), "TFLOP/s", fp64, fp64_src)
         # reduction: one FP64 complex add per slot and output coefficient; the kernel is bound
         # by the FP64 issue rate (ncu: FP64 pipe 82 %, DRAM 47 %), where an add costs an FMA's slot
-        put("reduce", "alu", 2.0 * slots * 3 * ns * B, "TFLOP/s", fp64 / 2, fp64_src + " (adds: half)")
+        if shape == 5:  # the slots' partial sums of four streams per row, read once
+            put("reduce", "hbm", slots * 64.0 * rows_of(N) * ((B + 7) // 8 * 8) + 2 * spec_b, "GB/s", hbm, src + " HBM copy")
+        else:
+            put("reduce", "alu", 2.0 * slots * 3 * ns * B, "TFLOP/s", fp64 / 2, fp64_src + " (adds: half)")
     return out
 
 
@@ -586,7 +600,7 @@ def main():
         kname = "solve_kernel<true> (float-float banded solves + pole sum)"
         roof_unit, peak_source = "Tops/s", "derived: 152 SMs x 128 FP32 lanes x sm_max_mhz (ops = adds, mults, FMAs)"
     else:
-        amount, peak = FLOPS_PER_ROW * B * P * rows_of(W["N"]), fp64_tf or fp64_peak_tflops(sm_mhz)
+        amount, peak = solve_flops_per_row(r["shape"], B) * B * P * rows_of(W["N"]), fp64_tf or fp64_peak_tflops(sm_mhz)
         traffic_tab, kname = SOLVE_TRAFFIC, "solve_kernel<false> (FP64 banded solves + pole sum)"
         roof_unit = "TFLOP/s"
         peak_source = ("measured: rexi_measure_fp64_fma, best of 5 per shape (FP64 FMA chains)" if fp64_tf else
@@ -608,6 +622,10 @@ def main():
         # the captures hold one pole group; NG groups add their partial sums, written once
         # and read once: B x NG x rows x 4 streams x 16 bytes each way
         traffic += 2 * B * groups * rows_of(W["N"]) * 64
+    if r["shape"] == 5 and r["solve_arith"] == "fp64":
+        kname = "solve_digits_kernel (FP64 recurrences; right-hand sides and pole sums as digit products)" if B > 4 \
+            else "solve_limbs_kernel (FP64 recurrences; right-hand sides and pole sums in integer limbs)"
+        traffic = None  # not captured at this size
     if fused:
         kname = "solve_fused_kernel (FP64 banded solves, beta-weighted pole sum on chip)"
     dtypes = {"mixed": "f64 solves + pole sum; 3xtf32 legendre; f32 fft", "fp64": "f64",
@@ -616,8 +634,11 @@ def main():
         "form at stated error" % (W["N"], W["M"], B, "s" if B > 1 else "")
     if not default_workload:
         traffic = None  # the captured traffic is for 16 states; it does not scale by rows alone
-    # one kernel per timed stage, plus the float-float solve's state split
+    # one kernel per timed stage, plus the state kernels of the float-float and the fixed-point
+    # solve, and the latter's sum of the slots where it is timed with the solve
     launches = sum(1 for v in r["stages"].values() if v > 0) + (1 if r["solve_arith"] == "fp32x2" else 0)
+    if r["shape"] == 5:
+        launches += 1 if r["stages"].get("reduce", 0.0) > 0 else 2
     sharded = args.shard == "poles" and world > 1
     jobs = 1 if sharded else world  # replicas each step a batch; shards step one batch together
     cfg = workload_config()
@@ -645,12 +666,14 @@ def main():
         "solve_stage": {"ms": solve_ms + r["stages"].get("reduce", 0.0),
                         "achieved": amount / ((solve_ms + r["stages"].get("reduce", 0.0)) * 1e-3) / 1e12,
                         "frac": amount / ((solve_ms + r["stages"].get("reduce", 0.0)) * 1e-3) / 1e12 / peak,
-                        "unit": roof_unit, "kernels": "solve_fused_kernel" if fused else "solve_kernel + reduce_kernel"},
+                        "unit": roof_unit, "kernels": "solve_fused_kernel" if fused else
+                        "state, sweep and finishing kernel" if r["shape"] == 5 else "solve_kernel + reduce_kernel"},
         "fp64_peak": {"tflops": fp64_tf, "ms": fp64_ms, "clocks": fp64_clocks,
                       "derived_tflops_at_max_clock": fp64_peak_tflops(sm_mhz)},
         "state_steps_per_s": jobs * B * 1e3 / r["ms"],
         "stage_ms": r["stages"],
-        "kernels": kernel_rooflines(r["precision"], r["stages"], r["slots"], sm_mhz, r["solve_arith"], fp64_tf),
+        "kernels": kernel_rooflines(r["precision"], r["stages"], r["slots"], sm_mhz, r["solve_arith"], fp64_tf,
+                                    r["shape"]),
         "e2e": {"value": jobs * 1e3 / r["ms_e2e"], "unit": "steps/s", "h2d_bytes_per_step": r["bytes"],
                 "d2h_bytes_per_step": r["bytes"], "copies": "pinned host, own streams, overlapping compute",
                 "result_matches_device_step": r["e2e_same"]},
@@ -663,7 +686,7 @@ def main():
                                 "dtype": dtypes[name], "solve_layout": solve_layout(f),
                                 "clocks": f["clocks"],
                                 "kernels": kernel_rooflines(f["precision"], f["stages"], f["slots"], sm_mhz,
-                                                            f["solve_arith"], fp64_tf)}
+                                                            f["solve_arith"], fp64_tf, f["shape"])}
     if "ff_solve_form" in line:
         line["ff_solve_form"]["note"] = ("float-float solves and pole sum on the FP32 pipes: an extension outside "
                                          "the precision contract (binary64 solves), timed for comparison")
