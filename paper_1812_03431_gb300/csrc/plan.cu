@@ -800,7 +800,7 @@ rexi_status tune_layout(Plan &pl, int B, int *slots_out, int *shape_out) {
   if (const DigitLayout *D0 = set_digit_slots(pl, B, 0)) {
     const int def = D0->slots;
     std::vector<int> tries = {def, std::max(1, def / 2), 2 * def, 4 * def};
-    if (pl.limbs) tries = {65536, 2 * 65536};
+    if (pl.limbs) tries = {65536, 2 * 65536, 3 * 65536};
     for (int slots : tries) {
       const DigitLayout *D = set_digit_slots(pl, B, slots);
       if (!D) break;
