@@ -22,8 +22,8 @@
 // in fragment order.  Everything is copied ahead with cp.async: a warp's next table fragment, also
 // across products and barriers, and the next group's inputs while the products run.
 //
-// Measured on GB300 (analysis, synthesis; against the FP64 kernels): T341 x 16 0.84, 0.70 / 4.37, 4.07
-// ms; T255 x 8 0.212, 0.193 / 1.01, 0.86; T639 x 1 0.52, 0.48; T170 x 1 0.031, 0.033 / 0.114, 0.169;
+// Measured on GB300 (analysis, synthesis; against the FP64 kernels): T341 x 16 0.84, 0.71 / 4.37, 4.07
+// ms; T255 x 8 0.212, 0.197 / 1.01, 0.86; T639 x 1 0.52, 0.48; T170 x 1 0.031, 0.033 / 0.114, 0.169;
 // T63 x 1 0.012, 0.014 / 0.037, 0.065.  Without the copies ahead and the shared tile: 0.92, 0.79;
 // 0.234, 0.204; T170 x 1 0.058, 0.076; T63 x 1 0.020, 0.027.  At T255 x 8 the tensor pipe is 35 %, the
 // issue slots 45 % busy (ncu): four warps per scheduler, which wait for each other at the groups'
@@ -57,6 +57,15 @@ constexpr int kZd = 2 * 2 * (kGroup / 2) * kPitch * 16, kDig = kZd + 2 * kGroup 
 constexpr int kRing = kExp + 48 * 4, kSmem = kRing + kWarps * 2 * kFrag;
 static_assert(2 * (kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
 
+// The synthesis' groups run over degrees, along which H grows like n and spectra fall: tables are
+// divided and data multiplied by the power of two below n + 1, or the products of a smooth field's
+// few large coefficients would be small against the group's largest product.
+// A balanced zonal flow's u at T42 against a 113-bit reference: 3.3e-16, without it 1.25e-15 (FP64
+// sums: 4.0e-16); a hundredth of the synthesis' time.
+__device__ __forceinline__ double degree_scale(int n) {
+  return __longlong_as_double((long long)(1023 + 31 - __clz(n + 1)) << 52);
+}
+
 struct TabArgs {
   const double *tab[2];          // Pbar, H: [nspec][J]
   uint4 *dig;                    // [fragment][P, H][4 registers][32 lanes]
@@ -79,7 +88,8 @@ __global__ void __launch_bounds__(32) legendre_digits_setup(TabArgs a) {
   auto val = [&](int r, int k) {
     if (r >= rows || k >= len) return 0.0;
     const int deg = a.synthesis ? k : r, lat = a.synthesis ? r : k;
-    return a.tab[x][(idx0 + cls + 2 * deg) * a.J + lat];
+    const double v = a.tab[x][(idx0 + cls + 2 * deg) * a.J + lat];
+    return a.synthesis ? v * (1.0 / degree_scale(m + cls + 2 * deg)) : v;
   };
   double v[4][4][2];  // k16 step, register, pair
   int e[2] = {0, 0};
@@ -385,11 +395,11 @@ __global__ void __launch_bounds__(256, 2) legendre_digits_synthesis(LegArgs a) {
       for (int h = 0; h < 2; ++h) {
         v[h] = make_double2(0, 0);
         if (ONE && f == 3) continue;
+        const int d = 2 * (2 * lane + h) + odd;
         v[h] = raw[raw_at(odd, 2 * lane + h, f * NS + st)];
-        if (f > 0) {
-          const double s = zds[2 * (2 * lane + h) + odd];
-          v[h] = make_double2(s * v[h].x, s * v[h].y);
-        }
+        double s = degree_scale(m + 2 * r0 + d);
+        if (f > 0) s *= zds[d];
+        v[h] = make_double2(s * v[h].x, s * v[h].y);
       }
       cut_pair(v[0], v[1], dig, cexp, odd * CT + (ONE ? 0 : f), 2 * (ONE ? f : st), lane);
     }

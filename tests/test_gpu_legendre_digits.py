@@ -118,3 +118,19 @@ def test_longitude_transforms(env, nlon):
         assert np.linalg.norm(grid[b, 0] - want[b, 0]) < TOL * np.linalg.norm(want[b, 0])
         assert np.linalg.norm(grid[b, 1:] - want[b, 1:]) < TOL * np.linalg.norm(want[b, 1:])
     plan.close()
+
+
+@pytest.mark.parametrize("N,nlat,nlon", [(42, 64, 128), (63, 96, 192)])
+@pytest.mark.parametrize("B", [1, 2])
+def test_a_smooth_flow_among_small_coefficients(env, N, nlat, nlon, B):
+    """One zonal coefficient, alone and with noise of 1e-4 of it in every degree: the winds are those of
+    either alone, within three roundings (the synthesis' groups hold low and high degrees)."""
+    torch, rexi = env
+    plan = rexi.Plan(N, nlat, nlon, M=8, max_batch=B)
+    small = inputs.random_spectral(N, B, 9) * 1e-4
+    big = np.zeros_like(small)
+    big[:, 1, 1] = 10 * np.abs(inputs.random_spectral(N, B, 9)[:, 1]).max()
+    wind = lambda s: plan.synthesize(torch.from_numpy(s).cuda()).cpu().numpy()[:, 1:]
+    both, alone = wind(big + small), wind(big)
+    assert np.linalg.norm(both - wind(small) - alone) < 3 * 2.0**-52 * np.linalg.norm(alone)
+    plan.close()
