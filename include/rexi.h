@@ -123,10 +123,11 @@ typedef struct {
                            matches cos to the fit level */
   int32_t pole_slots;   /* 0: the default solve -- with binary64 solves of the delta solver on
                            the rotating sphere the fixed-point solve (shape 5 of
-                           rexi_set_pole_slots) where its factors fit (64 to 164 B of device
+                           rexi_set_pole_slots) where its factors fit (68 to 156 B of device
                            memory per row and pole, at most 32 GiB and a third of what is
-                           free) and the poles are of like scale, except for batches of up to
-                           four states in plans with max_batch >= 5; else for up to four
+                           free) and the poles are of like scale, except for batches of one and
+                           two (below 400,000 rows times poles: up to four) states in plans
+                           with max_batch >= 5; else for up to four
                            states the fused solve that keeps the pole sum on chip (one
                            kernel, every output written once), else the pole-slot solve
                            (rexi_tune picks per batch); > 0: the pole-slot solve with this
@@ -287,9 +288,10 @@ rexi_status rexi_tune(rexi_plan *plan, int32_t batch, int32_t *slots, int32_t *s
  * passes), the last CTA of a tile to finish adding the groups' partial sums in group
  * order, or shape 5 for the fixed-point solve (binary64 delta solver on the rotating sphere:
  * the right-hand sides and the pole sums as exact fixed-point products, on the tensor cores in
- * plans with max_batch >= 5, for batches of five and more by default, and in integer limbs in
- * plans of up to four states, by default; slots: the items each system's poles are split over,
- * plus 65536 x the poles per lane for the limbs, 0: the defaults), or shape 3 for its lean form (three or four CTAs of four warps per SM, fewer
+ * plans with max_batch >= 5 and in integer limbs in plans of up to four states; slots: the
+ * items each system's poles are split over, plus for the limbs 65536 x their packing -- 1 or 2
+ * poles per lane, or 3: one, the warps of a CTA sharing each window's rows --, 0: the
+ * defaults), or shape 3 for its lean form (three or four CTAs of four warps per SM, fewer
  * registers, the next rows prefetched into the caches; tiles of up to 8 states), or shape
  * 4 for the lean form on CTAs of two warps (seven or eight per SM; tiles of up to 4
  * states; a tile of 2 states puts each state on a warp of its own, so no CTA splits its
