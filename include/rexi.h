@@ -309,10 +309,11 @@ rexi_status rexi_plan_info(const rexi_plan *plan, int64_t *info, int32_t n);
 /* Ragged batches (mixed truncations and pole counts): the banded solves of
  * every state of several plans run as ONE persistent launch over the merged
  * work list of every plan's items sorted longest first (Sec. 5: every (pole, m)
- * system is independent).  With binary64 solves that launch runs each plan's fixed-point
- * solve (shape 5 of rexi_set_pole_slots) where every plan has one and the states fill its
- * tiles well enough, each plan's inputs prepared before it and its sums put together after it
- * by small kernels; else it is the fused solve:
+ * system is independent).  With binary64 solves each plan's fixed-point solve (shape 5 of
+ * rexi_set_pole_slots) runs where every plan has one and the states fill its tiles well
+ * enough: one launch for the plans of five states and more and one for the smaller ones, each
+ * plan's inputs prepared before them and its sums put together after them by small kernels.
+ * Else the launch is the fused solve:
  * items are (system, tile of 2 states, plan), the pole sum stays on chip and no
  * reduction follows, provided the largest plan's running sums leave seven CTAs of two
  * warps, or three of four warps, per SM.  Otherwise (and with float-float solves) it is the pole-slot solve over

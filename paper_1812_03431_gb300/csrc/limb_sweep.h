@@ -36,7 +36,7 @@ struct LimbSweep {
   const int4 *inv_alpha;    // [P padded]
   const int4 *dig;
   const int *uexp;
-  const int4 *sys, *items;  // {system, tile, first window | windows << 16, slot}
+  const int4 *sys, *items;  // {system, state, first window | windows << 16, slot}
   double *part;             // [slots][nrows][B][4 streams][re, im]
   double2 *ybuf;            // per resident warp: [lmax][2][32]
   unsigned *counter;
@@ -98,15 +98,14 @@ __device__ __forceinline__ void cmad(long long &rh, long long &rl, long long &ih
 }
 
 // r = delta0 + Phi'/alpha + zeta'_{n-1}/s_{n-1} + zeta'_{n+1}/s_{n+1} at one row for the lane's KC
-// poles (the inputs carry the row's real factors), and l, from the row's stage and the next;
-// s: the lane's state
+// poles (the inputs carry the row's real factors), and l, from the row's stage and the next
 template <int KC>
 __device__ __forceinline__ void right_hand_sides(const char *stage, const char *next, const char *inv_alpha, int e0,
-                                                 const int (&one)[2], int s, int lane, double2 (&r)[2], double2 (&l)[2]) {
+                                                 const int (&one)[2], int lane, double2 (&r)[2], double2 (&l)[2]) {
   int4 in[4];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) in[j] = reinterpret_cast<const int4 *>(stage + kSIn)[s * 4 + j];
-  const int e = reinterpret_cast<const int *>(stage + kSU)[s] + e0 - 57;
+  for (int j = 0; j < 4; ++j) in[j] = reinterpret_cast<const int4 *>(stage + kSIn)[j];
+  const int e = *reinterpret_cast<const int *>(stage + kSU) + e0 - 57;
 #pragma unroll
   for (int c = 0; c < KC; ++c) {
     // delta: its weight 1 is one limb (0 past the last pole)
@@ -123,17 +122,16 @@ __device__ __forceinline__ void right_hand_sides(const char *stage, const char *
   }
 }
 
-// The window's sums over the lanes of each state of u = (beta/d') x, u/alpha, u/s_{n+1} and
+// The window's sums over the lanes of u = (beta/d') x, u/alpha, u/s_{n+1} and
 // u/s_{n-1}, x a row's solutions: returns the one of the eight (stream, part) values that this lane
 // ends up with (index: see sum_index).  prev: the stage of the row before (n + 2); be: the
 // exponents of beta/d'; fine: the bits by which the block's reciprocals are below 2^e0; sexp: the
 // exponent of the lane's stream.  beta, 1/d' and x vary over the poles by some bits each and not
 // together, so each pole's u has an exponent of its own and the window's unit is that of its
 // largest u.
-template <int SB, int KC>
+template <int KC>
 __device__ __forceinline__ double weighted_sums(const char *stage, const char *prev, const char *inv_alpha,
                                                 const int (&be)[2], int fine, int sexp, const double2 (&x)[2], int lane) {
-  constexpr int LPS = 32 / SB;  // lanes per state
   long long ur[2], ui[2];
   int eu[2], E = -(1 << 20);
 #pragma unroll
@@ -149,7 +147,7 @@ __device__ __forceinline__ double weighted_sums(const char *stage, const char *p
     ui[c] = ih + (il >> 30);
   }
 #pragma unroll
-  for (int o = 1; o < LPS; o <<= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
+  for (int o = 1; o < 32; o <<= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
   // sums over up to 64 poles of numbers below 2^59: kept in units of 2^3
   long long hh[8], hl[8], t[8];
   t[0] = t[1] = 4;
@@ -172,7 +170,7 @@ __device__ __forceinline__ double weighted_sums(const char *stage, const char *p
   for (int j = 0; j < 8; ++j) t[j] = (j < 2 ? t[j] : (hh[j] << fine) + (hl[j] >> (30 - fine)) + 4) >> 3;
   int n = 8;
 #pragma unroll
-  for (int o = LPS / 2; o > 0; o >>= 1) {
+  for (int o = 32 / 2; o > 0; o >>= 1) {
     if (n > 1) {  // keep one half of the values, add the partner's
       n >>= 1;
       const bool up = lane & o;
@@ -190,38 +188,33 @@ __device__ __forceinline__ double weighted_sums(const char *stage, const char *p
 }
 
 // the value a lane holds after weighted_sums (2 stream + part), -1 for lanes that repeat another's
-template <int SB>
 __device__ __forceinline__ int sum_index(int lane) {
-  constexpr int LPS = 32 / SB;
-  const int k = lane & (LPS - 1), rest = LPS / 8;
-  return (k & (rest - 1)) ? -1 : k / rest;
+  return lane & 3 ? -1 : lane >> 2;
 }
 
-template <int SB, int KC>
-__device__ void sweep_window(const LimbSweep &a, int sysid, int64_t row0, int len, int p0, int b0, int idx, double *part,
+template <int KC>
+__device__ void sweep_window(const LimbSweep &a, int sysid, int64_t row0, int len, int p0, int b, int idx, double *part,
                              bool first, double2 *yb, char *smem, int lane) {
-  constexpr int LPS = 32 / SB;
-  const int k = lane & (LPS - 1), s = lane / LPS, blk = p0 / kBlock, pk = p0 % kBlock + k;
+  const int blk = p0 / kBlock, pk = p0 % kBlock + lane;
   const int64_t rec = row0 * a.nblk + (int64_t)blk * len;
   const char *inv0 = a.inv + ((row0 + sysid) * a.nblk + (int64_t)blk * (len + 1)) * kRec + pk * 16;
   const unsigned sm = (unsigned)__cvta_generic_to_shared(smem);
   const char *ia = smem + kInvAlpha;
   {  // forward: y_i = r_i - l y_{i-1}; row i + 1's r is formed beside the FMAs of row i
     const char *f = a.fwd + rec * kRec + pk * 16, *inv = inv0;
-    const int4 *dig = a.dig + (row0 * a.B + b0) * 4;
-    const int *uexp = a.uexp + row0 * a.B + b0;
-    const int ns = min(SB, a.B - b0);  // states with inputs of their own
+    const int4 *dig = a.dig + (row0 * a.B + b) * 4;
+    const int *uexp = a.uexp + row0 * a.B + b;
     int j = 0;                         // next stage to copy, 0..len
     auto issue = [&]() {
       if (j <= len) {
         const unsigned to = sm + (j & 3) * kStage;
 #pragma unroll
-        for (int c = 0; c < KC; ++c) copy_async<16>(to + (c * 32 + lane) * 16, inv + c * LPS * 16);
+        for (int c = 0; c < KC; ++c) copy_async<16>(to + (c * 32 + lane) * 16, inv + c * 32 * 16);
         if (j < len) {
 #pragma unroll
-          for (int c = 0; c < KC; ++c) copy_async<16>(to + ((2 + c) * 32 + lane) * 16, f + c * LPS * 16);
-          if (lane < 4 * ns) copy_async<16>(to + kSIn + lane * 16, dig + lane);
-          else if (lane >= 16 && lane < 16 + ns) copy_async<4>(to + kSU + (lane - 16) * 4, uexp + lane - 16);
+          for (int c = 0; c < KC; ++c) copy_async<16>(to + ((2 + c) * 32 + lane) * 16, f + c * 32 * 16);
+          if (lane < 4) copy_async<16>(to + kSIn + lane * 16, dig + lane);
+          else if (lane == 4) copy_async<4>(to + kSU, uexp);
         }
         inv += kRec;
         f += kRec;
@@ -233,12 +226,11 @@ __device__ void sweep_window(const LimbSweep &a, int sysid, int64_t row0, int le
     };
     __syncwarp();  // every lane has read the stages of the window before
 #pragma unroll
-    for (int c = 0; c < KC; ++c) copy_async<16>(sm + kInvAlpha + (c * 32 + lane) * 16, a.inv_alpha + p0 + k + c * LPS);
+    for (int c = 0; c < KC; ++c) copy_async<16>(sm + kInvAlpha + (c * 32 + lane) * 16, a.inv_alpha + p0 + lane + c * 32);
     issue();
     issue();
     issue();
-    const int mine = min(s, ns - 1);
-    const int one[2] = {p0 + k < a.P ? 1 << (28 - a.e0) : 0, p0 + k + LPS < a.P ? 1 << (28 - a.e0) : 0};
+    const int one[2] = {p0 + lane < a.P ? 1 << (28 - a.e0) : 0, p0 + lane + 32 < a.P ? 1 << (28 - a.e0) : 0};
     double2 *yp = yb;
     double2 y[2] = {make_double2(0, 0), make_double2(0, 0)}, r[2], l[2];
     for (int i = 0; i <= len; ++i) {
@@ -250,7 +242,7 @@ __device__ void sweep_window(const LimbSweep &a, int sysid, int64_t row0, int le
         copy_wait<1>();
         __syncwarp();  // stages i and i + 1 have landed for every lane; i - 1 has been read
         issue();
-        right_hand_sides<KC>(smem + (i & 3) * kStage, smem + ((i + 1) & 3) * kStage, ia, a.e0, one, mine, lane, r, l);
+        right_hand_sides<KC>(smem + (i & 3) * kStage, smem + ((i + 1) & 3) * kStage, ia, a.e0, one, lane, r, l);
       }
       if (i > 0) {
 #pragma unroll
@@ -265,18 +257,18 @@ __device__ void sweep_window(const LimbSweep &a, int sysid, int64_t row0, int le
     const int fine = min(a.e0 - __ldg(a.eblk + blk), 8), sexp = idx > 1 ? a.e0 - fine - 51 : -53;
     int be[2], bn[2];
 #pragma unroll
-    for (int c = 0; c < KC; ++c) be[c] = bn[c] = __ldg(we + c * LPS);
+    for (int c = 0; c < KC; ++c) be[c] = bn[c] = __ldg(we + c * 32);
     int j = len;  // next stage to copy, len..0; the lane's own copies only
     auto issue = [&]() {
       if (j >= 0) {
         const unsigned to = sm + (j & 3) * kStage + lane * 16;
 #pragma unroll
-        for (int c = 0; c < KC; ++c) copy_async<16>(to + c * 512, inv + c * LPS * 16);
+        for (int c = 0; c < KC; ++c) copy_async<16>(to + c * 512, inv + c * 32 * 16);
         if (j < len) {
 #pragma unroll
           for (int c = 0; c < KC; ++c) {
-            copy_async<16>(to + (KC + c) * 512, f + c * LPS * 16);
-            copy_async<16>(to + (2 * KC + c) * 512, f + kRec + c * LPS * 16);
+            copy_async<16>(to + (KC + c) * 512, f + c * 32 * 16);
+            copy_async<16>(to + (2 * KC + c) * 512, f + kRec + c * 32 * 16);
           }
           f -= kBwd;
         }
@@ -305,7 +297,7 @@ __device__ void sweep_window(const LimbSweep &a, int sysid, int64_t row0, int le
       we = reinterpret_cast<const int *>(reinterpret_cast<const char *>(we) - kBwd);
       if (i > 0) {
 #pragma unroll
-        for (int c = 0; c < KC; ++c) bn[c] = __ldg(we + c * LPS);
+        for (int c = 0; c < KC; ++c) bn[c] = __ldg(we + c * 32);
       }
       copy_wait<1>();  // stages i + 1 and i
       issue();         // stage i - 2, in the place of i + 2
@@ -316,7 +308,7 @@ __device__ void sweep_window(const LimbSweep &a, int sysid, int64_t row0, int le
         xn[c] = cfms(y[c], reinterpret_cast<const double2 *>(stage)[(KC + c) * 32 + lane], x[c]);
         if (i > 1) y[c] = yp[c * 32 - 128];
       }
-      const double v = weighted_sums<SB, KC>(stage, smem + ((i + 1) & 3) * kStage, ia, be, fine, sexp, x, lane);
+      const double v = weighted_sums<KC>(stage, smem + ((i + 1) & 3) * kStage, ia, be, fine, sexp, x, lane);
       if (idx >= 0) *part = sum + v;
       part -= a.B * 8;
       yp -= 64;
@@ -329,21 +321,18 @@ __device__ void sweep_window(const LimbSweep &a, int sysid, int64_t row0, int le
   }
 }
 
-// One item: {system, tile, first window | windows << 16, slot}; yb: the lane's place in the warp's
+// One item: {system, state, first window | windows << 16, slot}; yb: the lane's place in the warp's
 // sweep buffer, smem: the warp's stages.
-template <int SB>
 __device__ __forceinline__ void limb_item(const LimbSweep &a, int4 item, int lane, double2 *yb, char *smem) {
-  constexpr int LPS = 32 / SB;
-  const int per = a.kc * LPS;  // poles per window
+  const int per = a.kc * 32;  // poles per window
   const int4 sy = a.sys[item.x];
   const int w0 = item.z & 0xffff, w1 = w0 + (item.z >> 16);
-  // lanes of a state past the batch repeat the last one and write nothing
-  const int b0 = item.y * SB, state = b0 + lane / LPS, idx = state < a.B ? sum_index<SB>(lane) : -1;
-  double *part = a.part + (((int64_t)item.w * a.nrows + sy.w) * a.B + min(state, a.B - 1)) * 8;
+  const int b = item.y, idx = sum_index(lane);
+  double *part = a.part + (((int64_t)item.w * a.nrows + sy.w) * a.B + b) * 8;
   for (int w = w0; w < w1; ++w) {
     const int p0 = w * per;
-    if (a.kc == 2 && p0 + LPS < a.P) sweep_window<SB, 2>(a, item.x, sy.w, sy.z, p0, b0, idx, part, w == w0, yb, smem, lane);
-    else sweep_window<SB, 1>(a, item.x, sy.w, sy.z, p0, b0, idx, part, w == w0, yb, smem, lane);
+    if (a.kc == 2 && p0 + 32 < a.P) sweep_window<2>(a, item.x, sy.w, sy.z, p0, b, idx, part, w == w0, yb, smem, lane);
+    else sweep_window<1>(a, item.x, sy.w, sy.z, p0, b, idx, part, w == w0, yb, smem, lane);
   }
 }
 
@@ -351,14 +340,12 @@ __device__ __forceinline__ void limb_item(const LimbSweep &a, int4 item, int lan
 // hide a row's chain (1800 cycles where one warp does all of it): one warp carries the two
 // recurrences, 4 FP64 FMAs per row, the others form the right-hand sides and the sums of three
 // rows at a time beside it, both through shared memory.  The arithmetic and the order of the
-// sums are those of sweep_window.  role: 0 for the recurrences; smem: the CTA's stages; mine: this
-// warp's among them; rows: the recurrences' warp's, [2][3 rows][32].
+// sums are those of sweep_window.  role: 0 for the recurrences; ring: the warp's stages; rows: in
+// those of the recurrences' warp, [2][3 rows][32].
 constexpr int kRowsAhead = 3;
-template <int SB>
-__device__ void sweep_window_split(const LimbSweep &a, int sysid, int64_t row0, int len, int p0, int b0, int idx, double *part,
+inline __device__ void sweep_window_split(const LimbSweep &a, int sysid, int64_t row0, int len, int p0, int b, int idx, double *part,
                                    bool first, double2 *yb, char *ring, double2 *rows, int role, int lane) {
-  constexpr int LPS = 32 / SB;
-  const int k = lane & (LPS - 1), s = lane / LPS, blk = p0 / kBlock, pk = p0 % kBlock + k;
+  const int blk = p0 / kBlock, pk = p0 % kBlock + lane;
   const int64_t rec = row0 * a.nblk + (int64_t)blk * len;
   const char *inv = a.inv + ((row0 + sysid) * a.nblk + (int64_t)blk * (len + 1)) * kRec + pk * 16;
   const int chunks = (len + kRowsAhead - 1) / kRowsAhead;
@@ -414,7 +401,7 @@ __device__ void sweep_window_split(const LimbSweep &a, int sysid, int64_t row0, 
   }
   const unsigned sm = (unsigned)__cvta_generic_to_shared(ring);
   const char *ia = ring + kInvAlpha;
-  const int ns = min(SB, a.B - b0), mine = min(s, ns - 1), c0 = role - 1;
+  const int c0 = role - 1;
   // two stages per row (its own factors, and 1/s of the row after), the next row's being copied
   auto issue = [&](int i, int set) {
     if (i >= 0 && i < len) {
@@ -427,15 +414,15 @@ __device__ void sweep_window_split(const LimbSweep &a, int sysid, int64_t row0, 
     issue(i, set);
     if (i < len) {
       const unsigned to = sm + 2 * set * kStage;
-      const int64_t st = (row0 + i) * a.B + b0;
-      if (lane < 4 * ns) copy_async<16>(to + kSIn + lane * 16, a.dig + st * 4 + lane);
-      else if (lane >= 16 && lane < 16 + ns) copy_async<4>(to + kSU + (lane - 16) * 4, a.uexp + st + lane - 16);
+      const int64_t st = (row0 + i) * a.B + b;
+      if (lane < 4) copy_async<16>(to + kSIn + lane * 16, a.dig + st * 4 + lane);
+      else if (lane == 4) copy_async<4>(to + kSU, a.uexp + st);
     }
     copy_commit();
   };
-  const int one[2] = {p0 + k < a.P ? 1 << (28 - a.e0) : 0, 0};
+  const int one[2] = {p0 + lane < a.P ? 1 << (28 - a.e0) : 0, 0};
   __syncwarp();  // every lane has read the stages of the window before
-  copy_async<16>(sm + kInvAlpha + lane * 16, a.inv_alpha + p0 + k);
+  copy_async<16>(sm + kInvAlpha + lane * 16, a.inv_alpha + p0 + lane);
   issue_inputs(c0, 0);
   for (int t = 0; t < chunks; ++t) {
     const int i = kRowsAhead * t + c0;
@@ -445,7 +432,7 @@ __device__ void sweep_window_split(const LimbSweep &a, int sysid, int64_t row0, 
     if (i < len) {
       double2 r[2], l[2];
       const char *stage = ring + 2 * (t & 1) * kStage;
-      right_hand_sides<1>(stage, stage + kStage, ia, a.e0, one, mine, lane, r, l);
+      right_hand_sides<1>(stage, stage + kStage, ia, a.e0, one, lane, r, l);
       *at(t, c0) = r[0];
     }
     __syncthreads();
@@ -475,7 +462,7 @@ __device__ void sweep_window_split(const LimbSweep &a, int sysid, int64_t row0, 
     if (i >= 0) {
       const double2 x[2] = {*at(t, c0), make_double2(0, 0)};
       const char *stage = ring + 2 * (t & 1) * kStage;
-      const double v = weighted_sums<SB, 1>(stage, stage + kStage, ia, be, fine, sexp, x, lane);
+      const double v = weighted_sums<1>(stage, stage + kStage, ia, be, fine, sexp, x, lane);
       if (idx >= 0) *p = sum + v;
     }
   }
@@ -483,16 +470,14 @@ __device__ void sweep_window_split(const LimbSweep &a, int sysid, int64_t row0, 
 }
 
 // One item by a CTA of four warps (kc 3); smem: the CTA's stages
-template <int SB>
 __device__ __forceinline__ void limb_item_split(const LimbSweep &a, int4 item, int lane, int warp, int lead, double2 *yb,
                                                 char *smem) {
-  constexpr int LPS = 32 / SB;
   const int4 sy = a.sys[item.x];
   const int w0 = item.z & 0xffff, w1 = w0 + (item.z >> 16);
-  const int b0 = item.y * SB, state = b0 + lane / LPS, idx = state < a.B ? sum_index<SB>(lane) : -1;
-  double *part = a.part + (((int64_t)item.w * a.nrows + sy.w) * a.B + min(state, a.B - 1)) * 8;
+  const int b = item.y, idx = sum_index(lane);
+  double *part = a.part + (((int64_t)item.w * a.nrows + sy.w) * a.B + b) * 8;
   for (int w = w0; w < w1; ++w)
-    sweep_window_split<SB>(a, item.x, sy.w, sy.z, w * LPS, b0, idx, part, w == w0, yb, smem + warp * kSmemWarp,
+    sweep_window_split(a, item.x, sy.w, sy.z, w * 32, b, idx, part, w == w0, yb, smem + warp * kSmemWarp,
                            reinterpret_cast<double2 *>(smem + lead * kSmemWarp), (warp - lead) & 3, lane);
 }
 

@@ -96,7 +96,7 @@ void free_plan(Plan *pl);
 
 // The smallest batch the digit solve takes by default: its warps carry tiles of eight states;
 // five of them still take a third of the pole-slot solve's time (T85: 0.18 / 0.62 ms).  Plans of
-// up to four states use the limb solve (T170, four states: 0.80 ms against 2.08 fused).  Then the
+// up to four states use the limb solve (T170, four states: 0.81 ms against 2.08 fused).  Then the
 // most device memory either's factors may take: 156 and 68 B per row and pole beside the
 // binary64 factors' 144.
 constexpr int kDigitMinBatch = 5;

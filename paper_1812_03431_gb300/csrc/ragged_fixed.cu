@@ -1,6 +1,6 @@
-// Ragged batches with the fixed-point solves: one persistent launch over the merged items of
-// every plan, each item swept as its plan's own step would (solve_digits.cu above four states,
-// solve_limbs.cu for plans of up to four).  Before it each plan's inputs are put into fixed
+// Ragged batches with the fixed-point solves: a persistent launch over the merged items of every
+// plan of a kind (solve_digits.cu above four states, solve_limbs.cu for plans of up to four), each
+// item swept as its plan's own step would.  Before it each plan's inputs are put into fixed
 // point, after it each plan's slots are summed.
 #include <cuda_runtime.h>
 
@@ -22,7 +22,7 @@ LimbSweep limb_sweep(Plan &pl, const DigitLayout &L, bool adjoint, int B);
 namespace {
 
 struct View {
-  int states;  // per warp: 8 digits, 1, 2 or 4 limbs
+  int states;  // per warp: 8 digits, 1 limbs
   union {
     DigitSweep d;
     LimbSweep l;
@@ -32,15 +32,7 @@ constexpr int kCtas = 4;
 constexpr int kViewBytes = (sizeof(View) + 15) / 16 * 16;
 constexpr int kWarpBytes = limb_solve::kSmemWarp + kViewBytes;
 
-// Not inlined: the sweeps side by side in one body spill (3 % slower).
-__device__ __noinline__ void sweep_digits(const DigitSweep &a, int4 item, int lane, double2 *yb, char *smem) {
-  digit_solve::digit_item(a, item, lane, yb, smem);
-}
-template <int SB>
-__device__ __noinline__ void sweep_limbs(const LimbSweep &a, int4 item, int lane, double2 *yb, char *smem) {
-  limb_solve::limb_item<SB>(a, item, lane, yb, smem);
-}
-
+template <bool DIGITS>
 __global__ void __launch_bounds__(128, kCtas)
     ragged_fixed_kernel(const View *views, const int4 *items, const int *plan_of, int nitems, unsigned *counter, double2 *ybuf,
                         int lmax) {
@@ -65,12 +57,8 @@ __global__ void __launch_bounds__(128, kCtas)
       have = p;
     }
     const int4 item = items[it];
-    switch (view->states) {
-      case 8: sweep_digits(view->d, item, lane, yb, smem); break;
-      case 4: sweep_limbs<4>(view->l, item, lane, yb, smem); break;
-      case 2: sweep_limbs<2>(view->l, item, lane, yb, smem); break;
-      default: sweep_limbs<1>(view->l, item, lane, yb, smem); break;
-    }
+    if constexpr (DIGITS) digit_solve::digit_item(view->d, item, lane, yb, smem);
+    else limb_solve::limb_item(view->l, item, lane, yb, smem);
   }
 }
 
@@ -84,19 +72,19 @@ void free_fixed_ragged(FixedRagged &R) {
 
 // False where a plan has no fixed-point factors, or where the tiles' padding makes the fused
 // solve the cheaper one: per row and pole a digit tile costs about 8 x 12 FP64 FMAs' time
-// whatever its states, a limb tile 14 per state it has room for, the fused solve 39 per state
+// whatever its states, limbs 14 per state, the fused solve 39 per state
 // (T170: 8 states 1.25 ms, 4 states 0.80, fused 0.52 per state).
 bool build_fixed_ragged(const std::vector<Plan *> &plans, const std::vector<int> &counts, FixedRagged &R) {
   R = FixedRagged{};
   double fixed_cost = 0, fused_cost = 0, work[9] = {};  // per kind: states per warp
-  auto kind = [&](size_t p) { return plans[p]->limbs ? limb_tile(counts[p]) : 8; };
+  auto kind = [&](size_t p) { return plans[p]->limbs ? 1 : 8; };
   for (size_t p = 0; p < plans.size(); ++p) {
     const int c = counts[p];
     if (c == 0) continue;
     const Plan &pl = *plans[p];
     if (!pl.dig_fwd.fwd || pl.nrows == 0 || (pl.limbs && c > 4)) return false;
     const double rows = (double)pl.nrows * pl.P;
-    fixed_cost += rows * (pl.limbs ? 14.0 * limb_tile(c) : 96.0 * ((c + 7) / 8));
+    fixed_cost += rows * (pl.limbs ? 14.0 * c : 96.0 * ((c + 7) / 8));
     fused_cost += rows * 39.0 * c;
     work[kind(p)] += (double)digit_work(pl, c, 2);
   }
@@ -119,9 +107,10 @@ bool build_fixed_ragged(const std::vector<Plan *> &plans, const std::vector<int>
     else views[p].d = digit_sweep(pl, R.layouts[p], false, c);
     R.lmax = std::max(R.lmax, pl.lmax);
   }
-  // one kind of sweep after the other, longest first within each: warps that run different
-  // sweeps side by side miss the instruction caches (48 states, T63 to T341: 20.6 ms with all
-  // items longest first)
+  // one kind of sweep after the other, in a launch each, longest first within it: warps that run
+  // different sweeps side by side miss the instruction caches (48 states, T63 to T341: 20.6 ms with
+  // all items longest first), and one kernel that calls both spills in either (12.5 ms;
+  // two 11.0)
   std::stable_sort(all.begin(), all.end(), [&](const Tagged &x, const Tagged &y) {
     const int kx = views[x.plan].states, ky = views[y.plan].states;
     return kx != ky ? kx > ky : x.it.work > y.it.work;
@@ -133,14 +122,15 @@ bool build_fixed_ragged(const std::vector<Plan *> &plans, const std::vector<int>
     plan_of.push_back(t.plan);
   }
   R.nitems = (int)items.size();
+  R.ndigits = (int)std::count_if(all.begin(), all.end(), [&](const Tagged &t) { return views[t.plan].states == 8; });
   const size_t n = items.size();
   cudaError_t e = cudaMalloc(&R.views_dev, views.size() * sizeof(View));
   if (e == cudaSuccess) e = cudaMalloc(&R.items_dev, n * (sizeof(int4) + sizeof(int)));
   if (e == cudaSuccess) e = cudaMemcpy(R.views_dev, views.data(), views.size() * sizeof(View), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(R.items_dev, items.data(), n * sizeof(int4), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(R.items_dev + n, plan_of.data(), n * sizeof(int), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(ragged_fixed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * kWarpBytes);
+  for (auto k : {ragged_fixed_kernel<true>, ragged_fixed_kernel<false>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * kWarpBytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
     free_fixed_ragged(R);
@@ -152,18 +142,24 @@ bool build_fixed_ragged(const std::vector<Plan *> &plans, const std::vector<int>
 // every plan's s_in -> s_out; ybuf: [resident warps][lmax of the ragged object][2][32]
 cudaError_t launch_fixed_ragged(const std::vector<Plan *> &plans, const std::vector<int> &counts, const FixedRagged &R,
                                 double2 *ybuf, unsigned *counter, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned), st);
+  cudaError_t e = cudaSuccess;
   int num_sms = 1;
   for (size_t p = 0; p < plans.size() && e == cudaSuccess; ++p) {
     num_sms = std::max(num_sms, plans[p]->num_sms);
     if (counts[p] > 0) e = launch_digit_state(*plans[p], false, plans[p]->s_in, counts[p], nullptr, st);
   }
   if (e != cudaSuccess) return e;
-  const int ctas = std::max(1, std::min(num_sms * kCtas, (R.nitems + 3) / 4));
-  ragged_fixed_kernel<<<(unsigned)ctas, 128, 4 * kWarpBytes, st>>>(
-      static_cast<const View *>(R.views_dev), R.items_dev, reinterpret_cast<const int *>(R.items_dev + R.nitems), R.nitems,
-      counter, ybuf, R.lmax);
-  e = cudaGetLastError();
+  for (int kind = 0; kind < 2 && e == cudaSuccess; ++kind) {
+    const int first = kind == 0 ? 0 : R.ndigits, n = kind == 0 ? R.ndigits : R.nitems - R.ndigits;
+    if (n == 0) continue;
+    e = cudaMemsetAsync(counter, 0, sizeof(unsigned), st);
+    if (e != cudaSuccess) return e;
+    (kind == 0 ? ragged_fixed_kernel<true> : ragged_fixed_kernel<false>)<<<
+        (unsigned)std::min(num_sms * kCtas, (n + 3) / 4), 128, 4 * kWarpBytes, st>>>(
+        static_cast<const View *>(R.views_dev), R.items_dev + first,
+        reinterpret_cast<const int *>(R.items_dev + R.nitems) + first, n, counter, ybuf, R.lmax);
+    e = cudaGetLastError();
+  }
   for (size_t p = 0; p < plans.size() && e == cudaSuccess; ++p)
     if (counts[p] > 0)
       e = launch_finish_digits(*plans[p], R.layouts[p], false, plans[p]->s_in, plans[p]->s_out, counts[p], st);

@@ -347,11 +347,10 @@ size_t digit_state_bytes(const Plan &pl, int B);
 size_t digit_slot_bytes(const Plan &pl, int B);
 cudaError_t build_digit_factors(Plan &pl, bool adjoint, const double2 *fac, DigitFactors &D);
 void free_digit_factors(DigitFactors &D);
-int limb_tile(int B);
-int limb_window(int B, int kc);
+int limb_window(int kc);
 size_t limb_factor_bytes(const Plan &pl);
 size_t limb_state_bytes(const Plan &pl, int B);
-cudaError_t limb_configure(int B, int kc);
+cudaError_t limb_configure(int kc);
 cudaError_t launch_limb_factors(Plan &pl, bool adjoint, const double2 *fac, DigitFactors &D, int *bad);
 cudaError_t launch_limb_state(Plan &pl, bool adjoint, const double2 *sin, int B, unsigned *counter, cudaStream_t st);
 cudaError_t launch_solve_limbs(Plan &pl, const DigitLayout &L, bool adjoint, int B, cudaStream_t st);
@@ -366,7 +365,7 @@ int64_t digit_work(const Plan &pl, int B, int kc);
 struct FixedRagged {
   void *views_dev = nullptr;        // per plan
   int4 *items_dev = nullptr;        // items, then their plans (int each)
-  int nitems = 0, lmax = 0;
+  int nitems = 0, ndigits = 0, lmax = 0;  // the digit solves' items come first
   std::vector<DigitLayout> layouts; // per plan (slots and poles per lane; no work list of its own)
 };
 bool build_fixed_ragged(const std::vector<Plan *> &plans, const std::vector<int> &counts, FixedRagged &R);

@@ -348,10 +348,10 @@ __global__ void digit_finish_kernel(FinishArgs a) {
 constexpr int kCtas = 4;
 
 // states per tile and poles per window of this plan's windowed solve
-int tile_of(const Plan &pl, int B) { return pl.limbs ? limb_tile(B) : kTile; }
-int tiles_of(const Plan &pl, int B) { return (B + tile_of(pl, B) - 1) / tile_of(pl, B); }
+int tile_of(const Plan &pl) { return pl.limbs ? 1 : kTile; }
+int tiles_of(const Plan &pl, int B) { return (B + tile_of(pl) - 1) / tile_of(pl); }
 int windows_of(const Plan &pl, int B, int kc) {
-  const int w = pl.limbs ? limb_window(B, kc) : kWin;
+  const int w = pl.limbs ? limb_window(kc) : kWin;
   return (pl.P + w - 1) / w;
 }
 
@@ -465,7 +465,7 @@ int64_t digit_work(const Plan &pl, int B, int kc) {
 // resident CTA (its barriers cost more than the shorter chains give beyond that): T63 x 1 with 71
 // poles 0.038 against 0.056 ms for one warp, with 279 poles (7.6 windows per SM) 0.047 / 0.068; T127 x
 // 1 with 151 poles (8.4) 0.078 / 0.134, T255 x 1 (17) 0.226 / 0.328; T127 x 1 with 535 poles (29) 0.208 /
-// 0.183, T63 x 4 with 279 (29) 0.135 / 0.115.  Otherwise one pole per lane halves a warp's chain of
+// 0.183, T63 x 4 with 279 (30) 0.119 / 0.101.  Otherwise one pole per lane halves a warp's chain of
 // FP64 FMAs per row at 0.7 of the whole row's instructions, which pays where items of two are
 // fewer than 1.6 per resident warp (26 per SM): T170 x 1 with 535 poles 0.266 / 0.360 ms (20 per SM);
 // T128 x 1 with 1047 poles 0.293 / 0.288 (29), T341 x 1 1.14 / 1.09 (40).
@@ -476,7 +476,7 @@ rexi_status build_digit_layout(Plan &pl, int B, int slots, DigitLayout &L) {
     L.kc = std::min(3, slots >> 16);
     auto windows = [&](int kc) { return (int64_t)pl.sys.size() * windows_of(pl, B, kc) * tiles_of(pl, B); };
     if (L.kc == 0) L.kc = windows(3) < 22 * (int64_t)pl.num_sms ? 3 : windows(2) < 26 * (int64_t)pl.num_sms ? 1 : 2;
-    if (limb_configure(B, L.kc) != cudaSuccess) {
+    if (limb_configure(L.kc) != cudaSuccess) {
       cudaGetLastError();
       return REXI_OK;
     }

@@ -21,15 +21,17 @@
 // per pole they agree with the tensor-core solve's to 3e-16, for 4 B per row and pole more.
 //
 // Measured on GB300 (solve with its sums, against the fused FP64 solve): T341, 535 poles, one state
-// 0.82 / 2.10 ms, four states 3.15 / 8.12; T170 x 1 0.27 / 0.56, T128 x 1 with 1047 poles 0.29 / 0.61,
+// 0.82 / 2.10 ms, four states 3.11 / 8.12; T170 x 1 0.26 / 0.56, T128 x 1 with 1047 poles 0.28 / 0.61,
 // T639 x 1 2.77 / 7.87 (slot solve), T63 x 1 with 279 poles 0.047 / 0.089.  With every factor of a
 // row stored (148 B per row and pole) one state waited on HBM: T639 3.05 ms, T341 0.91.  Now the
 // integer pipe is 59 % and the FP64 unit 57 % busy (ncu, T341 x 1) and the rest is latency.  Small
 // truncations waited on the row-to-row chain of their few warps (T63 0.066 ms): there a CTA's four
 // warps share a window (sweep_window_split).
 //
-// Lanes of a warp are (state, pole): SB states x 32 / SB poles, two poles per lane where the
-// window is full (poles k and k + 32 / SB), one for a short last window.
+// Lanes of a warp are poles of one state: two per lane where the window is full (poles k and
+// k + 32), one for a short last window.  Two or four states by a warp's lanes, which read each
+// factor once for them, were no faster (T341 x 4 3.18 / 3.14 ms, T170 x 4 0.86 / 0.83, T42 x 4 0.053 /
+// 0.055) and padded three states to four (T341 x 3 3.13 / 2.38, T170 x 3 0.82 / 0.63).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -170,8 +172,10 @@ __global__ void limb_state_kernel(StateArgs a) {
 }
 
 // ---- per step: the sweeps (limb_sweep.h) ----------------------------------------------------------
-template <int SB, int CTAS>
-__global__ void __launch_bounds__(128, CTAS) solve_limbs_kernel(LimbSweep a) {
+// resident CTAs of four warps per SM
+constexpr int kCtas = 4;
+
+__global__ void __launch_bounds__(128, kCtas) solve_limbs_kernel(LimbSweep a) {
   const int lane = threadIdx.x & 31;
   const int wslot = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   double2 *yb = a.ybuf + (int64_t)wslot * a.lmax * 64 + lane;
@@ -182,16 +186,12 @@ __global__ void __launch_bounds__(128, CTAS) solve_limbs_kernel(LimbSweep a) {
     if (lane == 0) it = atomicAdd(a.counter, 1u);
     it = __shfl_sync(0xffffffffu, it, 0);
     if (it >= (unsigned)a.nitems) break;
-    limb_item<SB>(a, a.items[it], lane, yb, smem);
+    limb_item(a, a.items[it], lane, yb, smem);
   }
 }
 
-// resident CTAs of four warps per SM
-constexpr int kCtas = 4;
-
 // The recurrences' warp differs between an SM's CTAs (blocks fill the SMs in turn), so that
 // each scheduler's FP64 unit gets one of the four.
-template <int SB>
 __global__ void __launch_bounds__(128, kCtas) solve_limbs_split_kernel(LimbSweep a) {
   __shared__ unsigned next;
   extern __shared__ __align__(16) char stages[];
@@ -202,31 +202,20 @@ __global__ void __launch_bounds__(128, kCtas) solve_limbs_split_kernel(LimbSweep
     __syncthreads();
     const unsigned it = next;
     if (it >= (unsigned)a.nitems) break;
-    limb_item_split<SB>(a, a.items[it], lane, warp, lead, yb, stages);
+    limb_item_split(a, a.items[it], lane, warp, lead, yb, stages);
   }
 }
 
-}  // namespace
-
-int limb_tile(int B) { return B >= 3 ? 4 : B; }                    // states per warp
-
-namespace {
-void (*kernel_for(int B, bool split))(LimbSweep) {
-  switch (limb_tile(B)) {
-    case 1: return split ? solve_limbs_split_kernel<1> : solve_limbs_kernel<1, kCtas>;
-    case 2: return split ? solve_limbs_split_kernel<2> : solve_limbs_kernel<2, kCtas>;
-    default: return split ? solve_limbs_split_kernel<4> : solve_limbs_kernel<4, kCtas>;
-  }
-}
 }  // namespace
 
 // raises the kernel's shared-memory limit, when a layout is built
-cudaError_t limb_configure(int B, int kc) {
-  return cudaFuncSetAttribute(kernel_for(B, kc == 3), cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * kSmemWarp);
+cudaError_t limb_configure(int kc) {
+  return cudaFuncSetAttribute(kc == 3 ? solve_limbs_split_kernel : solve_limbs_kernel,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * kSmemWarp);
 }
 
 // poles per window: kc per lane; 3: one per lane, a CTA per window
-int limb_window(int B, int kc) { return (kc == 2 ? 2 : 1) * 32 / limb_tile(B); }
+int limb_window(int kc) { return kc == 2 ? 64 : 32; }
 namespace {
 int blocks_of(const Plan &pl) { return (pl.P + kBlock - 1) / kBlock; }
 size_t inv_bytes(const Plan &pl) { return (size_t)(pl.nrows + (int64_t)pl.sys.size()) * blocks_of(pl) * kRec; }
@@ -329,7 +318,7 @@ LimbSweep limb_sweep(Plan &pl, const DigitLayout &L, bool adjoint, int B) {
 cudaError_t launch_solve_limbs(Plan &pl, const DigitLayout &L, bool adjoint, int B, cudaStream_t st) {
   const bool split = L.kc == 3;
   const unsigned ctas = (unsigned)std::max(1, std::min(pl.num_sms * kCtas, split ? L.nitems : (L.nitems + 3) / 4));
-  kernel_for(B, split)<<<ctas, 128, 4 * kSmemWarp, st>>>(limb_sweep(pl, L, adjoint, B));
+  (split ? solve_limbs_split_kernel : solve_limbs_kernel)<<<ctas, 128, 4 * kSmemWarp, st>>>(limb_sweep(pl, L, adjoint, B));
   return cudaGetLastError();
 }
 

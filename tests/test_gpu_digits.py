@@ -139,7 +139,7 @@ def test_values_that_are_not_finite_stay_in_their_state_and_order(env, value, B,
     plan.close()
 
 
-# rows around chunks of three, poles around windows of 32, 16 and 8, a part-filled state tile
+# rows around chunks of three, poles around windows of 32, one to four states
 @pytest.mark.parametrize("N,P,B", [(1, 1, 1), (2, 32, 1), (3, 33, 1), (5, 64, 1), (7, 65, 1), (13, 100, 1), (63, 149, 1),
                                    (5, 16, 2), (13, 33, 2), (5, 9, 3), (21, 31, 4), (31, 57, 3)])
 def test_windows_shared_by_a_block(env, N, P, B):
