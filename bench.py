@@ -117,7 +117,7 @@ def solve_flops_per_row(shape, batch):
     """FP64 work per (state, pole, row) of a binary64 solve layout."""
     if shape != 5:
         return FLOPS_PER_ROW
-    return DIGIT_FLOPS_PER_ROW if batch > 4 else LIMB_FLOPS_PER_ROW
+    return DIGIT_FLOPS_PER_ROW if batch > 5 else LIMB_FLOPS_PER_ROW
 
 
 def kernel_rooflines(form, stages, slots, sm_mhz, solve_arith="fp64", fp64_peak=None, shape=None):
@@ -623,7 +623,7 @@ def main():
         # and read once: B x NG x rows x 4 streams x 16 bytes each way
         traffic += 2 * B * groups * rows_of(W["N"]) * 64
     if r["shape"] == 5 and r["solve_arith"] == "fp64":
-        kname = "solve_digits_kernel (FP64 recurrences; right-hand sides and pole sums as digit products)" if B > 4 \
+        kname = "solve_digits_kernel (FP64 recurrences; right-hand sides and pole sums as digit products)" if B > 5 \
             else "solve_limbs_kernel (FP64 recurrences; right-hand sides and pole sums in integer limbs)"
         traffic = None  # not captured at this size
     if fused:

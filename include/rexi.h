@@ -127,7 +127,7 @@ typedef struct {
                            memory per row and pole, at most 32 GiB and a third of what is
                            free) and the poles are of like scale, except for batches of one and
                            two (below 400,000 rows times poles: up to four) states in plans
-                           with max_batch >= 5; else for up to four
+                           with max_batch >= 6; else for up to four
                            states the fused solve that keeps the pole sum on chip (one
                            kernel, every output written once), else the pole-slot solve
                            (rexi_tune picks per batch); > 0: the pole-slot solve with this
@@ -288,7 +288,7 @@ rexi_status rexi_tune(rexi_plan *plan, int32_t batch, int32_t *slots, int32_t *s
  * passes), the last CTA of a tile to finish adding the groups' partial sums in group
  * order, or shape 5 for the fixed-point solve (binary64 delta solver on the rotating sphere:
  * the right-hand sides and the pole sums as exact fixed-point products, on the tensor cores in
- * plans with max_batch >= 5 and in integer limbs in plans of up to four states; slots: the
+ * plans with max_batch >= 6 and in integer limbs in plans of up to five states; slots: the
  * items each system's poles are split over, plus for the limbs 65536 x their packing -- 1 or 2
  * poles per lane, or 3: one, the warps of a CTA sharing each window's rows --, 0: the
  * defaults), or shape 3 for its lean form (three or four CTAs of four warps per SM, fewer
@@ -311,7 +311,7 @@ rexi_status rexi_plan_info(const rexi_plan *plan, int64_t *info, int32_t n);
  * work list of every plan's items sorted longest first (Sec. 5: every (pole, m)
  * system is independent).  With binary64 solves each plan's fixed-point solve (shape 5 of
  * rexi_set_pole_slots) runs where every plan has one and the states fill its tiles well
- * enough: one launch for the plans of five states and more and one for the smaller ones, each
+ * enough: one launch for the plans of six states and more and one for the smaller ones, each
  * plan's inputs prepared before them and its sums put together after them by small kernels.
  * Else the launch is the fused solve:
  * items are (system, tile of 2 states, plan), the pole sum stays on chip and no
@@ -338,7 +338,7 @@ void rexi_ragged_destroy(rexi_ragged *rg);
 /* Optional per-stage timing (no counterpart in the paper): with max_calls > 0 the next max_calls calls of
  * rexi_step / rexi_step_adjoint record CUDA events on their stream around each
  * stage (0 FFT forward, 1 Legendre analysis, 2 banded solve + pole sum,
- * 3 slot reduction (zero with the fused solve, which has none, and in plans of up to four
+ * 3 slot reduction (zero with the fused solve, which has none, and in plans of up to five
  * states, which count it with the solve), 4 Legendre
  * synthesis, 5 FFT inverse, 6/7 layout transposes).  max_calls = 0 turns it off.  rexi_profile_read waits for the
  * recorded events, writes the summed milliseconds per stage to stage_ms[0..n)

@@ -94,11 +94,14 @@ __global__ void alp_tables_kernel(const double *mu_all, int N, int J, double *ta
 
 void free_plan(Plan *pl);
 
-// The smallest batch the digit solve takes by default: its warps carry tiles of eight states;
-// five of them still take a third of the pole-slot solve's time (T85: 0.18 / 0.62 ms).  Plans of
-// up to four states use the limb solve (T170, four states: 0.81 ms against 2.08 fused).  Then the
-// most device memory either's factors may take: 156 and 68 B per row and pole beside the
-// binary64 factors' 144.
+// Plans of up to five states use the limb solve, whose time grows with the states, larger ones the
+// digit solve, whose warps carry tiles of eight: T341 x 5 3.93 against 4.41 ms, T170 x 5 1.01 / 1.16, T85 x
+// 5 with 215 poles 0.154 / 0.165, T42 x 5 0.061 / 0.076; with six states T170 1.20 / 1.17, T85 0.195 /
+// 0.167, T42 0.067 / 0.076.
+constexpr int kLimbMostBatch = 5;
+// The smallest batch of a larger plan for its digit solve (five states take a quarter of the
+// pole-slot solve's time).  Then the most device memory either's factors may take: 156 and 68 B
+// per row and pole beside the binary64 factors' 144.
 constexpr int kDigitMinBatch = 5;
 // Larger plans' batches of three and four: the digit solve, its tiles padded, from this many rows
 // times poles (T63, 279 poles, 0.58 million: three states 0.144 / 0.159 ms, four 0.144 / 0.199; T170 x
@@ -341,7 +344,7 @@ rexi_status build_plan(const rexi_params &prm, Plan *pl) {
   }
 
   // the digit solve's factors, for plans that step batches it serves by default
-  pl->limbs = prm.max_batch < kDigitMinBatch;
+  pl->limbs = prm.max_batch <= kLimbMostBatch;
   if (pl->fac_fwd && !pl->ff && prm.solver == REXI_SOLVER_DELTA) {
     size_t mem_free = 0, mem_total = 0;
     if ((e = cudaMemGetInfo(&mem_free, &mem_total))) return fail("memory", e);

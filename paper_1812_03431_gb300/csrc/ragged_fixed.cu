@@ -1,5 +1,5 @@
 // Ragged batches with the fixed-point solves: a persistent launch over the merged items of every
-// plan of a kind (solve_digits.cu above four states, solve_limbs.cu for plans of up to four), each
+// plan of a kind (solve_limbs.cu for plans of up to five states, solve_digits.cu above), each
 // item swept as its plan's own step would.  Before it each plan's inputs are put into fixed
 // point, after it each plan's slots are summed.
 #include <cuda_runtime.h>
@@ -82,7 +82,7 @@ bool build_fixed_ragged(const std::vector<Plan *> &plans, const std::vector<int>
     const int c = counts[p];
     if (c == 0) continue;
     const Plan &pl = *plans[p];
-    if (!pl.dig_fwd.fwd || pl.nrows == 0 || (pl.limbs && c > 4)) return false;
+    if (!pl.dig_fwd.fwd || pl.nrows == 0 || c > pl.prm.max_batch) return false;
     const double rows = (double)pl.nrows * pl.P;
     fixed_cost += rows * (pl.limbs ? 14.0 * c : 96.0 * ((c + 7) / 8));
     fused_cost += rows * 39.0 * c;

@@ -1,4 +1,4 @@
-// Banded shifted solves of small batches (one to four states) with their two contractions in
+// Banded shifted solves of small batches (one to five states) with their two contractions in
 // exact integer arithmetic (paper Sec. 4.2, Sec. 5, Algorithm 1; binary64 delta solver).
 //
 // As in solve_digits.cu, only the 8 FP64 FMAs per (state, pole, row) of the two recurrences stay

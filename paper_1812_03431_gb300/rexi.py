@@ -314,7 +314,7 @@ class Plan:
         """rexi_set_pole_slots: use this pole-slot count and layout shape (0: the same groups
         for every zonal order, 1: in proportion to the system length) for this batch size,
         or shape 5: the fixed-point solve (``slots``: items per system, 0: default, plus
-        65536 x the packing in plans of up to four states), or shape 2
+        65536 x the packing in plans of up to five states), or shape 2
         (3: its lean form, 4: the lean form on two-warp CTAs): the fused solve with
         ``slots`` states per CTA tile (0: default) and each tile's poles split over ``groups``
         CTAs (0: default).  For shapes 2 to 4 returns tile + 256 x groups as used (``slots``

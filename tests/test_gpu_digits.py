@@ -1,5 +1,5 @@
 """The fixed-point solves (both contractions of the shifted solves exactly: on the tensor cores
-above four states, in integer limbs up to four) against the pole-slot solve, the oracle and its own linearity."""
+above five states, in integer limbs up to five) against the pole-slot solve, the oracle and its own linearity."""
 import numpy as np
 import pytest
 
@@ -38,9 +38,9 @@ def spectral_plan(rexi, N, B, al, be, tau=1800.0, **k):
     return rexi.Plan(N, nlon // 2, nlon, tau=tau, max_batch=B, layout="spectral", alpha=al, beta=be, **k)
 
 
-# truncations down to one row per system; pole counts around a window of eight (above four
-# states) and around 16, 32 and 64 (up to four); batches around a tile of eight states
-@pytest.mark.parametrize("N,P,B", [(1, 1, 5), (1, 9, 8), (2, 7, 9), (3, 8, 5), (8, 16, 16), (13, 17, 7), (21, 31, 17),
+# truncations down to one row per system; pole counts around a window of eight (above five
+# states) and around 32 and 64 (up to five); batches around a tile of eight states
+@pytest.mark.parametrize("N,P,B", [(1, 1, 5), (1, 1, 6), (1, 9, 8), (2, 7, 9), (3, 8, 5), (3, 8, 6), (8, 16, 16), (13, 17, 7), (21, 31, 17),
                                    (42, 57, 8), (63, 149, 6),
                                    (1, 1, 1), (2, 31, 1), (8, 32, 1), (13, 33, 1), (21, 64, 1), (42, 65, 1), (63, 149, 1),
                                    (3, 15, 2), (13, 17, 2), (21, 33, 2), (31, 100, 2), (5, 8, 3), (21, 9, 3), (31, 57, 4),
@@ -50,7 +50,7 @@ def test_matches_slot_solve(env, N, P, B):
     al, be = poles(P)
     x = torch.from_numpy(inputs.random_spectral(N, B, 7)).cuda()
     plan = spectral_plan(rexi, N, B, al, be)
-    got, adj = plan.step(x).cpu().numpy(), plan.step_adjoint(x).cpu().numpy()  # the default above four states
+    got, adj = plan.step(x).cpu().numpy(), plan.step_adjoint(x).cpu().numpy()  # the default
     for slots in (1, 2, 0, 1000):
         assert plan.set_pole_slots(B, slots, 5) >= 1
         y = plan.step(x).cpu().numpy()
@@ -139,9 +139,9 @@ def test_values_that_are_not_finite_stay_in_their_state_and_order(env, value, B,
     plan.close()
 
 
-# rows around chunks of three, poles around windows of 32, one to four states
+# rows around chunks of three, poles around windows of 32, one to five states
 @pytest.mark.parametrize("N,P,B", [(1, 1, 1), (2, 32, 1), (3, 33, 1), (5, 64, 1), (7, 65, 1), (13, 100, 1), (63, 149, 1),
-                                   (5, 16, 2), (13, 33, 2), (5, 9, 3), (21, 31, 4), (31, 57, 3)])
+                                   (5, 16, 2), (13, 33, 2), (5, 9, 3), (21, 31, 4), (31, 57, 3), (8, 40, 5)])
 def test_windows_shared_by_a_block(env, N, P, B):
     """Packing 3 (a block's warps share a window's rows) does the arithmetic of packing 1 in its order."""
     torch, rexi = env
