@@ -520,8 +520,9 @@ rexi_status rexi_plan_info(const rexi_plan *plan, int64_t *info, int32_t n) {
   auto it = pl.layouts.find(pl.prm.max_batch);
   auto us = pl.use_slots.find(pl.prm.max_batch);
   if (it != pl.layouts.end() && us != pl.use_slots.end() && us->second) slots = it->second.slots;
-  const int64_t v[8] = {pl.N, pl.nspec, pl.P, pl.nlat, pl.nlon, pl.prm.max_batch, slots, (int64_t)pl.bytes};
-  for (int i = 0; i < n && i < 8; ++i) info[i] = v[i];
+  const int fixed = !pl.dig_fwd.fwd ? 0 : (pl.limbs ? 1 : 2);
+  const int64_t v[9] = {pl.N, pl.nspec, pl.P, pl.nlat, pl.nlon, pl.prm.max_batch, slots, (int64_t)pl.bytes, fixed};
+  for (int i = 0; i < n && i < 9; ++i) info[i] = v[i];
   return REXI_OK;
 }
 

@@ -289,15 +289,21 @@ class Plan:
         ``self.layout_shape[batch]``).
 
         ``cache``: path of a JSON file of earlier choices keyed by the plan's shape (N,
-        grid, P, batch, precision, solver, solve arithmetic) and the GPU's name; a hit sets the layout
-        without timing (rexi_set_pole_slots), a miss tunes and records the result."""
+        grid, P, batch, largest batch, precision, solver, solve arithmetic), the solves it has to choose
+        from (its fixed-point factors, which depend on max_batch, on the poles' scales and on the
+        memory that was free) and the GPU's name; a hit sets the layout without timing
+        (rexi_set_pole_slots), a miss or an entry that the plan refuses tunes and records the result."""
         key = None
         if cache:
             key = self._tune_key(batch)
             table = _read_json(cache)
             if key in table:
                 slots, shape = table[key]
-                return self.set_pole_slots(batch, int(slots), int(shape))
+                try:
+                    return self.set_pole_slots(batch, int(slots), int(shape))
+                except RexiError as err:
+                    if err.status != REXI_EINVAL:
+                        raise
         n, sh = _I32(), _I32()
         _check("rexi_tune", load().rexi_tune(self._h, batch, ctypes.byref(n), ctypes.byref(sh)))
         self.layout_shape[batch] = sh.value
@@ -330,13 +336,15 @@ class Plan:
         import torch
         i = self.info()
         gpu = torch.cuda.get_device_name(torch.cuda.current_device())
-        return "N%d_%dx%d_P%d_B%d_%s_%s_%s_%s_%s" % (i["N"], i["nlon"], i["nlat"], i["P"], batch, self.precision,
-                                                     self.solver, self.solve_arith, self.layout, gpu)
+        solves = ("binary64", "limbs", "digits")[i["fixed_factors"]]
+        return "N%d_%dx%d_P%d_B%dof%d_%s_%s_%s_%s_%s_%s" % (
+            i["N"], i["nlon"], i["nlat"], i["P"], batch, i["max_batch"], self.precision, self.solver, self.solve_arith,
+            solves, self.layout, gpu)
 
     def info(self):
-        v = (ctypes.c_int64 * 8)()
-        _check("rexi_plan_info", load().rexi_plan_info(self._h, v, 8))
-        keys = ["N", "nspec", "P", "nlat", "nlon", "max_batch", "pole_slots", "device_bytes"]
+        v = (ctypes.c_int64 * 9)()
+        _check("rexi_plan_info", load().rexi_plan_info(self._h, v, 9))
+        keys = ["N", "nspec", "P", "nlat", "nlon", "max_batch", "pole_slots", "device_bytes", "fixed_factors"]
         return dict(zip(keys, list(v)))
 
     def check_device(self):
