@@ -291,7 +291,7 @@ rexi_status rexi_tune(rexi_plan *plan, int32_t batch, int32_t *slots, int32_t *s
  * plans with max_batch >= 6 and in integer limbs in plans of up to five states; slots: the
  * items each system's poles are split over, plus for the limbs 65536 x their packing -- 1 or 2
  * poles per lane, or 3: one, the warps of a CTA sharing each window's rows --, 0: the
- * defaults), or shape 3 for its lean form (three or four CTAs of four warps per SM, fewer
+ * defaults; a packing is REXI_EINVAL in plans with max_batch >= 6), or shape 3 for its lean form (three or four CTAs of four warps per SM, fewer
  * registers, the next rows prefetched into the caches; tiles of up to 8 states), or shape
  * 4 for the lean form on CTAs of two warps (seven or eight per SM; tiles of up to 4
  * states; a tile of 2 states puts each state on a warp of its own, so no CTA splits its

@@ -667,6 +667,10 @@ const FusedLayout *set_fused_tile(Plan &pl, int B, int tile, int form = 0, int g
 // where it does not apply), with slots = tile + 256 x pole groups.
 rexi_status set_layout(Plan &pl, int B, int slots, int shape, int *used) {
   if (shape == 5) {
+    if (slots >> 16 > (pl.limbs ? 3 : 0)) {
+      set_error("rexi_set_pole_slots: shape 5 takes a packing (65536 x 1 to 3) in plans of up to five states only");
+      return REXI_EINVAL;
+    }
     const DigitLayout *D = set_digit_slots(pl, B, slots);
     if (!D) {
       set_error("rexi_set_pole_slots: the digit solve (shape 5) does not apply to this plan");

@@ -473,7 +473,7 @@ rexi_status build_digit_layout(Plan &pl, int B, int slots, DigitLayout &L) {
   L = DigitLayout{};
   if (pl.nrows == 0) return REXI_OK;  // not available
   if (pl.limbs) {
-    L.kc = std::min(3, slots >> 16);
+    L.kc = slots >> 16;
     auto windows = [&](int kc) { return (int64_t)pl.sys.size() * windows_of(pl, B, kc) * tiles_of(pl, B); };
     if (L.kc == 0) L.kc = windows(3) < 22 * (int64_t)pl.num_sms ? 3 : windows(2) < 26 * (int64_t)pl.num_sms ? 1 : 2;
     if (limb_configure(L.kc) != cudaSuccess) {

@@ -187,3 +187,20 @@ def test_small_batches_of_a_larger_plan(env, N, M, B):
     assert fieldwise(plan.step_adjoint(x).cpu().numpy(), slots.step_adjoint(x).cpu().numpy()) < ORDER
     plan.close()
     slots.close()
+
+
+@pytest.mark.parametrize("B,slots", [(8, 65536), (8, 2 * 65536 + 3), (2, 4 * 65536), (2, 7 * 65536 + 1)])
+def test_packings_that_a_plan_does_not_have_are_refused(env, B, slots):
+    """Packings are the limbs' (1 to 3); the layout in use stays."""
+    torch, rexi = env
+    al, be = poles(45)
+    plan = spectral_plan(rexi, 13, B, al, be)
+    x = torch.from_numpy(inputs.random_spectral(13, B, 3)).cuda()
+    used = plan.set_pole_slots(B, 2, 5)
+    y = plan.step(x).cpu().numpy()
+    with pytest.raises(rexi.RexiError) as e:
+        plan.set_pole_slots(B, slots, 5)
+    assert e.value.status == rexi.REXI_EINVAL
+    np.testing.assert_array_equal(plan.step(x).cpu().numpy(), y)
+    assert plan.set_pole_slots(B, used, 5) == used  # what the call returned is taken back
+    plan.close()
