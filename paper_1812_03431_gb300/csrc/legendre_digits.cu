@@ -508,13 +508,20 @@ void free_legendre_digits(LegendreDigits &t) {
   t = LegendreDigits{};
 }
 
-// The tables in fragment order for one direction, from pl.tabP and pl.tabH; t stays empty (and
-// the FP64 kernels of legendre.cu serve the plan) where the device memory does not suffice.
-cudaError_t build_legendre_digits(Plan &pl, bool synthesis, LegendreDigits &t) {
-  t = LegendreDigits{};
+namespace {
+
+// where each system's fragments and exponents lie, for one direction
+struct TabLayout {
   std::vector<int4> sys;
-  int64_t frags = 0, groups = 0, nfrag = 0, nexp = 0;
+  int64_t nfrag = 0, nexp = 0;
   int most = 0;
+  bool ok = true;
+  size_t bytes() const { return (size_t)nfrag * 2 * kFrag + (size_t)nexp * 32 * sizeof(int); }
+};
+
+TabLayout tab_layout(const Plan &pl, bool synthesis) {
+  TabLayout L;
+  int64_t frags = 0, groups = 0;
   const int jt = (pl.J + 15) / 16, jg = (pl.J + kGroup - 1) / kGroup;
   for (int m = 0; m <= pl.N; ++m)
     for (int c = 0; c < 2; ++c) {
@@ -522,17 +529,32 @@ cudaError_t build_legendre_digits(Plan &pl, bool synthesis, LegendreDigits &t) {
       // fragment (k, tile) of the system is at (first + k) tiles + tile: `first` counts in the
       // system's own tiles, so the offset is rounded up to them
       const int tiles = std::max(1, synthesis ? jt : rt), kfr = synthesis ? rt : jt, kg = synthesis ? rg : jg;
-      frags = (nfrag + tiles - 1) / tiles;
-      groups = (nexp + tiles - 1) / tiles;
-      sys.push_back(make_int4(rows, (int)frags, (int)groups, 0));
-      if (frags > INT32_MAX || groups > INT32_MAX) return cudaSuccess;
-      nfrag = (frags + kfr) * tiles;
-      nexp = (groups + kg) * tiles;
-      most = std::max(most, 2 * tiles * kg);
+      frags = (L.nfrag + tiles - 1) / tiles;
+      groups = (L.nexp + tiles - 1) / tiles;
+      L.sys.push_back(make_int4(rows, (int)frags, (int)groups, 0));
+      if (frags > INT32_MAX || groups > INT32_MAX) L.ok = false;
+      L.nfrag = (frags + kfr) * tiles;
+      L.nexp = (groups + kg) * tiles;
+      L.most = std::max(L.most, 2 * tiles * kg);
     }
+  return L;
+}
+
+}  // namespace
+
+// of both directions
+size_t legendre_digit_bytes(const Plan &pl) { return tab_layout(pl, false).bytes() + tab_layout(pl, true).bytes(); }
+
+// The tables in fragment order for one direction, from pl.tabP and pl.tabH; t stays empty (and
+// the FP64 kernels of legendre.cu serve the plan) where the device memory does not suffice.
+cudaError_t build_legendre_digits(Plan &pl, bool synthesis, LegendreDigits &t) {
+  t = LegendreDigits{};
+  const TabLayout L = tab_layout(pl, synthesis);
+  const std::vector<int4> &sys = L.sys;
+  if (!L.ok) return cudaSuccess;
   cudaError_t e = cudaSuccess;
-  if (cudaMalloc(&t.dig, (size_t)nfrag * 2 * kFrag) != cudaSuccess ||
-      cudaMalloc(&t.exps, (size_t)nexp * 32 * sizeof(int)) != cudaSuccess ||
+  if (cudaMalloc(&t.dig, (size_t)L.nfrag * 2 * kFrag) != cudaSuccess ||
+      cudaMalloc(&t.exps, (size_t)L.nexp * 32 * sizeof(int)) != cudaSuccess ||
       cudaMalloc(&t.sys, sys.size() * sizeof(int4)) != cudaSuccess) {
     cudaGetLastError();
     free_legendre_digits(t);
@@ -549,14 +571,14 @@ cudaError_t build_legendre_digits(Plan &pl, bool synthesis, LegendreDigits &t) {
   a.J = pl.J;
   a.synthesis = synthesis;
   if (e == cudaSuccess) {
-    legendre_digits_setup<<<dim3((unsigned)most, (unsigned)sys.size()), 32>>>(a);
+    legendre_digits_setup<<<dim3((unsigned)L.most, (unsigned)sys.size()), 32>>>(a);
     e = cudaGetLastError();
   }
   for (auto k : {legendre_digits_analysis<true>, legendre_digits_analysis<false>, legendre_digits_synthesis<true>,
                  legendre_digits_synthesis<false>})
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   if (e != cudaSuccess) free_legendre_digits(t);
-  t.bytes = (size_t)nfrag * 2 * kFrag + (size_t)nexp * 32 * sizeof(int);
+  t.bytes = L.bytes();
   return e;
 }
 

@@ -111,6 +111,17 @@ constexpr int kDigitMinBatchLarge = 3;
 constexpr int64_t kDigitLarge = 400000;
 constexpr size_t kDigitMostBytes = (size_t)32 << 30;
 
+// Whether a form that a plan can do without may take `need` bytes: a third of what is free, and
+// `keep` bytes must stay.
+bool spare_memory(size_t need, size_t keep) {
+  size_t mem_free = 0, mem_total = 0;
+  if (cudaMemGetInfo(&mem_free, &mem_total) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return need <= std::min(kDigitMostBytes, mem_free / 3) && need + keep <= mem_free;
+}
+
 rexi_status build_plan(const rexi_params &prm, Plan *pl) {
   pl->prm = prm;
   pl->ff = prm.solve_arith == REXI_SOLVE_FP32X2;
@@ -343,23 +354,6 @@ rexi_status build_plan(const rexi_params &prm, Plan *pl) {
     }
   }
 
-  // the digit solve's factors, for plans that step batches it serves by default
-  pl->limbs = prm.max_batch <= kLimbMostBatch;
-  if (pl->fac_fwd && !pl->ff && prm.solver == REXI_SOLVER_DELTA) {
-    size_t mem_free = 0, mem_total = 0;
-    if ((e = cudaMemGetInfo(&mem_free, &mem_total))) return fail("memory", e);
-    const size_t need = digit_factor_bytes(*pl) + digit_state_bytes(*pl, prm.max_batch);
-    if (need <= std::min(kDigitMostBytes, mem_free / 3)) {
-      if ((e = build_digit_factors(*pl, false, pl->fac_fwd, pl->dig_fwd))) return fail("digit factors", e);
-      if (pl->dig_fwd.fwd && cudaMalloc(&pl->dig_state, digit_state_bytes(*pl, prm.max_batch)) != cudaSuccess) {
-        cudaGetLastError();
-        pl->dig_state = nullptr;
-        free_digit_factors(pl->dig_fwd);
-      }
-      if (pl->dig_fwd.fwd) bytes += need;
-    }
-  }
-
   // ---- grid, Legendre tables, FFT
   {  // tables serve the grid layout and rexi_analyze / rexi_synthesize
     std::vector<double> mu, w;
@@ -435,22 +429,7 @@ rexi_status build_plan(const rexi_params &prm, Plan *pl) {
     if ((e = legendre_configure())) return fail("legendre configure", e);
   }
 
-  if (prm.precision == REXI_MIXED) {
-    if ((e = tc_setup(*pl))) return fail("tensor-core tables", e);
-  } else {
-    // the tables as digits, in place of the binary64 ones where both directions fit
-    if ((e = build_legendre_digits(*pl, false, pl->leg_ana))) return fail("Legendre digits", e);
-    if (pl->leg_ana.dig && (e = build_legendre_digits(*pl, true, pl->leg_syn))) return fail("Legendre digits", e);
-    if (pl->leg_syn.dig) {
-      if ((e = cudaDeviceSynchronize())) return fail("Legendre digits", e);
-      cudaFree(pl->tabP);
-      cudaFree(pl->tabH);
-      pl->tabP = pl->tabH = nullptr;
-      bytes += pl->leg_ana.bytes + pl->leg_syn.bytes - 2 * (size_t)NS * pl->J * sizeof(double);
-    } else {
-      free_legendre_digits(pl->leg_ana);
-    }
-  }
+  if (prm.precision == REXI_MIXED && (e = tc_setup(*pl))) return fail("tensor-core tables", e);
 
   // ---- workspaces
   const int B = prm.max_batch;
@@ -465,7 +444,6 @@ rexi_status build_plan(const rexi_params &prm, Plan *pl) {
   cap = std::min(cap, P);
   pl->partial_cap = (size_t)cap;
   pl->partial_elems = (size_t)cap * 3 * NS * B;
-  if (pl->dig_fwd.fwd) pl->partial_elems = std::max(pl->partial_elems, digit_slot_bytes(*pl, B) / sizeof(double2));
   if ((e = dalloc(&pl->partial, pl->partial_elems, &bytes))) return fail("partials", e);
   pl->resident_warps = pl->num_sms * 16;
   // forward-sweep intermediates: sweep_width poles per lane per row
@@ -473,6 +451,46 @@ rexi_status build_plan(const rexi_params &prm, Plan *pl) {
     return fail("scratch", e);
   if ((e = dalloc(&pl->counter, 1, &bytes))) return fail("counter", e);
   pl->slots_override = prm.pole_slots;
+
+  // ---- the fixed-point forms, which a plan can do without: what it needs comes first
+  pl->limbs = B <= kLimbMostBatch;
+  if (pl->fac_fwd && !pl->ff && prm.solver == REXI_SOLVER_DELTA) {
+    const size_t state = digit_state_bytes(*pl, B), need = digit_factor_bytes(*pl) + state;
+    const size_t fac = (size_t)F_NCOMP * pl->nrows * P * sizeof(double2);  // as the adjoint will need
+    if (spare_memory(need, fac) && (e = build_digit_factors(*pl, false, pl->fac_fwd, pl->dig_fwd)))
+      return fail("digit factors", e);
+    // the sums of one slot: more than the buffer of the slot solve only where that holds a single one
+    const size_t sums = digit_slot_bytes(*pl, B) / sizeof(double2);
+    double2 *part = nullptr;
+    if (pl->dig_fwd.fwd && (cudaMalloc(&pl->dig_state, state) != cudaSuccess ||
+                            (sums > pl->partial_elems && cudaMalloc(&part, sums * sizeof(double2)) != cudaSuccess))) {
+      cudaGetLastError();
+      if (pl->dig_state) cudaFree(pl->dig_state);
+      pl->dig_state = nullptr;
+      free_digit_factors(pl->dig_fwd);
+    }
+    if (pl->dig_fwd.fwd) bytes += need;
+    if (part) {
+      cudaFree(pl->partial);
+      bytes += (sums - pl->partial_elems) * sizeof(double2);
+      pl->partial = part;
+      pl->partial_elems = sums;
+    }
+  }
+  if (prm.precision != REXI_MIXED && spare_memory(legendre_digit_bytes(*pl), 0)) {
+    // the Legendre tables as digits, in place of the binary64 ones where both directions fit
+    if ((e = build_legendre_digits(*pl, false, pl->leg_ana))) return fail("Legendre digits", e);
+    if (pl->leg_ana.dig && (e = build_legendre_digits(*pl, true, pl->leg_syn))) return fail("Legendre digits", e);
+    if (pl->leg_syn.dig) {
+      if ((e = cudaDeviceSynchronize())) return fail("Legendre digits", e);
+      cudaFree(pl->tabP);
+      cudaFree(pl->tabH);
+      pl->tabP = pl->tabH = nullptr;
+      bytes += pl->leg_ana.bytes + pl->leg_syn.bytes - 2 * (size_t)NS * pl->J * sizeof(double);
+    } else {
+      free_legendre_digits(pl->leg_ana);
+    }
+  }
   if ((e = cudaDeviceSynchronize())) return fail("setup", e);
   return REXI_OK;
 }

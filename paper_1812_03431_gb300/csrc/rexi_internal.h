@@ -342,6 +342,7 @@ cudaError_t launch_solve_fused(Plan &pl, const FusedLayout &F, bool adjoint, con
                                int B, cudaStream_t st);
 // digit solve (solve_digits.cu): sin -> slot sums in pl.partial, then the ordered sum of the
 // slots with the pole-independent terms
+bool spare_memory(size_t need, size_t keep);
 size_t digit_factor_bytes(const Plan &pl);
 size_t digit_state_bytes(const Plan &pl, int B);
 size_t digit_slot_bytes(const Plan &pl, int B);
@@ -408,6 +409,7 @@ cudaError_t launch_leg_ana(Plan &pl, const double2 *four, double2 *sint, int B,
                            const double *zdscale, cudaStream_t st);
 cudaError_t launch_leg_syn(Plan &pl, const double2 *sint, double2 *four, int B,
                            const double *zdscale, cudaStream_t st);
+size_t legendre_digit_bytes(const Plan &pl);
 cudaError_t build_legendre_digits(Plan &pl, bool synthesis, LegendreDigits &t);
 void free_legendre_digits(LegendreDigits &t);
 cudaError_t launch_leg_ana_digits(Plan &pl, const double2 *four, double2 *sint, int B, const double *zd,
