@@ -125,7 +125,8 @@ typedef struct {
                            the rotating sphere the fixed-point solve (shape 5 of
                            rexi_set_pole_slots) where its factors fit (68 to 156 B of device
                            memory per row and pole, at most 32 GiB and a third of what is
-                           free) and the poles are of like scale, except for batches of one and
+                           free when the plan's workspaces, or for the adjoint its binary64
+                           factors, are allocated) and the poles are of like scale, except for batches of one and
                            two (below 400,000 rows times poles: up to four) states in plans
                            with max_batch >= 6; else for up to four
                            states the fused solve that keeps the pole sum on chip (one

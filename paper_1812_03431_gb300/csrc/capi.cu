@@ -106,6 +106,7 @@ rexi_status ensure_adjoint_factors(Plan &pl) {
   if (pl.fac_adj || pl.prm.fsphere) {
     if (pl.fac_adj && pl.dig_fwd.fwd && !pl.dig_adj_tried) {
       pl.dig_adj_tried = true;
+      if (!spare_memory(digit_factor_bytes(pl), 0)) return REXI_OK;  // as for the forward ones
       cudaError_t e = build_digit_factors(pl, true, pl.fac_adj, pl.dig_adj);
       if (e != cudaSuccess) return cuda_fail("adjoint digit factors", e);
       if (pl.dig_adj.fwd) pl.bytes += digit_factor_bytes(pl);

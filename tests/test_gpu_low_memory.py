@@ -86,3 +86,29 @@ def test_transforms_and_steps_without_any_fixed_point_form(env):
     assert low["fixed_factors"] == 0 and low["device_bytes"] < info["device_bytes"] - tables
     for a, b in zip(got, want):  # sums of up to 192 terms and two transforms: as against the oracle elsewhere
         assert fieldwise(a, b) < 1e-11
+
+
+@pytest.mark.parametrize("B", [8, 2])
+def test_the_adjoint_takes_no_more_than_its_share(env, B):
+    """Room for the adjoint's binary64 factors and as much as its fixed-point ones take: more than a third."""
+    torch, rexi = env
+    N, P = 127, 151
+    al, be, _ = rc.rexi_coefficients(64, 0.2)
+    k = (al.size - P) // 2
+    make = lambda: rexi.Plan(N, 192, 384, tau=1200.0, max_batch=B, layout="spectral", alpha=al[k:k + P], beta=be[k:k + P])  # noqa: E731
+    g = torch.from_numpy(inputs.random_spectral(N, B, 6)).cuda()
+    full = make()
+    want = full.step_adjoint(g).cpu().numpy()
+    with_both = full.info()["device_bytes"]
+    full.close()
+    plan = make()
+    before = plan.info()["device_bytes"]
+    binary64 = 9 * 16 * P * ((N + 1) * (N + 2) // 2 - 1)
+    fixed = with_both - before - binary64
+    assert fixed > 40 * MB
+    out = torch.empty_like(g)
+    with only(torch, binary64 + fixed + 32 * MB):
+        got = plan.step_adjoint(g, out=out).cpu().numpy()
+        assert plan.info()["device_bytes"] - before < binary64 + 2 * MB
+    assert fieldwise(got, want) < ORDER
+    plan.close()
