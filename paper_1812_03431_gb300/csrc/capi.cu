@@ -24,6 +24,7 @@ rexi_status step_static(Plan &pl, const void *in, void *out, int B, cudaStream_t
 rexi_status tune_layout(Plan &pl, int B, int *slots_out, int *shape_out);
 rexi_status set_layout(Plan &pl, int B, int slots, int shape, int *used);
 const FusedLayout *fused_layout(Plan &pl, int B);
+bool digits_chosen(const Plan &pl, int B);
 const DigitLayout *digit_layout(Plan &pl, int B, bool adjoint);
 
 namespace {
@@ -102,27 +103,30 @@ rexi_status check_io2(const Plan &pl, const void *in, const void *out, int B, bo
   return REXI_OK;
 }
 
-rexi_status ensure_adjoint_factors(Plan &pl) {
-  if (pl.fac_adj || pl.prm.fsphere) {
-    if (pl.fac_adj && pl.dig_fwd.fwd && !pl.dig_adj_tried) {
-      pl.dig_adj_tried = true;
-      if (!spare_memory(digit_factor_bytes(pl), 0)) return REXI_OK;  // as for the forward ones
-      cudaError_t e = build_digit_factors(pl, true, pl.fac_adj, pl.dig_adj);
-      if (e != cudaSuccess) return cuda_fail("adjoint digit factors", e);
-      if (pl.dig_adj.fwd) pl.bytes += digit_factor_bytes(pl);
-    }
-    return REXI_OK;
-  }
+// The adjoint's factors, on the first call; in fixed point when a batch of the digit solve first
+// asks for them (the read of their flag waits for both).
+rexi_status ensure_adjoint_factors(Plan &pl, int B) {
+  if (pl.prm.fsphere) return REXI_OK;
+  const bool fixed = !pl.dig_adj_tried && digits_chosen(pl, B);
+  if (pl.fac_adj && !fixed) return REXI_OK;
+  cudaError_t e = cudaSuccess;
   const size_t n = (size_t)fac_ncomp(pl) * pl.nrows * pl.P;
-  cudaError_t e = cudaMalloc(&pl.fac_adj, n * sizeof(double2));
-  if (e != cudaSuccess) {
-    pl.fac_adj = nullptr;
-    set_error(std::string("adjoint factors: ") + cudaGetErrorString(e));
-    return REXI_ENOMEM;
+  if (!pl.fac_adj) {
+    if (cudaMalloc(&pl.fac_adj, n * sizeof(double2)) != cudaSuccess) {
+      pl.fac_adj = nullptr;
+      set_error(std::string("adjoint factors: ") + cudaGetErrorString(cudaGetLastError()));
+      return REXI_ENOMEM;
+    }
+    pl.bytes += n * sizeof(double2);
+    e = launch_factor_setup(pl, true, 0);
   }
-  pl.bytes += n * sizeof(double2);
-  e = launch_factor_setup(pl, true, 0);
-  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  if (fixed) {
+    pl.dig_adj_tried = true;
+    if (e == cudaSuccess && spare_memory(digit_factor_bytes(pl), 0))  // the rule of the forward ones
+      e = build_digit_factors(pl, true, pl.fac_adj, pl.dig_adj);
+    if (pl.dig_adj.fwd) pl.bytes += digit_factor_bytes(pl);
+  }
+  if (e == cudaSuccess && !pl.dig_adj.fwd) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return cuda_fail("adjoint factor setup", e);
   if (pl.ff) {
     const rexi_status r = take_range_error(pl, "adjoint float-float factors");
@@ -133,7 +137,7 @@ rexi_status ensure_adjoint_factors(Plan &pl) {
       return r;
     }
   }
-  return ensure_adjoint_factors(pl);  // then the same factors as digits
+  return REXI_OK;
 }
 
 // Spectral REXI core on the plan's internal layout: s_in -> s_out.
@@ -226,7 +230,7 @@ rexi_status step_impl(rexi_plan *plan, const void *in, void *out, int32_t B, voi
     set_error("rexi_step_adjoint: not available for REXI_SOLVER_PHI plans");
     return REXI_EINVAL;
   }
-  if (adjoint && (r = ensure_adjoint_factors(pl)) != REXI_OK) return r;
+  if (adjoint && (r = ensure_adjoint_factors(pl, B)) != REXI_OK) return r;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   Marks mk(pl, st);
   if (grid) {
@@ -489,6 +493,7 @@ rexi_status rexi_tune(rexi_plan *plan, int32_t batch, int32_t *slots, int32_t *s
   rexi_status r = tune_layout(pl, batch, &s, &sh);
   if (r == REXI_OK && slots) *slots = s;
   if (r == REXI_OK && shape) *shape = sh;
+  if (r == REXI_OK && pl.fac_adj) r = ensure_adjoint_factors(pl, batch);
   return r;
 }
 
@@ -511,6 +516,7 @@ rexi_status rexi_set_pole_slots(rexi_plan *plan, int32_t batch, int32_t slots, i
   int u = 0;
   rexi_status r = set_layout(pl, batch, slots, shape, &u);
   if (r == REXI_OK && used) *used = u;
+  if (r == REXI_OK && pl.fac_adj) r = ensure_adjoint_factors(pl, batch);  // as a first adjoint call with it would
   return r;
 }
 

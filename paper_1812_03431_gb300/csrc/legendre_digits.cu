@@ -503,8 +503,7 @@ LegArgs leg_args(const Plan &pl, const LegendreDigits &t, const double2 *four, c
 }  // namespace
 
 void free_legendre_digits(LegendreDigits &t) {
-  for (void *p : {(void *)t.dig, (void *)t.exps, (void *)t.sys})
-    if (p) cudaFree(p);
+  if (t.dig) cudaFree(t.dig);  // the others lie behind it
   t = LegendreDigits{};
 }
 
@@ -516,7 +515,9 @@ struct TabLayout {
   int64_t nfrag = 0, nexp = 0;
   int most = 0;
   bool ok = true;
-  size_t bytes() const { return (size_t)nfrag * 2 * kFrag + (size_t)nexp * 32 * sizeof(int); }
+  size_t dig_bytes() const { return (size_t)nfrag * 2 * kFrag; }
+  size_t exp_bytes() const { return (size_t)nexp * 32 * sizeof(int); }
+  size_t bytes() const { return dig_bytes() + exp_bytes() + sys.size() * sizeof(int4); }
 };
 
 TabLayout tab_layout(const Plan &pl, bool synthesis) {
@@ -552,15 +553,15 @@ cudaError_t build_legendre_digits(Plan &pl, bool synthesis, LegendreDigits &t) {
   const TabLayout L = tab_layout(pl, synthesis);
   const std::vector<int4> &sys = L.sys;
   if (!L.ok) return cudaSuccess;
-  cudaError_t e = cudaSuccess;
-  if (cudaMalloc(&t.dig, (size_t)L.nfrag * 2 * kFrag) != cudaSuccess ||
-      cudaMalloc(&t.exps, (size_t)L.nexp * 32 * sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&t.sys, sys.size() * sizeof(int4)) != cudaSuccess) {
+  char *mem = nullptr;
+  if (cudaMalloc(&mem, L.bytes()) != cudaSuccess) {
     cudaGetLastError();
-    free_legendre_digits(t);
     return cudaSuccess;
   }
-  e = cudaMemcpy(t.sys, sys.data(), sys.size() * sizeof(int4), cudaMemcpyHostToDevice);
+  t.dig = reinterpret_cast<uint4 *>(mem);
+  t.exps = reinterpret_cast<int *>(mem + L.dig_bytes());
+  t.sys = reinterpret_cast<int4 *>(mem + L.dig_bytes() + L.exp_bytes());
+  cudaError_t e = cudaMemcpy(t.sys, sys.data(), sys.size() * sizeof(int4), cudaMemcpyHostToDevice);
   TabArgs a;
   a.tab[0] = pl.tabP;
   a.tab[1] = pl.tabH;

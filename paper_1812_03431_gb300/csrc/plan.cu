@@ -630,14 +630,20 @@ const FusedLayout *fused_layout(Plan &pl, int B) {
   return it->second.st > 0 ? &it->second : nullptr;
 }
 
-// The digit solve's work list for steps of B states, or null where another kernel serves them:
-// no digit factors (see build_plan), an explicit pole_slots, another layout chosen for this
-// batch, or without a choice a batch below kDigitMinBatch (kDigitMinBatchLarge).
-const DigitLayout *digit_layout(Plan &pl, int B, bool adjoint) {
-  if (!(adjoint ? pl.dig_adj : pl.dig_fwd).fwd) return nullptr;
+// Whether steps of B states take the digit solve: the plan has its factors (see build_plan), and
+// it was chosen for this batch or, without a choice, there is no explicit pole_slots and the batch
+// is not below kDigitMinBatch (kDigitMinBatchLarge).
+bool digits_chosen(const Plan &pl, int B) {
+  if (!pl.dig_fwd.fwd) return false;
   auto ud = pl.use_digits.find(B);
+  if (ud != pl.use_digits.end()) return ud->second;
   const int least = pl.limbs ? 1 : (pl.nrows * pl.P >= kDigitLarge ? kDigitMinBatchLarge : kDigitMinBatch);
-  if (ud != pl.use_digits.end() ? !ud->second : (pl.slots_override > 0 || B < least)) return nullptr;
+  return pl.slots_override <= 0 && B >= least;
+}
+
+// The digit solve's work list for steps of B states, or null where another kernel serves them.
+const DigitLayout *digit_layout(Plan &pl, int B, bool adjoint) {
+  if (!digits_chosen(pl, B) || (adjoint && !pl.dig_adj.fwd)) return nullptr;
   auto it = pl.digits.find(B);
   if (it == pl.digits.end()) {
     DigitLayout L;

@@ -124,7 +124,7 @@ struct FusedRagged {
 // of coupling and weight digits, and the rows' input scales.  Empty (fwd null) where it does
 // not serve the plan.
 struct DigitFactors {
-  char *fwd = nullptr, *bwd = nullptr;
+  char *fwd = nullptr, *bwd = nullptr;  // all in one allocation, fwd first
   int *vexp = nullptr;
   // limbs only: reciprocals of the shifts, of the poles, their exponent, the rows' real factors
   char *inv = nullptr;
@@ -277,7 +277,7 @@ struct Plan {
   std::map<int, int> fused_form;  // 0: register form; lean form with CTAs of 1: four warps, 2: two warps
   std::map<int, int> fused_groups; // requested CTAs per system's poles (0: the default)
 
-  // digit solve: the factors as digits (adjoint on first use), the step's inputs as digits,
+  // digit solve: the factors as digits (adjoint when a batch that they serve first asks for it), the step's inputs as digits,
   // per batch size the work list and whether rexi_tune / rexi_set_pole_slots chose it
   DigitFactors dig_fwd, dig_adj;
   bool dig_adj_tried = false;

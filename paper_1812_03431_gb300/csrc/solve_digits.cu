@@ -358,8 +358,7 @@ int windows_of(const Plan &pl, int B, int kc) {
 }  // namespace
 
 void free_digit_factors(DigitFactors &D) {
-  for (void *p : {(void *)D.fwd, (void *)D.bwd, (void *)D.vexp, (void *)D.inv, (void *)D.inv_alpha, (void *)D.scale})
-    if (p) cudaFree(p);
+  if (D.fwd) cudaFree(D.fwd);  // the others lie behind it
   D = DigitFactors{};
 }
 
@@ -372,10 +371,8 @@ namespace {
 cudaError_t launch_digit_factors(Plan &pl, const double2 *fac, DigitFactors &D, int *bad) {
   const int nwin = (pl.P + kWin - 1) / kWin;
   const size_t nrec = (size_t)pl.nrows * nwin;
-  cudaError_t e = cudaMalloc(&D.fwd, nrec * kFwdRec);
-  if (e == cudaSuccess) e = cudaMalloc(&D.bwd, nrec * kBwdRec);
-  if (e == cudaSuccess) e = cudaMalloc(&D.vexp, (size_t)pl.nrows * 4 * sizeof(int));
-  if (e != cudaSuccess) return e;
+  D.bwd = D.fwd + nrec * kFwdRec;
+  D.vexp = reinterpret_cast<int *>(D.bwd + nrec * kBwdRec);
   SetupArgs a;
   a.fac = fac;
   a.sys = pl.sys_dev;
@@ -403,12 +400,15 @@ cudaError_t launch_digit_factors(Plan &pl, const double2 *fac, DigitFactors &D, 
 cudaError_t build_digit_factors(Plan &pl, bool adjoint, const double2 *fac, DigitFactors &D) {
   D = DigitFactors{};
   if (pl.nrows == 0 || (pl.P + kWin - 1) / kWin > 0x7fff || pl.sys.size() > 0xffff) return cudaSuccess;
-  int *bad = nullptr, hbad = 0;
-  cudaError_t e = cudaMalloc(&bad, sizeof(int));
+  // one allocation, the flag at its end; the read of the flag waits for the factors
+  const size_t bytes = digit_factor_bytes(pl);
+  int hbad = 0;
+  cudaError_t e = cudaMalloc(&D.fwd, bytes + sizeof(int));
+  int *bad = reinterpret_cast<int *>(D.fwd + bytes);
+  if (e != cudaSuccess) D.fwd = nullptr;
   if (e == cudaSuccess) e = cudaMemsetAsync(bad, 0, sizeof(int), 0);
   if (e == cudaSuccess) e = pl.limbs ? launch_limb_factors(pl, adjoint, fac, D, bad) : launch_digit_factors(pl, fac, D, bad);
   if (e == cudaSuccess) e = cudaMemcpy(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost);
-  if (bad) cudaFree(bad);
   if (e != cudaSuccess || hbad) free_digit_factors(D);
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();

@@ -220,6 +220,7 @@ namespace {
 int blocks_of(const Plan &pl) { return (pl.P + kBlock - 1) / kBlock; }
 size_t inv_bytes(const Plan &pl) { return (size_t)(pl.nrows + (int64_t)pl.sys.size()) * blocks_of(pl) * kRec; }
 size_t scale_bytes(const Plan &pl) { return (size_t)pl.nrows * 6 * sizeof(double); }
+int *block_exponents(const Plan &pl, const DigitFactors &D) { return reinterpret_cast<int *>(D.scale + (size_t)pl.nrows * 6); }
 }  // namespace
 size_t limb_factor_bytes(const Plan &pl) {
   return (size_t)pl.nrows * blocks_of(pl) * (kRec + kBwd) + inv_bytes(pl) + scale_bytes(pl) +
@@ -235,16 +236,13 @@ int limb_exponent(const Plan &pl) {
   return least > 0.0 ? std::max(0, std::ilogb(1.0 / least)) : kMaxSpread + 1;
 }
 
-// The factor set as limbs; `bad` set where it does not serve.  cudaErrorMemoryAllocation where
-// it does not fit.
+// The factor set as limbs, in the limb_factor_bytes at D.fwd; `bad` set where it does not serve.
 cudaError_t launch_limb_factors(Plan &pl, bool adjoint, const double2 *fac, DigitFactors &D, int *bad) {
   const size_t nrec = (size_t)pl.nrows * blocks_of(pl);
-  cudaError_t e = cudaMalloc(&D.fwd, nrec * kRec);
-  if (e == cudaSuccess) e = cudaMalloc(&D.bwd, nrec * kBwd);
-  if (e == cudaSuccess) e = cudaMalloc(&D.inv, inv_bytes(pl));
-  if (e == cudaSuccess) e = cudaMalloc(&D.inv_alpha, (size_t)blocks_of(pl) * (kBlock * sizeof(int4) + sizeof(int)));
-  if (e == cudaSuccess) e = cudaMalloc(&D.scale, scale_bytes(pl));
-  if (e != cudaSuccess) return e;
+  D.bwd = D.fwd + nrec * kRec;
+  D.inv = D.bwd + nrec * kBwd;
+  D.inv_alpha = reinterpret_cast<int4 *>(D.inv + inv_bytes(pl));
+  D.scale = reinterpret_cast<double *>(D.inv_alpha + (size_t)blocks_of(pl) * kBlock);  // every part a multiple of 16 B so far
   SetupArgs a;
   a.fac = fac;
   a.alpha = pl.alpha_dev;
@@ -254,7 +252,7 @@ cudaError_t launch_limb_factors(Plan &pl, bool adjoint, const double2 *fac, Digi
   a.bwd = D.bwd;
   a.inv = D.inv;
   a.inv_alpha = D.inv_alpha;
-  a.eblk = reinterpret_cast<int *>(D.inv_alpha + (size_t)blocks_of(pl) * kBlock);
+  a.eblk = block_exponents(pl, D);
   a.scale = D.scale;
   a.bad = bad;
   a.P = pl.P;
@@ -266,8 +264,8 @@ cudaError_t launch_limb_factors(Plan &pl, bool adjoint, const double2 *fac, Digi
   a.tau = pl.prm.tau;
   a.q = 2.0 * pl.prm.omega * pl.prm.tau;
   a.phibar = pl.prm.gravity * pl.prm.mean_depth;
-  if (a.e0 > kMaxSpread) return cudaMemset(bad, 1, 1);
-  e = cudaMemset(a.eblk, 0x80, blocks_of(pl) * sizeof(int));  // a very negative number
+  if (a.e0 > kMaxSpread) return cudaMemsetAsync(bad, 1, 1, 0);
+  const cudaError_t e = cudaMemsetAsync(a.eblk, 0x80, blocks_of(pl) * sizeof(int), 0);  // a very negative number
   if (e != cudaSuccess) return e;
   limb_factor_kernel<<<dim3((unsigned)((pl.lmax + 1) * a.nblk), (unsigned)pl.sys.size()), kBlock>>>(a);
   return cudaGetLastError();
@@ -296,7 +294,7 @@ LimbSweep limb_sweep(Plan &pl, const DigitLayout &L, bool adjoint, int B) {
   a.inv = D.inv;
   a.inv_alpha = D.inv_alpha;
   a.e0 = D.e0;
-  a.eblk = reinterpret_cast<const int *>(D.inv_alpha + (size_t)blocks_of(pl) * kBlock);
+  a.eblk = block_exponents(pl, D);
   a.dig = reinterpret_cast<const int4 *>(pl.dig_state);
   a.uexp = reinterpret_cast<const int *>(pl.dig_state + (size_t)pl.nrows * B * 4 * sizeof(int4));
   a.sys = pl.sys_dev;

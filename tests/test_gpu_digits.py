@@ -204,3 +204,28 @@ def test_packings_that_a_plan_does_not_have_are_refused(env, B, slots):
     np.testing.assert_array_equal(plan.step(x).cpu().numpy(), y)
     assert plan.set_pole_slots(B, used, 5) == used  # what the call returned is taken back
     plan.close()
+
+
+def test_the_adjoints_factors_wait_for_a_batch_that_they_serve(env):
+    """One state in a plan for eight takes the binary64 factors only; eight states, or a call that
+    chooses the fixed-point solve for one, the others as well; results as the slot solve's throughout."""
+    torch, rexi = env
+    N, P, B = 42, 149, 8
+    al, be = poles(P)
+    x = torch.from_numpy(inputs.random_spectral(N, B, 17)).cuda()
+    slots = spectral_plan(rexi, N, B, al, be, pole_slots=4)
+    want = slots.step_adjoint(x).cpu().numpy()
+    binary64 = 9 * 16 * P * ((N + 1) * (N + 2) // 2 - 1)
+    for choose in (False, True):
+        plan = spectral_plan(rexi, N, B, al, be)
+        start = plan.info()["device_bytes"]
+        assert fieldwise(plan.step_adjoint(x[:1]).cpu().numpy(), want[:1]) < ORDER
+        assert plan.info()["device_bytes"] == start + binary64
+        if choose:
+            plan.set_pole_slots(1, 0, 5)
+        else:
+            assert fieldwise(plan.step_adjoint(x).cpu().numpy(), want) < ORDER
+        assert plan.info()["device_bytes"] > start + 2 * binary64
+        assert fieldwise(plan.step_adjoint(x[:1]).cpu().numpy(), want[:1]) < ORDER
+        plan.close()
+    slots.close()
