@@ -18,7 +18,8 @@
 // degrees or latitudes.  A tile of the product's columns is one field of the four states (re,
 // im), so that a lane ends up with all fields of one state and combines them in registers.  With
 // one state that tile would be three quarters padding: there the three fields share one, and two
-// products (P and H times all fields) do for the five.  Tables: 8 B per value as in the FP64 form,
+// products (P and H times all fields) do for the five.  Small batches take that form state by
+// state (one_state below).  Tables: 8 B per value as in the FP64 form,
 // in fragment order.  Everything is copied ahead with cp.async: a warp's next table fragment, also
 // across products and barriers, and the next group's inputs while the products run.
 //
@@ -226,7 +227,7 @@ __device__ __forceinline__ double2 of_field(double2 v, int lane, int f) {
 }
 
 // Analysis: out[n] = sum_j; blockIdx.x: states, .y: row tiles (eight per CTA, classes 0, 1), .z: m.
-// ONE: a batch of one state.  Its three fields share a column tile (lane q holds field q), which
+// ONE: one state per CTA.  Its three fields share a column tile (lane q holds field q), which
 // makes two products, P and H times all fields, of the five.
 template <bool ONE>
 __global__ void __launch_bounds__(256, 2) legendre_digits_analysis(LegArgs a) {
@@ -235,7 +236,7 @@ __global__ void __launch_bounds__(256, 2) legendre_digits_analysis(LegArgs a) {
   const double2 *raw = reinterpret_cast<const double2 *>(smem);
   uint4 *dig = reinterpret_cast<uint4 *>(smem + kDig);
   int *cexp = reinterpret_cast<int *>(smem + kExp);
-  const int m = blockIdx.z, b0 = blockIdx.x * 4, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int m = blockIdx.z, b0 = blockIdx.x * (ONE ? 1 : 4), tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int4 s0 = a.sys[2 * m], s1 = a.sys[2 * m + 1];
   const int t0 = (s0.x + 15) / 16, t1 = (s1.x + 15) / 16;
   if ((int)blockIdx.y * kWarps >= t0 + t1) return;
@@ -330,7 +331,7 @@ __global__ void __launch_bounds__(256, 2) legendre_digits_analysis(LegArgs a) {
       add_im(delta[i], fm, pu.x, pu.y);
     }
   }
-  const int b = ONE ? 0 : b0 + q;
+  const int b = ONE ? b0 : b0 + q;
   if (b >= a.B) return;
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
@@ -353,7 +354,7 @@ __global__ void __launch_bounds__(256, 2) legendre_digits_synthesis(LegArgs a) {
   const double *zds = reinterpret_cast<const double *>(smem + kZd);
   uint4 *dig = reinterpret_cast<uint4 *>(smem + kDig);
   int *cexp = reinterpret_cast<int *>(smem + kExp);
-  const int m = blockIdx.z, b0 = blockIdx.x * 4, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int m = blockIdx.z, b0 = blockIdx.x * (ONE ? 1 : 4), tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int tiles = (a.J + 15) / 16, tile = blockIdx.y * kWarps + warp, q = lane & 3, row = lane >> 2;
   const bool live = tile < tiles;
   const int64_t idx0 = (int64_t)m * (2 * a.N + 3 - m) / 2;
@@ -452,7 +453,7 @@ __global__ void __launch_bounds__(256, 2) legendre_digits_synthesis(LegArgs a) {
     }
   }
   if (!live) return;
-  const int b = ONE ? 0 : b0 + q, M1 = a.N + 1, ncol = 3 * a.B;
+  const int b = ONE ? b0 : b0 + q, M1 = a.N + 1, ncol = 3 * a.B;
   if constexpr (ONE) {  // lane q takes field q: Phi; U = i m P chi' - H psi'; V = i m P psi' + H chi'
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
@@ -583,17 +584,33 @@ cudaError_t build_legendre_digits(Plan &pl, bool synthesis, LegendreDigits &t) {
   return e;
 }
 
+namespace {
+// One state per CTA in place of four: a batch of one, and batches whose CTAs then still find their
+// places at once (two per SM), where a CTA's chain of two products in place of five is what counts.
+// Analysis, synthesis with the FFT, us, one / four states per CTA: T21 x 2 13.8 / 19.9, 14.6 / 24.5 (of
+// the FP64 kernels: 18.5, 22.0); T63 x 4 (256 CTAs) 20.8 / 26.0, 22.5 / 32.7; T24 x 12 (300) 19.2 / 24.0,
+// 22.0 / 29.7; past the line T24 x 16 (400) 27.1 / 25.7, 30.4 / 32.0, T48 x 8 (392) 29.9 / 29.4, 33.7 /
+// 37.2, T127 x 8 (1024) 91.6 / 73.5, 86.9 / 74.6.
+bool one_state(const Plan &pl, int B, unsigned rows) {
+  return B == 1 || (int64_t)(pl.N + 1) * rows * B <= 2 * pl.num_sms;
+}
+}  // namespace
+
 cudaError_t launch_leg_ana_digits(Plan &pl, const double2 *four, double2 *sint, int B, const double *zd, cudaStream_t st) {
   const int tiles = (pl.N / 2 + 1 + 15) / 16 + ((pl.N + 1) / 2 + 15) / 16;
-  const dim3 g((unsigned)((B + 3) / 4), (unsigned)((tiles + kWarps - 1) / kWarps), (unsigned)(pl.N + 1));
-  (B == 1 ? legendre_digits_analysis<true> : legendre_digits_analysis<false>)<<<g, 32 * kWarps, kSmem, st>>>(
+  const unsigned rows = (unsigned)((tiles + kWarps - 1) / kWarps);
+  const bool one = one_state(pl, B, rows);
+  const dim3 g((unsigned)(one ? B : (B + 3) / 4), rows, (unsigned)(pl.N + 1));
+  (one ? legendre_digits_analysis<true> : legendre_digits_analysis<false>)<<<g, 32 * kWarps, kSmem, st>>>(
       leg_args(pl, pl.leg_ana, four, sint, B, zd));
   return cudaGetLastError();
 }
 
 cudaError_t launch_leg_syn_digits(Plan &pl, const double2 *sint, double2 *four, int B, const double *zd, cudaStream_t st) {
-  const dim3 g((unsigned)((B + 3) / 4), (unsigned)(((pl.J + 15) / 16 + kWarps - 1) / kWarps), (unsigned)(pl.N + 1));
-  (B == 1 ? legendre_digits_synthesis<true> : legendre_digits_synthesis<false>)<<<g, 32 * kWarps, kSmem, st>>>(
+  const unsigned rows = (unsigned)(((pl.J + 15) / 16 + kWarps - 1) / kWarps);
+  const bool one = one_state(pl, B, rows);
+  const dim3 g((unsigned)(one ? B : (B + 3) / 4), rows, (unsigned)(pl.N + 1));
+  (one ? legendre_digits_synthesis<true> : legendre_digits_synthesis<false>)<<<g, 32 * kWarps, kSmem, st>>>(
       leg_args(pl, pl.leg_syn, four, sint, B, zd));
   return cudaGetLastError();
 }

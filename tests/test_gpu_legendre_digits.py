@@ -134,3 +134,23 @@ def test_a_smooth_flow_among_small_coefficients(env, N, nlat, nlon, B):
     both, alone = wind(big + small), wind(big)
     assert np.linalg.norm(both - wind(small) - alone) < 3 * 2.0**-52 * np.linalg.norm(alone)
     plan.close()
+
+
+# batches whose CTAs of one state fill two places per SM (304) or just do not, and the same states fewer at a time
+@pytest.mark.parametrize("N,nlat,nlon,B,few", [(1, 2, 4, 153, 152), (2, 4, 8, 103, 7), (15, 32, 48, 20, 3), (16, 36, 48, 18, 17),
+                                               (31, 64, 96, 10, 9), (33, 128, 108, 9, 4), (37, 76, 120, 9, 8),
+                                               (66, 132, 200, 5, 2), (127, 192, 384, 3, 2), (130, 132, 400, 3, 2)])
+def test_one_and_four_states_per_block(env, N, nlat, nlon, B, few):
+    """Each product is exact up to 2^-59 of its group and rounded alike in both forms, the sums over the
+    groups are in another order (up to four of them)."""
+    torch, rexi = env
+    plan = rexi.Plan(N, nlat, nlon, M=8, max_batch=B)
+    x = torch.from_numpy(inputs.random_grid(B, nlat, nlon, 11)).cuda()
+    S = torch.from_numpy(inputs.random_spectral(N, B, 12, slope=0.0)).cuda()
+    for f, v in ((plan.analyze, x), (plan.synthesize, S)):
+        four = f(v).cpu().numpy()
+        one = np.concatenate([f(v[i:i + few].contiguous()).cpu().numpy() for i in range(0, B, few)])
+        for b in range(B):
+            for k in range(3):
+                assert np.linalg.norm(one[b, k] - four[b, k]) <= 4 * 2.0**-52 * np.linalg.norm(four[b, k])
+    plan.close()
