@@ -140,6 +140,17 @@ rexi_status ensure_adjoint_factors(Plan &pl, int B) {
   return REXI_OK;
 }
 
+// The fixed-point solve and its sums, sin -> sout ([B][3][nspec] where by_state, else [3][nspec][B]).
+rexi_status fixed_core(Plan &pl, const DigitLayout &dl, int B, bool adjoint, const double2 *sin, double2 *sout, bool by_state,
+                       cudaStream_t st, Marks &mk) {
+  mk.mark(ST_SOLVE);
+  cudaError_t e = launch_solve_digits(pl, dl, adjoint, sin, by_state, B, st);
+  if (e != cudaSuccess) return cuda_fail("fixed-point solve", e);
+  if (!pl.limbs) mk.mark(ST_REDUCE);  // small batches count it with the solve
+  e = launch_finish_digits(pl, dl, adjoint, sin, sout, by_state, B, st);
+  return e == cudaSuccess ? REXI_OK : cuda_fail("fixed-point sums", e);
+}
+
 // Spectral REXI core on the plan's internal layout: s_in -> s_out.
 rexi_status core(Plan &pl, int B, bool adjoint, cudaStream_t st, Marks &mk) {
   if (pl.prm.fsphere) {
@@ -147,14 +158,8 @@ rexi_status core(Plan &pl, int B, bool adjoint, cudaStream_t st, Marks &mk) {
     cudaError_t e = launch_fsphere(pl, adjoint, pl.s_in, pl.s_out, B, false, 0, st);
     return e == cudaSuccess ? REXI_OK : cuda_fail("f-sphere solve", e);
   }
-  if (const DigitLayout *dl = digit_layout(pl, B, adjoint)) {  // both contractions on the tensor cores
-    mk.mark(ST_SOLVE);
-    cudaError_t e = launch_solve_digits(pl, *dl, adjoint, pl.s_in, B, st);
-    if (e != cudaSuccess) return cuda_fail("digit solve", e);
-    if (!pl.limbs) mk.mark(ST_REDUCE);  // small batches count it with the solve
-    e = launch_finish_digits(pl, *dl, adjoint, pl.s_in, pl.s_out, B, st);
-    return e == cudaSuccess ? REXI_OK : cuda_fail("digit sums", e);
-  }
+  if (const DigitLayout *dl = digit_layout(pl, B, adjoint))
+    return fixed_core(pl, *dl, B, adjoint, pl.s_in, pl.s_out, false, st, mk);
   SolveLayout *lay = nullptr;
   rexi_status r = get_layout(pl, B, false, &lay);
   if (r != REXI_OK) return r;
@@ -235,6 +240,12 @@ rexi_status step_impl(rexi_plan *plan, const void *in, void *out, int32_t B, voi
   Marks mk(pl, st);
   if (grid) {
     if ((r = analyze(pl, static_cast<const double *>(in), B, adjoint, st, mk)) != REXI_OK) return r;
+  } else if (const DigitLayout *dl = pl.limbs ? digit_layout(pl, B, adjoint) : nullptr) {
+    // limbs read and write the caller's layout: without the two transposes a step of few rows
+    // has the three launches it had with the fused solve
+    r = fixed_core(pl, *dl, B, adjoint, static_cast<const double2 *>(in), static_cast<double2 *>(out), true, st, mk);
+    if (r == REXI_OK) mk.mark(kStages);
+    return r;
   } else {
     mk.mark(ST_TRANS_IN);
     cudaError_t e = launch_transpose_in(static_cast<const double2 *>(in), pl.s_in, pl.nspec, B, st);

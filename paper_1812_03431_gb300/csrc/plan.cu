@@ -837,8 +837,8 @@ rexi_status tune_layout(Plan &pl, int B, int *slots_out, int *shape_out) {
       if (!D) break;
       for (int rep = 0; rep < 3; ++rep) {
         if (rep == 1) cudaEventRecord(e0, st);
-        launch_solve_digits(pl, *D, false, pl.s_in, B, st);
-        launch_finish_digits(pl, *D, false, pl.s_in, pl.s_out, B, st);
+        launch_solve_digits(pl, *D, false, pl.s_in, false, B, st);
+        launch_finish_digits(pl, *D, false, pl.s_in, pl.s_out, false, B, st);
       }
       cudaEventRecord(e1, st);
       float ms = 1e30f;

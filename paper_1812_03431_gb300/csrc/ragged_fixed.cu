@@ -146,7 +146,7 @@ cudaError_t launch_fixed_ragged(const std::vector<Plan *> &plans, const std::vec
   int num_sms = 1;
   for (size_t p = 0; p < plans.size() && e == cudaSuccess; ++p) {
     num_sms = std::max(num_sms, plans[p]->num_sms);
-    if (counts[p] > 0) e = launch_digit_state(*plans[p], false, plans[p]->s_in, counts[p], nullptr, st);
+    if (counts[p] > 0) e = launch_digit_state(*plans[p], false, plans[p]->s_in, false, counts[p], nullptr, st);
   }
   if (e != cudaSuccess) return e;
   for (int kind = 0; kind < 2 && e == cudaSuccess; ++kind) {
@@ -162,7 +162,7 @@ cudaError_t launch_fixed_ragged(const std::vector<Plan *> &plans, const std::vec
   }
   for (size_t p = 0; p < plans.size() && e == cudaSuccess; ++p)
     if (counts[p] > 0)
-      e = launch_finish_digits(*plans[p], R.layouts[p], false, plans[p]->s_in, plans[p]->s_out, counts[p], st);
+      e = launch_finish_digits(*plans[p], R.layouts[p], false, plans[p]->s_in, plans[p]->s_out, false, counts[p], st);
   return e;
 }
 

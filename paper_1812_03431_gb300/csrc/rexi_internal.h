@@ -353,9 +353,11 @@ size_t limb_factor_bytes(const Plan &pl);
 size_t limb_state_bytes(const Plan &pl, int B);
 cudaError_t limb_configure(int kc);
 cudaError_t launch_limb_factors(Plan &pl, bool adjoint, const double2 *fac, DigitFactors &D, int *bad);
-cudaError_t launch_limb_state(Plan &pl, bool adjoint, const double2 *sin, int B, unsigned *counter, cudaStream_t st);
+cudaError_t launch_limb_state(Plan &pl, bool adjoint, const double2 *sin, bool by_state, int B, unsigned *counter,
+                              cudaStream_t st);
 cudaError_t launch_solve_limbs(Plan &pl, const DigitLayout &L, bool adjoint, int B, cudaStream_t st);
-cudaError_t launch_digit_state(Plan &pl, bool adjoint, const double2 *sin, int B, unsigned *counter, cudaStream_t st);
+cudaError_t launch_digit_state(Plan &pl, bool adjoint, const double2 *sin, bool by_state, int B, unsigned *counter,
+                               cudaStream_t st);
 struct DigitItem {
   int4 it;       // system, tile, first window | windows << 16, slot
   int64_t work;  // rows x windows
@@ -375,10 +377,10 @@ cudaError_t launch_fixed_ragged(const std::vector<Plan *> &plans, const std::vec
                                 double2 *ybuf, unsigned *counter, cudaStream_t st);
 rexi_status build_digit_layout(Plan &pl, int B, int slots, DigitLayout &L);
 void free_digit_layout(DigitLayout &L);
-cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, int B,
+cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, bool by_state, int B,
                                 cudaStream_t st);
 cudaError_t launch_finish_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, double2 *sout,
-                                 int B, cudaStream_t st);
+                                 bool by_state, int B, cudaStream_t st);
 cudaError_t launch_solve_ragged(const SolveView *views_dev, const WorkItem *items, int nitems, double2 *ybuf,
                                 int lmax, unsigned *counter, int resident_warps, bool ff, cudaStream_t st);
 // float-float solves: convert n complex values in place (factors), or split n binary64

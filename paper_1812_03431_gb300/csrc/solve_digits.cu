@@ -285,6 +285,7 @@ struct FinishArgs {
   double2 sphi;
   int64_t nspec, nrows;
   const double *scale;  // limbs: per row the sums' real factors at 3..5 (see solve_limbs.cu), else null
+  bool by_state;        // sin, sout: [B][3][nspec], else [3][nspec][B]
   int B, tile, tiles, unit, sstr, pstr, slots, N;
 };
 
@@ -297,8 +298,9 @@ __global__ void digit_finish_kernel(FinishArgs a) {
   const int first = threadIdx.x % SPLIT;
   for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / SPLIT; t < total;
        t += (int64_t)gridDim.x * blockDim.x / SPLIT) {
-    const int b = (int)(t % a.B);
-    const int64_t fi = t / a.B;
+    const int64_t inner = a.by_state ? 3 * a.nspec : a.B, outer = t / inner, rest = t - outer * inner;
+    const int b = (int)(a.by_state ? outer : rest);
+    const int64_t fi = a.by_state ? rest : outer;
     const int f = (int)(fi / a.nspec);
     const int64_t ix = fi - (int64_t)f * a.nspec;
     const uint8_t fl = a.rflags[fi];
@@ -504,9 +506,11 @@ void free_digit_layout(DigitLayout &L) {
   L = DigitLayout{};
 }
 
-// the batch's inputs in fixed point, and *counter = 0
-cudaError_t launch_digit_state(Plan &pl, bool adjoint, const double2 *sin, int B, unsigned *counter, cudaStream_t st) {
-  if (pl.limbs) return launch_limb_state(pl, adjoint, sin, B, counter, st);
+// the batch's inputs in fixed point, and *counter = 0.  by_state (limbs only): sin is [B][3][nspec], as
+// rexi_step takes it, else [3][nspec][B].
+cudaError_t launch_digit_state(Plan &pl, bool adjoint, const double2 *sin, bool by_state, int B, unsigned *counter,
+                               cudaStream_t st) {
+  if (pl.limbs) return launch_limb_state(pl, adjoint, sin, by_state, B, counter, st);
   const int tiles = tiles_of(pl, B);
   StateArgs s;
   s.sin = sin;
@@ -544,8 +548,9 @@ DigitSweep digit_sweep(Plan &pl, const DigitLayout &L, bool adjoint, int B) {
   return a;
 }
 
-cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, int B, cudaStream_t st) {
-  cudaError_t e = launch_digit_state(pl, adjoint, sin, B, pl.counter, st);
+cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, bool by_state, int B,
+                                cudaStream_t st) {
+  cudaError_t e = launch_digit_state(pl, adjoint, sin, by_state, B, pl.counter, st);
   if (e != cudaSuccess) return e;
   if (pl.limbs) return launch_solve_limbs(pl, L, adjoint, B, st);
   const int ctas = std::min(pl.num_sms * kCtas, (L.nitems + 3) / 4);
@@ -553,8 +558,8 @@ cudaError_t launch_solve_digits(Plan &pl, const DigitLayout &L, bool adjoint, co
   return cudaGetLastError();
 }
 
-cudaError_t launch_finish_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, double2 *sout, int B,
-                                 cudaStream_t st) {
+cudaError_t launch_finish_digits(Plan &pl, const DigitLayout &L, bool adjoint, const double2 *sin, double2 *sout,
+                                 bool by_state, int B, cudaStream_t st) {
   FinishArgs f;
   f.part = reinterpret_cast<const double *>(pl.partial);
   f.sin = sin;
@@ -566,6 +571,7 @@ cudaError_t launch_finish_digits(Plan &pl, const DigitLayout &L, bool adjoint, c
   f.sphi = adjoint ? pl.sphi_adj : pl.sphi_fwd;
   f.nspec = pl.nspec;
   f.nrows = pl.nrows;
+  f.by_state = by_state;
   f.B = B;
   f.tile = pl.limbs ? 1 : kTile;
   f.tiles = pl.limbs ? B : tiles_of(pl, B);

@@ -130,13 +130,13 @@ __global__ void __launch_bounds__(kBlock) limb_factor_kernel(SetupArgs a) {
 
 // ---- per step: the row inputs as limbs ----------------------------------------------------------
 struct StateArgs {
-  const double2 *sin;  // [3][nspec][B]
+  const double2 *sin;  // [3][nspec] places `place` apart, states `state` apart
   const int4 *sys;
   const double *scale;
   int4 *dig;           // [nrows][B][4 inputs]
   int *uexp;           // [nrows][B]
   unsigned *counter;   // the sweep's next item, set to zero here (null: not)
-  int64_t nspec;
+  int64_t nspec, place, state;
   int B, N;
 };
 
@@ -152,7 +152,7 @@ __global__ void limb_state_kernel(StateArgs a) {
   double2 x = make_double2(0, 0);
   if (live && nn >= nmin && nn <= a.N) {
     const int64_t ix = (int64_t)m * (2 * a.N + 3 - m) / 2 + (nn - m);
-    x = __ldg(a.sin + ((int64_t)field * a.nspec + ix) * a.B + b);
+    x = __ldg(a.sin + ((int64_t)field * a.nspec + ix) * a.place + b * a.state);
   }
   if (live && q > 0) {
     const double v = a.scale[((int64_t)sy.w + i) * 6 + q - 1];
@@ -271,7 +271,8 @@ cudaError_t launch_limb_factors(Plan &pl, bool adjoint, const double2 *fac, Digi
   return cudaGetLastError();
 }
 
-cudaError_t launch_limb_state(Plan &pl, bool adjoint, const double2 *sin, int B, unsigned *counter, cudaStream_t st) {
+cudaError_t launch_limb_state(Plan &pl, bool adjoint, const double2 *sin, bool by_state, int B, unsigned *counter,
+                              cudaStream_t st) {
   StateArgs s;
   s.sin = sin;
   s.sys = pl.sys_dev;
@@ -280,6 +281,8 @@ cudaError_t launch_limb_state(Plan &pl, bool adjoint, const double2 *sin, int B,
   s.uexp = reinterpret_cast<int *>(pl.dig_state + (size_t)pl.nrows * B * 4 * sizeof(int4));
   s.counter = counter;
   s.nspec = pl.nspec;
+  s.place = by_state ? 1 : B;
+  s.state = by_state ? 3 * pl.nspec : 1;
   s.B = B;
   s.N = pl.N;
   limb_state_kernel<<<dim3((unsigned)((pl.lmax * B * 4 + 255) / 256), (unsigned)pl.sys.size()), 256, 0, st>>>(s);

@@ -229,3 +229,18 @@ def test_the_adjoints_factors_wait_for_a_batch_that_they_serve(env):
         assert fieldwise(plan.step_adjoint(x[:1]).cpu().numpy(), want[:1]) < ORDER
         plan.close()
     slots.close()
+
+
+@pytest.mark.parametrize("N,P,B", [(1, 1, 1), (3, 26, 1), (8, 45, 2), (21, 31, 3), (31, 149, 4), (42, 65, 5)])
+def test_small_batches_are_stepped_in_the_callers_layout(env, N, P, B):
+    """No transposes around the limb solve, and the bits of the step that has them (rexi_integrate)."""
+    torch, rexi = env
+    al, be = poles(P)
+    plan = spectral_plan(rexi, N, B, al, be)
+    x = torch.from_numpy(inputs.random_spectral(N, B, 19)).cuda()
+    plan.profile_enable(1)
+    y = plan.step(x).cpu().numpy()
+    st, _ = plan.profile_read()
+    assert st["transpose_in"] == 0.0 and st["transpose_out"] == 0.0
+    np.testing.assert_array_equal(y, plan.integrate(x, 1).cpu().numpy())
+    plan.close()
