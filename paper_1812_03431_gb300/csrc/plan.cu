@@ -109,6 +109,10 @@ constexpr int kDigitMinBatch = 5;
 // 0.067).  Two states: 4.4 / 4.1 ms at T341.
 constexpr int kDigitMinBatchLarge = 3;
 constexpr int64_t kDigitLarge = 400000;
+// Up to this truncation the FP64 Legendre kernels are the faster ones at any batch, with the FFT and in a
+// graph (FP64 / digits): T1 x 1 analysis 8.3 / 10.3 us, synthesis 8.9 / 12.4; T3 x 16 10.4 / 11.9, 11.6 / 13.9; T5 x
+// 2 11.4 / 11.4, 12.6 / 13.6, x 64 synthesis 27.8 / 31.2.  T8 x 2 13.9 / 11.9, 15.2 / 13.4.
+constexpr int kTinyTruncation = 5;
 constexpr size_t kDigitMostBytes = (size_t)32 << 30;
 
 // Whether a form that a plan can do without may take `need` bytes: a third of what is free, and
@@ -477,7 +481,7 @@ rexi_status build_plan(const rexi_params &prm, Plan *pl) {
       pl->partial_elems = sums;
     }
   }
-  if (prm.precision != REXI_MIXED && spare_memory(legendre_digit_bytes(*pl), 0)) {
+  if (prm.precision != REXI_MIXED && N > kTinyTruncation && spare_memory(legendre_digit_bytes(*pl), 0)) {
     // the Legendre tables as digits, in place of the binary64 ones where both directions fit
     if ((e = build_legendre_digits(*pl, false, pl->leg_ana))) return fail("Legendre digits", e);
     if (pl->leg_ana.dig && (e = build_legendre_digits(*pl, true, pl->leg_syn))) return fail("Legendre digits", e);
