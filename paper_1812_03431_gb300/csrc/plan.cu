@@ -109,6 +109,11 @@ constexpr int kDigitMinBatch = 5;
 // 0.067).  Two states: 4.4 / 4.1 ms at T341.
 constexpr int kDigitMinBatchLarge = 3;
 constexpr int64_t kDigitLarge = 400000;
+// Grid plans of few rows per system keep the fused solve, one launch to the limbs' three: up to two rows
+// (T4) at up to four states, up to four (T8) at one.  Steps in a row, us, fused / limbs: T3 x 1 to 4 38.8 to
+// 42.8 / 46.1 to 47.7 (replayed in a graph 31.2 / 31.3), T5 x 1 44.0 / 46.1, T6 x 1 46.2 / 49.2, T8 x 1 mixed
+// 43.2 / 45.7; past the lines T5 x 2 46.3 / 46.1, T8 x 2 54.5 / 49.9, T10 x 1 56.3 / 50.1.
+constexpr int kFewRows = 2, kFewRowsOne = 4;
 // Up to this truncation the FP64 Legendre kernels are the faster ones at any batch, with the FFT and in a
 // graph (FP64 / digits): T1 x 1 analysis 8.3 / 10.3 us, synthesis 8.9 / 12.4; T3 x 16 10.4 / 11.9, 11.6 / 13.9; T5 x
 // 2 11.4 / 11.4, 12.6 / 13.6, x 64 synthesis 27.8 / 31.2.  T8 x 2 13.9 / 11.9, 15.2 / 13.4.
@@ -641,7 +646,9 @@ bool digits_chosen(const Plan &pl, int B) {
   if (!pl.dig_fwd.fwd) return false;
   auto ud = pl.use_digits.find(B);
   if (ud != pl.use_digits.end()) return ud->second;
-  const int least = pl.limbs ? 1 : (pl.nrows * pl.P >= kDigitLarge ? kDigitMinBatchLarge : kDigitMinBatch);
+  const bool grid = pl.prm.layout == REXI_GRID;
+  const int least = pl.limbs ? (grid && pl.lmax <= kFewRows ? kFusedDefaultMaxBatch + 1 : grid && pl.lmax <= kFewRowsOne ? 2 : 1)
+                             : (pl.nrows * pl.P >= kDigitLarge ? kDigitMinBatchLarge : kDigitMinBatch);
   return pl.slots_override <= 0 && B >= least;
 }
 

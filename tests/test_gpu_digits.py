@@ -244,3 +244,18 @@ def test_small_batches_are_stepped_in_the_callers_layout(env, N, P, B):
     assert st["transpose_in"] == 0.0 and st["transpose_out"] == 0.0
     np.testing.assert_array_equal(y, plan.integrate(x, 1).cpu().numpy())
     plan.close()
+
+
+@pytest.mark.parametrize("N", [4, 5, 8, 9])
+@pytest.mark.parametrize("B", [1, 2, 4, 5])
+def test_grid_steps_of_few_rows(env, N, B):
+    """On both sides of the lines below which grid plans keep the fused solve."""
+    torch, rexi = env
+    al, be = poles(45)
+    make = lambda **k: rexi.Plan(N, 12, 24, tau=1800.0, max_batch=B, alpha=al, beta=be, **k)  # noqa: E731
+    plan, slots = make(), make(pole_slots=2)
+    x = torch.from_numpy(inputs.random_grid(B, 12, 24, 3)).cuda()
+    for f, g in ((plan.step, slots.step), (plan.step_adjoint, slots.step_adjoint)):
+        assert fieldwise(f(x).cpu().numpy(), g(x).cpu().numpy()) < ORDER
+    plan.close()
+    slots.close()
