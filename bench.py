@@ -173,6 +173,7 @@ def kernel_rooflines(form, stages, slots, sm_mhz, solve_arith="fp64", fp64_peak=
         # by the FP64 issue rate (ncu: FP64 pipe 82 %, DRAM 47 %), where an add costs an FMA's slot
         if shape == 5:  # the slots' partial sums of four streams per row, read once
             put("reduce", "hbm", slots * 64.0 * rows_of(N) * ((B + 7) // 8 * 8) + 2 * spec_b, "GB/s", hbm, src + " HBM copy")
+            put("sums", "hbm", (slots & 0xffff) * 64.0 * rows_of(N) * B + 2 * spec_b, "GB/s", hbm, src + " HBM copy")
         else:
             put("reduce", "alu", 2.0 * slots * 3 * ns * B, "TFLOP/s", fp64 / 2, fp64_src + " (adds: half)")
     return out
@@ -593,6 +594,7 @@ def main():
     r = results[chosen]
     P = 2 * (W["M"] + 11) + 1
     solve_ms = r["stages"]["solve"]
+    sums_ms = r["stages"].get("reduce", 0.0) + r["stages"].get("sums", 0.0)  # one or the other
     sm_mhz = (r["clocks"] or {}).get("sm_max_mhz") or 2070.0
     if r["solve_arith"] == "fp32x2":
         amount, peak = FF_OPS_PER_ROW * B * P * rows_of(W["N"]), fp32_peak_tops(sm_mhz)
@@ -634,11 +636,10 @@ def main():
         "form at stated error" % (W["N"], W["M"], B, "s" if B > 1 else "")
     if not default_workload:
         traffic = None  # the captured traffic is for 16 states; it does not scale by rows alone
-    # one kernel per timed stage, plus the state kernels of the float-float and the fixed-point
-    # solve, and the latter's sum of the slots where it is timed with the solve
+    # one kernel per timed stage, plus the state kernels of the float-float and the fixed-point solve
     launches = sum(1 for v in r["stages"].values() if v > 0) + (1 if r["solve_arith"] == "fp32x2" else 0)
     if r["shape"] == 5:
-        launches += 1 if r["stages"].get("reduce", 0.0) > 0 else 2
+        launches += 1
     sharded = args.shard == "poles" and world > 1
     jobs = 1 if sharded else world  # replicas each step a batch; shards step one batch together
     cfg = workload_config()
@@ -663,9 +664,9 @@ def main():
                      "peak_source": peak_source, "algorithmic_per_launch": amount, "launch_ms": solve_ms},
         # the whole S4 stage (banded solves and the complete pole sum): the fused solve's time
         # alone, or the slot kernel's plus its reduction -- the two paths compared like for like
-        "solve_stage": {"ms": solve_ms + r["stages"].get("reduce", 0.0),
-                        "achieved": amount / ((solve_ms + r["stages"].get("reduce", 0.0)) * 1e-3) / 1e12,
-                        "frac": amount / ((solve_ms + r["stages"].get("reduce", 0.0)) * 1e-3) / 1e12 / peak,
+        "solve_stage": {"ms": solve_ms + sums_ms,
+                        "achieved": amount / ((solve_ms + sums_ms) * 1e-3) / 1e12,
+                        "frac": amount / ((solve_ms + sums_ms) * 1e-3) / 1e12 / peak,
                         "unit": roof_unit, "kernels": "solve_fused_kernel" if fused else
                         "state, sweep and finishing kernel" if r["shape"] == 5 else "solve_kernel + reduce_kernel"},
         "fp64_peak": {"tflops": fp64_tf, "ms": fp64_ms, "clocks": fp64_clocks,

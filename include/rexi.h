@@ -341,9 +341,9 @@ void rexi_ragged_destroy(rexi_ragged *rg);
 /* Optional per-stage timing (no counterpart in the paper): with max_calls > 0 the next max_calls calls of
  * rexi_step / rexi_step_adjoint record CUDA events on their stream around each
  * stage (0 FFT forward, 1 Legendre analysis, 2 banded solve + pole sum,
- * 3 slot reduction (zero with the fused solve, which has none, and in plans of up to five
- * states, which count it with the solve), 4 Legendre
- * synthesis, 5 FFT inverse, 6/7 layout transposes).  max_calls = 0 turns it off.  rexi_profile_read waits for the
+ * 3 slot reduction (zero with the fused solve, which has none), 4 Legendre
+ * synthesis, 5 FFT inverse, 6/7 layout transposes, 8 the sum of the slots after the limb solves
+ * of plans of up to five states; larger plans' is stage 3).  max_calls = 0 turns it off.  rexi_profile_read waits for the
  * recorded events, writes the summed milliseconds per stage to stage_ms[0..n)
  * and the number of timed calls to *calls, and restarts the count. */
 rexi_status rexi_profile_enable(rexi_plan *plan, int32_t max_calls);

@@ -42,7 +42,7 @@ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 // Stage boundaries of one call: NVTX ranges (a host-side timeline for profilers; no cost
 // without one attached) and, when rexi_profile_enable is on, CUDA events on the stream.
 const char *const kStageNames[kStages] = {"fft_fwd", "leg_ana", "solve", "reduce",
-                                          "leg_syn", "fft_inv", "transpose_in", "transpose_out"};
+                                          "leg_syn", "fft_inv", "transpose_in", "transpose_out", "sums"};
 
 struct Marks {
   Plan &pl;
@@ -146,7 +146,7 @@ rexi_status fixed_core(Plan &pl, const DigitLayout &dl, int B, bool adjoint, con
   mk.mark(ST_SOLVE);
   cudaError_t e = launch_solve_digits(pl, dl, adjoint, sin, by_state, B, st);
   if (e != cudaSuccess) return cuda_fail("fixed-point solve", e);
-  if (!pl.limbs) mk.mark(ST_REDUCE);  // small batches count it with the solve
+  mk.mark(pl.limbs ? ST_SUMS : ST_REDUCE);
   e = launch_finish_digits(pl, dl, adjoint, sin, sout, by_state, B, st);
   return e == cudaSuccess ? REXI_OK : cuda_fail("fixed-point sums", e);
 }

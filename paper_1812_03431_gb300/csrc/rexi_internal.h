@@ -299,7 +299,7 @@ struct Plan {
 inline int fac_ncomp(const Plan &pl) { return pl.ff ? F_NCOMPACT : F_NCOMP; }
 
 enum Stage { ST_FFT_FWD = 0, ST_LEG_ANA, ST_SOLVE, ST_REDUCE, ST_LEG_SYN, ST_FFT_INV, ST_TRANS_IN,
-             ST_TRANS_OUT, kStages };
+             ST_TRANS_OUT, ST_SUMS, kStages };
 
 // ---- kernels (launchers) ------------------------------------------------------------
 cudaError_t launch_factor_setup(Plan &pl, bool adjoint, cudaStream_t st);

@@ -357,15 +357,16 @@ class Plan:
         error word from the host, for tests of check_device."""
         _check("rexi_inject_device_error", load().rexi_inject_device_error(self._h, int(bits)))
 
-    STAGES = ["fft_fwd", "leg_ana", "solve", "reduce", "leg_syn", "fft_inv", "transpose_in", "transpose_out"]
+    STAGES = ["fft_fwd", "leg_ana", "solve", "reduce", "leg_syn", "fft_inv", "transpose_in", "transpose_out",
+              "sums"]
 
     def profile_enable(self, max_calls):
         _check("rexi_profile_enable", load().rexi_profile_enable(self._h, max_calls))
 
     def profile_read(self):
-        ms = np.zeros(8)
+        ms = np.zeros(len(self.STAGES))
         n = _I32()
-        _check("rexi_profile_read", load().rexi_profile_read(self._h, ms.ctypes.data_as(_DP), 8, ctypes.byref(n)))
+        _check("rexi_profile_read", load().rexi_profile_read(self._h, ms.ctypes.data_as(_DP), ms.size, ctypes.byref(n)))
         return dict(zip(self.STAGES, ms.tolist())), n.value
 
     def close(self):

@@ -259,3 +259,20 @@ def test_grid_steps_of_few_rows(env, N, B):
         assert fieldwise(f(x).cpu().numpy(), g(x).cpu().numpy()) < ORDER
     plan.close()
     slots.close()
+
+
+@pytest.mark.parametrize("layout", ["spectral", "grid"])
+def test_every_kernel_of_a_limb_step_has_its_stage(env, layout):
+    """Up to five states the default is the limb solve, whose slots a second kernel sums."""
+    torch, rexi = env
+    N, B = 31, 4
+    plan = rexi.Plan(N, 48, 96, M=32, max_batch=B, layout=layout)
+    assert plan.info()["fixed_factors"] == 1
+    S = torch.from_numpy(inputs.random_spectral(N, B, 9)).cuda()
+    x = S if layout == "spectral" else plan.synthesize(S)
+    plan.profile_enable(1)
+    plan.step(x)
+    st, n = plan.profile_read()
+    ran = {"spectral": {"solve", "sums"}, "grid": {"fft_fwd", "leg_ana", "solve", "sums", "leg_syn", "fft_inv"}}[layout]
+    assert n == 1 and {k for k, v in st.items() if v > 0} == ran
+    plan.close()
