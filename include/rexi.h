@@ -304,7 +304,7 @@ rexi_status rexi_set_pole_slots(rexi_plan *plan, int32_t batch, int32_t slots, i
 
 /* Host-side description of a plan (no counterpart in the paper): writes up to 9 int64 values
  * {N, nspec, P, nlat, nlon, max_batch, pole_slots, device bytes held, fixed-point factors};
- * pole_slots is that of steps with max_batch states, 0 when they use the fused solve; the last
+ * pole_slots is that of steps with max_batch states, 0 when they use the fixed-point or the fused solve; the last
  * value is 0 where the plan has no factors for the fixed-point solve (shape 5 of
  * rexi_set_pole_slots is REXI_EINVAL), 1 for integer limbs, 2 for tensor-core digits. */
 rexi_status rexi_plan_info(const rexi_plan *plan, int64_t *info, int32_t n);

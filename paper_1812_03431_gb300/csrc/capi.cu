@@ -534,10 +534,11 @@ rexi_status rexi_set_pole_slots(rexi_plan *plan, int32_t batch, int32_t slots, i
 rexi_status rexi_plan_info(const rexi_plan *plan, int64_t *info, int32_t n) {
   if (!plan || !plan->pl || !info) { set_error("null argument"); return REXI_EINVAL; }
   const Plan &pl = *plan->pl;
-  int slots = 0;  // 0 when steps of max_batch states use the fused solve (no slot partials)
+  int slots = 0;  // 0 when steps of max_batch states use the fixed-point or the fused solve
   auto it = pl.layouts.find(pl.prm.max_batch);
   auto us = pl.use_slots.find(pl.prm.max_batch);
-  if (it != pl.layouts.end() && us != pl.use_slots.end() && us->second) slots = it->second.slots;
+  if (it != pl.layouts.end() && us != pl.use_slots.end() && us->second && !digits_chosen(pl, pl.prm.max_batch))
+    slots = it->second.slots;
   const int fixed = !pl.dig_fwd.fwd ? 0 : (pl.limbs ? 1 : 2);
   const int64_t v[9] = {pl.N, pl.nspec, pl.P, pl.nlat, pl.nlon, pl.prm.max_batch, slots, (int64_t)pl.bytes, fixed};
   for (int i = 0; i < n && i < 9; ++i) info[i] = v[i];

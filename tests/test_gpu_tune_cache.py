@@ -63,3 +63,14 @@ def test_an_entry_that_the_plan_refuses_is_a_miss(rexi, tmp_path):
     plan.tune(B, cache=str(cache))
     assert json.loads(cache.read_text())[key][1] != 5
     plan.close()
+
+
+@pytest.mark.parametrize("max_batch", [3, 8])
+def test_pole_slots_are_those_of_the_solve_in_use(rexi, max_batch):
+    """A slot layout chosen earlier is not reported once the fixed-point solve has been."""
+    plan = plan_of(rexi, *alike(), max_batch)
+    used = plan.set_pole_slots(max_batch, 4, 0)
+    assert plan.info()["pole_slots"] == used > 0
+    plan.set_pole_slots(max_batch, 0, 5)
+    assert plan.info()["pole_slots"] == 0
+    plan.close()
