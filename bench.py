@@ -103,11 +103,15 @@ def measured_peaks():
 
 
 def solve_layout(r):
-    """The tuned solve layout of a form's record: pole slots and shape, or for the fused
-    solve (shapes 2 to 4) its form, CTA tile and the CTAs that split each tile's poles."""
+    """The tuned solve layout of a form's record: pole slots and shape, for the fused
+    solve (shapes 2 to 4) its form, CTA tile and the CTAs that split each tile's poles, for the
+    fixed-point solve (shape 5) its kind."""
     if r["shape"] in (2, 3, 4):
         return {"fused": {2: "register", 3: "lean", 4: "lean, two-warp CTAs"}[r["shape"]],
                 "tile": r["slots"] % 256, "pole_groups": r["slots"] // 256, "layout_shape": r["shape"]}
+    if r["shape"] == 5 and r["slots"] >> 16:  # limbs: 65536 x the packing
+        return {"limbs": {1: "one pole per lane", 2: "two poles per lane", 3: "one pole per lane, a block per window"}[
+            r["slots"] >> 16], "pole_slots": r["slots"] & 0xffff, "layout_shape": 5}
     if r["shape"] == 5:
         return {"digits": "contractions on the tensor cores", "pole_slots": r["slots"], "layout_shape": 5}
     return {"pole_slots": r["slots"], "layout_shape": r["shape"]}

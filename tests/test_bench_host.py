@@ -57,3 +57,12 @@ def test_solve_layout_and_kernel_rooflines():
     # the mixed FFT moves the FP64 grid and the FP32 Fourier array once each
     assert k["fft_fwd"]["algorithmic"] == 16 * 3 * 512 * 1024 * 8 + 512 * 342 * 48 * 8
     assert "reduce" not in k and "leg_ana" not in k  # stages without a time are left out
+
+
+def test_solve_layout_of_the_fixed_point_solves():
+    import bench
+    assert bench.solve_layout({"slots": 6, "shape": 5}) == {
+        "digits": "contractions on the tensor cores", "pole_slots": 6, "layout_shape": 5}
+    limbs = [bench.solve_layout({"slots": 65536 * k + 9, "shape": 5}) for k in (1, 2, 3)]
+    assert all(v["pole_slots"] == 9 and "digits" not in v for v in limbs)
+    assert len({v["limbs"] for v in limbs}) == 3
