@@ -7,17 +7,20 @@ namespace rexi {
 
 // a / d as the product by 1/d, corrected by its remainder (Markstein, IBM J. Res. Dev. 34, 1990: with
 // 1/d correctly rounded the corrected quotient is), three FP64 instructions each after the one
-// division.  Divisors whose reciprocal or remainders leave the normal range are divided by.
+// division.  Where the reciprocal, the quotient or the remainder could leave the normal range (biased
+// exponents outside [200, 1800], or a's and d's more than 900 apart), a is divided.
 struct Recip {
   double d, r;
-  bool plain;
+  int least, most;  // exponents of a for the product
   __device__ __forceinline__ explicit Recip(double d_) : d(d_), r(1.0 / d_) {
     const int e = (__double2hiint(d_) >> 20) & 0x7ff;
-    plain = e < 200 || e > 1800;
+    const bool plain = e < 200 || e > 1800;
+    least = plain ? 2048 : (e > 1100 ? e - 900 : 200);
+    most = e < 900 ? e + 900 : 1800;
   }
   __device__ __forceinline__ double of(double a) const {
     const int e = (__double2hiint(a) >> 20) & 0x7ff;
-    if (plain || e < 200 || e > 1800) return a / d;
+    if (e < least || e > most) return a / d;
     const double q = a * r;
     return fma(fma(-q, d, a), r, q);
   }
