@@ -192,3 +192,70 @@ def test_autotuner_keeps_results(env):
     sel = np.concatenate([np.arange(idx(m, m, N), idx(m, N, N) + 1) for m in [0, 5, 64, 127]])
     assert max(rel(after[0, f, sel], ref[0, f, sel]) for f in range(3)) < TOL
     plan.close()
+
+
+def unlike(n=45):
+    """Poles whose couplings differ by more than the fixed-point factors cover."""
+    k = np.arange(n)
+    return -(2.0 ** (k % 3 * 10.0 - 10.0)) + 1j * k, np.full(n, 1.0 / n) + 0j
+
+
+@pytest.mark.parametrize("case", ["few states of large plans", "poles of unlike scale", "one plan of them"])
+def test_ragged_without_the_fixed_point_solves(env, case):
+    """The fused launch over every plan's items: one or two states of plans for eight, whose digit tiles would
+    be mostly padding, and plans that have no fixed-point factors."""
+    torch, rexi = env
+    Ns, max_batch = (42, 63, 21), 8 if case.startswith("few") else 3
+    plans = []
+    for i, N in enumerate(Ns):
+        al, be, _ = rc.rexi_coefficients(32, 0.2)
+        if case == "poles of unlike scale" or (case == "one plan of them" and i == 1):
+            al, be = unlike()
+        plans.append(rexi.Plan(N, 96, 192, tau=1200.0, max_batch=max_batch, layout="spectral", alpha=al, beta=be))
+    assert [p.info()["fixed_factors"] for p in plans] == {"few states of large plans": [2, 2, 2], "poles of unlike scale": [0, 0, 0],
+                                                          "one plan of them": [1, 0, 1]}[case]
+    rg = rexi.Ragged(plans, 5)
+    for state_plan in ([0, 1, 2, 1, 0], [1], [2, 1]):
+        states = [torch.from_numpy(inputs.random_spectral(Ns[p], 1, 5000 + s)[0]).cuda() for s, p in enumerate(state_plan)]
+        outs = [torch.empty_like(x) for x in states]
+        rg.step(states, outs, state_plan)
+        torch.cuda.synchronize()
+        for p, plan in enumerate(plans):
+            idx = [s for s in range(len(state_plan)) if state_plan[s] == p]
+            if not idx:
+                continue
+            Y = plan.step(torch.stack([states[s] for s in idx])).cpu().numpy()
+            for r, s in enumerate(idx):
+                assert rel(outs[s].cpu().numpy(), Y[r]) < 1e-13
+    rg.close()
+    for plan in plans:
+        plan.close()
+
+
+@pytest.mark.parametrize("layout,B", [("grid", 9), ("spectral", 9), ("spectral", 3)])
+@pytest.mark.parametrize("adjoint", [False, True])
+def test_fixed_point_steps_in_cuda_graph(env, layout, B, adjoint):
+    """The digit solve's and the limb solve's kernels (the work counter is reset by one of them)."""
+    torch, rexi = env
+    N = 42
+    plan = rexi.Plan(N, 64, 128, M=32, tau=1200.0, max_batch=B, layout=layout)
+    assert plan.info()["fixed_factors"] == (2 if B > 5 else 1)
+    S = torch.from_numpy(inputs.random_spectral(N, B, 5)).cuda()
+    x = S if layout == "spectral" else plan.synthesize(S)
+    y = torch.empty_like(x)
+    f = plan.step_adjoint if adjoint else plan.step
+    eager = f(x, out=y).clone()  # the first call with this batch builds the work list
+    g = torch.cuda.CUDAGraph()
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        f(x, out=y)
+    torch.cuda.current_stream().wait_stream(side)
+    with torch.cuda.graph(g):
+        f(x, out=y)
+    for _ in range(2):
+        y.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(y, eager)
+    plan.close()
