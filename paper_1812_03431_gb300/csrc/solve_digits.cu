@@ -285,22 +285,23 @@ struct FinishArgs {
   double2 sphi;
   int64_t nspec, nrows;
   const double *scale;  // limbs: per row the sums' real factors at 3..5 (see solve_limbs.cu), else null
-  bool by_state;        // sin, sout: [B][3][nspec], else [3][nspec][B]
   int B, tile, tiles, unit, sstr, pstr, slots, N;
 };
 
 // SPLIT threads per output, each over every SPLIT-th slot: one where the outputs fill the chip (HBM
 // bounds it: T341 x 16 with 8 slots 0.123 to 0.131 ms, 0.137 without four slots' loads in flight), four where
 // they are few and the slots many (T85 x 5 with 27 20 / 31 us, T42 x 8 with 19 12 / 16 us).
-template <int SPLIT>
+// BY_STATE: sin and sout are [B][3][nspec], else [3][nspec][B] (a kernel of its own: chosen at run time it
+// cost every step 0.7 us at T170 x 1).
+template <int SPLIT, bool BY_STATE>
 __global__ void digit_finish_kernel(FinishArgs a) {
   const int64_t total = 3 * a.nspec * a.B, slot = a.nrows * a.tiles * a.unit, step = slot * SPLIT;
   const int first = threadIdx.x % SPLIT;
   for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / SPLIT; t < total;
        t += (int64_t)gridDim.x * blockDim.x / SPLIT) {
-    const int64_t inner = a.by_state ? 3 * a.nspec : a.B, outer = t / inner, rest = t - outer * inner;
-    const int b = (int)(a.by_state ? outer : rest);
-    const int64_t fi = a.by_state ? rest : outer;
+    const int64_t per = BY_STATE ? 3 * a.nspec : a.B;
+    const int b = (int)(BY_STATE ? t / per : t % per);
+    const int64_t fi = BY_STATE ? t % per : t / per;
     const int f = (int)(fi / a.nspec);
     const int64_t ix = fi - (int64_t)f * a.nspec;
     const uint8_t fl = a.rflags[fi];
@@ -571,7 +572,6 @@ cudaError_t launch_finish_digits(Plan &pl, const DigitLayout &L, bool adjoint, c
   f.sphi = adjoint ? pl.sphi_adj : pl.sphi_fwd;
   f.nspec = pl.nspec;
   f.nrows = pl.nrows;
-  f.by_state = by_state;
   f.B = B;
   f.tile = pl.limbs ? 1 : kTile;
   f.tiles = pl.limbs ? B : tiles_of(pl, B);
@@ -583,8 +583,9 @@ cudaError_t launch_finish_digits(Plan &pl, const DigitLayout &L, bool adjoint, c
   f.N = pl.N;
   const int64_t total = 3 * pl.nspec * B;
   const int split = L.slots >= 8 && total <= 2048 * (int64_t)pl.num_sms ? 4 : 1;
-  (split > 1 ? digit_finish_kernel<4> : digit_finish_kernel<1>)<<<
-      (unsigned)std::min<int64_t>((total * split + 255) / 256, 1 << 20), 256, 0, st>>>(f);
+  auto k = by_state ? (split > 1 ? digit_finish_kernel<4, true> : digit_finish_kernel<1, true>)
+                    : (split > 1 ? digit_finish_kernel<4, false> : digit_finish_kernel<1, false>);
+  k<<<(unsigned)std::min<int64_t>((total * split + 255) / 256, 1 << 20), 256, 0, st>>>(f);
   return cudaGetLastError();
 }
 
