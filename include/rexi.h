@@ -31,6 +31,9 @@
  *   south (mu_j = sin(lat_j) are the Gauss-Legendre nodes, descending),
  *   longitude lambda_i = 2 pi i / nlon.  Robert's cos(lat) scaling (Sec. 3) is
  *   applied inside.
+ * Range: the fixed-point forms (the default solve of binary64 plans, and the transforms of REXI_FP64) scale
+ *   each group of numbers by its largest.  Subnormal numbers, and what is below 2^-61 of its group's
+ *   largest or below 2^-959, count as zero in them; magnitudes should stay below 2^1000.
  * Device pointers: every in/out pointer below named *_dev is a device pointer
  *   to caller-owned, contiguous, 16-byte aligned memory; in and out must not
  *   overlap (REXI_EINVAL).  The plan owns every other allocation.
@@ -126,9 +129,12 @@ typedef struct {
                            rexi_set_pole_slots) where its factors fit (68 to 156 B of device
                            memory per row and pole, at most 32 GiB and a third of what is
                            free when the plan's workspaces, or for the adjoint its binary64
-                           factors, are allocated) and the poles are of like scale, except for batches of one and
+                           factors, are allocated) and the poles are of like scale (couplings
+                           within eight bits of each other: with the computed poles M up to some
+                           1150, in plans of up to five states 1270), except for batches of one and
                            two (below 400,000 rows times poles: up to four) states in plans
-                           with max_batch >= 6; else for up to four
+                           with max_batch >= 6, and grid plans up to T4 with up to four states and up
+                           to T8 with one; else for up to four
                            states the fused solve that keeps the pole sum on chip (one
                            kernel, every output written once), else the pole-slot solve
                            (rexi_tune picks per batch); > 0: the pole-slot solve with this
@@ -310,13 +316,13 @@ rexi_status rexi_set_pole_slots(rexi_plan *plan, int32_t batch, int32_t slots, i
 rexi_status rexi_plan_info(const rexi_plan *plan, int64_t *info, int32_t n);
 
 /* Ragged batches (mixed truncations and pole counts): the banded solves of
- * every state of several plans run as ONE persistent launch over the merged
+ * every state of several plans run in persistent launches over a merged
  * work list of every plan's items sorted longest first (Sec. 5: every (pole, m)
  * system is independent).  With binary64 solves each plan's fixed-point solve (shape 5 of
  * rexi_set_pole_slots) runs where every plan has one and the states fill its tiles well
  * enough: one launch for the plans of six states and more and one for the smaller ones, each
  * plan's inputs prepared before them and its sums put together after them by small kernels.
- * Else the launch is the fused solve:
+ * Else one launch of the fused solve:
  * items are (system, tile of 2 states, plan), the pole sum stays on chip and no
  * reduction follows, provided the largest plan's running sums leave seven CTAs of two
  * warps, or three of four warps, per SM.  Otherwise (and with float-float solves) it is the pole-slot solve over

@@ -44,7 +44,7 @@ __device__ __forceinline__ int fdiv(int x, uint32_t mag, int d) { return d == 1 
 __device__ __forceinline__ void mad_wide(long long &acc, int a, int b) {
   asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
 }
-// acc (hi sums, rounded middle sums) += v t for a limb pair t, |v| < 2^60
+// acc (hi sums, rounded middle sums) += v t for a limb pair t, |v| < 2^61 (4 sqrt(2) 2^kTop in radix 8)
 struct Acc {
   long long hh = 0, hl = 1 << 29;
   __device__ __forceinline__ void add(int2 v, int2 t) {

@@ -10,7 +10,9 @@ namespace rexi {
 namespace fixed {
 
 constexpr int kNotFinite = 1 << 20;  // exponent of a group that holds an Inf or NaN
-constexpr int kMaxSpread = 8;        // bits by which a pole's couplings may differ in scale
+// Bits by which a pole's couplings may differ in scale from the middle pole's, and reciprocals of the
+// shifts from the largest: |alpha| up to some 2^8.
+constexpr int kMaxSpread = 8;
 
 __device__ __forceinline__ int bexp(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 

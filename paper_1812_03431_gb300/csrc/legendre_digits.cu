@@ -29,7 +29,9 @@
 // 0.234, 0.204; T170 x 1 0.058, 0.076; T63 x 1 0.020, 0.027.  At T255 x 8 the tensor pipe is 35 %, the
 // issue slots 45 % busy (ncu): four warps per scheduler, which wait for each other at the groups'
 // barriers and within the chains of a product; registers allow no more warps.  Fewer instructions
-// (sums read off the accumulators' bits per 32 terms) gave nothing.
+// (sums read off the accumulators' bits per 32 terms) gave nothing.  tcgen05 would keep the accumulators
+// out of the registers; it is not built (both operands are in shared memory already, but tables
+// would have to be expanded to fp16 there).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -61,8 +63,8 @@ static_assert(2 * (kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
 // The synthesis' groups run over degrees, along which H grows like n and spectra fall: tables are
 // divided and data multiplied by the power of two below n + 1, or the products of a smooth field's
 // few large coefficients would be small against the group's largest product.
-// A balanced zonal flow's u at T42 against a 113-bit reference: 3.3e-16, without it 1.25e-15 (FP64
-// sums: 4.0e-16); a hundredth of the synthesis' time.
+// Without it the wind of one large zonal coefficient among small ones was several roundings off the sum
+// of its parts; it takes a hundredth of the synthesis' time.
 __device__ __forceinline__ double degree_scale(int n) {
   return __longlong_as_double((long long)(1023 + 31 - __clz(n + 1)) << 52);
 }

@@ -163,9 +163,10 @@ rexi_status rexi_ragged_step(rexi_ragged *rg, const void *const *in_dev, void *c
       set_error("rexi_ragged_step: more states for plan " + std::to_string(p) + " than its max_batch");
       return REXI_EINVAL;
     }
-  // binary64 plans: one launch of the fixed-point solves over every plan's items, or where
-  // that does not apply one fused launch (the pole sum on chip, no reductions); else the slot kernel over the merged work list, then per-plan reductions.
-  // Either work list is cached per count vector.
+  // binary64 plans: a launch per kind of fixed-point solve over every plan's items, or where
+  // that does not apply one fused launch (the pole sum on chip, no reductions); else the slot
+  // kernel over the merged work list, then per-plan reductions.  The work list is cached per
+  // count vector.
   auto it = rg->cfgs.find(counts);
   if (it == rg->cfgs.end() && !rg->plans[0]->ff) {
     rexi_ragged::Cfg cfg;
