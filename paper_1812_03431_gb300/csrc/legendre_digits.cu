@@ -587,21 +587,22 @@ cudaError_t build_legendre_digits(Plan &pl, bool synthesis, LegendreDigits &t) {
 }
 
 namespace {
-// One state per CTA in place of four: a batch of one, and batches whose CTAs then still find their
-// places at once (two per SM), where a CTA's chain of two products in place of five is what counts.
-// Analysis, synthesis with the FFT, us, one / four states per CTA: T21 x 2 13.8 / 19.9, 14.6 / 24.5 (of
-// the FP64 kernels: 18.5, 22.0); T63 x 4 (256 CTAs) 20.8 / 26.0, 22.5 / 32.7; T24 x 12 (300) 19.2 / 24.0,
-// 22.0 / 29.7; past the line T24 x 16 (400) 27.1 / 25.7, 30.4 / 32.0, T48 x 8 (392) 29.9 / 29.4, 33.7 /
-// 37.2, T127 x 8 (1024) 91.6 / 73.5, 86.9 / 74.6.
-bool one_state(const Plan &pl, int B, unsigned rows) {
-  return B == 1 || (int64_t)(pl.N + 1) * rows * B <= 2 * pl.num_sms;
+// One state per CTA in place of four: a batch of one, and batches with few CTAs, where a CTA's chain of
+// two products in place of five is what counts: up to two CTAs of one state per SM, which find their
+// places at once, for the analysis, four for the synthesis.  With the FFT, us, one / four states per CTA:
+// analysis T21 x 2 13.8 / 19.9 (FP64 kernels 18.5), T63 x 4 (256 CTAs) 20.8 / 26.0, T24 x 12 (300) 19.2 / 24.0;
+// past the line T28 x 12 (348) 27.8 / 26.6, T24 x 16 (400) 27.1 / 25.7, T127 x 8 (1024) 91.6 / 73.5.
+// Synthesis T21 x 2 14.6 / 24.5 (22.0), T63 x 4 22.5 / 32.7, T48 x 8 (392) 33.7 / 37.2, T85 x 6 (516) 44.0 / 52.7,
+// T48 x 12 (588) 37.2 / 39.0; past the line T42 x 16 (688) 40.5 / 38.9, T63 x 12 (768) 47.6 / 42.9.
+bool one_state(const Plan &pl, int B, unsigned rows, int per_sm) {
+  return B == 1 || (int64_t)(pl.N + 1) * rows * B <= (int64_t)per_sm * pl.num_sms;
 }
 }  // namespace
 
 cudaError_t launch_leg_ana_digits(Plan &pl, const double2 *four, double2 *sint, int B, const double *zd, cudaStream_t st) {
   const int tiles = (pl.N / 2 + 1 + 15) / 16 + ((pl.N + 1) / 2 + 15) / 16;
   const unsigned rows = (unsigned)((tiles + kWarps - 1) / kWarps);
-  const bool one = one_state(pl, B, rows);
+  const bool one = one_state(pl, B, rows, 2);
   const dim3 g((unsigned)(one ? B : (B + 3) / 4), rows, (unsigned)(pl.N + 1));
   (one ? legendre_digits_analysis<true> : legendre_digits_analysis<false>)<<<g, 32 * kWarps, kSmem, st>>>(
       leg_args(pl, pl.leg_ana, four, sint, B, zd));
@@ -610,7 +611,7 @@ cudaError_t launch_leg_ana_digits(Plan &pl, const double2 *four, double2 *sint, 
 
 cudaError_t launch_leg_syn_digits(Plan &pl, const double2 *sint, double2 *four, int B, const double *zd, cudaStream_t st) {
   const unsigned rows = (unsigned)(((pl.J + 15) / 16 + kWarps - 1) / kWarps);
-  const bool one = one_state(pl, B, rows);
+  const bool one = one_state(pl, B, rows, 4);
   const dim3 g((unsigned)(one ? B : (B + 3) / 4), rows, (unsigned)(pl.N + 1));
   (one ? legendre_digits_synthesis<true> : legendre_digits_synthesis<false>)<<<g, 32 * kWarps, kSmem, st>>>(
       leg_args(pl, pl.leg_syn, four, sint, B, zd));

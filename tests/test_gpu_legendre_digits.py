@@ -136,10 +136,13 @@ def test_a_smooth_flow_among_small_coefficients(env, N, nlat, nlon, B):
     plan.close()
 
 
-# batches whose CTAs of one state fill two places per SM (304) or just do not, and the same states fewer at a time
+# batches whose CTAs of one state fill two (304, analysis) or four (608, synthesis) places per SM or just do
+# not, and the same states fewer at a time
 @pytest.mark.parametrize("N,nlat,nlon,B,few", [(1, 2, 4, 153, 152), (2, 4, 8, 103, 7), (15, 32, 48, 20, 3), (16, 36, 48, 18, 17),
                                                (31, 64, 96, 10, 9), (33, 128, 108, 9, 4), (37, 76, 120, 9, 8),
-                                               (66, 132, 200, 5, 2), (127, 192, 384, 3, 2), (130, 132, 400, 3, 2)])
+                                               (66, 132, 200, 5, 2), (127, 192, 384, 3, 2), (130, 132, 400, 3, 2),
+                                               (15, 32, 48, 39, 38), (16, 36, 48, 36, 35), (31, 64, 96, 20, 19), (33, 128, 108, 18, 5),
+                                               (66, 132, 200, 10, 9), (127, 192, 384, 5, 4)])
 def test_one_and_four_states_per_block(env, N, nlat, nlon, B, few):
     """Each product is exact up to 2^-59 of its group and rounded alike in both forms, the sums over the
     groups are in another order (up to four of them)."""
