@@ -97,7 +97,7 @@ void free_plan(Plan *pl);
 // Plans of up to five states use the limb solve, whose time grows with the states, larger ones the
 // digit solve, whose warps carry tiles of eight: T341 x 5 3.93 against 4.41 ms, T170 x 5 1.01 / 1.16, T85 x
 // 5 with 215 poles 0.154 / 0.165, T42 x 5 0.061 / 0.076; with six states T170 1.20 / 1.17, T85 0.195 /
-// 0.167, T42 0.067 / 0.076.
+// 0.167, T42 0.067 / 0.076 (one line for all sizes: only below T85 would a sixth state gain).
 constexpr int kLimbMostBatch = 5;
 // The smallest batch of a larger plan for its digit solve (five states take a quarter of the
 // pole-slot solve's time).  Then the most device memory either's factors may take: 156 and 68 B

@@ -73,7 +73,10 @@ void free_fixed_ragged(FixedRagged &R) {
 // False where a plan has no fixed-point factors, or where the tiles' padding makes the fused
 // solve the cheaper one: per row and pole a digit tile costs about 8 x 12 FP64 FMAs' time
 // whatever its states, limbs 14 per state, the fused solve 39 per state
-// (T170: 8 states 1.25 ms, 4 states 0.80, fused 0.52 per state).
+// (T170: 8 states 1.25 ms, 4 states 0.80, fused 0.52 per state).  Over 170 random calls (one to eight
+// states of one to three plans, T10 to T250, 55 to 535 poles) the choice took 0.10 to 1.06 times the fused
+// launch's time, median 0.28.  Limbs hold two poles per lane here whatever the windows: the launch
+// has every plan's items.
 bool build_fixed_ragged(const std::vector<Plan *> &plans, const std::vector<int> &counts, FixedRagged &R) {
   R = FixedRagged{};
   double fixed_cost = 0, fused_cost = 0, work[9] = {};  // per kind: states per warp
@@ -108,7 +111,7 @@ bool build_fixed_ragged(const std::vector<Plan *> &plans, const std::vector<int>
     R.lmax = std::max(R.lmax, pl.lmax);
   }
   // one kind of sweep after the other, in a launch each, longest first within it: warps that run
-  // different sweeps side by side miss the instruction caches (48 states, T63 to T341: 20.6 ms with
+  // different sweeps side by side miss the instruction caches (48 states, T63 to T341: 19.6 ms with
   // all items longest first), and one kernel that calls both spills in either (12.5 ms;
   // two 11.0)
   std::stable_sort(all.begin(), all.end(), [&](const Tagged &x, const Tagged &y) {
